@@ -419,6 +419,16 @@ constexpr double kRingRecordsPerLane = SKIM_RING_RECORDS_PER_LANE;
 // entries side by side (traverse.cu: table_slot)
 constexpr uint32_t kNodeHashWords = SKIM_NODE_HASH_WORDS;
 
+// Residual searches over materialised rows run as one block per instance
+// (reach.cu) except where few instances are large: a block then walks alone
+// what the global queue spreads over the GPU.  Time of the searches of 30
+// seeds, queue / blocks in ms: R-MAT 20 wc (0.55 M live pairs per instance)
+// 3.8 / 2.5 with l = 1, 9.8 / 5.6 with l = 64; R-MAT 20 p = 0.05 (0.8 M)
+// 1.9 / 5.1 with l = 8, 2.4 / 4.6 with l = 16, 6.6 / 2.6 with l = 64; R-MAT 22
+// p = 0.01 (0.65 M) 1.6 / 3.2 with l = 1, 6.2 / 2.4 with l = 64.
+constexpr uint32_t kReachInst = 32;
+constexpr uint64_t kReachPairs = 600000;
+
 int ensure_idx(skim_ctx *c, uint64_t need);
 
 bool trace_batches() {
@@ -740,12 +750,34 @@ int residual(skim_ctx *c, uint32_t x, uint64_t *cov) {
         cudaEventCreate(&t1);
         cudaEventRecord(t0, c->st);
     }
-    CK(c, launch_fwd_source(a, x, c->st));
-    {
+    if (c->mat && (c->l >= kReachInst || c->live_total <= kReachPairs * c->l)) {
         KTimer kt(c, SKIM_K_FWD);
-        CK(c, launch_traverse(a, true, c->grid_fwd, c->st));
+        ReachArgs r{};
+        r.off = c->foff;
+        r.rows = c->flive;
+        r.l = c->l;
+        r.mask = c->covered;
+        // scratch: the visited table (a SKIM batch's lane bits were gathered
+        // when it was searched), up to the work queue's capacity
+        r.list = reinterpret_cast<uint2 *>(c->hkeys);
+        r.cap = static_cast<uint32_t>(std::min<uint64_t>(std::min(c->hcap, c->qcap) / c->l, c->n));
+        r.pend_trav = c->pend_trav;
+        r.seg_start = c->seg_start;
+        r.seg_len = c->seg_len;
+        r.size = c->size;
+        r.idx_nodes = c->idx;
+        r.chosen = c->chosen;
+        r.ctl = c->ctl;
+        r.timeout_ns = c->timeout_ns;
+        CK(c, launch_reach(r, x, c->st));
+    } else {
+        CK(c, launch_fwd_source(a, x, c->st));
+        {
+            KTimer kt(c, SKIM_K_FWD);
+            CK(c, launch_traverse(a, true, c->grid_fwd, c->st));
+        }
+        CK(c, cudaMemsetAsync(c->chosen + x, 1, 1, c->st));
     }
-    CK(c, cudaMemsetAsync(c->chosen + x, 1, 1, c->st));
     c->pend_res = true;
     c->pend_cov = cov;
     if (trace_batches()) {  // one line per residual search, waited for

@@ -149,6 +149,26 @@ int rev_ring_grid();
 cudaError_t launch_rev_ring(const TravArgs &a, const uint32_t *lane_pair, uint32_t B, uint32_t l,
                             const uint64_t *covered, uint64_t *alive, bool sources, int grid, cudaStream_t s);
 
+// reach.cu: the residual search of seed x over materialised rows, one block per
+// instance (the seed is marked chosen)
+struct ReachArgs {
+    const uint32_t *off;        // row bounds per (v, i) in the search direction
+    const uint32_t *rows;
+    uint32_t l;
+    uint64_t *mask;             // per node: instances in which it has been reached (covered)
+    uint2 *list;                // scratch: 2 * cap entries per instance
+    uint32_t cap;
+    uint64_t *pend_trav;        // per node: instances whose rows did not fit the scratch
+    const uint64_t *seg_start;  // index segment of every pair: first entry, entries
+    uint32_t *seg_len;
+    uint32_t *size;
+    const uint32_t *idx_nodes;
+    uint8_t *chosen;
+    DevCtl *ctl;
+    uint64_t timeout_ns;
+};
+cudaError_t launch_reach(const ReachArgs &a, uint32_t x, cudaStream_t s);
+
 // batch.cu
 cudaError_t launch_lane_inst(const uint32_t *lane_pair, const uint64_t *lane_rank, uint32_t B, uint32_t l,
                              uint8_t *lane_inst, uint64_t *lane_g, cudaStream_t s);
