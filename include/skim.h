@@ -70,8 +70,9 @@ typedef struct {
  *   rank_key   rank of pair (v,i) is fmix(rank_key + (v*l+i)*G), read as
  *              a real in [0,1) after scaling by 2^-64 (ranks never tie);
  *   prob_key   trivalency class of edge (u,v): fmix(prob_key ^ (u<<32|v)) % 3;
- *   batch_lanes  ranks per batched search, 0 = automatic (2M; 4M on graphs of
- *              2^23 nodes or more);
+ *   batch_lanes  ranks per batched search, 0 = automatic (sketch builds over
+ *              materialised instances: up to 16M; otherwise 2M, and 4M on
+ *              graphs of 2^23 nodes or more);
  *   rank_mode  SKIM_RANKS_*: how the pairs are ordered and what a sketch holds.
  *     SKIM_RANKS_UNIFORM (0): the uniform 64-bit ranks above.
  *     SKIM_RANKS_PERMUTATION (1): structured permutation ranks (Section 3.1).
@@ -131,16 +132,19 @@ int skim_autotune_batch_lanes(skim_ctx *ctx, const uint32_t *candidates, uint32_
 
 /* Switches of the rank-batched searches (Algorithms 1 and 2 run a batch of
  * consecutive ranks as one search; none of these changes a result):
- *   batch_lanes            ranks per batch, 0 = automatic (2M, 4M on graphs
- *                          of 2^23 nodes or more, or fewer when the previous
- *                          batch's records per lane say so);
- *   ring_records_per_lane  a batch whose searches are expected to leave at
- *                          most this many visit records per lane (from the
- *                          previous batch) runs with per-warp work queues in
- *                          shared memory; larger searches share one global
- *                          queue over the whole GPU (default 8; 0 = always
- *                          the global queue);
- *   node_sort_density      a batch's visit records are placed by node
+ *   batch_lanes            ranks per batch, 0 = automatic (see skim_params, or
+ *                          fewer when the previous batch's records per lane
+ *                          say so);
+ *   ring_records_per_lane  searches with a global visited table (SKIM's, builds
+ *                          without materialised instances, a build's first
+ *                          batches and the lanes whose search is too large for
+ *                          a warp) that are expected to make at most this many
+ *                          visits per lane (from the previous ones) run with
+ *                          per-warp work queues in shared memory; larger
+ *                          searches share one global queue over the whole GPU
+ *                          (default 8; 0 = always the global queue);
+ *   node_sort_density      SKIM, and builds without materialised instances: a
+ *                          batch's visit records are placed by node
  *                          buckets (a counting pass over buckets of 2^s
  *                          consecutive nodes, s chosen for about one bucket
  *                          per record) when the buckets number at most
@@ -289,9 +293,9 @@ int skim_oracle_query_batch(skim_ctx *ctx, const uint64_t *offsets, uint32_t q,
                             const uint32_t *seeds, double *est_out, int on_device);
 
 /* Counters of the last build / greedy call (see SKIM_STAT_* indices). */
-#define SKIM_STAT_REV_VISITS 0      /* (node, rank) visits of reverse searches */
+#define SKIM_STAT_REV_VISITS 0      /* (node, rank) visits that reverse searches made */
 #define SKIM_STAT_REV_COINS 1       /* coins evaluated by reverse searches */
-#define SKIM_STAT_INSERTIONS 2      /* sketch insertions (build) or commits (greedy) */
+#define SKIM_STAT_INSERTIONS 2      /* ranks entered into sketches (build) or commits (greedy) */
 #define SKIM_STAT_FWD_VISITS 3      /* (node, instance) pairs covered by residual searches */
 #define SKIM_STAT_FWD_COINS 4       /* coins evaluated by residual searches */
 #define SKIM_STAT_BATCHES 5         /* rank batches */

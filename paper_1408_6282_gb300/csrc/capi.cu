@@ -95,6 +95,15 @@ struct skim_ctx {
     uint64_t *full = nullptr, *X = nullptr;
     uint32_t *xlen = nullptr;
     bool built = false;
+    // build over materialised rows (build.cu): need masks, overflow places,
+    // hit and deferred-lane bitmaps, source pairs of deferred lanes, the
+    // contracted components (component and upstream masks, hit lists)
+    void *need_ws = nullptr;  // a need pass's tasks, where the visited table is small
+    uint64_t need_ws_bytes = 0;
+    uint64_t *over_buf = nullptr, *nonempty = nullptr, *need = nullptr, *comp = nullptr, *comp_up = nullptr;
+    uint32_t *over_seg = nullptr, *full_list = nullptr, *hitbits = nullptr, *defbits = nullptr, *defpair = nullptr;
+    uint32_t *node_off = nullptr;  // graphs of a batch: first nodes
+    void *comp_ws = nullptr;
     // SKIM
     bool sk_init = false;
     uint64_t *covered = nullptr, *seg_start = nullptr, *pend_trav = nullptr, *pend_erase = nullptr;
@@ -322,7 +331,6 @@ TravArgs base_args(skim_ctx *c, bool forward) {
     a.col = c->mat ? (forward ? c->flive : c->rlive) : (forward ? c->fcol : c->rcol);
     a.mat = c->mat ? 1 : 0;
     a.loff = forward ? c->foff : c->loff;
-    a.lmask = forward ? c->fmask : nullptr;
     a.cm = c->cm;
     a.q = c->q;
     a.qcap = c->qcap;
@@ -349,6 +357,24 @@ TravArgs base_args(skim_ctx *c, bool forward) {
     a.pend_trav = c->pend_trav;
     a.pend_erase = c->pend_erase;
     return a;
+}
+
+// Forward walk of every instance marking the reached nodes in mask, in a launch
+// of `ways` walks per instance.  Scratch: the visited table, up to the work
+// queue's capacity (a SKIM batch's lane bits are gathered when it is searched,
+// so nothing reads the table between batches).
+ReachArgs reach_args(skim_ctx *c, uint64_t *mask, uint32_t ways) {
+    ReachArgs r{};
+    r.off = c->foff;
+    r.rows = c->flive;
+    r.l = c->l;
+    r.n = c->n;
+    r.mask = mask;
+    r.list = reinterpret_cast<uint2 *>(c->hkeys);
+    r.cap = static_cast<uint32_t>(std::min<uint64_t>(std::min(c->hcap, c->qcap) / (ways * c->l), c->n));
+    r.ctl = c->ctl;
+    r.timeout_ns = c->timeout_ns;
+    return r;
 }
 
 // Source lanes of a reverse batch taken by the per-warp-queue search.
@@ -387,7 +413,7 @@ int run_traversal(skim_ctx *c, TravArgs &a, bool forward, uint64_t *R_out, const
         if (forward)
             CK(c, launch_respill_fwd(a, c->n, c->st));
         else
-            CK(c, launch_respill_rev(a, h.rec_count.v, c->st));
+            CK(c, launch_respill_rev(a, c->st));
     }
 }
 
@@ -594,6 +620,9 @@ int pull_stats(skim_ctx *c) {
 int reset_stats(skim_ctx *c) {
     CK(c, cudaMemsetAsync(c->ctl->stats, 0, sizeof(c->ctl->stats), c->st));
     std::fill(c->hstats, c->hstats + SKIM_STAT_COUNT, 0);
+    // the host's copy too (differences are taken before the first read-back;
+    // no copy into it is in flight between calls)
+    std::fill(std::begin(c->hctl->stats), std::end(c->hctl->stats), 0ull);
     c->vis_seen = 0;
     return SKIM_OK;
 }
@@ -752,23 +781,13 @@ int residual(skim_ctx *c, uint32_t x, uint64_t *cov) {
     }
     if (c->mat && (c->l >= kReachInst || c->live_total <= kReachPairs * c->l)) {
         KTimer kt(c, SKIM_K_FWD);
-        ReachArgs r{};
-        r.off = c->foff;
-        r.rows = c->flive;
-        r.l = c->l;
-        r.mask = c->covered;
-        // scratch: the visited table (a SKIM batch's lane bits were gathered
-        // when it was searched), up to the work queue's capacity
-        r.list = reinterpret_cast<uint2 *>(c->hkeys);
-        r.cap = static_cast<uint32_t>(std::min<uint64_t>(std::min(c->hcap, c->qcap) / c->l, c->n));
+        ReachArgs r = reach_args(c, c->covered, 1);
         r.pend_trav = c->pend_trav;
         r.seg_start = c->seg_start;
         r.seg_len = c->seg_len;
         r.size = c->size;
         r.idx_nodes = c->idx;
         r.chosen = c->chosen;
-        r.ctl = c->ctl;
-        r.timeout_ns = c->timeout_ns;
         CK(c, launch_reach(r, x, c->st));
     } else {
         CK(c, launch_fwd_source(a, x, c->st));
@@ -924,6 +943,7 @@ int make_instances(skim_ctx *c) {
         RC(dalloc(c, &c->fmask, std::max<uint64_t>(c->m, 1)));
         RC(dalloc(c, &c->loff, c->nl + 1));
         RC(dalloc(c, &c->foff, c->nl + 1));
+        RC(dalloc(c, &c->nonempty, c->n));
         RC(dalloc_bytes(c, &c->pieces, live_pieces_bytes(c->m)));
     }
     // counts per (v, i) scanned into 64-bit offsets, kept as 32-bit offsets
@@ -936,7 +956,7 @@ int make_instances(skim_ctx *c) {
     CK(c, exclusive_scan_u64(off, off, c->nl + 1, nullptr, c->ws, c->st));
     CK(c, cudaMemcpyAsync(&c->live_total, off + c->nl, sizeof(uint64_t), cudaMemcpyDeviceToHost, c->st));
     CK(c, cudaStreamSynchronize(c->st));
-    if (c->live_total > kRowMask) {  // offsets would not fit 31 bits: coins are drawn in the searches
+    if (c->live_total > kMaxLive) {  // offsets would not fit 31 bits: coins are drawn in the searches
         dfree(c, off);
         return SKIM_OK;
     }
@@ -950,6 +970,7 @@ int make_instances(skim_ctx *c) {
     }
     CK(c, launch_live_fill(c->rptr, c->rcol, c->rmask, c->n, c->m, c->l, off, c->rlive, c->pieces, c->st));
     CK(c, launch_offsets_u32(off, c->nl, c->loff, c->st));
+    CK(c, launch_nonempty(c->loff, c->n, c->l, c->nonempty, c->st));
     // the same live pairs by tail: rows of live out-neighbours for the residual
     CK(c, launch_live_count(c->fptr, c->fmask, c->n, c->m, c->l, off, c->pieces, c->st));
     CK(c, cudaMemsetAsync(off + c->nl, 0, sizeof(uint64_t), c->st));
@@ -1055,6 +1076,9 @@ int skim_destroy(skim_ctx *c) {
     dfree(c, c->ncnt); dfree(c, c->noff); dfree(c, c->nlist); dfree(c, c->nlist_cnt);
     dfree(c, c->ws);
     dfree(c, c->lane_inst); dfree(c, c->lane_g); dfree(c, c->alive); dfree(c, c->lane_cnt); dfree(c, c->lane_off); dfree(c, c->lane_fill);
+    dfree(c, c->nonempty); dfree(c, c->need); dfree(c, c->comp); dfree(c, c->comp_up);
+    dfree(c, c->over_seg); dfree(c, c->over_buf); dfree(c, c->full_list); dfree(c, c->hitbits); dfree(c, c->defbits); dfree(c, c->defpair);
+    dfree(c, c->node_off); dfree(c, c->comp_ws); dfree(c, c->need_ws);
     dfree(c, c->lcnt); dfree(c, c->full); dfree(c, c->X); dfree(c, c->xlen);
     dfree(c, c->covered); dfree(c, c->seg_start); dfree(c, c->pend_trav); dfree(c, c->pend_erase);
     dfree(c, c->size); dfree(c, c->seg_len); dfree(c, c->idx); dfree(c, c->chosen);
@@ -1355,7 +1379,7 @@ int skim_create_batch(const skim_graph *graphs, const skim_params *prm, uint32_t
              launch_rank_bases(b, c->n, c->l, c->rbase, c->st) == cudaSuccess;
     }
     if (ok) ok = cudaStreamSynchronize(c->st) == cudaSuccess;
-    dfree(c, d_off);
+    c->node_off = d_off;
     dfree(c, d_ng);
     dfree(c, d_keys);
     dfree(c, d_model);
@@ -1479,27 +1503,365 @@ int skim_instance_stats(skim_ctx *c, uint64_t *live_pairs, int *materialised) {
     return SKIM_OK;
 }
 
-int skim_build_sketches(skim_ctx *c) {
-    if (!c) return SKIM_EINVAL;
-    if (c->broken) return SKIM_ECUDA;
-    if (!c->X) {
-        RC(dalloc(c, &c->lcnt, c->nl));
-        RC(dalloc(c, &c->full, c->n));
-        RC(dalloc(c, &c->X, static_cast<size_t>(c->n) * c->k));
-        RC(dalloc(c, &c->xlen, c->n));
+}  // extern "C"
+
+namespace {
+
+// ---- Algorithm 2 over materialised rows (build.cu) ---------------------------
+
+#ifndef SKIM_ROWS_GROWTH
+#define SKIM_ROWS_GROWTH 32
+#endif
+#ifndef SKIM_ROWS_REFRESH
+#define SKIM_ROWS_REFRESH 1.5
+#endif
+#ifndef SKIM_ROWS_LANES
+#define SKIM_ROWS_LANES (1u << 24)
+#endif
+#ifndef SKIM_ROWS_VISITS
+#define SKIM_ROWS_VISITS (16u << 20)
+#endif
+constexpr uint32_t kRowsGrowth = SKIM_ROWS_GROWTH;  // lanes of a batch over the last one, at most
+// need is recomputed when the processed ranks grew by kRowsRefresh, until half
+// of them are done, or when the searches since the last time made kRowsVisits
+// visits (about twice what the pass costs)
+constexpr double kRowsRefresh = SKIM_ROWS_REFRESH;
+constexpr uint64_t kRowsVisits = SKIM_ROWS_VISITS;
+#ifndef SKIM_ROWS_DIRECT
+#define SKIM_ROWS_DIRECT (1u << 18)
+#endif
+// A batch of few lanes with larger searches goes to the searches with a global
+// table at once: the warps' own searches take 0.2 ms for it however few they
+// are, and defer much of it.
+constexpr uint32_t kRowsDirect = SKIM_ROWS_DIRECT;
+constexpr double kRowsDirectVisits = 4.0;
+#ifndef SKIM_ROWS_CHEAP
+#define SKIM_ROWS_CHEAP 2097152.0
+#endif
+constexpr double kRowsCheap = SKIM_ROWS_CHEAP;      // visits that a batch may make however much it grows
+#ifndef SKIM_ROWS_LAST
+#define SKIM_ROWS_LAST 0.5
+#endif
+constexpr uint32_t kRowsLanes = SKIM_ROWS_LANES;    // lanes of a batch unless the caller says otherwise
+// Visits per lane of the first batch from which components are contracted.
+// They are far apart: 11-22 on weighted cascades (R-MAT 18 to 20) and near-critical
+// Erdos-Renyi graphs, hundreds to tens of thousands above the threshold.
+constexpr double kGiantMean = 64.0;
+
+int rows_buffers(skim_ctx *c) {
+    if (c->need) return SKIM_OK;
+    RC(dalloc(c, &c->over_seg, c->n));
+    RC(dalloc(c, &c->over_buf, c->rcap));
+    RC(dalloc(c, &c->full_list, c->n));
+    RC(dalloc(c, &c->hitbits, c->lane_cap / 32 + 1));
+    RC(dalloc(c, &c->defbits, c->lane_cap / 32 + 1));
+    RC(dalloc(c, &c->defpair, c->lane_cap));
+    if (!c->nlist) RC(dalloc(c, &c->nlist, c->n));
+    // a task is 24 bytes; about a third of the pairs can be one
+    const uint64_t tasks = std::min<uint64_t>(8 * c->nl, 4ull << 30);
+    if (tasks > c->hcap * 2 * sizeof(uint64_t)) {
+        RC(dalloc_bytes(c, &c->need_ws, tasks));
+        c->need_ws_bytes = tasks;
     }
-    if (c->batch_active) {  // a SKIM batch holds the visited table: release it
-        RC(commit_lanes(c, c->blo, c->bB - 1));
-        RC(clear_batch(c));
-        c->batch_active = false;
+    return dalloc(c, &c->need, c->n);
+}
+
+// What a build with contracted components keeps per graph, in one allocation.
+struct CompSpace {
+    unsigned long long *best;           // 64 per graph
+    uint64_t *topen, *hits, *sorted, *places;
+    uint32_t *pivot, *count, *tlen, *total, *list, *seg;
+};
+
+size_t comp_space(uint32_t graphs, uint32_t l, uint32_t k, void *ws, CompSpace *sp) {
+    size_t at = 0;
+    const auto take = [&](auto *&p, size_t count) {
+        p = reinterpret_cast<std::decay_t<decltype(p)>>(static_cast<char *>(ws) + at);
+        at += (count * sizeof(*p) + 15) & ~static_cast<size_t>(15);
+    };
+    const size_t lists = static_cast<size_t>(graphs) * 64;
+    take(sp->best, lists);
+    take(sp->topen, graphs);
+    take(sp->hits, lists * k);
+    take(sp->sorted, static_cast<size_t>(graphs) * l * k);
+    take(sp->places, lists * ((l * k + 63) / 64));
+    take(sp->pivot, lists);
+    take(sp->count, 128);
+    take(sp->tlen, lists);
+    take(sp->total, graphs);
+    take(sp->list, lists);
+    take(sp->seg, lists);
+    return at;
+}
+
+// Contract the component around each instance's pivot (of every graph); *on =
+// false if none is worth it.
+int contract_components(skim_ctx *c, BuildNode &g, CompSpace *sp, bool *on) {
+    *on = false;
+    if (!c->comp) {
+        RC(dalloc(c, &c->comp_up, c->n));
+        RC(dalloc_bytes(c, &c->comp_ws, comp_space(g.graphs, c->l, c->k, nullptr, sp)));
+        RC(dalloc(c, &c->comp, c->n));
+    }
+    comp_space(g.graphs, c->l, c->k, c->comp_ws, sp);
+    g.tlen = sp->tlen;
+    g.topen = sp->topen;
+    CK(c, cudaMemsetAsync(c->comp, 0, c->n * sizeof(uint64_t), c->st));
+    CK(c, cudaMemsetAsync(c->comp_up, 0, c->n * sizeof(uint64_t), c->st));
+    CK(c, cudaMemsetAsync(sp->tlen, 0, g.graphs * 64ull * sizeof(uint32_t), c->st));
+    {
+        KTimer kt(c, SKIM_K_REV);
+        CK(c, launch_pivots(g, sp->best, sp->pivot, c->st));
+        ReachArgs r = reach_args(c, c->comp, 2);
+        r.back_off = c->loff;
+        r.back_rows = c->rlive;
+        r.back_mask = c->comp_up;
+        uint64_t *pend = nullptr;
+        RC(dalloc(c, &pend, 2ull * c->n));
+        CK(c, cudaMemsetAsync(pend, 0, 2ull * c->n * sizeof(uint64_t), c->st));
+        r.pend_trav = pend;
+        r.back_pend = pend + c->n;
+        CK(c, launch_reach_from(r, sp->pivot, g.graphs, sp->count, c->st));
+        dfree(c, pend);
+        CK(c, launch_components(g, c->comp, c->comp_up, sp->count, sp->count + 64, c->ctl, c->st));
+    }
+    RC(sync_ctl(c));
+    if (c->hctl->err & kErrTimeout) {
+        c->broken = true;
+        return SKIM_ETIMEOUT;
+    }
+    *on = c->hctl->b.n_open != 0;
+    return SKIM_OK;
+}
+
+// The deferred lanes of a batch (D of them, after R0 records), searched from
+// their sources with a global visited table of about four slots per expected
+// visit (vpl visits per lane in the last such search; 0: unknown, the whole
+// table).  words: all lanes of the batch, records per table entry.  *retry: the
+// batch has to be run again with fewer lanes.
+int search_deferred(skim_ctx *c, uint64_t p0, uint32_t D, uint64_t R0, const BuildArgs &ba, double *vpl, bool words,
+                    uint64_t *R, bool *retry) {
+    *retry = false;
+    const uint32_t T = (D + 63) / 64;
+    CK(c, launch_deferred_lanes(ba.deflist, D, D == ba.B, c->spair + p0, c->l, c->defpair, c->lane_inst, c->st));
+    TravArgs a = base_args(c, false);
+    a.tbits = bitlen(T - 1);
+    a.hnode = T <= kNodeHashWords ? 1 : 0;
+    a.need = ba.need;
+    a.lmask = ba.lmask;
+    a.scc = ba.scc;
+    a.hit = ba.hit;
+    a.lane_of = ba.deflist;
+    a.lbits = ba.lbits;
+    a.own = ba.own;
+    a.words = words ? 1 : 0;
+    for (bool whole = *vpl <= 0;; whole = true) {
+        uint64_t want = c->hcap;
+        if (!whole)
+            want = static_cast<uint64_t>(std::min(std::max(65536.0, kTableSlots * *vpl * D), static_cast<double>(c->hcap)));
+        a.hmask = pow2_at_least(std::min(want, c->hcap)) - 1;  // (hcap is a power of two)
+        CK(c, clear_table(c, a.hmask + 1));
+        CK(c, cudaMemsetAsync(&c->ctl->src_next, 0, 3 * sizeof(HotCounter), c->st));  // src_next, busy, beat
+        const uint64_t v0 = c->hctl->stats[kStRevVisits];
+        if (*vpl > 0 && *vpl <= c->ring_rpl) {
+            const RevSources rs{c->defpair, D, nullptr, nullptr};
+            RC(run_traversal(c, a, false, R, &rs));
+        } else {
+            {
+                KTimer kt(c, SKIM_K_SOURCES);
+                CK(c, launch_rev_sources(a, c->defpair, D, c->l, nullptr, nullptr, c->st));
+            }
+            RC(run_traversal(c, a, false, R));
+        }
+        const DevCtl &h = *c->hctl;
+        const unsigned err = h.err & kErrRetryable;
+        RC(reset_queue(c, h.q_tail.v));
+        if (!err) {
+            *vpl = std::max(1.0, static_cast<double>(h.stats[kStRevVisits] - v0) / D);
+            return SKIM_OK;
+        }
+        CK(c, cudaMemsetAsync(c->pend, 0, c->hcap * sizeof(uint64_t), c->st));
+        if (whole || (err & kErrRecords)) {
+            *vpl = 0;
+            *retry = true;
+            return SKIM_OK;
+        }
+        // more visits than expected: once more with the whole table
+        c->hstats[SKIM_STAT_RETRIES]++;
+        CK(c, cudaMemsetAsync(&c->ctl->err, 0, sizeof(unsigned), c->st));
+        c->hctl->rec_count.v = R0;
+        CK(c, cudaMemcpyAsync(&c->ctl->rec_count, &c->hctl->rec_count, sizeof(uint64_t), cudaMemcpyHostToDevice,
+                              c->st));
+    }
+}
+
+int build_rows(skim_ctx *c) {
+    RC(rows_buffers(c));
+    const bool own_rec = c->rank_mode != SKIM_RANKS_UNIFORM;  // positions: not recomputable from the pair
+    const uint64_t lmask = c->l == 64 ? ~0ull : (1ull << c->l) - 1;
+    CK(c, cudaMemsetAsync(c->xlen, 0, c->n * sizeof(uint32_t), c->st));
+    CK(c, cudaMemsetAsync(&c->ctl->b, 0, sizeof(BuildCtl), c->st));
+    CK(c, launch_need_start(c->need, c->n, lmask, c->st));
+    BuildArgs a{};
+    a.l = c->l;
+    a.n = c->n;
+    a.loff = c->loff;
+    a.rlive = c->rlive;
+    a.nonempty = c->nonempty;
+    a.need = c->need;
+    a.lmask = lmask;
+    a.hit = c->hitbits;
+    a.rec = c->rkey;
+    a.rcap = c->rcap;
+    a.own = own_rec ? 1 : 0;
+    a.deflist = c->lane_fill;
+    a.defbits = c->defbits;
+    a.ctl = c->ctl;
+    BuildNode g{};
+    g.n = c->n;
+    g.l = c->l;
+    g.k = c->k;
+    g.loff = c->loff;
+    g.rlive = c->rlive;
+    g.foff = c->foff;
+    g.flive = c->flive;
+    g.nonempty = c->nonempty;
+    g.len = c->xlen;
+    g.rank_key = c->rank_key;
+    g.rbase = c->rbase;
+    g.own = own_rec ? 0 : 1;
+    g.graphs = c->batch_count ? c->batch_count : 1;
+    g.node_off = c->node_off;
+    CompSpace cs{};
+    const BuildScratch sc{c->rkey2, c->rval2, c->over_buf, c->nlist, c->over_seg};
+    uint64_t bmax = c->batch_cfg ? c->batch_cfg : kRowsLanes;
+    bmax = std::max<uint64_t>(64, std::min<uint64_t>(bmax, c->lane_cap));
+    uint64_t B = std::min<uint64_t>(bmax, kBuildFirst), p0 = 0, last = 0, since = 0;
+    double per = 1e9;  // visits per lane of the last batch
+    double vpl = 0, vpl_def = 0;  // visits per lane of the last batch searched whole, of the last deferred lanes
+    bool giant = false;
+    bool force = false;  // after an overflow: a global table with a record per entry, which needs the least room
+    while (p0 < c->nbuild) {
+        const uint32_t b = static_cast<uint32_t>(std::min<uint64_t>(B, c->nbuild - p0));
+        RC(reset_ctl(c));
+        CK(c, cudaMemsetAsync(&c->ctl->b, 0, 5 * sizeof(unsigned), c->st));  // the batch's counts
+        CK(c, cudaMemsetAsync(c->defbits, 0, (b / 32 + 1) * sizeof(uint32_t), c->st));
+        const bool hits = giant && c->hctl->b.n_open != 0;
+        if (hits) CK(c, cudaMemsetAsync(c->hitbits, 0, (b / 32 + 1) * sizeof(uint32_t), c->st));
+        a.pair = c->spair + p0;
+        a.B = b;
+        a.lbits = static_cast<uint32_t>(bitlen(b - 1));
+        const uint64_t v0 = c->hctl->stats[kStRevVisits];
+        bool retry = false;
+        uint64_t R0 = 0, v1 = v0;
+        uint32_t D = b;
+        const bool direct = force || (b <= kRowsDirect && per >= kRowsDirectVisits);
+        const bool words = force || (direct && p0 == 0);
+        if (!direct) {
+            {
+                KTimer kt(c, SKIM_K_REV);
+                CK(c, launch_build_search(a, c->st));
+            }
+            RC(sync_ctl(c));
+            retry = (c->hctl->err & kErrRetryable) != 0;
+            R0 = c->hctl->rec_count.v;
+            v1 = c->hctl->stats[kStRevVisits];
+            D = c->hctl->b.n_def;
+        }
+        uint64_t R = R0;
+        if (!retry && D) RC(search_deferred(c, p0, D, R0, a, direct ? &vpl : &vpl_def, words, &R, &retry));
+        if (c->hctl->b.failed) {  // the last need pass gave up
+            c->broken = true;
+            return SKIM_ETIMEOUT;
+        }
+        if (c->hctl->b.n_full == c->n) break;  // every node has its k ranks: the batch found nothing
+        if (retry) {
+            if (b <= 64 && force) return SKIM_ENOMEM;  // even the smallest batch overflows the tables
+            c->hstats[SKIM_STAT_RETRIES]++;
+            B = std::max<uint32_t>(64, b / 4);
+            force = true;
+            continue;
+        }
+        force = false;
+        const uint64_t v2 = c->hctl->stats[kStRevVisits];
+        if (trace_batches())
+            fprintf(stderr, "skim rows p0=%llu B=%u records=%llu visits=%llu deferred=%u their visits=%llu full=%u\n",
+                    static_cast<unsigned long long>(p0), b, static_cast<unsigned long long>(R),
+                    static_cast<unsigned long long>(v1 - v0), D, static_cast<unsigned long long>(v2 - v1),
+                    c->hctl->b.n_full);
+        const uint64_t *ranks = c->srank + p0;
+        {
+            KTimer kt(c, SKIM_K_ACCEPT);
+            CK(c, launch_append(c->rkey, 0, R0, a.lbits, D ? c->defbits : nullptr, ranks, c->k, c->xlen, c->X, sc,
+                                c->ctl, c->st));
+            if (words) {
+                // a record appends at most k ranks, and a part of the records
+                // as many as there is room for should all of them overflow
+                const uint64_t part = std::max<uint64_t>(1, c->rcap / std::min(c->k, 64u));
+                for (uint64_t r = 0; r < R; r += part) {
+                    const uint64_t m = std::min(part, R - r);
+                    if (r) CK(c, cudaMemsetAsync(&c->ctl->b.n_over, 0, 3 * sizeof(unsigned), c->st));
+                    CK(c, launch_append_words(c->rkey + r, c->rval + r, m, bitlen((b + 63) / 64 - 1), c->hvals, a.pair,
+                                              c->l, a.own, a.lbits, ranks, c->k, c->xlen, c->X, sc, c->ctl, c->st));
+                    CK(c, launch_overflow(m, a.lbits, ranks, c->k, c->xlen, c->X, R <= part, sc, c->ctl, c->st));
+                }
+            } else {
+                CK(c, launch_append(c->rkey, R0, R, a.lbits, nullptr, ranks, c->k, c->xlen, c->X, sc, c->ctl, c->st));
+                CK(c, launch_overflow(R, a.lbits, ranks, c->k, c->xlen, c->X, true, sc, c->ctl, c->st));
+            }
+            if (hits) {
+                const BuildScratch hs{c->rkey2, c->rval2, c->over_buf, cs.list, cs.seg};
+                CK(c, launch_hits(g, c->hitbits, a.pair, ranks, b, a.lbits, c->rkey, cs.hits, hs, c->ctl, c->st));
+            }
+        }
+        if (p0 == 0 && static_cast<double>(v2 - v0) >= kGiantMean * b) {
+            RC(contract_components(c, g, &cs, &giant));
+            if (giant) {
+                a.scc = g.scc = c->comp;
+                g.up = c->comp_up;
+                bmax = std::min(bmax, std::max<uint64_t>(64, c->rcap));  // (a record per hit)
+            }
+        }
+        p0 += b;
+        c->hstats[SKIM_STAT_BATCHES]++;
+        c->hstats[SKIM_STAT_RANKS] += b;
+        // next batch: larger, with the records near a quarter of their table
+        // and the deferred visits near an eighth of theirs
+        const double recs = static_cast<double>(std::max<uint64_t>(R, 1)) / b;
+        const double defs = static_cast<double>(std::max<uint64_t>(v2 - v1, 1)) / b;
+        const uint64_t fit = static_cast<uint64_t>(std::min(c->rcap / 4.0 / recs, c->hcap / 8.0 / defs));
+        // (visits per lane as measured, unless a component has just been contracted)
+        per = static_cast<double>(std::max<uint64_t>(v2 - v0, 1)) / b;
+        uint64_t next = kRowsGrowth * static_cast<uint64_t>(b);
+        if (per >= kRowsDirectVisits && !(giant && p0 == b)) next = std::max(next, static_cast<uint64_t>(kRowsCheap / per));
+        B = std::max<uint64_t>(64, std::min<uint64_t>({bmax, next, fit}));
+        since += v2 - v0;
+        if (p0 < c->nbuild && ((static_cast<double>(p0) < SKIM_ROWS_LAST * static_cast<double>(c->nbuild) &&
+                                static_cast<double>(p0) >= kRowsRefresh * static_cast<double>(last)) ||
+                               since >= kRowsVisits)) {
+            since = 0;
+            last = p0;
+            KTimer kt(c, SKIM_K_ACCEPT);
+            CK(c, launch_need(g, c->srank + p0, c->need, c->full_list, c->need_ws ? c->need_ws : c->hkeys,
+                              c->need_ws ? c->need_ws_bytes : c->hcap * 2 * sizeof(uint64_t), c->ctl, c->timeout_ns,
+                              c->st));
+        }
+    }
+    KTimer kt(c, SKIM_K_ACCEPT);
+    CK(c, launch_merge(g, c->X, cs.hits, cs.sorted, cs.places, cs.total, c->ctl, c->st));
+    return SKIM_OK;
+}
+
+// Algorithm 2 with coins drawn in the searches.
+int build_coins(skim_ctx *c) {
+    if (!c->lcnt) {
+        RC(dalloc(c, &c->full, c->n));
+        RC(dalloc(c, &c->lcnt, c->nl));
     }
     CK(c, cudaMemsetAsync(c->lcnt, 0, c->nl, c->st));
     CK(c, cudaMemsetAsync(c->full, 0, c->n * sizeof(uint64_t), c->st));
-    if (c->mat) CK(c, launch_clear_row_flags(c->loff, c->nl, c->st));
     CK(c, cudaMemsetAsync(c->X, 0, static_cast<size_t>(c->n) * c->k * sizeof(uint64_t), c->st));
     CK(c, cudaMemsetAsync(c->xlen, 0, c->n * sizeof(uint32_t), c->st));
-    RC(reset_stats(c));
-    c->built = false;
     const uint32_t Bmax = default_lanes(c);
     // The first batch is small: the searches of the lowest ranks can each
     // reach a large part of the graph (thousands of records per lane on
@@ -1526,7 +1888,7 @@ int skim_build_sketches(skim_ctx *c) {
                 cudaEventRecord(t0, c->st);
             }
             CK(c, launch_accept(c->rkey, c->rval, c->hvals, c->bR, c->btbits, c->lane_inst, c->srank + p0, c->l,
-                                c->k, c->lcnt, c->full, c->mat ? c->loff : nullptr, c->X, c->xlen, c->ctl, c->st));
+                                c->k, c->lcnt, c->full, c->X, c->xlen, c->ctl, c->st));
             if (trace_batches()) {
                 cudaEventRecord(t1, c->st);
                 cudaEventSynchronize(t1);
@@ -1553,6 +1915,28 @@ int skim_build_sketches(skim_ctx *c) {
         const uint64_t fit = static_cast<uint64_t>(static_cast<double>(c->rcap) / SKIM_BUILD_FILL / per_lane);
         B = static_cast<uint32_t>(std::max<uint64_t>(64, std::min<uint64_t>({Bmax, kBuildGrowth * B, fit})));
     }
+    return SKIM_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int skim_build_sketches(skim_ctx *c) {
+    if (!c) return SKIM_EINVAL;
+    if (c->broken) return SKIM_ECUDA;
+    if (!c->X) {
+        RC(dalloc(c, &c->xlen, c->n));
+        RC(dalloc(c, &c->X, static_cast<size_t>(c->n) * c->k));
+    }
+    if (c->batch_active) {  // a SKIM batch holds the visited table: release it
+        RC(commit_lanes(c, c->blo, c->bB - 1));
+        RC(clear_batch(c));
+        c->batch_active = false;
+    }
+    RC(reset_stats(c));
+    c->built = false;
+    RC(c->mat ? build_rows(c) : build_coins(c));
     uint64_t batches = c->hstats[SKIM_STAT_BATCHES], ranks = c->hstats[SKIM_STAT_RANKS],
              retries = c->hstats[SKIM_STAT_RETRIES];
     RC(pull_stats(c));

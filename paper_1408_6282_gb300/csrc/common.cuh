@@ -22,12 +22,12 @@ inline void note_launch() { g_kernel_launches.fetch_add(1, std::memory_order_rel
 
 constexpr uint64_t kGolden = 0x9E3779B97F4A7C15ull;
 constexpr uint64_t kEmptyKey = ~0ull;
-// Materialised live rows: 32-bit offsets into the row array; the top bit of
-// row r's start (r = v * l + i) says that the instance-local sketch of (v, i)
-// holds k ranks (Algorithm 2's pruning), so one load gives the row and the
-// pruning decision.  Offsets therefore stay below 2^31.
-constexpr uint32_t kRowMask = 0x7FFFFFFFu;
-constexpr uint32_t kRowFull = 0x80000000u;
+// Materialised live rows have 32-bit offsets; a context with more live pairs
+// than this keeps none.
+constexpr uint64_t kMaxLive = 0x7FFFFFFFull;
+// Row lengths of a sketch build: the node holds k ranks and takes no more.
+constexpr uint32_t kRowDone = 0x80000000u;
+constexpr uint32_t kRowListed = 0x40000000u;  // and is in the list of full nodes (implies kRowDone)
 // key of the within-chunk node order of permutation ranks: fmix(rank_key ^ salt)
 constexpr uint64_t kPermSalt = 0x7065726d75746531ull;
 constexpr unsigned kFull = 0xffffffffu;
@@ -102,6 +102,18 @@ struct alignas(128) HotCounter {
     unsigned long long pad[15];
 };
 
+// Control of a sketch build over materialised rows (build.cu).
+struct BuildCtl {
+    // of a batch: deferred lanes; overflow records, nodes with overflow, space
+    // given to it; hit records
+    unsigned n_def, n_over, n_list, over_total, n_hit;
+    // of a need pass: tasks (short and long rows), the grid barrier, change flags, worklist lengths
+    unsigned n_task, n_long, bar, changed[3], wl[3];
+    // of the build: full nodes and open hit lists, now and at the last need pass
+    unsigned n_full, n_open, n_full_last, n_open_last;
+    unsigned failed;                // a need pass ran into the wait limit
+};
+
 // Device control block: queue cursors, counters, flags, reductions.
 // src_next, busy and beat serve the reverse searches with per-warp queues:
 // the next unclaimed source lane of the batch, the warps that hold work, and
@@ -117,6 +129,7 @@ struct DevCtl {
     unsigned int err;
     unsigned int spill;   // some work was parked in pending masks
     unsigned int pad[2];
+    BuildCtl b;
 };
 
 enum Stat { kStRevVisits = 0, kStRevCoins, kStInsert, kStFwdVisits, kStFwdCoins, kStRevEdges, kStFwdEdges };

@@ -57,12 +57,20 @@ struct TravArgs {
     uint64_t *pend_trav;        // per node: instances whose expansion was spilled
     uint64_t *pend_erase;       // per node: instances whose index erasure was spilled
     // materialised instances (mat != 0): reverse searches walk the live
-    // in-neighbours of (node v, instance i), col[loff[v*l+i] .. loff[v*l+i+1])
-    // (offsets masked by kRowMask; kRowFull on a row start marks a full local
-    // sketch), forward searches the live out-neighbours the same way
+    // in-neighbours of (node v, instance i), col[loff[v*l+i] .. loff[v*l+i+1]),
+    // forward searches the live out-neighbours the same way
     int mat;
     const uint32_t *loff;
-    const uint64_t *lmask;
+    // sketch build over materialised instances (need != null): lane q of the
+    // search is lane lane_of[q] of the batch; need, scc, hit, lbits, own as in
+    // BuildArgs; words: records node << tbits | word per table entry instead
+    const uint64_t *need;
+    uint64_t lmask;
+    const uint64_t *scc;
+    uint32_t *hit;
+    const uint32_t *lane_of;
+    uint32_t lbits;
+    int own, words;
 };
 
 // graph.cu
@@ -95,10 +103,8 @@ cudaError_t launch_live_count(const uint32_t *ptr, const uint64_t *mask, uint32_
                               uint64_t *off, void *pieces_ws, cudaStream_t s);
 cudaError_t launch_live_fill(const uint32_t *ptr, const uint32_t *col, const uint64_t *mask, uint32_t n, uint64_t m,
                              uint32_t l, const uint64_t *off, uint32_t *live, void *pieces_ws, cudaStream_t s);
-// off32[r] = off[r] for r <= count (offsets below 2^31; no row flagged full)
+// off32[r] = off[r] for r <= count (offsets below 2^31)
 cudaError_t launch_offsets_u32(const uint64_t *off, uint64_t count, uint32_t *off32, cudaStream_t s);
-// clear the full flags (kRowFull) of rows 0 .. count - 1
-cudaError_t launch_clear_row_flags(uint32_t *off32, uint64_t count, cudaStream_t s);
 
 // Rank order of all pairs: bucket by the top bits, then sort each bucket.
 // rank of pair x = v*l+i is fmix(rank_key + G*x), or fmix(rbase[v] + G*i)
@@ -136,8 +142,9 @@ cudaError_t launch_rev_sources(const TravArgs &a, const uint32_t *lane_pair, uin
                                const uint64_t *covered, uint64_t *alive, cudaStream_t s);
 cudaError_t launch_fwd_source(const TravArgs &a, uint32_t x, cudaStream_t s);
 cudaError_t launch_traverse(const TravArgs &a, bool forward, int grid, cudaStream_t s);
-// Re-queue spilled work (after a drained traversal that set DevCtl::spill).
-cudaError_t launch_respill_rev(const TravArgs &a, uint64_t R, cudaStream_t s);
+// Re-queue spilled work (after a drained traversal that set DevCtl::spill);
+// reverse searches find it by their table slots.
+cudaError_t launch_respill_rev(const TravArgs &a, cudaStream_t s);
 cudaError_t launch_respill_fwd(const TravArgs &a, uint32_t n, cudaStream_t s);
 int traverse_grid(bool forward);  // resident blocks for the persistent traversal
 // Reverse searches over materialised live rows with per-warp queues in shared
@@ -156,9 +163,12 @@ struct ReachArgs {
     const uint32_t *rows;
     uint32_t l;
     uint64_t *mask;             // per node: instances in which it has been reached (covered)
+    const uint32_t *back_off, *back_rows;
+    uint64_t *back_mask;
     uint2 *list;                // scratch: 2 * cap entries per instance
     uint32_t cap;
-    uint64_t *pend_trav;        // per node: instances whose rows did not fit the scratch
+    uint64_t *pend_trav, *back_pend;  // per node: instances whose rows did not fit the scratch
+    uint32_t n;
     const uint64_t *seg_start;  // index segment of every pair: first entry, entries
     uint32_t *seg_len;
     uint32_t *size;
@@ -168,20 +178,99 @@ struct ReachArgs {
     uint64_t timeout_ns;
 };
 cudaError_t launch_reach(const ReachArgs &a, uint32_t x, cudaStream_t s);
+// What the nodes pivot[64 * q + i], q < starts, reach in instance i, for every
+// instance: its bit in mask
+// (zero before), the number of nodes to count[i].  A walk that does not fit the
+// scratch sets its bit in BuildCtl::reach_fail.  Uses off, rows, l, mask, list,
+// cap, ctl and timeout_ns of a.
+cudaError_t launch_reach_from(const ReachArgs &a, const uint32_t *pivot, uint32_t starts, uint32_t *count,
+                              cudaStream_t s);
+
+// build.cu: Algorithm 2 over materialised rows
+struct BuildArgs {
+    const uint32_t *pair;   // the batch's pairs v*l + i in rank order
+    uint32_t B, l, n;
+    const uint32_t *loff, *rlive;
+    const uint64_t *nonempty;  // per node: instances in which its row is not empty
+    const uint64_t *need;   // per node: instances in which something upstream still needs ranks
+    uint64_t lmask;         // all l instances (need == lmask: the node itself may)
+    const uint64_t *scc;    // per node: instances in which it is in the contracted component (null: none)
+    uint32_t *hit;          // bitmap of the lanes that hit an open component
+    uint64_t *rec;          // records node << lbits | lane
+    uint64_t rcap;
+    uint32_t lbits;
+    int own;                // sources leave records too (ranks that k_merge cannot recompute)
+    uint32_t *deflist, *defbits;  // deferred lanes: list, bitmap
+    DevCtl *ctl;
+};
+struct BuildNode {
+    uint32_t n, l, k;
+    const uint32_t *loff, *rlive, *foff, *flive;
+    const uint64_t *nonempty;
+    uint32_t *len;          // row lengths (kRowDone, kRowListed)
+    uint64_t rank_key;
+    const uint64_t *rbase;
+    int own;                // own ranks are not recorded: they are merged
+    // contracted components (up null: none): per node the instances in which it
+    // reaches / is in the component of its graph; per graph (first nodes
+    // node_off, null for one graph) and instance the length of the hit list,
+    // per graph the open lists
+    const uint64_t *up, *scc;
+    uint32_t graphs;
+    const uint32_t *node_off;
+    uint32_t *tlen;         // [graph][64]
+    uint64_t *topen;
+};
+struct BuildScratch {
+    uint64_t *over_key;     // one entry per record of a batch
+    uint32_t *over_pos;
+    uint64_t *buf;
+    uint32_t *list, *seg;   // n entries
+};
+cudaError_t launch_build_search(const BuildArgs &a, cudaStream_t s);
+// source pairs and instances of the D deferred lanes
+cudaError_t launch_deferred_lanes(uint32_t *deflist, uint32_t D, bool all, const uint32_t *pair, uint32_t l,
+                                  uint32_t *defpair, uint8_t *lane_inst, cudaStream_t s);
+cudaError_t launch_append(const uint64_t *rec, uint64_t r0, uint64_t r1, uint32_t lbits, const uint32_t *defbits,
+                          const uint64_t *lane_rank, uint32_t k, uint32_t *len, uint64_t *X, const BuildScratch &b,
+                          DevCtl *ctl, cudaStream_t s);
+// records node << tbits | word of a search of all lanes of a batch (slots
+// rec_val, lane bits hvals): the ranks of each one's lanes, without the node's
+// own unless `own`
+cudaError_t launch_append_words(const uint64_t *rec, const uint32_t *rec_val, uint64_t R, uint32_t tbits,
+                                const uint64_t *hvals, const uint32_t *pair, uint32_t l, int own, uint32_t lbits, const uint64_t *lane_rank, uint32_t k, uint32_t *len,
+                                uint64_t *X, const BuildScratch &b, DevCtl *ctl, cudaStream_t s);
+// rows that received more than k ranks keep the k smallest (R: records appended;
+// done: and are full)
+cudaError_t launch_overflow(uint64_t R, uint32_t lbits, const uint64_t *lane_rank, uint32_t k, uint32_t *len,
+                            uint64_t *X, bool done, const BuildScratch &b, DevCtl *ctl, cudaStream_t s);
+cudaError_t launch_need_start(uint64_t *need, uint32_t n, uint64_t lmask, cudaStream_t s);
+cudaError_t launch_nonempty(const uint32_t *loff, uint32_t n, uint32_t l, uint64_t *nonempty, cudaStream_t s);
+// *next (device): the first rank not yet processed; full_list: n entries kept
+// from pass to pass
+cudaError_t launch_need(const BuildNode &g, const uint64_t *next, uint64_t *need, uint32_t *full_list, void *scratch,
+                        uint64_t scratch_bytes, DevCtl *ctl, uint64_t timeout_ns, cudaStream_t s);
+// best, pivot: 64 entries per graph
+cudaError_t launch_pivots(const BuildNode &g, unsigned long long *best, uint32_t *pivot, cudaStream_t s);
+// down becomes the component, up is cleared where it is not contracted
+cudaError_t launch_components(const BuildNode &g, uint64_t *down, uint64_t *up, const uint32_t *ndown,
+                              const uint32_t *nup, DevCtl *ctl, cudaStream_t s);
+// a batch's hits into the lists hits[graph][64][k] (rec: one entry per lane of the batch)
+cudaError_t launch_hits(const BuildNode &g, const uint32_t *hit, const uint32_t *pair, const uint64_t *lane_rank,
+                        uint32_t B, uint32_t lbits, uint64_t *rec, uint64_t *hits, const BuildScratch &b, DevCtl *ctl,
+                        cudaStream_t s);
+// hits_sorted: [graph][l * k]; places: [graph][64][(l * k + 63) / 64]; total: [graph]
+cudaError_t launch_merge(const BuildNode &g, uint64_t *X, uint64_t *hits, uint64_t *hits_sorted, uint64_t *places,
+                         uint32_t *total, DevCtl *ctl, cudaStream_t s);
 
 // batch.cu
 cudaError_t launch_lane_inst(const uint32_t *lane_pair, const uint64_t *lane_rank, uint32_t B, uint32_t l,
                              uint8_t *lane_inst, uint64_t *lane_g, cudaStream_t s);
-// Algorithm 2 acceptance of a batch's sorted records.  flag: R + 1 uint64 and
-// starts: R + 1 uint32 of scratch; scan_ws: scan workspace for R + 1 entries.
-// Algorithm 2's acceptance of a batch's sorted records; record r's lane bits
-// are hvals[2 * rec_val[r]].
-// row_flag (may be null): live-row offsets whose kRowFull bit is set with the
-// full bit of (v, i).
+// Algorithm 2's acceptance of a batch's sorted records where coins are drawn
+// in the searches; record r's lane bits are hvals[2 * rec_val[r]].
 cudaError_t launch_accept(const uint64_t *rec_key, const uint32_t *rec_val, const uint64_t *hvals, uint64_t R,
                           uint32_t tbits, const uint8_t *lane_inst, const uint64_t *lane_rank, uint32_t l, uint32_t k,
-                          uint8_t *lcnt, uint64_t *full, uint32_t *row_flag, uint64_t *X, uint32_t *xlen, DevCtl *ctl,
-                          cudaStream_t s);
+                          uint8_t *lcnt, uint64_t *full, uint64_t *X, uint32_t *xlen, DevCtl *ctl, cudaStream_t s);
 
 // recsort.cu: order a batch's R records by key, node by node.  cnt: n + 1
 // counters, all zero on entry and on return; off: n + 1 node offsets (out);

@@ -38,13 +38,16 @@ struct ReachShared {
     uint2 erase[kEraseCap];           // {pair, index entries}
     uint2 longs[kLongCap];
     uint32_t seen[kSeen];
-    uint32_t n_rows[3], n_erase, n_long;
+    uint32_t n_rows[3], n_erase, n_long, parked;
     unsigned long long visits, edges;
 };
 
+template <bool RES>
 struct Reach {
     const ReachArgs &A;
     ReachShared &sh;
+    const uint32_t *off, *rows;
+    uint64_t *mask, *pend;
     uint32_t inst;
     uint64_t bit;
     uint32_t par;                     // parity the new rows are written to
@@ -52,7 +55,7 @@ struct Reach {
     uint64_t visits = 0, edges = 0;   // per lane
 
     SKIM_DEV uint2 *spill_list(uint32_t p) const {
-        return A.list + (static_cast<uint64_t>(inst) * 2 + p) * A.cap;
+        return A.list + (static_cast<uint64_t>(blockIdx.x) * 2 + p) * A.cap;
     }
 
     // Warp-collective: lanes with `has` reach node x.
@@ -71,10 +74,10 @@ struct Reach {
             // independent requests, in flight together; an index is erased
             // only by the lane whose OR newly covers its pair, so reading its
             // length first is safe
-            const uint64_t old = atomicOr(reinterpret_cast<unsigned long long *>(&A.mask[x]), bit);
-            b = A.off[r];
-            len = A.off[r + 1] - b;
-            sl = A.seg_len[r];
+            const uint64_t old = atomicOr(reinterpret_cast<unsigned long long *>(&mask[x]), bit);
+            b = off[r];
+            len = off[r + 1] - b;
+            if (RES) sl = A.seg_len[r];
             fresh = !(old & bit);
         }
         visits += fresh ? 1 : 0;
@@ -90,13 +93,16 @@ struct Reach {
                     sh.front[par][at] = make_uint2(b, len);
                 } else if (at - kFrontCap < A.cap) {
                     spill_list(par)[at - kFrontCap] = make_uint2(b, len);
+                } else if (!RES) {  // parked: taken up when the frontier runs dry
+                    atomicOr(reinterpret_cast<unsigned long long *>(&pend[x]), bit);
+                    sh.parked = 1;
                 } else {  // parked: re-queued by the host
                     atomicOr(reinterpret_cast<unsigned long long *>(&A.pend_trav[x]), bit);
                     A.ctl->spill = 1;
                 }
             }
         }
-        if (fresh && sl) {
+        if (RES && fresh && sl) {
             const uint32_t at = atomicAdd(&sh.n_erase, 1u);
             if (at < kEraseCap)
                 sh.erase[at] = make_uint2(static_cast<uint32_t>(r), sl);
@@ -155,20 +161,47 @@ struct Reach {
             }
             const uint32_t sb = __shfl_sync(kFull, first, sl);
             const bool has = o < total;
-            visit(has, has ? A.rows[sb + o] : 0);
+            visit(has, has ? rows[sb + o] : 0);
         }
     }
 
     // Warp-collective: entries t, t + step, .. of a row (t of lane 0 the same
     // for the whole warp up to the lane).
     SKIM_DEV void sweep(uint32_t b, uint32_t len, uint32_t t, uint32_t step) {
-        uint32_t x = t < len ? A.rows[b + t] : 0;
+        uint32_t x = t < len ? rows[b + t] : 0;
         for (uint32_t k0 = t - (threadIdx.x & 31); k0 < len; k0 += step) {
             const uint32_t k = k0 + (threadIdx.x & 31);
-            const uint32_t xn = k + step < len ? A.rows[b + k + step] : 0;
+            const uint32_t xn = k + step < len ? rows[b + k + step] : 0;
             visit(k < len, x);
             x = xn;
         }
+    }
+
+    // Block-collective: rows parked for want of room become the frontier of
+    // level t, as many as it holds; returns how many.
+    SKIM_DEV uint32_t unpark(uint32_t t) {
+        __syncthreads();
+        if (threadIdx.x == 0) sh.parked = 0;
+        par = t & 1;
+        n_next = &sh.n_rows[t % 3];
+        __syncthreads();
+        for (uint32_t v0 = 0; v0 < A.n; v0 += kReachThreads) {
+            const uint32_t v = v0 + threadIdx.x;
+            const bool mine = v < A.n && (*reinterpret_cast<volatile uint64_t *>(&pend[v]) & bit);
+            if (!mine) continue;
+            const uint32_t at = atomicAdd(n_next, 1u);
+            if (at >= kFrontCap + A.cap) {
+                sh.parked = 1;
+                continue;
+            }
+            atomicAnd(reinterpret_cast<unsigned long long *>(&pend[v]), ~bit);
+            const uint64_t r = static_cast<uint64_t>(v) * A.l + inst;
+            const uint2 it = make_uint2(off[r], off[r + 1] - off[r]);
+            if (at < kFrontCap) sh.front[par][at] = it;
+            else spill_list(par)[at - kFrontCap] = it;
+        }
+        __syncthreads();
+        return min(sh.n_rows[t % 3], kFrontCap + A.cap);
     }
 
     // Block-collective: erase the kept index segments, a warp per segment (a
@@ -186,22 +219,35 @@ struct Reach {
     }
 };
 
-// Block i searches instance i from node x.  The wait of a level's barrier is
-// bounded like every other wait: a level that takes longer than the limit
-// ends the search with the error flag.
-__global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_t x) {
+// Block i searches instance i, from node x (RES: the residual search of seed
+// x) or from the pivots of instance i (blocks from l on: against the edges).  The wait of a level's barrier is bounded like every
+// other wait: a level that takes longer than the limit ends the search with
+// the error flag.
+template <bool RES>
+__global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_t x, const uint32_t *pivot,
+                                                            uint32_t starts, uint32_t *count) {
     extern __shared__ char s_raw[];
     ReachShared &sh = *reinterpret_cast<ReachShared *>(s_raw);
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    Reach R{A, sh, blockIdx.x, 1ull << blockIdx.x, 0, &sh.n_rows[0]};
+    const bool back = !RES && blockIdx.x >= A.l;
+    const uint32_t inst = back ? blockIdx.x - A.l : blockIdx.x;
+    Reach<RES> R{A, sh, back ? A.back_off : A.off, back ? A.back_rows : A.rows, back ? A.back_mask : A.mask,
+                 back ? A.back_pend : A.pend_trav, inst, 1ull << inst, 0, &sh.n_rows[0]};
     for (uint32_t q = threadIdx.x; q < kSeen; q += kReachThreads) sh.seen[q] = 0xFFFFFFFFu;
     if (threadIdx.x == 0) {
-        sh.n_rows[0] = sh.n_rows[1] = sh.n_rows[2] = sh.n_erase = sh.n_long = 0;
+        sh.n_rows[0] = sh.n_rows[1] = sh.n_rows[2] = sh.n_erase = sh.n_long = sh.parked = 0;
         sh.visits = sh.edges = 0;
-        if (blockIdx.x == 0) A.chosen[x] = 1;
+        if (RES && blockIdx.x == 0) A.chosen[x] = 1;
     }
     __syncthreads();
-    if (warp == 0) R.visit(lane == 0, x);
+    if (RES) {
+        if (warp == 0) R.visit(lane == 0, x);
+    } else {
+        for (uint32_t q0 = warp * 32; q0 < starts; q0 += kReachThreads) {
+            const bool in = q0 + lane < starts;
+            R.visit(in, in ? pivot[(q0 + lane) * 64 + inst] : 0);
+        }
+    }
     __syncthreads();
     // Level t reads its rows from parity t & 1 and their number from
     // n_rows[t % 3], adds the next level's to n_rows[(t + 1) % 3] and empties
@@ -210,7 +256,8 @@ __global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_
     // the wait limit) is handled behind it.
     uint64_t t_level = globaltimer();
     for (uint32_t t = 0;; t++) {
-        const uint32_t m = min(sh.n_rows[t % 3], kFrontCap + A.cap);
+        uint32_t m = min(sh.n_rows[t % 3], kFrontCap + A.cap);
+        if (!RES && m == 0 && sh.parked) m = R.unpark(t);
         if (m == 0) break;
         R.par = (t + 1) & 1;
         R.n_next = &sh.n_rows[(t + 1) % 3];
@@ -251,6 +298,10 @@ __global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_
         if (R.edges) atomicAdd(&sh.edges, R.edges);
     }
     __syncthreads();
+    if (!RES) {
+        if (threadIdx.x == 0) count[(back ? 64 : 0) + inst] = static_cast<uint32_t>(sh.visits);
+        return;
+    }
     if (threadIdx.x == 0) {
         if (sh.visits) {
             atomicAdd(&A.ctl->stats[kStFwdVisits], sh.visits);
@@ -263,11 +314,21 @@ __global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_
 }  // namespace
 
 cudaError_t launch_reach(const ReachArgs &a, uint32_t x, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_reach, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_reach<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(sizeof(ReachShared)));
     if (e != cudaSuccess) return e;
     note_launch();
-    k_reach<<<a.l, kReachThreads, sizeof(ReachShared), s>>>(a, x);
+    k_reach<true><<<a.l, kReachThreads, sizeof(ReachShared), s>>>(a, x, nullptr, 1, nullptr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reach_from(const ReachArgs &a, const uint32_t *pivot, uint32_t starts, uint32_t *count,
+                              cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(k_reach<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(sizeof(ReachShared)));
+    if (e != cudaSuccess) return e;
+    note_launch();
+    k_reach<false><<<2 * a.l, kReachThreads, sizeof(ReachShared), s>>>(a, 0, pivot, starts, count);
     return cudaGetLastError();
 }
 

@@ -21,6 +21,7 @@
 // Reverse searches of small batches use per-warp queues instead (k_rev_ring),
 // and residual searches keep a few items per block in shared memory (FwdRing).
 // Every wait is bounded by a timeout that sets an error flag.
+#include <algorithm>
 #include <type_traits>
 
 #include "internal.cuh"
@@ -400,7 +401,7 @@ SKIM_DEV unsigned ring_take(const TravArgs &A, FwdRing *R, unsigned freel, bool 
 // Live in-neighbour row of (u, lane j of word t) in the materialised instances.
 SKIM_DEV uint32_t live_row_len(const TravArgs &A, uint32_t u, uint32_t t, int j) {
     const uint64_t r = static_cast<uint64_t>(u) * A.l + A.lane_inst[static_cast<size_t>(t) * 64 + j];
-    return (A.loff[r + 1] & kRowMask) - (A.loff[r] & kRowMask);
+    return A.loff[r + 1] - A.loff[r];
 }
 
 // A materialised reverse item names its row directly: v = first entry of the
@@ -440,7 +441,7 @@ SKIM_DEV void push_rev(const TravArgs &A, Acc &acc, uint32_t u, uint32_t t, uint
             const int j = __ffsll(m) - 1;
             const uint32_t inst = A.lane_inst[static_cast<size_t>(t) * 64 + j];
             const uint64_t r = static_cast<uint64_t>(u) * A.l + inst;
-            const uint64_t b0 = A.loff[r] & kRowMask, b1 = A.loff[r + 1] & kRowMask;
+            const uint64_t b0 = A.loff[r], b1 = A.loff[r + 1];
             write_row_items(A, s + c, b0, b1, t, j, inst);
             c += n_chunks(static_cast<uint32_t>(b1 - b0));
         }
@@ -530,24 +531,34 @@ struct FwdSink {
 };
 
 // Warp-collective, materialised reverse searches: lanes with `act` reach node
-// u for lane j of word t (instance inst).  The row bounds of (u, inst) and the
-// pruning word are loaded together, before the visited-table update.
+// u for lane j of word t (instance inst).  The row bounds of (u, inst) are
+// loaded before the visited-table update, in a sketch build together with the
+// node's need word, which says whether the search goes on there and whether a
+// visit leaves a record: node << lbits | batch lane (not a `source`'s unless
+// `own`), or like a SKIM search one per table entry (`words`).
 template <class SK>
 SKIM_DEV void emit_rev_mat(const TravArgs &A, Acc &acc, SK &sk, bool act, uint32_t u, uint32_t t, int j,
-                           uint32_t inst) {
+                           uint32_t inst, bool source = false) {
     if (!__any_sync(kFull, act)) return;
     const uint64_t key = (static_cast<uint64_t>(u) << A.tbits) | t;
-    uint64_t b0 = 0, b1 = 0, h0 = 0, k0 = 0, v0 = 0;
+    uint64_t b0 = 0, b1 = 0, h0 = 0, k0 = 0, v0 = 0, nd = 0;
     if (act) {
-        // the first visited-table slot, and the row of (u, inst) with
-        // Algorithm 2's pruning flag: independent loads, in flight together
+        // the first visited-table slot and the row of (u, inst): independent
+        // loads, in flight together
         h0 = table_slot(key, A.tbits, A.hnode, A.hmask);
         load_slot(A.hkeys, h0, &k0, &v0);
         const uint64_t r = static_cast<uint64_t>(u) * A.l + inst;
-        const uint32_t w0 = A.loff[r], w1 = A.loff[r + 1];
-        b0 = w0 & kRowMask;
-        b1 = w1 & kRowMask;
-        if (A.prune && (w0 & kRowFull)) act = false;  // Algorithm 2: local sketch full
+        b0 = A.loff[r];
+        b1 = A.loff[r + 1];
+        if (A.need) {
+            nd = A.need[u];
+            if (!((nd >> inst) & 1ull)) act = false;
+            if (A.scc && ((A.scc[u] >> inst) & 1ull)) {
+                const uint32_t ln = A.lane_of[t * 64u + j];
+                if (act) atomicOr(&A.hit[ln >> 5], 1u << (ln & 31));
+                act = false;
+            }
+        }
     }
     const uint64_t bit = 1ull << j;
     bool fresh = false, first = false;
@@ -559,7 +570,11 @@ SKIM_DEV void emit_rev_mat(const TravArgs &A, Acc &acc, SK &sk, bool act, uint32
         else
             atomicOr(&A.ctl->err, kErrHash);
     }
-    sk.record(A, first, key, slot);
+    if (A.need && !A.words)
+        sk.record(A, fresh && nd == A.lmask && (!source || A.own),
+                  static_cast<uint64_t>(u) << A.lbits | A.lane_of[t * 64u + j], 0);
+    else
+        sk.record(A, first && (!A.need || nd == A.lmask), key, slot);
     acc.visits += fresh ? 1 : 0;
     const uint32_t ni = fresh ? n_chunks(static_cast<uint32_t>(b1 - b0)) : 0;
     sk.rows(A, acc, ni, b0, b1, t, j, inst, slot);
@@ -1186,7 +1201,7 @@ SKIM_DEV bool ring_take_sources(const TravArgs &A, Acc &acc, RingSink &sk, const
             atomicOr(reinterpret_cast<unsigned long long *>(&S.alive[j0 >> 6]),
                      static_cast<unsigned long long>(b) << (((j0 >> 5) & 1) * 32));
     }
-    emit_rev_mat(A, acc, sk, act, u, j >> 6, static_cast<int>(j & 63), i);
+    emit_rev_mat(A, acc, sk, act, u, j >> 6, static_cast<int>(j & 63), i, true);
     return true;
 }
 
@@ -1605,24 +1620,25 @@ __global__ void k_rev_sources(TravArgs A, const uint32_t *lane_pair, uint32_t B,
         }
         GlobalSink gsink;
         if (A.mat)
-            emit_rev_mat(A, acc, gsink, act, u, j >> 6, static_cast<int>(j & 63), i);
+            emit_rev_mat(A, acc, gsink, act, u, j >> 6, static_cast<int>(j & 63), i, true);
         else
             emit_rev<false>(A, acc, act, u, j >> 6, 1ull << (j & 63));
     }
     flush_acc(A, acc, false);
 }
 
-__global__ void k_respill_rev(TravArgs A, uint64_t R) {
-    const int lane = threadIdx.x & 31;
+// Parked reverse work, found by the table slots that hold it.
+__global__ void k_respill_rev(TravArgs A) {
+    const uint32_t lane = threadIdx.x & 31;
     const uint64_t warps = static_cast<uint64_t>(gridDim.x) * (blockDim.x / 32);
     const uint64_t tmask = (1ull << A.tbits) - 1;
-    for (uint64_t w = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); w * 32 < R; w += warps) {
-        const uint64_t r = w * 32 + lane;
-        uint64_t p = 0, slot = 0, key = 0;
-        if (r < R) {
-            slot = A.rec_val[r];
-            key = A.rec_key[r];
-            p = atomicExch(reinterpret_cast<unsigned long long *>(&A.pend[slot]), 0ull);
+    for (uint64_t w = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5); w * 32 <= A.hmask; w += warps) {
+        const uint64_t slot = w * 32 + lane;
+        uint64_t p = 0, key = 0;
+        if (slot <= A.hmask && A.pend[slot]) {
+            p = A.pend[slot];
+            A.pend[slot] = 0;
+            key = A.hkeys[2 * slot] - 1;
         }
         Acc acc;
         if (A.mat)
@@ -1679,13 +1695,10 @@ cudaError_t launch_rev_sources(const TravArgs &a, const uint32_t *lane_pair, uin
     return cudaGetLastError();
 }
 
-cudaError_t launch_respill_rev(const TravArgs &a, uint64_t R, cudaStream_t s) {
-    if (R == 0) return cudaSuccess;
-    uint64_t warps = (R + 31) / 32;
-    uint64_t blocks = (warps + 7) / 8;
-    if (blocks > 152 * 16) blocks = 152 * 16;
+cudaError_t launch_respill_rev(const TravArgs &a, cudaStream_t s) {
+    const uint64_t blocks = std::min<uint64_t>((a.hmask + 256) / 256, 152 * 16);
     note_launch();
-    k_respill_rev<<<static_cast<unsigned>(blocks), 256, 0, s>>>(a, R);
+    k_respill_rev<<<static_cast<unsigned>(blocks), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

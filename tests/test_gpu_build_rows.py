@@ -1,0 +1,85 @@
+"""The sketch build over materialised rows (build.cu) at the sizes where it can
+go wrong: row capacities (k at 64 and 255, fewer and more ranks than k), one
+instance and 64, components contracted in one graph and in many (uniform ranks
+and positions), walks that do not fit their scratch, tiny record and task
+tables, node ids past the 32-bit keys of the warps' reached sets.  Sketches are
+whole numbers and must equal the oracle's, or the build with coins drawn in the
+searches where the oracle would take too long."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(n, src, dst, l, k, model, p, mode=0, bl=0, seed=31):
+    import paper_1408_6282_gb300 as pkg
+    ks = synth.Keys.from_seed(seed)
+    pb = oracle.Problem(n, src, dst, l, k, model, p, ks.coin, ks.rank, ks.prob)
+    ox, oln, _ = oracle.build_sketches(pb, rank_mode=mode)
+    with pkg.Skim(n, src, dst, l, k, model, p, ks.coin, ks.rank, ks.prob, batch_lanes=bl, rank_mode=mode) as sk:
+        for _ in range(2):  # a context builds again from its own leftovers
+            sk.build_sketches()
+            x, ln = sk.sketches()
+            assert np.array_equal(ln, oln) and np.array_equal(x, ox)
+
+
+GRAPHS = {
+    "rmat12": lambda: synth.rmat(12, 16, 5),
+    "er5000": lambda: synth.erdos_renyi(5003, 40009, 6),
+    "cycle": lambda: synth.cycle(700),
+    "clique": lambda: synth.clique(90),
+}
+
+
+@pytest.mark.parametrize("name", list(GRAPHS))
+@pytest.mark.parametrize("l,k,model,p", [(64, 64, 0, 0.1), (64, 65, 1, 0.0), (33, 255, 0, 0.3), (1, 64, 0, 0.5),
+                                         (64, 2, 2, 0.0), (5, 7, 0, 1.0)])
+@pytest.mark.parametrize("mode,bl", [(0, 0), (1, 0), (0, 100)])
+def test_rows_match_oracle(name, l, k, model, p, mode, bl):
+    g = GRAPHS[name]()
+    _check(g.n, g.src, g.dst, l, k, model, p, mode, bl)
+
+
+@pytest.mark.parametrize("hook,value", [("SKIM_QUEUE_ITEMS", "600"), ("SKIM_RECORD_ITEMS", "4096")])
+@pytest.mark.parametrize("name", ["rmat12", "cycle"])
+def test_small_scratch(monkeypatch, hook, value, name):
+    monkeypatch.setenv(hook, value)
+    g = GRAPHS[name]()
+    _check(g.n, g.src, g.dst, 16, 16, 0, 0.2)
+
+
+@pytest.mark.parametrize("count", [2, 70])
+def test_components_of_many_graphs(count):
+    """A component, hit lists and pivots per graph; sizes from one node up."""
+    import paper_1408_6282_gb300 as pkg
+    gs = [synth.empty_graph(1), synth.clique(40)] + [synth.rmat(6 + g % 4, 12, 900 + g) for g in range(count)]
+    l, k = 64, 32
+    keys = [synth.Keys.from_seed(200 + g) for g in range(len(gs))]
+    models = [g % 3 for g in range(len(gs))]
+    with pkg.Skim.batch([(g.n, g.src, g.dst) for g in gs], l, k, models, [0.3] * len(gs), [q.coin for q in keys],
+                        [q.rank for q in keys], [q.prob for q in keys]) as sk:
+        sk.build_sketches()
+        x, ln = sk.sketches()
+        for g, m, q, o in zip(gs, models, keys, sk.offsets):
+            pb = oracle.Problem(g.n, g.src, g.dst, l, k, m, 0.3, q.coin, q.rank, q.prob)
+            ox, oln, _ = oracle.build_sketches(pb)
+            assert np.array_equal(ln[o:o + g.n], oln) and np.array_equal(x[o:o + g.n], ox)
+
+
+def test_node_ids_past_24_bits():
+    """2^24 + 9 nodes with edges among the highest ids (64-bit reached-set keys),
+    against the build with coins drawn in the searches."""
+    import paper_1408_6282_gb300 as pkg
+    n = (1 << 24) + 9
+    g = synth.rmat(15, 8, 77)
+    src, dst = g.src + np.uint32(n - g.n), g.dst + np.uint32(n - g.n)
+    with pkg.Skim(n, src, dst, 2, 8, 0, 0.25, 3, 4, 5) as sk:
+        sk.build_sketches()
+        x, ln = sk.sketches()
+        sk.set_live_rows(False)
+        sk.build_sketches()
+        y, lm = sk.sketches()
+        assert np.array_equal(ln, lm) and np.array_equal(x, y)
