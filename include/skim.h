@@ -355,9 +355,9 @@ int skim_context_shape(skim_ctx *ctx, uint32_t *n, uint32_t *k, uint32_t *l);
 /* ---- Serving: the influence oracle as a continuous-batching request loop ----
  * (queries of Section 5.1, Eq. unionest, over sketches resident on the GPU).
  * A server thread admits submitted seed sets into launch groups while
- * in-flight slots (max_inflight queries) and scratch memory (scratch_slots
- * hash-table slots of 16 bytes, split over `streams` streams; a query of |S|
- * seeds needs the next power of two >= 2|S|(k-1)+2) allow, and launches each
+ * in-flight slots (max_inflight queries) and hash-table slots (scratch_slots,
+ * split over `streams` streams; a query of |S| seeds counts as the next power
+ * of two >= 2|S|(k-1)+2) allow, and launches each
  * group on a free stream.  Groups on different streams run concurrently; a
  * request that arrives while others are on the GPU joins the next group as
  * soon as slots and memory free up.  Each result is bitwise identical to

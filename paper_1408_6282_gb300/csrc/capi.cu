@@ -139,15 +139,13 @@ struct skim_ctx {
     bool pend_res = false;
     uint64_t *pend_cov = nullptr;
     // queries
-    uint64_t *qk = nullptr, *qv = nullptr;
-    uint64_t qtcap = 0;
     uint32_t *qseeds = nullptr;
     uint64_t qseeds_cap = 0;
-    uint64_t *qoff = nullptr;  // seed, table and chunk offsets (3 x (q+1))
+    uint64_t *qoff = nullptr;  // seed and block offsets (2 x (q+1))
     double *qout = nullptr;
+    double *hq = nullptr;        // pinned, behind hctl: a single query's estimate
     uint64_t qmeta_cap = 0;
-    uint64_t *qtop = nullptr;
-    unsigned *qtopu = nullptr;
+    unsigned *qdone = nullptr;   // finished blocks per query, zero between calls
     void *qpart = nullptr;
     uint64_t qpart_cap = 0;
     // counters of the last build/greedy call
@@ -997,43 +995,35 @@ int rank_order(skim_ctx *c) {
     return SKIM_OK;
 }
 
-int ensure_query_space(skim_ctx *c, uint64_t seeds, uint64_t q, uint64_t table, uint64_t chunks) {
-    if (chunks > c->qpart_cap) {
+int ensure_query_space(skim_ctx *c, uint64_t seeds, uint64_t q, uint64_t blocks) {
+    if (blocks > c->qpart_cap) {
         dfree(c, c->qpart);
-        c->qpart_cap = std::max<uint64_t>(chunks, 1024);
-        const int rc = dalloc_bytes(c, &c->qpart, c->qpart_cap * query_partial_bytes());
-        if (rc != SKIM_OK) {
-            c->qpart_cap = 0;
-            return rc;
-        }
+        c->qpart_cap = 0;
+        const uint64_t cap = std::max<uint64_t>(blocks, 1024);
+        RC(dalloc_bytes(c, &c->qpart, cap * query_partial_bytes()));
+        c->qpart_cap = cap;
     }
     if (seeds > c->qseeds_cap) {
         dfree(c, c->qseeds);
-        c->qseeds_cap = std::max<uint64_t>(seeds, 4096);
-        RC(dalloc(c, &c->qseeds, c->qseeds_cap));
+        c->qseeds_cap = 0;
+        const uint64_t cap = std::max<uint64_t>(seeds, 4096);
+        RC(dalloc(c, &c->qseeds, cap));
+        c->qseeds_cap = cap;
     }
     if (q + 1 > c->qmeta_cap) {
         dfree(c, c->qoff);
         dfree(c, c->qout);
-        dfree(c, c->qtop);
-        dfree(c, c->qtopu);
-        c->qmeta_cap = std::max<uint64_t>(q + 1, 1024);
-        RC(dalloc(c, &c->qoff, 3 * c->qmeta_cap));  // seed, table and chunk offsets in one upload
-        RC(dalloc(c, &c->qout, c->qmeta_cap));
-        RC(dalloc(c, &c->qtop, c->qmeta_cap));
-        RC(dalloc(c, &c->qtopu, c->qmeta_cap));
-    }
-    if (table > c->qtcap) {
-        dfree(c, c->qk);
-        dfree(c, c->qv);
-        c->qtcap = std::max<uint64_t>(table, 1ull << 16);
-        RC(dalloc(c, &c->qk, c->qtcap));
-        RC(dalloc(c, &c->qv, c->qtcap));
+        dfree(c, c->qdone);
+        c->qmeta_cap = 0;
+        const uint64_t cap = std::max<uint64_t>(q + 1, 1024);
+        RC(dalloc(c, &c->qoff, 2 * cap));  // seed and block offsets in one upload
+        RC(dalloc(c, &c->qout, cap));
+        RC(dalloc(c, &c->qdone, cap));
+        CK(c, cudaMemsetAsync(c->qdone, 0, cap * sizeof(unsigned), c->st));
+        c->qmeta_cap = cap;
     }
     return SKIM_OK;
 }
-
-uint64_t query_table(uint64_t s, uint32_t k) { return pow2_at_least(std::max<uint64_t>(64, 2 * s * (k - 1) + 2)); }
 
 }  // namespace
 
@@ -1086,8 +1076,8 @@ int skim_destroy(skim_ctx *c) {
     dfree(c, c->rmask); dfree(c, c->fmask); dfree(c, c->loff); dfree(c, c->rlive); dfree(c, c->rrow); dfree(c, c->rev2fwd);
     dfree(c, c->foff); dfree(c, c->flive);
     dfree(c, c->pieces);
-    dfree(c, c->qk); dfree(c, c->qv); dfree(c, c->qseeds); dfree(c, c->qoff); dfree(c, c->qout);
-    dfree(c, c->qtop); dfree(c, c->qtopu);
+    dfree(c, c->qseeds); dfree(c, c->qoff); dfree(c, c->qout);
+    dfree(c, c->qdone);
     dfree(c, c->qpart);
     for (auto &p : c->kpend) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
     for (auto e : c->kpool) cudaEventDestroy(e);
@@ -1166,7 +1156,8 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
     } while (0)
     {
         TRY(dalloc(c, &c->ctl, 1));
-        TRYC(cudaMallocHost(reinterpret_cast<void **>(&c->hctl), sizeof(DevCtl)));
+        TRYC(cudaMallocHost(reinterpret_cast<void **>(&c->hctl), sizeof(DevCtl) + sizeof(double)));
+        c->hq = reinterpret_cast<double *>(c->hctl + 1);
         TRYC(cudaMemsetAsync(c->ctl, 0, sizeof(DevCtl), c->st));
         TRY(dalloc(c, &c->dflag, 1));
         // edges on the device
@@ -2086,15 +2077,13 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
     if (!c->built) return SKIM_ENOTBUILT;
     if (q == 0) return SKIM_OK;
     if (offsets[0] != 0) return SKIM_EINVAL;
-    // one host block: seed offsets | table offsets | chunk offsets
+    // one host block: seed offsets | block offsets
     const size_t q1 = static_cast<size_t>(q) + 1;
-    std::vector<uint64_t> meta(3 * q1, 0);
-    uint64_t *toff = meta.data() + q1, *coff = meta.data() + 2 * q1;
+    std::vector<uint64_t> meta(2 * q1, 0);
+    uint64_t *boff = meta.data() + q1;
     for (uint32_t i = 0; i < q; i++) {
         if (offsets[i + 1] < offsets[i]) return SKIM_EINVAL;
-        const uint64_t H = query_table(offsets[i + 1] - offsets[i], c->k);
-        toff[i + 1] = toff[i] + H;
-        coff[i + 1] = coff[i] + query_chunks(H);
+        boff[i + 1] = boff[i] + query_blocks(offsets[i + 1] - offsets[i], c->k);
     }
     std::copy(offsets, offsets + q1, meta.data());
     const uint64_t total = offsets[q];
@@ -2103,35 +2092,51 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
         for (uint64_t i = 0; i < total; i++)
             if (seeds[i] >= c->n) return SKIM_EINVAL;
     }
-    RC(ensure_query_space(c, total, q, toff[q], coff[q]));
+    RC(ensure_query_space(c, total, q, boff[q]));
     const uint32_t *dseeds = seeds;
     if (!on_device && total) {
         CK(c, cudaMemcpyAsync(c->qseeds, seeds, total * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st));
         dseeds = c->qseeds;
     }
-    uint64_t *d_off = c->qoff, *d_toff = c->qoff + q1, *d_coff = c->qoff + 2 * q1;
+    uint64_t *d_off = c->qoff, *d_boff = c->qoff + q1;
     CK(c, cudaMemcpyAsync(d_off, meta.data(), meta.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, c->st));
-    CK(c, cudaMemsetAsync(c->dflag, 0, sizeof(unsigned), c->st));
+    unsigned *flag = c->dflag;
+    CK(c, cudaMemsetAsync(flag, 0, sizeof(unsigned), c->st));
     double *dout = on_device ? est_out : c->qout;
     {
         KTimer kt(c, SKIM_K_QUERY);
-        QueryScratch qs{c->qk, c->qv, c->qtop, c->qtopu, c->qpart, c->dflag};
-        CK(c, launch_query_multi(c->X, c->xlen, c->n, c->k, query_terms_of(c), dseeds, d_off, d_toff, d_coff, q, toff[q], total,
-                                 static_cast<uint32_t>(coff[q]), qs, dout, c->st));
+        QueryScratch qs{c->qpart, c->qdone, flag};
+        CK(c, launch_query_multi(c->X, c->xlen, c->n, c->k, query_terms_of(c), dseeds, d_off, d_boff, q,
+                                 static_cast<uint32_t>(boff[q]), qs, dout, c->st));
     }
     unsigned bad = 0;
-    CK(c, cudaMemcpyAsync(&bad, c->dflag, sizeof(unsigned), cudaMemcpyDeviceToHost, c->st));
+    CK(c, cudaMemcpyAsync(&bad, flag, sizeof(unsigned), cudaMemcpyDeviceToHost, c->st));
     if (!on_device)
         CK(c, cudaMemcpyAsync(est_out, c->qout, q * sizeof(double), cudaMemcpyDeviceToHost, c->st));
     CK(c, cudaStreamSynchronize(c->st));
     resolve_timers(c);
+    if (bad & 2u) return fail_cuda(c, cudaErrorUnknown);
     return bad ? SKIM_EINVAL : SKIM_OK;
 }
 
 int skim_oracle_query(skim_ctx *c, const uint32_t *seeds, uint32_t n_seeds, double *est_out) {
     if (!c || !est_out || (n_seeds && !seeds)) return SKIM_EINVAL;
-    uint64_t off[2] = {0, n_seeds};
-    return skim_oracle_query_batch(c, off, 1, seeds, est_out, 0);
+    if (c->broken) return SKIM_ECUDA;
+    if (!c->built) return SKIM_ENOTBUILT;
+    if (!query_fits_args(n_seeds, c->k)) {
+        uint64_t off[2] = {0, n_seeds};
+        return skim_oracle_query_batch(c, off, 1, seeds, est_out, 0);
+    }
+    for (uint32_t i = 0; i < n_seeds; i++)
+        if (seeds[i] >= c->n) return SKIM_EINVAL;
+    {
+        KTimer kt(c, SKIM_K_QUERY);
+        CK(c, launch_query_one(c->X, c->xlen, c->n, c->k, query_terms_of(c), seeds, n_seeds, c->hq, c->st));
+    }
+    CK(c, cudaStreamSynchronize(c->st));
+    resolve_timers(c);
+    *est_out = *c->hq;
+    return SKIM_OK;
 }
 
 int skim_kernel_launches(uint64_t *out) {

@@ -307,18 +307,15 @@ cudaError_t launch_second_size(const uint32_t *idx_nodes, const uint64_t *idx_ba
                                uint32_t *out, cudaStream_t s);
 
 // query.cu
-// Scratch of the multi-block query path: hash tables (total_slots keys and
-// values), per-query top-rank slots, per-chunk partial sums, an error flag.
+// Scratch of the queries: per-block partial sums, counters of the larger queries'
+// finished blocks (zero between calls), an error flag.
 struct QueryScratch {
-    uint64_t *hkeys;
-    uint64_t *hvals;
-    uint64_t *top_tau;
-    unsigned *top_used;
     void *partial;
+    unsigned *done;
     unsigned *err;
 };
-uint32_t query_chunks(uint64_t table_slots);  // chunks of one query's table
-size_t query_partial_bytes();                  // bytes per chunk partial
+uint32_t query_blocks(uint64_t seeds, uint32_t k);  // blocks of a larger query, 0 for one that takes a single block
+size_t query_partial_bytes();
 // How a threshold becomes a term of Eq. unionest, and the final divisor:
 //  mode 0 (uniform 64-bit ranks): 1 / (h * 2^-64), divided by l;
 //  mode 1 (structured permutation, Section 3.1): num / h with num = n*l - 1,
@@ -333,9 +330,14 @@ struct QueryTerms {
 QueryTerms query_terms_of(const skim_ctx *c);
 cudaError_t launch_node_estimates(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, uint32_t l,
                                   int mode, double *out, cudaStream_t s);
+// block_off: prefix sums of query_blocks; blocks: their total
 cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
-                               const uint32_t *seeds, const uint64_t *offsets, const uint64_t *table_off,
-                               const uint64_t *chunk_off, uint32_t q, uint64_t total_slots, uint64_t total_seeds,
-                               uint32_t total_chunks, const QueryScratch &qs, double *out, cudaStream_t s);
+                               const uint32_t *seeds, const uint64_t *offsets, const uint64_t *block_off, uint32_t q,
+                               uint32_t blocks, const QueryScratch &qs, double *out, cudaStream_t s);
+// One query with few enough seeds (host) to be kernel arguments; out_host: pinned.
+constexpr uint32_t kQueryArgSeeds = 960;
+bool query_fits_args(uint64_t seeds, uint32_t k);
+cudaError_t launch_query_one(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
+                             const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st);
 
 }  // namespace skim

@@ -5,7 +5,7 @@
 // is divided by l.  tau_u is the k-th smallest rank of a full sketch and 1 for
 // a sketch with fewer than k ranks (Eq. combinedthresh).
 //
-// A hash table per query in global scratch keeps, per distinct z, the
+// A hash table per query keeps, per distinct z, the
 // largest tau (as a 64-bit integer; the integer order equals the order of
 // the reals h/2^64 and the rounding to double is monotone).  Each term 1/tau is
 // formed in double exactly as h -> double -> scale by 2^-64 -> 1/x, then added
@@ -58,15 +58,13 @@ SKIM_DEV double term_of(const QueryTerms &t, uint64_t h) {
 
 // exact fixed-point image (value * 2^64) of a double in [2^-12, 2^64]
 SKIM_DEV U192 to_fixed(double v) {
-    uint64_t bits = static_cast<uint64_t>(__double_as_longlong(v));
-    int e = static_cast<int>((bits >> 52) & 0x7ff) - 1023;
-    uint64_t mant = (bits & ((1ull << 52) - 1)) | (1ull << 52);
-    int sh = e + 12;  // value * 2^64 = mant * 2^(e - 52 + 64)
-    U192 r{{0, 0, 0}};
-    int q = sh >> 6, rb = sh & 63;
-    r.w[q] = mant << rb;
-    if (rb && q + 1 < 3) r.w[q + 1] = mant >> (64 - rb);
-    return r;
+    const uint64_t bits = static_cast<uint64_t>(__double_as_longlong(v));
+    const int e = static_cast<int>((bits >> 52) & 0x7ff) - 1023;
+    const uint64_t mant = (bits & ((1ull << 52) - 1)) | (1ull << 52);
+    const int sh = e + 12;  // value * 2^64 = mant * 2^(e - 52 + 64)
+    const int q = sh >> 6, rb = sh & 63;
+    const uint64_t lo = mant << rb, hi = rb ? mant >> (64 - rb) : 0;
+    return U192{{q == 0 ? lo : 0, q == 0 ? hi : q == 1 ? lo : 0, q == 1 ? hi : q == 2 ? lo : 0}};
 }
 
 SKIM_DEV int top_bit(const U192 &a) {
@@ -93,8 +91,10 @@ SKIM_DEV double fixed_to_double(const U192 &a) {
     if (p < 0) return 0.0;
     if (p <= 52) return ldexp(static_cast<double>(a.w[0]), -64);
     int sh = p - 52;
-    uint64_t mant = 0;
-    for (int b = 0; b < 53; b++) mant |= bit_at(a, sh + b) << b;
+    const int w = sh >> 6, b = sh & 63;
+    uint64_t mant = a.w[w] >> b;
+    if (b && w + 1 < 3) mant |= a.w[w + 1] << (64 - b);
+    mant &= (1ull << 53) - 1;
     bool rnd = bit_at(a, sh - 1);
     bool sticky = any_below(a, sh - 1);
     if (rnd && (sticky || (mant & 1ull))) {
@@ -107,12 +107,38 @@ SKIM_DEV double fixed_to_double(const U192 &a) {
     return ldexp(static_cast<double>(mant), sh - 64);
 }
 
-// ---- multi-block form: the work of a group of queries is spread over the
-// whole GPU.  Each query owns a hash table of H_q slots (a power of two) in
-// one scratch array; table q is cut into chunks of kQChunk slots whose
-// partial sums (exact, 192-bit) are added per query at the end.
+// ---- hash tables of rank -> term -------------------------------------------------
+//
+// A slot holds a rank and the term of the threshold it is charged to, as the
+// double's bits (all ones: empty).  Terms fall as thresholds rise, in every
+// rank reading, so the largest threshold of equal ranks is the smallest term, and
+// the order of non-negative doubles is that of their bits.  So the one division
+// is made per seed, 32 at a time (FP64 runs at a thirty-second of the integer
+// rate), and not per rank.
+//
+// The table is in shared memory.  A query of up to kSmallEntries ranks takes one
+// block; a larger one is cut by the hash of the rank into parts of about
+// kPartEntries, a block each: every block reads all of the query's sketches (from
+// L2 after the first) and keeps the ranks of its part, so nothing is scattered
+// through global memory, and the last block of a query adds the parts.  A part that
+// does not fit its table is cut finer and read again.
+//
+// Measured: 1000 queries of 1 to 1000 seeds (145 K sketches of 64 ranks, R-MAT 20),
+// kernels: 1.03 ms with a table per query in global memory (two arrays, two
+// atomics per rank, a pass to clear and one to sum), 0.66 ms with 16-byte slots and
+// terms per seed there (0.54 ms of it the atomics: 15 G/s, also where the tables
+// stay in L2), 0.44 ms so (0.58 ms before a warp collected 32 ranks of its part).  One query of 10 seeds, host to host: 48 us with four
+// kernels, two uploads and two downloads, 19 us with one kernel that has the seeds
+// as arguments and writes the estimate to host memory.
 
-constexpr uint32_t kQChunk = 2048;
+constexpr uint32_t kSmallEntries = 2700, kSmallSlots = 4095;  // 64 KB: three blocks per SM
+constexpr int kSmallThreads = 256;
+#ifndef SKIM_PART_ENTRIES
+#define SKIM_PART_ENTRIES 8000
+#endif
+constexpr uint32_t kPartEntries = SKIM_PART_ENTRIES, kPartSlots = 12287;   // 192 KB
+constexpr int kPartThreads = 1024;
+constexpr uint32_t kStage = 64;  // pairs a warp collects
 
 SKIM_DEV uint32_t upper_bound_u64(const uint64_t *a, uint32_t n, uint64_t x) {  // first i with a[i] > x
     uint32_t lo = 0, hi = n;
@@ -124,101 +150,203 @@ SKIM_DEV uint32_t upper_bound_u64(const uint64_t *a, uint32_t n, uint64_t x) {  
     return lo;
 }
 
-__global__ void k_q_clear(uint64_t *hkeys, uint64_t *hvals, uint64_t total, unsigned long long *top_tau,
-                          unsigned *top_used, uint32_t q) {
-    for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < total;
-         i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        hkeys[i] = kEmptyKey;
-        hvals[i] = 0;
+// Rank z (hash h) with stored term t into a table of H slots: the smallest term
+// of equal ranks stays.  False if the table is full.
+SKIM_DEV uint32_t rank_hash(uint64_t z) {
+    uint32_t h = static_cast<uint32_t>(z ^ (z >> 32)) * 0x9E3779B1u;
+    h = (h ^ (h >> 15)) * 0x85EBCA77u;
+    return h ^ (h >> 13);
+}
+SKIM_DEV bool table_put(uint64_t *keys, uint64_t *terms, uint32_t H, uint32_t at, uint64_t z, uint64_t t) {
+    if (z == kEmptyKey) at = H;  // a place of its own
+    for (uint32_t p = 0; p < H; p++) {
+        uint64_t k = *reinterpret_cast<volatile uint64_t *>(&keys[at]);
+        if (k == kEmptyKey && at != H)
+            k = atomicCAS(reinterpret_cast<unsigned long long *>(&keys[at]), kEmptyKey, z);
+        if (k == kEmptyKey || k == z) {
+            if (*reinterpret_cast<volatile uint64_t *>(&terms[at]) > t)
+                atomicMin(reinterpret_cast<unsigned long long *>(&terms[at]), t);
+            return true;
+        }
+        if (++at == H) at = 0;
     }
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < q; i += gridDim.x * blockDim.x) {
-        top_tau[i] = 0;
-        top_used[i] = 0;
-    }
+    return false;
 }
 
-__global__ void k_q_insert(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const uint32_t *seeds,
-                           const uint64_t *offsets, const uint64_t *table_off, uint32_t q, uint64_t *hkeys,
-                           uint64_t *hvals, unsigned long long *top_tau, unsigned *top_used, unsigned *err) {
-    const uint64_t total = offsets[q] * k;
-    for (uint64_t e = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; e < total;
-         e += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const uint64_t j = e / k;
-        const uint32_t pos = static_cast<uint32_t>(e % k);
-        const uint32_t u = seeds[j];
-        if (u >= n) {
-            atomicOr(err, 1u);
-            continue;
-        }
-        const uint32_t ln = xlen[u];
-        const uint32_t body = ln == k ? k - 1 : ln;
-        if (pos >= body) continue;
-        const uint32_t qi = upper_bound_u64(offsets + 1, q, j);  // query holding seed j
-        const uint64_t z = X[static_cast<uint64_t>(u) * k + pos];
-        const uint64_t tau = ln == k ? X[static_cast<uint64_t>(u) * k + k - 1] : ~0ull;
-        if (z == kEmptyKey) {
-            atomicMax(&top_tau[qi], static_cast<unsigned long long>(tau));
-            top_used[qi] = 1;
-            continue;
-        }
-        const uint64_t base = table_off[qi], H = table_off[qi + 1] - base;
-        uint64_t *tk = hkeys + base;
-        uint64_t *tv = hvals + base;
-        uint64_t h = fmix(z) & (H - 1);
-        for (uint64_t p = 0; p < H; p++) {
-            unsigned long long prev = atomicCAS(reinterpret_cast<unsigned long long *>(&tk[h]),
-                                                static_cast<unsigned long long>(kEmptyKey),
-                                                static_cast<unsigned long long>(z));
-            if (prev == kEmptyKey || prev == z) {
-                atomicMax(reinterpret_cast<unsigned long long *>(&tv[h]), static_cast<unsigned long long>(tau));
-                break;
-            }
-            h = (h + 1) & (H - 1);
-        }
-    }
+// What a lane has of its seed: the row, its ranks below the threshold, the
+// stored term.
+struct SeedRow {
+    uint32_t u, body;
+    uint64_t term;
+};
+SKIM_DEV SeedRow seed_row(const uint64_t *X, const uint32_t *xlen, uint32_t k, const QueryTerms &terms, uint32_t u) {
+    const uint32_t ln = xlen[u];
+    const uint64_t tau = ln == k ? X[static_cast<uint64_t>(u) * k + k - 1] : ~0ull;
+    return SeedRow{u, ln == k ? k - 1 : ln, static_cast<uint64_t>(__double_as_longlong(term_of(terms, tau)))};
 }
 
-// one block per chunk: partial[c] = exact sum of the chunk's terms
-__global__ void __launch_bounds__(256) k_q_sum(const uint64_t *hkeys, const uint64_t *hvals, const uint64_t *table_off,
-                                               const uint64_t *chunk_off, uint32_t q,
-                                               const unsigned long long *top_tau, const unsigned *top_used,
-                                               QueryTerms terms, U192 *partial) {
-    __shared__ U192 wsum[8];
-    const uint32_t c = blockIdx.x;
-    const uint32_t qi = upper_bound_u64(chunk_off + 1, q, c);
-    const uint64_t first = chunk_off[qi];
-    const uint64_t lo = table_off[qi] + (c - first) * kQChunk;
-    const uint64_t hi = min(lo + kQChunk, table_off[qi + 1]);
-    U192 acc{{0, 0, 0}};
-    for (uint64_t i = lo + threadIdx.x; i < hi; i += blockDim.x)
-        if (hkeys[i] != kEmptyKey) {
-            const double v = term_of(terms, hvals[i]);
-            if (v != 0.0) add192(acc, to_fixed(v));
-        }
-    if (c == first && threadIdx.x == 0 && top_used[qi]) {
-        const double v = term_of(terms, top_tau[qi]);
-        if (v != 0.0) add192(acc, to_fixed(v));
-    }
+SKIM_DEV U192 warp_sum192(U192 a) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         U192 other;
-        for (int w = 0; w < 3; w++) other.w[w] = __shfl_down_sync(kFull, acc.w[w], o);
-        add192(acc, other);
+        for (int w = 0; w < 3; w++) other.w[w] = __shfl_down_sync(kFull, a.w[w], o);
+        add192(a, other);
     }
-    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        U192 tot{{0, 0, 0}};
-        for (int w = 0; w < 8; w++) add192(tot, wsum[w]);
-        partial[c] = tot;
-    }
+    return a;
 }
 
-__global__ void k_q_final(const U192 *partial, const uint64_t *chunk_off, uint32_t q, double div, double *out) {
-    for (uint32_t qi = blockIdx.x * blockDim.x + threadIdx.x; qi < q; qi += gridDim.x * blockDim.x) {
-        U192 tot{{0, 0, 0}};
-        for (uint64_t c = chunk_off[qi]; c < chunk_off[qi + 1]; c++) add192(tot, partial[c]);
-        out[qi] = fixed_to_double(tot) / div;
+SKIM_DEV void add_term(U192 &acc, uint64_t stored) {
+    if (stored != kEmptyKey && stored) add192(acc, to_fixed(__longlong_as_double(static_cast<long long>(stored))));
+}
+
+// Block-collective: the exact sum over the ranks of a query whose hash lies in
+// part `part` of `parts` (thread 0's return value), table of H + 1 slots in tab.
+// PART: a row has few ranks of the part, so a warp collects 32 before it goes to
+// the table (kStage pairs per warp behind it).
+template <bool PART>
+SKIM_DEV U192 query_block(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
+                          const uint32_t *seeds, uint32_t s, uint64_t part, uint64_t parts, uint64_t *tab, uint32_t H,
+                          unsigned *err) {
+    __shared__ U192 wsum[32];
+    const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5, lane = threadIdx.x & 31;
+    uint64_t *keys = tab, *val = tab + H + 1;
+    ulonglong2 *st = reinterpret_cast<ulonglong2 *>(val + H + 1) + warp * kStage;
+    U192 acc{{0, 0, 0}};
+    for (uint64_t cut = 1, c = 0; c < cut;) {  // one piece, unless the table overflows
+        const uint64_t pieces = parts * cut, piece = part * cut + c;
+        const uint64_t lo = (piece << 32) / pieces, hi = ((piece + 1) << 32) / pieces;  // of the 32-bit hash
+        const uint32_t lo32 = static_cast<uint32_t>(lo), last = static_cast<uint32_t>(hi - lo - 1);
+        const uint64_t scale = (static_cast<uint64_t>(H) << 32) / (hi - lo);           // hash - lo -> slot
+        for (uint32_t i = threadIdx.x; i <= H; i += blockDim.x) keys[i] = val[i] = kEmptyKey;
+        __syncthreads();
+        bool full = false;
+        uint32_t nst = 0;
+        const auto slot_of = [&](uint32_t h) { return min(H - 1, static_cast<uint32_t>(((h - lo32) * scale) >> 32)); };
+        for (uint32_t j0 = 0; j0 + warp < s; j0 += warps * 32) {  // lane i: seed j0 + i warps + warp
+            const uint32_t j = j0 + lane * warps + warp;
+            SeedRow r{0, 0, 0};
+            if (j < s) {
+                const uint32_t u = seeds[j];
+                if (u < n) r = seed_row(X, xlen, k, terms, u);
+                else atomicOr(err, 1u);
+            }
+            const uint32_t cnt = min(32u, (s - j0 - warp + warps - 1) / warps);
+            for (uint32_t i = 0; i < cnt; i++) {
+                const uint32_t u = __shfl_sync(kFull, r.u, i), body = __shfl_sync(kFull, r.body, i);
+                const uint64_t t = __shfl_sync(kFull, r.term, i);
+                const uint64_t *row = X + static_cast<uint64_t>(u) * k;
+                for (uint32_t p0 = 0; p0 < body; p0 += 32) {
+                    const bool in = p0 + lane < body;
+                    const uint64_t z = in ? row[p0 + lane] : 0;
+                    const uint32_t h = rank_hash(z);
+                    const bool mine = in && h - lo32 <= last;
+                    if (!PART) {
+                        if (mine) full |= !table_put(keys, val, H, slot_of(h), z, t);
+                        continue;
+                    }
+                    const unsigned mb = __ballot_sync(kFull, mine);
+                    if (mine) st[nst + __popc(mb & lanemask_lt())] = make_ulonglong2(z, t);
+                    nst += __popc(mb);
+                    __syncwarp();
+                    if (nst < 32) continue;
+                    const ulonglong2 e = st[lane];
+                    full |= !table_put(keys, val, H, slot_of(rank_hash(e.x)), e.x, e.y);
+                    __syncwarp();
+                    if (lane < nst - 32) st[lane] = st[lane + 32];
+                    nst -= 32;
+                    __syncwarp();
+                }
+            }
+        }
+        if (PART && lane < nst) full |= !table_put(keys, val, H, slot_of(rank_hash(st[lane].x)), st[lane].x, st[lane].y);
+        if (__syncthreads_or(full)) {
+            if (hi - lo < 2) {  // (thousands of ranks of one hash)
+                if (threadIdx.x == 0 && err) atomicOr(err, 2u);
+                break;
+            }
+            cut *= 2;  // the pieces done so far stay done
+            c *= 2;
+            continue;
+        }
+        for (uint32_t i = threadIdx.x; i <= H; i += blockDim.x) add_term(acc, val[i]);
+        c++;
+        if (c < cut) __syncthreads();
+    }
+    acc = warp_sum192(acc);
+    if (lane == 0) wsum[warp] = acc;
+    __syncthreads();
+    if (warp == 0) {
+        U192 t{{0, 0, 0}};
+        if (threadIdx.x < warps) t = wsum[threadIdx.x];
+        acc = warp_sum192(t);
+    }
+    return acc;
+}
+
+SKIM_HD uint32_t small_slots(uint64_t entries) { return static_cast<uint32_t>(entries + entries / 2 + 32); }
+
+// One query whose seeds are kernel arguments; the estimate goes to host memory.
+template <uint32_t CAP>
+struct SeedArgs {
+    uint32_t s;
+    uint32_t seeds[CAP];
+};
+template <uint32_t CAP>
+__global__ void __launch_bounds__(1024) k_q_one(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k,
+                                                QueryTerms terms, const __grid_constant__ SeedArgs<CAP> a, double *out) {
+    extern __shared__ ulonglong2 s_tab[];
+    const U192 e = query_block<false>(X, xlen, n, k, terms, a.seeds, a.s, 0, 1, reinterpret_cast<uint64_t *>(s_tab),
+                               small_slots(static_cast<uint64_t>(a.s) * (k - 1)), nullptr);
+    if (threadIdx.x == 0) *out = fixed_to_double(e) / terms.div;
+}
+
+// Block q: query q, if it is small.
+__global__ void __launch_bounds__(kSmallThreads) k_q_small(const uint64_t *X, const uint32_t *xlen, uint32_t n,
+                                                           uint32_t k, QueryTerms terms, const uint32_t *seeds,
+                                                           const uint64_t *offsets, const uint64_t *block_off,
+                                                           double *out, unsigned *err) {
+    extern __shared__ ulonglong2 s_tab[];
+    const uint32_t q = blockIdx.x;
+    if (block_off[q + 1] != block_off[q]) return;
+    const uint64_t s0 = offsets[q];
+    const uint32_t s = static_cast<uint32_t>(offsets[q + 1] - s0);
+    const U192 e = query_block<false>(X, xlen, n, k, terms, seeds + s0, s, 0, 1, reinterpret_cast<uint64_t *>(s_tab),
+                               small_slots(static_cast<uint64_t>(s) * (k - 1)), err);
+    if (threadIdx.x == 0) out[q] = fixed_to_double(e) / terms.div;
+}
+
+// One block per part of the larger queries; the last block of a query (done
+// counts them, zero again after) adds the parts.
+__global__ void __launch_bounds__(kPartThreads) k_q_part(const uint64_t *X, const uint32_t *xlen, uint32_t n,
+                                                         uint32_t k, QueryTerms terms, const uint32_t *seeds,
+                                                         const uint64_t *offsets, const uint64_t *block_off,
+                                                         uint32_t q, U192 *partial, unsigned *done, double *out,
+                                                         unsigned *err) {
+    extern __shared__ ulonglong2 s_tab[];
+    __shared__ int s_last;
+    const uint32_t c = blockIdx.x;
+    const uint32_t qi = upper_bound_u64(block_off + 1, q, c);
+    const uint64_t first = block_off[qi], end = block_off[qi + 1], s0 = offsets[qi];
+    const U192 e = query_block<true>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(offsets[qi + 1] - s0), c - first,
+                               end - first, reinterpret_cast<uint64_t *>(s_tab), kPartSlots, err);
+    if (threadIdx.x == 0) {
+        partial[c] = e;
+        __threadfence();
+        s_last = atomicAdd(&done[qi], 1u) + 1 == static_cast<unsigned>(end - first);
+    }
+    __syncthreads();
+    if (!s_last || threadIdx.x >= 32) return;
+    __threadfence();
+    U192 tot{{0, 0, 0}};
+    for (uint64_t p = first + threadIdx.x; p < end; p += 32) {
+        U192 x;
+        for (int w = 0; w < 3; w++) x.w[w] = __ldcg(&partial[p].w[w]);
+        add192(tot, x);
+    }
+    tot = warp_sum192(tot);
+    if (threadIdx.x == 0) {
+        out[qi] = fixed_to_double(tot) / terms.div;
+        done[qi] = 0;
     }
 }
 
@@ -247,7 +375,10 @@ __global__ void k_node_estimates(const uint64_t *X, const uint32_t *xlen, uint32
 
 }  // namespace
 
-uint32_t query_chunks(uint64_t table_slots) { return static_cast<uint32_t>((table_slots + kQChunk - 1) / kQChunk); }
+uint32_t query_blocks(uint64_t seeds, uint32_t k) {
+    const uint64_t e = seeds * (k - 1);
+    return e <= kSmallEntries ? 0 : static_cast<uint32_t>((e + kPartEntries - 1) / kPartEntries);
+}
 
 size_t query_partial_bytes() { return sizeof(U192); }
 
@@ -259,26 +390,51 @@ cudaError_t launch_node_estimates(const uint64_t *X, const uint32_t *xlen, uint3
     return cudaGetLastError();
 }
 
+bool query_fits_args(uint64_t seeds, uint32_t k) { return seeds <= kQueryArgSeeds && seeds * (k - 1) <= 3 * kSmallEntries; }
+
+namespace {
+template <uint32_t CAP>
+cudaError_t one_launch(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
+                       const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st) {
+    SeedArgs<CAP> a;
+    a.s = s;
+    std::copy(seeds, seeds + s, a.seeds);
+    const size_t smem = (small_slots(static_cast<uint64_t>(s) * (k - 1)) + 1) * sizeof(ulonglong2);
+    if (smem > 32 * 1024) {  // (with the static part, 48 KB need no asking)
+        const cudaError_t e = cudaFuncSetAttribute(k_q_one<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   static_cast<int>((small_slots(3 * kSmallEntries) + 1) * sizeof(ulonglong2)));
+        if (e != cudaSuccess) return e;
+    }
+    const uint32_t threads = std::min<uint32_t>(1024, std::max<uint32_t>(128, s * 32));
+    note_launch();
+    k_q_one<CAP><<<1, threads, smem, st>>>(X, xlen, n, k, terms, a, out_host);
+    return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_query_one(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
+                             const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st) {
+    return s <= 60 ? one_launch<60>(X, xlen, n, k, terms, seeds, s, out_host, st)
+                   : one_launch<kQueryArgSeeds>(X, xlen, n, k, terms, seeds, s, out_host, st);
+}
+
 cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
-                               const uint32_t *seeds, const uint64_t *offsets, const uint64_t *table_off,
-                               const uint64_t *chunk_off, uint32_t q, uint64_t total_slots, uint64_t total_seeds,
-                               uint32_t total_chunks, const QueryScratch &qs, double *out, cudaStream_t s) {
+                               const uint32_t *seeds, const uint64_t *offsets, const uint64_t *block_off, uint32_t q,
+                               uint32_t blocks, const QueryScratch &qs, double *out, cudaStream_t s) {
     if (q == 0) return cudaSuccess;
-    auto grid = [](uint64_t work) {
-        uint64_t g = (work + 255) / 256;
-        return static_cast<unsigned>(g < 1 ? 1 : (g > 152 * 16 ? 152 * 16 : g));
-    };
-    unsigned long long *top_tau = reinterpret_cast<unsigned long long *>(qs.top_tau);
+    static_assert(kSmallSlots >= kSmallEntries + kSmallEntries / 2 + 32, "a small query's table");
+    const int smem = (kSmallSlots + 1) * sizeof(ulonglong2), part_smem =
+              (kPartSlots + 1 + kPartThreads / 32 * kStage) * sizeof(ulonglong2);
+    cudaError_t e = cudaFuncSetAttribute(k_q_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_q_part, cudaFuncAttributeMaxDynamicSharedMemorySize, part_smem);
+    if (e != cudaSuccess) return e;
+    if (blocks) {
+        note_launch();
+        k_q_part<<<blocks, kPartThreads, part_smem, s>>>(X, xlen, n, k, terms, seeds, offsets, block_off, q,
+                                                         static_cast<U192 *>(qs.partial), qs.done, out, qs.err);
+    }
     note_launch();
-    k_q_clear<<<grid(total_slots), 256, 0, s>>>(qs.hkeys, qs.hvals, total_slots, top_tau, qs.top_used, q);
-    note_launch();
-    k_q_insert<<<grid(total_seeds * k), 256, 0, s>>>(X, xlen, n, k, seeds, offsets, table_off, q, qs.hkeys, qs.hvals,
-                                                     top_tau, qs.top_used, qs.err);
-    note_launch();
-    k_q_sum<<<total_chunks, 256, 0, s>>>(qs.hkeys, qs.hvals, table_off, chunk_off, q, top_tau, qs.top_used, terms,
-                                         static_cast<U192 *>(qs.partial));
-    note_launch();
-    k_q_final<<<grid(q), 256, 0, s>>>(static_cast<const U192 *>(qs.partial), chunk_off, q, terms.div, out);
+    k_q_small<<<q, kSmallThreads, smem, s>>>(X, xlen, n, k, terms, seeds, offsets, block_off, out, qs.err);
     return cudaGetLastError();
 }
 

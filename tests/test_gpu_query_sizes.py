@@ -1,0 +1,36 @@
+"""Queries at the sizes where their kernels change: seeds as kernel arguments and
+in memory, one block and several parts, tables at their fill limits, seeds given
+twice, no seeds.  Alone and in a batch the same bits; within 1e-12 of the
+oracle's sum in double."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+REL = 1e-12
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("k", [2, 16, 64, 255])
+def test_sizes_around_the_limits(k, mode):
+    import paper_1408_6282_gb300 as pkg
+    g = synth.erdos_renyi(3001, 15000, 41)
+    ks = synth.Keys.from_seed(41)
+    l, p = 16, 0.15
+    pb = oracle.Problem(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
+    ox, oln, _ = oracle.build_sketches(pb, rank_mode=mode)
+    limits = [2700 // (k - 1), 8100 // (k - 1), 8000 // (k - 1), 16000 // (k - 1), 60, 960]
+    sizes = sorted({s for x in limits for s in (x - 1, x, x + 1) if 0 <= s <= 9000} | {0, 1, 31, 32, 33})
+    rng = np.random.default_rng(k)
+    sets = [rng.integers(0, g.n, s) if s > g.n else rng.choice(g.n, s, replace=False) for s in sizes]
+    sets.append(np.repeat(sets[-1][:40], 3))
+    with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, rank_mode=mode) as sk:
+        sk.build_sketches()
+        batch = sk.query_batch(sets)
+        for s, b in zip(sets, batch):
+            a = sk.query(s)
+            assert a == b
+            ref = oracle.union_estimate(ox, oln, l, s, rank_mode=mode)
+            assert abs(a - ref) <= REL * abs(ref)
