@@ -88,7 +88,7 @@ struct skim_ctx {
     uint64_t *alive = nullptr, *lane_cnt = nullptr, *lane_off = nullptr;
     uint32_t *lane_fill = nullptr;
     uint32_t lane_cap = 0;
-    int grid_rev = 0, grid_fwd = 0, grid_ring = 0;
+    int grid_rev = 0, grid_coin = 0, grid_fwd = 0, grid_ring = 0;
     uint64_t timeout_ns = 2000000000ull;
     // sketches
     uint8_t *lcnt = nullptr;
@@ -394,7 +394,7 @@ int run_traversal(skim_ctx *c, TravArgs &a, bool forward, uint64_t *R_out, const
                 CK(c, launch_rev_ring(a, rs->lane_pair, rs->B, c->l, rs->covered, rs->alive, first, c->grid_ring,
                                       c->st));
             else
-                CK(c, launch_traverse(a, forward, forward ? c->grid_fwd : c->grid_rev, c->st));
+                CK(c, launch_traverse(a, forward, forward ? c->grid_fwd : c->mat ? c->grid_rev : c->grid_coin, c->st));
         }
         RC(sync_ctl(c));
         const DevCtl &h = *c->hctl;
@@ -1277,9 +1277,10 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
         TRY(dalloc(c, &c->lane_cnt, c->lane_cap));
         TRY(dalloc(c, &c->lane_off, c->lane_cap));
         TRY(dalloc(c, &c->lane_fill, c->lane_cap));
-        c->grid_rev = traverse_grid(false);
+        c->grid_rev = traverse_grid(false, true);
+        c->grid_coin = traverse_grid(false, false);
         c->grid_ring = rev_ring_grid();
-        c->grid_fwd = traverse_grid(true);
+        c->grid_fwd = traverse_grid(true, true);
         TRYC(cudaStreamSynchronize(c->st));
     }
 #undef TRY

@@ -58,6 +58,21 @@ SKIM_HD uint64_t pair_rank(uint64_t rank_key, uint64_t x) { return fmix(rank_key
 SKIM_HD uint64_t edge_state(uint64_t coin_key, uint32_t u, uint32_t v) {
     return fmix(coin_key ^ ((static_cast<uint64_t>(u) << 32) | v));
 }
+// fmix(z) <= t, from the upper half of the last product where that decides (all
+// but one coin in 2^32): its lower half and the last shift of the output
+// function are not needed.
+SKIM_DEV bool fmix_le(uint64_t z, uint64_t t) {
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z ^= z >> 27;
+    constexpr uint32_t ml = 0x133111EBu, mh = 0x94D049BBu;
+    const uint32_t zl = static_cast<uint32_t>(z), zh = static_cast<uint32_t>(z >> 32);
+    uint32_t h = __umulhi(zl, ml) + zl * mh + zh * ml;
+    h ^= h >> 31;
+    const uint32_t th = static_cast<uint32_t>(t >> 32);
+    if (h != th) return h < th;
+    z *= 0x94D049BB133111EBull;
+    return (z ^ (z >> 31)) <= t;
+}
 SKIM_HD bool coin_live(uint64_t he, uint32_t inst, uint64_t tm1) {
     return fmix(he + kGolden * static_cast<uint64_t>(inst + 1)) <= tm1;
 }

@@ -110,10 +110,10 @@ __global__ void k_live_masks(const uint32_t *rrow, const uint32_t *rcol, const u
         uint64_t mk = 0;
         uint32_t i = 0;
         for (; i + 1 < l; i += 2) {
-            const uint64_t c0 = fmix(h + kGolden * (i + 1)), c1 = fmix(h + kGolden * (i + 2));
-            mk |= (static_cast<uint64_t>(c0 <= t1) << i) | (static_cast<uint64_t>(c1 <= t1) << (i + 1));
+            mk |= (static_cast<uint64_t>(fmix_le(h + kGolden * (i + 1), t1)) << i) |
+                  (static_cast<uint64_t>(fmix_le(h + kGolden * (i + 2), t1)) << (i + 1));
         }
-        if (i < l) mk |= static_cast<uint64_t>(fmix(h + kGolden * (i + 1)) <= t1) << i;
+        if (i < l) mk |= static_cast<uint64_t>(fmix_le(h + kGolden * (i + 1), t1)) << i;
         rmask[e] = mk;
         fmask[rev2fwd[e]] = mk;
     }

@@ -714,11 +714,10 @@ SKIM_DEV uint64_t live_lanes(uint64_t he, uint64_t m, uint64_t t1, const uint64_
             const int j2 = __ffsll(m) - 1;
             m &= m - 1;
             const uint64_t g2 = g[j2];
-            const uint64_t c1 = fmix(he + g1), c2 = fmix(he + g2);
-            live |= static_cast<uint64_t>(c1 <= t1) << j1;
-            live |= static_cast<uint64_t>(c2 <= t1) << j2;
+            live |= static_cast<uint64_t>(fmix_le(he + g1, t1)) << j1;
+            live |= static_cast<uint64_t>(fmix_le(he + g2, t1)) << j2;
         } else {
-            live |= static_cast<uint64_t>(fmix(he + g1) <= t1) << j1;
+            live |= static_cast<uint64_t>(fmix_le(he + g1, t1)) << j1;
         }
     }
     return live;
@@ -783,6 +782,9 @@ SKIM_DEV Desc shfl_desc(const Desc &d, int src) {
 #ifndef SKIM_TRAV_MIN_BLOCKS
 #define SKIM_TRAV_MIN_BLOCKS 3
 #endif
+#ifndef SKIM_COIN_MIN_BLOCKS
+#define SKIM_COIN_MIN_BLOCKS 3
+#endif
 constexpr int kUnroll = SKIM_UNROLL;  // edges per lane per step: independent hash chains
 
 // Coin test of CSR edge idx for item d: the lanes (reverse) or instances
@@ -815,7 +817,7 @@ SKIM_DEV uint64_t edge_live_xh(const TravArgs &A, const Desc &d, uint32_t idx, u
     if (MAT) return d.mask;
     if (FWD) return live_lanes(he, d.mask, edge_tm1_fwd(A, idx, d.v, x), ginst);
     const uint64_t t1 = edge_tm1_rev(A, idx, x, d.v, d.tm1);
-    if (d.single) return fmix(he + d.g1) <= t1 ? d.mask : 0;
+    if (d.single) return fmix_le(he + d.g1, t1) ? d.mask : 0;
     return live_lanes(he, d.mask, t1, A.lane_g + static_cast<size_t>(d.w >> kChunkBits) * 64);
 }
 
@@ -827,20 +829,152 @@ SKIM_DEV uint64_t edge_live(const TravArgs &A, const Desc &d, uint32_t idx, uint
     if (MAT) return d.mask;
     if (FWD) return live_lanes(he, d.mask, edge_tm1_fwd(A, idx, d.v, x), ginst);
     const uint64_t t1 = edge_tm1_rev(A, idx, x, d.v, d.tm1);
-    if (d.single) return fmix(he + d.g1) <= t1 ? d.mask : 0;
+    if (d.single) return fmix_le(he + d.g1, t1) ? d.mask : 0;
     return live_lanes(he, d.mask, t1, A.lane_g + static_cast<size_t>(d.w >> kChunkBits) * 64);
 }
 
 // Algorithm 2: drop lanes whose instance-local sketch at u already holds k ranks.
-SKIM_DEV uint64_t prune_full(const TravArgs &A, const Desc &d, uint32_t u, uint64_t live) {
+SKIM_DEV uint64_t prune_full(const TravArgs &A, uint32_t t, uint32_t u, uint64_t live) {
     const uint64_t fu = A.full[u];
     if (!fu) return live;
-    const uint8_t *li = A.lane_inst + static_cast<size_t>(d.w >> kChunkBits) * 64;
+    const uint8_t *li = A.lane_inst + static_cast<size_t>(t) * 64;
     for (uint64_t m = live; m; m &= m - 1) {
         const int j = __ffsll(m) - 1;
         if ((fu >> li[j]) & 1ull) live &= ~(1ull << j);
     }
     return live;
+}
+
+// ---- reverse items with coins drawn in the search ------------------------------
+//
+// A visit of a hub draws thousands of coins of which a few are live, so the live
+// edges are collected in shared memory and visited 32 at a time: visiting after
+// every 32 edges kept one lane of the warp busy (R-MAT 15, IC model, p = 0.01:
+// 22 G coins, 190 ms of search; 97 ms so, and 139 with the visits inlined four
+// times).  Rows of 32 edges and more are swept by
+// the warp, 128 edges a step (four independent hash chains per lane; an edge's
+// other end is read only where it is live), the edges of the others are spread
+// over the lanes.
+constexpr uint32_t kCoinStage = 32 + 4 * 32;  // live edges a warp holds
+
+// Warp-collective: visit the first min(n, 32) of the n live edges in st ({other
+// end | word << 32, lanes}) and move the others up; returns the lane's new visits.
+// (Not inlined: the loops that draw coins have to fit the instruction cache.)
+__device__ __noinline__ uint32_t coin_visit(const TravArgs &A, ulonglong2 *st, uint32_t n) {
+    const uint32_t lane = threadIdx.x & 31, c = min(n, 32u), rest = n - c;
+    __syncwarp();
+    const ulonglong2 e = lane < c ? st[lane] : make_ulonglong2(0, 0);
+    for (uint32_t q = 0; q < rest; q += 32) {  // (c is 32 here)
+        const ulonglong2 m = st[min(c + q + lane, kCoinStage - 1)];
+        __syncwarp();
+        if (q + lane < rest) st[q + lane] = m;
+        __syncwarp();
+    }
+    Acc acc;
+    emit_rev<false>(A, acc, lane < c, static_cast<uint32_t>(e.x), static_cast<uint32_t>(e.x >> 32), e.y);
+    return static_cast<uint32_t>(acc.visits);
+}
+
+struct CoinStage {
+    ulonglong2 *st;
+    uint32_t n;  // warp-uniform
+
+    // Warp-collective: lanes with live != 0 hold a live edge from x in word t.
+    SKIM_DEV void put(const TravArgs &A, uint64_t live, uint32_t x, uint32_t t) {
+        if (live && A.prune) live = prune_full(A, t, x, live);
+        const unsigned b = __ballot_sync(kFull, live != 0);
+        if (live) st[n + __popc(b & lanemask_lt())] = make_ulonglong2(static_cast<uint64_t>(t) << 32 | x, live);
+        n += __popc(b);
+    }
+    SKIM_DEV void visit(const TravArgs &A, Acc &acc) {
+        acc.visits += coin_visit(A, st, n);
+        n -= min(n, 32u);
+    }
+};
+
+SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have, const Item &it) {
+    const uint32_t lane = threadIdx.x & 31;
+    Desc d = describe<false, false>(A, have, it);
+    if (d.cnt) {
+        acc.edges += d.cnt;
+        acc.coins += static_cast<unsigned long long>(d.cnt) * __popcll(d.mask);
+        d.tm1 = A.cm.model == 1 ? A.cm.thr_wc[d.v] : A.cm.tm1_uniform;
+        d.single = (d.mask & (d.mask - 1)) == 0;
+        if (d.single) d.g1 = A.lane_g[static_cast<size_t>(d.w >> kChunkBits) * 64 + (__ffsll(d.mask) - 1)];
+    }
+    CoinStage S{st, 0};
+    const bool plain = A.cm.model < 2;  // the threshold is the row's
+    unsigned big = __ballot_sync(kFull, d.cnt >= 32);
+    while (big) {
+        const int src = __ffs(big) - 1;
+        big &= big - 1;
+        const Desc b = shfl_desc(d, src);
+        const uint32_t t = b.w >> kChunkBits;
+        if (b.single) {
+            const uint64_t *he = A.he + b.begin;
+            const uint32_t steps = (b.cnt + 31) / 32;
+            for (uint32_t s0 = 0; s0 < steps; s0 += 4) {
+                uint64_t h[4];
+#pragma unroll
+                for (uint32_t q = 0; q < 4; q++) h[q] = he[min((s0 + q) * 32 + lane, b.cnt - 1)];
+#pragma unroll
+                for (uint32_t q = 0; q < 4; q++) {
+                    if (s0 + q >= steps) break;
+                    const uint32_t k = (s0 + q) * 32 + lane;
+                    uint64_t t1 = b.tm1;
+                    if (!plain && k < b.cnt) t1 = edge_tm1_rev(A, b.begin + k, A.col[b.begin + k], b.v, 0);
+                    const bool live = fmix_le(h[q] + b.g1, t1) && k < b.cnt;
+                    if (__any_sync(kFull, live)) S.put(A, live ? b.mask : 0, live ? A.col[b.begin + k] : 0, t);
+                }
+                while (S.n >= 32) S.visit(A, acc);
+            }
+        } else {
+            for (uint32_t k0 = 0; k0 < b.cnt; k0 += 32) {
+                const uint32_t k = k0 + lane, idx = b.begin + k;
+                uint64_t live = 0;
+                uint32_t x = 0;
+                if (k < b.cnt) {
+                    x = A.col[idx];
+                    live = live_lanes(A.he[idx], b.mask, edge_tm1_rev(A, idx, x, b.v, b.tm1),
+                                      A.lane_g + static_cast<size_t>(t) * 64);
+                }
+                S.put(A, live, x, t);
+                if (S.n >= 32) S.visit(A, acc);
+            }
+        }
+    }
+    const uint32_t c = d.cnt < 32 ? d.cnt : 0;
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= static_cast<uint32_t>(o)) incl += y;
+    }
+    const uint32_t total = __shfl_sync(kFull, incl, 31), first = d.begin - (incl - c);
+    for (uint32_t g = 0; g < total; g += 32) {
+        const uint32_t o = g + lane;
+        uint32_t sl = 0;  // owner: the first lane whose inclusive count exceeds o
+#pragma unroll
+        for (uint32_t step = 16; step > 0; step >>= 1) {
+            const uint32_t v = __shfl_sync(kFull, incl, sl + step - 1);
+            if (v <= o) sl += step;
+        }
+        const uint32_t idx = __shfl_sync(kFull, first, sl) + o, v = __shfl_sync(kFull, d.v, sl);
+        const uint32_t t = __shfl_sync(kFull, d.w, sl) >> kChunkBits;
+        const uint64_t mask = __shfl_sync(kFull, d.mask, sl), tm1 = __shfl_sync(kFull, d.tm1, sl);
+        const uint64_t g1 = __shfl_sync(kFull, d.g1, sl);
+        uint64_t live = 0;
+        uint32_t x = 0;
+        if (o < total) {
+            x = A.col[idx];
+            const uint64_t t1 = edge_tm1_rev(A, idx, x, v, tm1), he = A.he[idx];
+            live = (mask & (mask - 1)) == 0 ? (fmix_le(he + g1, t1) ? mask : 0)
+                                            : live_lanes(he, mask, t1, A.lane_g + static_cast<size_t>(t) * 64);
+        }
+        S.put(A, live, x, t);
+        if (S.n >= 32) S.visit(A, acc);
+    }
+    while (S.n) S.visit(A, acc);  // before the items count as done
 }
 
 // Hand the live results of one step to the emitters (warp-collective).
@@ -851,11 +985,6 @@ SKIM_DEV void emit_step(const TravArgs &A, Acc &acc, SK &sk, const Desc &d, cons
         uint64_t live = lv[q];
         if constexpr (FWD) {
             emit_fwd<MAT>(A, acc, live != 0, tg[q], live, sk.ring);
-        } else if constexpr (MAT) {
-            emit_rev_mat(A, acc, sk, live != 0, tg[q], d.w >> kChunkBits, __ffsll(d.mask) - 1, d.inst);
-        } else {
-            if (live && A.prune) live = prune_full(A, d, tg[q], live);
-            emit_rev<MAT>(A, acc, live != 0, tg[q], d.w >> kChunkBits, live);
         }
     }
 }
@@ -1341,12 +1470,15 @@ constexpr unsigned long long kDoneBatch = 64;
 // room; a warp takes ring items into its lanes that hold no queue item.
 struct NoRing {};
 template <bool FWD, bool MAT>
-__global__ void __launch_bounds__(kTravThreads, FWD ? 1 : SKIM_TRAV_MIN_BLOCKS) k_traverse(TravArgs A) {
+__global__ void __launch_bounds__(kTravThreads, FWD ? 1 : MAT ? SKIM_TRAV_MIN_BLOCKS : SKIM_COIN_MIN_BLOCKS)
+    k_traverse(const __grid_constant__ TravArgs A) {
     constexpr bool kStaged = !FWD && MAT;
     constexpr bool kLocal = FWD && MAT && kFwdKeep > 0;
+    constexpr bool kCoins = !FWD && !MAT;
     __shared__ uint64_t ginst[64];  // (i + 1) * G for instance i (residual searches)
     __shared__ uint64_t s_rk[kStaged ? kTravThreads / 32 : 1][kStaged ? kRecStage : 1];
     __shared__ uint32_t s_rs[kStaged ? kTravThreads / 32 : 1][kStaged ? kRecStage : 1];
+    __shared__ ulonglong2 s_coin[kCoins ? kTravThreads / 32 : 1][kCoins ? kCoinStage : 1];
     __shared__ typename std::conditional<kLocal, FwdRing, NoRing>::type s_ring;
     FwdRing *ring = nullptr;
     if constexpr (kLocal) {
@@ -1358,7 +1490,6 @@ __global__ void __launch_bounds__(kTravThreads, FWD ? 1 : SKIM_TRAV_MIN_BLOCKS) 
     const int lane = threadIdx.x & 31;
     DevCtl *C = A.ctl;
     Acc acc;
-    GlobalSink gsink;
     FwdSink fsink{ring};
     const uint32_t wib = kStaged ? threadIdx.x >> 5 : 0;
     RingSink ssink{nullptr, s_rk[wib], s_rs[wib], 0, 0, 0, 0};
@@ -1401,7 +1532,7 @@ __global__ void __launch_bounds__(kTravThreads, FWD ? 1 : SKIM_TRAV_MIN_BLOCKS) 
                 else if constexpr (FWD)
                     process_items<FWD, MAT>(A, acc, fsink, have, it, ginst);
                 else
-                    process_items<FWD, MAT>(A, acc, gsink, have, it, ginst);
+                    coin_expand(A, acc, s_coin[threadIdx.x >> 5], have, it);
                 if constexpr (kLocal) {
                     // after the items' own pushes (their reservations are made)
                     __syncwarp();
@@ -1538,21 +1669,20 @@ __global__ void __launch_bounds__(kTravThreads, FWD ? 1 : SKIM_TRAV_MIN_BLOCKS) 
 // start leaves slots below the tail unclaimed, and the resident warps then
 // wait until the time limit and the call returns SKIM_ETIMEOUT (no hang).  So
 // the grid is at most the blocks that fit on the device by the occupancy of
-// every instantiation that may be launched with it, and another kernel that
+// the instantiation launched with it, and another kernel that
 // occupies SMs at the same time (another stream of this process, another
 // context) can break it the same way.  The reverse searches over materialised
 // rows (k_rev_ring) have no such requirement.
-int traverse_grid(bool forward) {
-    int dev = 0, sms = 0, per = 0, per2 = 0;
+int traverse_grid(bool forward, bool mat) {
+    int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // A residual search starts from one seed and stays narrow: one block per
     // SM keeps the idle warps (which poll) few.  Reverse searches of a batch
     // fill the machine: as many blocks as fit.
     if (forward) return sms;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, false>, kTravThreads, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per2, k_traverse<false, true>, kTravThreads, 0);
-    if (per2 < per) per = per2;
+    if (mat) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, true>, kTravThreads, 0);
+    else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, false>, kTravThreads, 0);
     if (per < 1) per = 1;
     return sms * per;
 }
