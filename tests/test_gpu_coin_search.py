@@ -1,0 +1,45 @@
+"""Reverse searches that draw their coins (no stored instances, and the IC model,
+which never stores any): rows of up to, at and past the 32, 64 and 128 edges a
+warp takes at a step, rows longer than a queue item takes at once, every edge live
+and few, one instance per item and many.  Sketches are whole numbers and must equal
+the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+DEGREES = [1, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 257, 1000, 2100]
+
+
+def _graph():
+    """DEGREES as in-degrees, 4 nodes of each, among 3000 nodes; a ring joins all."""
+    rng = np.random.default_rng(9)
+    n = 3000
+    src, dst = [np.arange(n, dtype=np.uint32)], [np.roll(np.arange(n, dtype=np.uint32), 1)]
+    for i, d in enumerate(DEGREES * 4):
+        v = 50 * i
+        u = rng.choice(np.setdiff1d(np.arange(n), [v, (v + 1) % n]), d - 1, replace=False).astype(np.uint32)
+        src.append(u)
+        dst.append(np.full(d - 1, v, np.uint32))
+    src, dst = np.concatenate(src), np.concatenate(dst)
+    order = np.lexsort((dst, src))
+    return n, src[order], dst[order]
+
+
+@pytest.mark.parametrize("mode,l,bl", [(2, 1, 0), (2, 1, 100), (0, 1, 0), (0, 64, 0), (1, 7, 64)])
+@pytest.mark.parametrize("model,p", [(0, 0.5), (0, 0.02), (1, 0.0), (2, 0.0)])
+def test_row_sizes(model, p, mode, l, bl):
+    import paper_1408_6282_gb300 as pkg
+    n, src, dst = _graph()
+    ks = synth.Keys.from_seed(17)
+    k = 33
+    pb = oracle.Problem(n, src, dst, l, k, model, p, ks.coin, ks.rank, ks.prob)
+    ox, oln, _ = oracle.build_ic_sketches(pb) if mode == 2 else oracle.build_sketches(pb, rank_mode=mode)
+    with pkg.Skim(n, src, dst, l, k, model, p, ks.coin, ks.rank, ks.prob, batch_lanes=bl, rank_mode=mode) as sk:
+        sk.set_live_rows(False)
+        for _ in range(2):
+            sk.build_sketches()
+            x, ln = sk.sketches()
+            assert np.array_equal(ln, oln) and np.array_equal(x, ox)
