@@ -148,6 +148,8 @@ struct skim_ctx {
     unsigned *qdone = nullptr;   // finished blocks per query, zero between calls
     void *qpart = nullptr;
     uint64_t qpart_cap = 0;
+    uint64_t *qtab = nullptr;  // table of the largest queries (16 bytes per slot)
+    uint64_t qtab_slots = 0;
     // counters of the last build/greedy call
     uint64_t hstats[SKIM_STAT_COUNT] = {0};
     // kernel timing (CUDA events on the context stream)
@@ -995,7 +997,14 @@ int rank_order(skim_ctx *c) {
     return SKIM_OK;
 }
 
-int ensure_query_space(skim_ctx *c, uint64_t seeds, uint64_t q, uint64_t blocks) {
+int ensure_query_space(skim_ctx *c, uint64_t seeds, uint64_t q, uint64_t blocks, uint64_t table_slots) {
+    if (table_slots > c->qtab_slots) {
+        dfree(c, c->qtab);
+        c->qtab_slots = 0;
+        RC(dalloc(c, &c->qtab, 2 * table_slots));
+        c->qtab_slots = table_slots;
+    }
+    blocks = query_partials(static_cast<uint32_t>(blocks), table_slots);
     if (blocks > c->qpart_cap) {
         dfree(c, c->qpart);
         c->qpart_cap = 0;
@@ -1079,6 +1088,7 @@ int skim_destroy(skim_ctx *c) {
     dfree(c, c->qseeds); dfree(c, c->qoff); dfree(c, c->qout);
     dfree(c, c->qdone);
     dfree(c, c->qpart);
+    dfree(c, c->qtab);
     for (auto &p : c->kpend) { cudaEventDestroy(p.a); cudaEventDestroy(p.b); }
     for (auto e : c->kpool) cudaEventDestroy(e);
     delete c;
@@ -2081,10 +2091,12 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
     // one host block: seed offsets | block offsets
     const size_t q1 = static_cast<size_t>(q) + 1;
     std::vector<uint64_t> meta(2 * q1, 0);
-    uint64_t *boff = meta.data() + q1;
+    uint64_t *boff = meta.data() + q1, table_slots = 0;
     for (uint32_t i = 0; i < q; i++) {
         if (offsets[i + 1] < offsets[i]) return SKIM_EINVAL;
-        boff[i + 1] = boff[i] + query_blocks(offsets[i + 1] - offsets[i], c->k);
+        const uint64_t cnt = offsets[i + 1] - offsets[i];
+        boff[i + 1] = boff[i] + query_blocks(cnt, c->k);
+        table_slots = std::max(table_slots, query_table_slots(cnt, c->k));
     }
     std::copy(offsets, offsets + q1, meta.data());
     const uint64_t total = offsets[q];
@@ -2093,7 +2105,7 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
         for (uint64_t i = 0; i < total; i++)
             if (seeds[i] >= c->n) return SKIM_EINVAL;
     }
-    RC(ensure_query_space(c, total, q, boff[q]));
+    RC(ensure_query_space(c, total, q, boff[q], table_slots));
     const uint32_t *dseeds = seeds;
     if (!on_device && total) {
         CK(c, cudaMemcpyAsync(c->qseeds, seeds, total * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st));
@@ -2106,8 +2118,8 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
     double *dout = on_device ? est_out : c->qout;
     {
         KTimer kt(c, SKIM_K_QUERY);
-        QueryScratch qs{c->qpart, c->qdone, flag};
-        CK(c, launch_query_multi(c->X, c->xlen, c->n, c->k, query_terms_of(c), dseeds, d_off, d_boff, q,
+        QueryScratch qs{c->qpart, c->qdone, flag, c->qtab, c->qtab_slots};
+        CK(c, launch_query_multi(c->X, c->xlen, c->n, c->k, query_terms_of(c), dseeds, d_off, d_boff, q, offsets,
                                  static_cast<uint32_t>(boff[q]), qs, dout, c->st));
     }
     unsigned bad = 0;
@@ -2136,6 +2148,10 @@ int skim_oracle_query(skim_ctx *c, const uint32_t *seeds, uint32_t n_seeds, doub
     }
     CK(c, cudaStreamSynchronize(c->st));
     resolve_timers(c);
+    if (*c->hq < 0) {  // a block's table was full
+        uint64_t off[2] = {0, n_seeds};
+        return skim_oracle_query_batch(c, off, 1, seeds, est_out, 0);
+    }
     *est_out = *c->hq;
     return SKIM_OK;
 }

@@ -313,8 +313,12 @@ struct QueryScratch {
     void *partial;
     unsigned *done;
     unsigned *err;
+    void *table;            // for the largest queries, 16 bytes per slot
+    uint64_t table_slots;
 };
-uint32_t query_blocks(uint64_t seeds, uint32_t k);  // blocks of a larger query, 0 for one that takes a single block
+uint32_t query_blocks(uint64_t seeds, uint32_t k);  // parts of a larger query, 0 for a small one and for the largest
+uint64_t query_table_slots(uint64_t seeds, uint32_t k);  // of the largest ones' table in global memory, else 0
+uint32_t query_partials(uint32_t blocks, uint64_t table_slots);  // places of `partial`
 size_t query_partial_bytes();
 // How a threshold becomes a term of Eq. unionest, and the final divisor:
 //  mode 0 (uniform 64-bit ranks): 1 / (h * 2^-64), divided by l;
@@ -330,12 +334,13 @@ struct QueryTerms {
 QueryTerms query_terms_of(const skim_ctx *c);
 cudaError_t launch_node_estimates(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, uint32_t l,
                                   int mode, double *out, cudaStream_t s);
-// block_off: prefix sums of query_blocks; blocks: their total
+// block_off: prefix sums of query_blocks; blocks: their total; h_offsets: offsets, on the host
 cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                                const uint32_t *seeds, const uint64_t *offsets, const uint64_t *block_off, uint32_t q,
-                               uint32_t blocks, const QueryScratch &qs, double *out, cudaStream_t s);
+                               const uint64_t *h_offsets, uint32_t blocks, const QueryScratch &qs, double *out,
+                               cudaStream_t s);
 // One query with few enough seeds (host) to be kernel arguments; out_host: pinned.
-constexpr uint32_t kQueryArgSeeds = 960;
+constexpr uint32_t kQueryArgSeeds = 8000;
 bool query_fits_args(uint64_t seeds, uint32_t k);
 cudaError_t launch_query_one(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                              const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st);

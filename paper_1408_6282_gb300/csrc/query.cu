@@ -18,6 +18,7 @@
 // formed as one double division (terms are at least 1/k >= 2^-8, so 64
 // fraction bits still hold them exactly).
 #include <algorithm>
+#include <cooperative_groups.h>
 
 #include "internal.cuh"
 
@@ -127,18 +128,35 @@ SKIM_DEV double fixed_to_double(const U192 &a) {
 // kernels: 1.03 ms with a table per query in global memory (two arrays, two
 // atomics per rank, a pass to clear and one to sum), 0.66 ms with 16-byte slots and
 // terms per seed there (0.54 ms of it the atomics: 15 G/s, also where the tables
-// stay in L2), 0.44 ms so (0.58 ms before a warp collected 32 ranks of its part).  One query of 10 seeds, host to host: 48 us with four
-// kernels, two uploads and two downloads, 19 us with one kernel that has the seeds
-// as arguments and writes the estimate to host memory.
+// stay in L2), 0.44 ms so (0.58 ms before a warp collected 32 ranks of its part).
+//
+// A single query is one kernel that has the seeds as arguments and writes the
+// estimate to host memory (host to host: 48 -> 19 us for 10 seeds; before, four
+// kernels, two uploads and two downloads).  Reading every sketch in every block is
+// what it would wait for, so a larger one takes a cluster of 16 blocks whose
+// warps share the seeds and put a rank into the table of the block that has its
+// hash, through distributed shared memory: 64 ranks per sketch, 445 seeds 61 -> 32
+// us, 1000 seeds 66 -> 40 us (clusters of 8: 66 us, of 4: 118 us; parts: 85 us).  A batch fills the
+// chip with parts and is slower with clusters (1000 queries, with copies: 0.52 ms;
+// clusters of 4, 8, 16: 0.63, 0.76, 1.07 ms), so clusters are for two queries, or
+// four of few parts (4 of 1000 seeds, 16 ranks per sketch: 67 us, in parts 91 us;
+// 64 ranks per sketch: 91 and 82 us; 8 of 200 seeds: 80 and 66 us).  Both
+// read a query once per part or round of clusters: from kBlockMost ranks on the
+// table is in global memory (64 ranks per sketch, 30000 seeds: 264 us, clusters
+// 555 us, parts 1100 us; 9000 seeds, clusters: 107 us).
+// One block is as fast as the cluster up to
+// kOneEntries (100 seeds of 16 ranks: 28 us both; 43 seeds of 64: 30 and 29 us).
 
 constexpr uint32_t kSmallEntries = 2700, kSmallSlots = 4095;  // 64 KB: three blocks per SM
 constexpr int kSmallThreads = 256;
-#ifndef SKIM_PART_ENTRIES
-#define SKIM_PART_ENTRIES 8000
-#endif
-constexpr uint32_t kPartEntries = SKIM_PART_ENTRIES, kPartSlots = 12287;   // 192 KB
+constexpr uint32_t kPartEntries = 8000, kPartSlots = 12287;  // 192 KB
 constexpr int kPartThreads = 1024;
 constexpr uint32_t kStage = 64;  // pairs a warp collects
+constexpr uint32_t kOneEntries = 1500;
+constexpr uint32_t kCluster = 16, kClusterSlots = kPartSlots, kClusterEntries = kCluster * 7800;
+constexpr uint32_t kClusterQueries = 4, kClusterParts = 8;
+constexpr uint64_t kBlockMost = 1 << 20;  // ranks, above that the table is in global memory
+constexpr uint32_t kTableBlocks = 152 * 2;
 
 SKIM_DEV uint32_t upper_bound_u64(const uint64_t *a, uint32_t n, uint64_t x) {  // first i with a[i] > x
     uint32_t lo = 0, hi = n;
@@ -173,6 +191,28 @@ SKIM_DEV bool table_put(uint64_t *keys, uint64_t *terms, uint32_t H, uint32_t at
     return false;
 }
 
+// The same from any block of the cluster.  Every access is a trip to the other
+// block, so an exchange is tried without looking first; and the minimum is a loop over the
+// 64-bit exchange, the one 64-bit operation that shared memory makes atomic
+// for local and remote callers alike (an atomicMin of 64 bits lost updates here).
+SKIM_DEV bool table_put_remote(uint64_t *keys, uint64_t *terms, uint32_t H, uint32_t at, uint64_t z, uint64_t t) {
+    if (z == kEmptyKey) at = H;
+    for (uint32_t p = 0; p < H; p++) {
+        const uint64_t k =
+            at == H ? z : atomicCAS(reinterpret_cast<unsigned long long *>(&keys[at]), kEmptyKey, z);
+        if (k == kEmptyKey || k == z) {
+            for (uint64_t v = kEmptyKey; v > t;) {
+                const uint64_t o = atomicCAS(reinterpret_cast<unsigned long long *>(&terms[at]), v, t);
+                if (o == v) break;
+                v = o;
+            }
+            return true;
+        }
+        if (++at == H) at = 0;
+    }
+    return false;
+}
+
 // What a lane has of its seed: the row, its ranks below the threshold, the
 // stored term.
 struct SeedRow {
@@ -199,6 +239,19 @@ SKIM_DEV void add_term(U192 &acc, uint64_t stored) {
     if (stored != kEmptyKey && stored) add192(acc, to_fixed(__longlong_as_double(static_cast<long long>(stored))));
 }
 
+SKIM_DEV U192 block_sum192(U192 acc) {  // valid in thread 0
+    __shared__ U192 wsum[32];
+    acc = warp_sum192(acc);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        U192 t{{0, 0, 0}};
+        if (threadIdx.x < (blockDim.x >> 5)) t = wsum[threadIdx.x];
+        acc = warp_sum192(t);
+    }
+    return acc;
+}
+
 // Block-collective: the exact sum over the ranks of a query whose hash lies in
 // part `part` of `parts` (thread 0's return value), table of H + 1 slots in tab.
 // PART: a row has few ranks of the part, so a warp collects 32 before it goes to
@@ -207,7 +260,6 @@ template <bool PART>
 SKIM_DEV U192 query_block(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                           const uint32_t *seeds, uint32_t s, uint64_t part, uint64_t parts, uint64_t *tab, uint32_t H,
                           unsigned *err) {
-    __shared__ U192 wsum[32];
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5, lane = threadIdx.x & 31;
     uint64_t *keys = tab, *val = tab + H + 1;
     ulonglong2 *st = reinterpret_cast<ulonglong2 *>(val + H + 1) + warp * kStage;
@@ -272,18 +324,82 @@ SKIM_DEV U192 query_block(const uint64_t *X, const uint32_t *xlen, uint32_t n, u
         c++;
         if (c < cut) __syncthreads();
     }
-    acc = warp_sum192(acc);
-    if (lane == 0) wsum[warp] = acc;
-    __syncthreads();
-    if (warp == 0) {
-        U192 t{{0, 0, 0}};
-        if (threadIdx.x < warps) t = wsum[threadIdx.x];
-        acc = warp_sum192(t);
+    return block_sum192(acc);
+}
+
+// Cluster-collective: the exact sum over the ranks of a query whose hash lies in
+// part `part` of `parts`, in the tables of the cluster's blocks (H + 1 slots each; a
+// block has a range of the hashes), in `cut` pieces or more.  Thread 0 of block 0
+// has the total; *bad: the ranks of some hash are more than fit.
+SKIM_DEV U192 query_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
+                            const uint32_t *seeds, uint32_t s, uint64_t part, uint64_t parts, uint64_t cut,
+                            uint64_t *tab, uint32_t H, unsigned *err, bool *bad) {
+    __shared__ U192 sums[kCluster];
+    __shared__ int s_full;
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    const uint32_t rank = cl.block_rank(), lane = threadIdx.x & 31;
+    const uint32_t w = rank * (blockDim.x >> 5) + (threadIdx.x >> 5), ways = kCluster * (blockDim.x >> 5);
+    uint64_t *keys = tab, *val = tab + H + 1;
+    U192 acc{{0, 0, 0}};
+    *bad = false;
+    for (uint64_t c = 0; c < cut;) {
+        const uint64_t pieces = parts * cut, piece = part * cut + c;
+        const uint64_t lo = (piece << 32) / pieces, hi = ((piece + 1) << 32) / pieces;  // of the 32-bit hash
+        const uint32_t lo32 = static_cast<uint32_t>(lo), last = static_cast<uint32_t>(hi - lo - 1);
+        const uint64_t scale = (static_cast<uint64_t>(kCluster * H) << 32) / (hi - lo);
+        for (uint32_t i = threadIdx.x; i <= H; i += blockDim.x) keys[i] = val[i] = kEmptyKey;
+        if (threadIdx.x == 0) s_full = 0;
+        cl.sync();
+        bool over = false;
+        for (uint32_t j0 = w; j0 < s; j0 += ways * 32) {  // lane i: seed j0 + i ways
+            const uint32_t j = j0 + lane * ways;
+            SeedRow r{0, 0, 0};
+            if (j < s) {
+                const uint32_t u = seeds[j];
+                if (u < n) r = seed_row(X, xlen, k, terms, u);
+                else atomicOr(err, 1u);
+            }
+            const uint32_t cnt = min(32u, (s - j0 + ways - 1) / ways);
+            for (uint32_t i = 0; i < cnt; i++) {
+                const uint32_t u = __shfl_sync(kFull, r.u, i), body = __shfl_sync(kFull, r.body, i);
+                const uint64_t t = __shfl_sync(kFull, r.term, i);
+                const uint64_t *row = X + static_cast<uint64_t>(u) * k;
+                for (uint32_t p = lane; p < body; p += 32) {
+                    const uint64_t z = row[p];
+                    const uint32_t h = rank_hash(z) - lo32;
+                    if (h > last) continue;
+                    const uint32_t at = static_cast<uint32_t>(__umul64hi(static_cast<uint64_t>(h) << 32, scale));
+                    const uint32_t g = min(kCluster * H - 1, at), b = g / H;
+                    over |= !table_put_remote(cl.map_shared_rank(keys, b), cl.map_shared_rank(val, b), H, g - b * H, z, t);
+                }
+            }
+        }
+        if (over) *cl.map_shared_rank(&s_full, 0) = 1;
+        cl.sync();
+        const bool again = *cl.map_shared_rank(&s_full, 0) != 0;
+        if (!again)
+            for (uint32_t i = threadIdx.x; i <= H; i += blockDim.x) add_term(acc, val[i]);
+        cl.sync();  // all have read the flag
+        if (!again) {
+            c++;
+        } else if (hi - lo < 2) {
+            *bad = true;
+            break;
+        } else {
+            cut *= 2;  // the pieces done so far stay done
+            c *= 2;
+        }
     }
+    acc = block_sum192(acc);
+    if (threadIdx.x == 0) *cl.map_shared_rank(&sums[rank], 0) = acc;
+    cl.sync();  // (a block leaves when nobody needs its memory any more)
+    if (rank == 0 && threadIdx.x == 0)
+        for (uint32_t r = 1; r < kCluster; r++) add192(acc, sums[r]);
     return acc;
 }
 
-SKIM_HD uint32_t small_slots(uint64_t entries) { return static_cast<uint32_t>(entries + entries / 2 + 32); }
+constexpr SKIM_HD uint32_t small_slots(uint64_t entries) { return static_cast<uint32_t>(entries + entries / 2 + 32); }
 
 // One query whose seeds are kernel arguments; the estimate goes to host memory.
 template <uint32_t CAP>
@@ -299,40 +415,40 @@ __global__ void __launch_bounds__(1024) k_q_one(const uint64_t *X, const uint32_
                                small_slots(static_cast<uint64_t>(a.s) * (k - 1)), nullptr);
     if (threadIdx.x == 0) *out = fixed_to_double(e) / terms.div;
 }
+// (an estimate is never negative: -1 tells the host to take the batch path)
+template <uint32_t CAP>
+__global__ void __launch_bounds__(1024)
+    k_q_one_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, QueryTerms terms,
+                    const __grid_constant__ SeedArgs<CAP> a, uint32_t H, double *out) {
+    extern __shared__ ulonglong2 s_tab[];
+    bool full;
+    const U192 e = query_cluster(X, xlen, n, k, terms, a.seeds, a.s, 0, 1, 1, reinterpret_cast<uint64_t *>(s_tab), H, nullptr, &full);
+    if (blockIdx.x == 0 && threadIdx.x == 0) *out = full ? -1.0 : fixed_to_double(e) / terms.div;
+}
 
 // Block q: query q, if it is small.
 __global__ void __launch_bounds__(kSmallThreads) k_q_small(const uint64_t *X, const uint32_t *xlen, uint32_t n,
                                                            uint32_t k, QueryTerms terms, const uint32_t *seeds,
-                                                           const uint64_t *offsets, const uint64_t *block_off,
-                                                           double *out, unsigned *err) {
+                                                           const uint64_t *offsets, double *out, unsigned *err) {
     extern __shared__ ulonglong2 s_tab[];
     const uint32_t q = blockIdx.x;
-    if (block_off[q + 1] != block_off[q]) return;
     const uint64_t s0 = offsets[q];
     const uint32_t s = static_cast<uint32_t>(offsets[q + 1] - s0);
+    if (static_cast<uint64_t>(s) * (k - 1) > kSmallEntries) return;
     const U192 e = query_block<false>(X, xlen, n, k, terms, seeds + s0, s, 0, 1, reinterpret_cast<uint64_t *>(s_tab),
                                small_slots(static_cast<uint64_t>(s) * (k - 1)), err);
     if (threadIdx.x == 0) out[q] = fixed_to_double(e) / terms.div;
 }
 
-// One block per part of the larger queries; the last block of a query (done
-// counts them, zero again after) adds the parts.
-__global__ void __launch_bounds__(kPartThreads) k_q_part(const uint64_t *X, const uint32_t *xlen, uint32_t n,
-                                                         uint32_t k, QueryTerms terms, const uint32_t *seeds,
-                                                         const uint64_t *offsets, const uint64_t *block_off,
-                                                         uint32_t q, U192 *partial, unsigned *done, double *out,
-                                                         unsigned *err) {
-    extern __shared__ ulonglong2 s_tab[];
+// Block-collective: part c (of first .. end) of a query has the sum e in thread 0;
+// the last one to come adds them up (*done counts, zero again after).
+SKIM_DEV void add_parts(const U192 &e, uint64_t c, uint64_t first, uint64_t end, U192 *partial, unsigned *done,
+                        double *out, double div) {
     __shared__ int s_last;
-    const uint32_t c = blockIdx.x;
-    const uint32_t qi = upper_bound_u64(block_off + 1, q, c);
-    const uint64_t first = block_off[qi], end = block_off[qi + 1], s0 = offsets[qi];
-    const U192 e = query_block<true>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(offsets[qi + 1] - s0), c - first,
-                               end - first, reinterpret_cast<uint64_t *>(s_tab), kPartSlots, err);
     if (threadIdx.x == 0) {
         partial[c] = e;
         __threadfence();
-        s_last = atomicAdd(&done[qi], 1u) + 1 == static_cast<unsigned>(end - first);
+        s_last = atomicAdd(done, 1u) + 1 == static_cast<unsigned>(end - first);
     }
     __syncthreads();
     if (!s_last || threadIdx.x >= 32) return;
@@ -345,9 +461,74 @@ __global__ void __launch_bounds__(kPartThreads) k_q_part(const uint64_t *X, cons
     }
     tot = warp_sum192(tot);
     if (threadIdx.x == 0) {
-        out[qi] = fixed_to_double(tot) / terms.div;
-        done[qi] = 0;
+        *out = fixed_to_double(tot) / div;
+        *done = 0;
     }
+}
+
+// A query of more than kBlockMost ranks: into a table of H + 1 slots in global
+// memory, then the sum over it.
+__global__ void __launch_bounds__(512) k_q_table(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k,
+                                                 QueryTerms terms, const uint32_t *seeds, uint64_t s, uint64_t *tab,
+                                                 uint32_t H, unsigned *err) {
+    const uint32_t lane = threadIdx.x & 31, ways = gridDim.x * (blockDim.x >> 5);
+    const uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    for (uint64_t j0 = static_cast<uint64_t>(w) * 32; j0 < s; j0 += static_cast<uint64_t>(ways) * 32) {
+        SeedRow r{0, 0, 0};
+        if (j0 + lane < s) {
+            const uint32_t u = seeds[j0 + lane];
+            if (u < n) r = seed_row(X, xlen, k, terms, u);
+            else atomicOr(err, 1u);
+        }
+        for (int i = 0; i < 32; i++) {
+            const uint32_t u = __shfl_sync(kFull, r.u, i), body = __shfl_sync(kFull, r.body, i);
+            const uint64_t t = __shfl_sync(kFull, r.term, i);
+            for (uint32_t p = lane; p < body; p += 32) {
+                const uint64_t z = X[static_cast<uint64_t>(u) * k + p];
+                if (!table_put(tab, tab + H + 1, H, __umulhi(rank_hash(z), H), z, t)) atomicOr(err, 2u);
+            }
+        }
+    }
+}
+__global__ void __launch_bounds__(512) k_q_table_sum(const uint64_t *val, uint32_t H, U192 *partial, unsigned *done,
+                                                     double *out, double div) {
+    U192 acc{{0, 0, 0}};
+    for (uint64_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= H; i += gridDim.x * blockDim.x) add_term(acc, val[i]);
+    add_parts(block_sum192(acc), blockIdx.x, 0, gridDim.x, partial, done, out, div);
+}
+
+// One block per part of the larger queries.
+__global__ void __launch_bounds__(kPartThreads) k_q_part(const uint64_t *X, const uint32_t *xlen, uint32_t n,
+                                                         uint32_t k, QueryTerms terms, const uint32_t *seeds,
+                                                         const uint64_t *offsets, const uint64_t *block_off,
+                                                         uint32_t q, U192 *partial, unsigned *done, double *out,
+                                                         unsigned *err) {
+    extern __shared__ ulonglong2 s_tab[];
+    const uint32_t c = blockIdx.x;
+    const uint32_t qi = upper_bound_u64(block_off + 1, q, c);
+    const uint64_t first = block_off[qi], end = block_off[qi + 1], s0 = offsets[qi];
+    const U192 e = query_block<true>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(offsets[qi + 1] - s0), c - first,
+                               end - first, reinterpret_cast<uint64_t *>(s_tab), kPartSlots, err);
+    add_parts(e, c, first, end, partial, &done[qi], &out[qi], terms.div);
+}
+
+// The same by clusters, `ways` for each query.
+__global__ void __launch_bounds__(kPartThreads) k_q_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n,
+                                                            uint32_t k, QueryTerms terms, const uint32_t *seeds,
+                                                            const uint64_t *offsets, const uint64_t *block_off,
+                                                            uint32_t ways, U192 *partial, unsigned *done, double *out,
+                                                            unsigned *err) {
+    extern __shared__ ulonglong2 s_tab[];
+    const uint32_t c = blockIdx.x / kCluster, qi = c / ways;
+    if (block_off[qi + 1] == block_off[qi]) return;
+    const uint64_t s0 = offsets[qi], s = offsets[qi + 1] - s0, room = static_cast<uint64_t>(kClusterEntries) * ways;
+    bool bad;
+    const U192 e = query_cluster(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(s), c % ways, ways,
+                                 (s * (k - 1) + room - 1) / room, reinterpret_cast<uint64_t *>(s_tab), kClusterSlots, err,
+                                 &bad);
+    if (blockIdx.x % kCluster) return;
+    if (bad && threadIdx.x == 0) atomicOr(err, 2u);
+    add_parts(e, c, qi * ways, (qi + 1) * ways, partial, &done[qi], &out[qi], terms.div);
 }
 
 // Single-node influence estimates from each node's own sketch: the bottom-k
@@ -377,7 +558,12 @@ __global__ void k_node_estimates(const uint64_t *X, const uint32_t *xlen, uint32
 
 uint32_t query_blocks(uint64_t seeds, uint32_t k) {
     const uint64_t e = seeds * (k - 1);
-    return e <= kSmallEntries ? 0 : static_cast<uint32_t>((e + kPartEntries - 1) / kPartEntries);
+    return e <= kSmallEntries || e > kBlockMost ? 0 : static_cast<uint32_t>((e + kPartEntries - 1) / kPartEntries);
+}
+
+uint64_t query_table_slots(uint64_t seeds, uint32_t k) {
+    const uint64_t e = seeds * (k - 1);
+    return e <= kBlockMost ? 0 : std::min<uint64_t>(e + e / 2, 0xfffffffeu) + 1;
 }
 
 size_t query_partial_bytes() { return sizeof(U192); }
@@ -390,52 +576,115 @@ cudaError_t launch_node_estimates(const uint64_t *X, const uint32_t *xlen, uint3
     return cudaGetLastError();
 }
 
-bool query_fits_args(uint64_t seeds, uint32_t k) { return seeds <= kQueryArgSeeds && seeds * (k - 1) <= 3 * kSmallEntries; }
+// 960 and 8000 seeds are 4 and 32 KB of arguments, the usual and the largest size.
+bool query_fits_args(uint64_t seeds, uint32_t k) {
+    return seeds <= kQueryArgSeeds && seeds * (k - 1) <= kClusterEntries;
+}
 
 namespace {
+
+template <class K, class... Args>
+cudaError_t cluster_launch(K kernel, unsigned clusters, uint32_t H, cudaStream_t st, const Args &...args) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (kClusterSlots + 1) * sizeof(ulonglong2));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kCluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(clusters * kCluster);
+    cfg.blockDim = dim3(kPartThreads);
+    cfg.dynamicSmemBytes = (H + 1) * sizeof(ulonglong2);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    note_launch();
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <uint32_t CAP>
 cudaError_t one_launch(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                        const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st) {
     SeedArgs<CAP> a;
     a.s = s;
     std::copy(seeds, seeds + s, a.seeds);
-    const size_t smem = (small_slots(static_cast<uint64_t>(s) * (k - 1)) + 1) * sizeof(ulonglong2);
-    if (smem > 32 * 1024) {  // (with the static part, 48 KB need no asking)
-        const cudaError_t e = cudaFuncSetAttribute(k_q_one<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   static_cast<int>((small_slots(3 * kSmallEntries) + 1) * sizeof(ulonglong2)));
-        if (e != cudaSuccess) return e;
+    const uint64_t entries = static_cast<uint64_t>(s) * (k - 1);
+    if (entries <= kOneEntries) {
+        static_assert((small_slots(kOneEntries) + 1) * sizeof(ulonglong2) < 40 * 1024, "needs no asking");
+        const uint32_t threads = std::min<uint32_t>(1024, std::max<uint32_t>(128, s * 32));
+        note_launch();
+        k_q_one<CAP><<<1, threads, (small_slots(entries) + 1) * sizeof(ulonglong2), st>>>(X, xlen, n, k, terms, a, out_host);
+        return cudaGetLastError();
     }
-    const uint32_t threads = std::min<uint32_t>(1024, std::max<uint32_t>(128, s * 32));
-    note_launch();
-    k_q_one<CAP><<<1, threads, smem, st>>>(X, xlen, n, k, terms, a, out_host);
-    return cudaGetLastError();
+    if constexpr (CAP > 60) {
+        const uint32_t H = static_cast<uint32_t>(std::min<uint64_t>(kClusterSlots, entries * 2 / kCluster + 64));
+        return cluster_launch(k_q_one_cluster<CAP>, 1, H, st, X, xlen, n, k, terms, a, H, out_host);
+    }
+    return cudaErrorInvalidValue;
 }
 }  // namespace
 
 cudaError_t launch_query_one(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                              const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st) {
-    return s <= 60 ? one_launch<60>(X, xlen, n, k, terms, seeds, s, out_host, st)
-                   : one_launch<kQueryArgSeeds>(X, xlen, n, k, terms, seeds, s, out_host, st);
+    if (s <= 60 && s * (k - 1) <= kOneEntries) return one_launch<60>(X, xlen, n, k, terms, seeds, s, out_host, st);
+    return s <= 960 ? one_launch<960>(X, xlen, n, k, terms, seeds, s, out_host, st)
+                    : one_launch<kQueryArgSeeds>(X, xlen, n, k, terms, seeds, s, out_host, st);
 }
 
 cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                                const uint32_t *seeds, const uint64_t *offsets, const uint64_t *block_off, uint32_t q,
-                               uint32_t blocks, const QueryScratch &qs, double *out, cudaStream_t s) {
+                               const uint64_t *h_offsets, uint32_t blocks, const QueryScratch &qs, double *out,
+                               cudaStream_t s) {
     if (q == 0) return cudaSuccess;
     static_assert(kSmallSlots >= kSmallEntries + kSmallEntries / 2 + 32, "a small query's table");
-    const int smem = (kSmallSlots + 1) * sizeof(ulonglong2), part_smem =
-              (kPartSlots + 1 + kPartThreads / 32 * kStage) * sizeof(ulonglong2);
-    cudaError_t e = cudaFuncSetAttribute(k_q_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_q_part, cudaFuncAttributeMaxDynamicSharedMemorySize, part_smem);
-    if (e != cudaSuccess) return e;
-    if (blocks) {
-        note_launch();
-        k_q_part<<<blocks, kPartThreads, part_smem, s>>>(X, xlen, n, k, terms, seeds, offsets, block_off, q,
-                                                         static_cast<U192 *>(qs.partial), qs.done, out, qs.err);
+    U192 *partial = static_cast<U192 *>(qs.partial);
+    cudaError_t e = cudaSuccess;
+    uint32_t tables = 0;
+    if (h_offsets[q] * (k - 1) > kBlockMost) {  // some query may be one of those
+        for (uint32_t i = 0; i < q && e == cudaSuccess; i++) {
+            const uint64_t cnt = h_offsets[i + 1] - h_offsets[i], slots = query_table_slots(cnt, k);
+            if (!slots) continue;
+            if (slots > qs.table_slots) return cudaErrorInvalidValue;
+            tables++;
+            e = cudaMemsetAsync(qs.table, 0xff, slots * sizeof(ulonglong2), s);
+            if (e != cudaSuccess) return e;
+            uint64_t *tab = static_cast<uint64_t *>(qs.table);
+            const uint32_t H = static_cast<uint32_t>(slots - 1);
+            note_launch();
+            note_launch();
+            k_q_table<<<kTableBlocks * 2, 512, 0, s>>>(X, xlen, n, k, terms, seeds + h_offsets[i], cnt, tab, H, qs.err);
+            k_q_table_sum<<<kTableBlocks, 512, 0, s>>>(tab + slots, H, partial + blocks, qs.done + i, out + i, terms.div);
+            e = cudaGetLastError();
+        }
     }
-    note_launch();
-    k_q_small<<<q, kSmallThreads, smem, s>>>(X, xlen, n, k, terms, seeds, offsets, block_off, out, qs.err);
-    return cudaGetLastError();
+    if (e == cudaSuccess && blocks && (q <= 2 || (q <= kClusterQueries && blocks <= kCluster))) {
+        const uint32_t ways = std::max(1u, std::min(kClusterParts / q, (blocks * kPartEntries - 1) / kClusterEntries + 1));
+        e = cluster_launch(k_q_cluster, q * ways, kClusterSlots, s, X, xlen, n, k, terms, seeds, offsets, block_off, ways,
+                           partial, qs.done, out, qs.err);
+    } else if (e == cudaSuccess && blocks) {
+        const int smem = (kPartSlots + 1 + kPartThreads / 32 * kStage) * sizeof(ulonglong2);
+        e = cudaFuncSetAttribute(k_q_part, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        note_launch();
+        k_q_part<<<blocks, kPartThreads, smem, s>>>(X, xlen, n, k, terms, seeds, offsets, block_off, q, partial, qs.done,
+                                                    out, qs.err);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess && (q > 1 || (!blocks && !tables))) {
+        const int smem = (kSmallSlots + 1) * sizeof(ulonglong2);
+        e = cudaFuncSetAttribute(k_q_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        note_launch();
+        k_q_small<<<q, kSmallThreads, smem, s>>>(X, xlen, n, k, terms, seeds, offsets, out, qs.err);
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
+uint32_t query_partials(uint32_t blocks, uint64_t table_slots) {
+    return std::max(blocks + (table_slots ? kTableBlocks : 0), kClusterParts);
 }
 
 }  // namespace skim

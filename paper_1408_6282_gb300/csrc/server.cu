@@ -49,6 +49,7 @@ struct Lane {  // one stream and its buffers
     unsigned *d_done = nullptr;  // finished blocks per query, zero between groups
     void *d_part = nullptr;
     uint64_t part_cap = 0;
+    void *d_table = nullptr;  // of queries above the shared-memory tables' limit (16 bytes per arena slot), or null
     uint32_t group_cap = 0;
     std::vector<uint64_t> tickets, boff;  // boff: the group's block offsets
 };
@@ -92,6 +93,7 @@ void free_lane(Lane &ln) {
     if (ln.d_err) cudaFree(ln.d_err);
     if (ln.d_done) cudaFree(ln.d_done);
     if (ln.d_part) cudaFree(ln.d_part);
+    if (ln.d_table) cudaFree(ln.d_table);
     if (ln.h_seeds) cudaFreeHost(ln.h_seeds);
     if (ln.h_meta) cudaFreeHost(ln.h_meta);
     if (ln.h_out) cudaFreeHost(ln.h_out);
@@ -161,8 +163,8 @@ bool admit(skim_server *s) {
     std::copy(ln->boff.begin(), ln->boff.end(), ln->h_meta + g1);
     ok &= cudaMemcpyAsync(ln->d_meta, ln->h_meta, 2 * g1 * sizeof(uint64_t), cudaMemcpyHostToDevice, ln->st) ==
           cudaSuccess;
-    QueryScratch qs{ln->d_part, ln->d_done, ln->d_err};
-    ok &= launch_query_multi(s->X, s->xlen, s->n, s->k, s->terms, ln->d_seeds, ln->d_meta, ln->d_meta + g1, cnt,
+    QueryScratch qs{ln->d_part, ln->d_done, ln->d_err, ln->d_table, ln->d_table ? ln->arena_slots : 0};
+    ok &= launch_query_multi(s->X, s->xlen, s->n, s->k, s->terms, ln->d_seeds, ln->d_meta, ln->d_meta + g1, cnt, ln->h_meta,
                              static_cast<uint32_t>(ln->boff.back()), qs, ln->d_out, ln->st) == cudaSuccess;
     ok &= cudaMemcpyAsync(ln->h_out, ln->d_out, cnt * sizeof(double), cudaMemcpyDeviceToHost, ln->st) == cudaSuccess;
     ok &= cudaEventRecord(ln->done, ln->st) == cudaSuccess;
@@ -225,7 +227,10 @@ int skim_server_start(skim_ctx *ctx, uint32_t max_inflight, uint64_t scratch_slo
         ok &= cudaStreamCreateWithFlags(&ln.st, cudaStreamNonBlocking) == cudaSuccess;
         ok &= cudaEventCreateWithFlags(&ln.done, cudaEventDisableTiming) == cudaSuccess;
         ok &= cudaMalloc(&ln.d_seeds, ln.seed_cap * sizeof(uint32_t)) == cudaSuccess;
-        ln.part_cap = arena / 2048 + gcap;  // a block per 8000 ranks, for which a query is charged 16000 slots
+        // a block per 8000 ranks, for which a query is charged 16000 slots
+        const uint64_t table = query_table_slots(arena / 2 / (k - 1), k);  // the largest query's
+        ln.part_cap = query_partials(static_cast<uint32_t>(arena / 2048 + gcap), table);
+        if (table) ok &= cudaMalloc(&ln.d_table, arena * 2 * sizeof(uint64_t)) == cudaSuccess;
         ok &= cudaMalloc(&ln.d_meta, 2 * (gcap + 1) * sizeof(uint64_t)) == cudaSuccess;
         ok &= cudaMalloc(&ln.d_out, gcap * sizeof(double)) == cudaSuccess;
         ok &= cudaMalloc(&ln.d_err, sizeof(unsigned)) == cudaSuccess;

@@ -1,5 +1,5 @@
 """Queries at the sizes where their kernels change: seeds as kernel arguments and
-in memory, one block and several parts, tables at their fill limits, seeds given
+in memory, one block, clusters, parts and the table in memory, tables at their fill limits, seeds given
 twice, no seeds.  Alone and in a batch the same bits; within 1e-12 of the
 oracle's sum in double."""
 import numpy as np
@@ -21,7 +21,7 @@ def test_sizes_around_the_limits(k, mode):
     l, p = 16, 0.15
     pb = oracle.Problem(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
     ox, oln, _ = oracle.build_sketches(pb, rank_mode=mode)
-    limits = [2700 // (k - 1), 8100 // (k - 1), 8000 // (k - 1), 16000 // (k - 1), 60, 960]
+    limits = [1500 // (k - 1), 2700 // (k - 1), 8000 // (k - 1), 124800 // (k - 1), 60, 960, 8000]
     sizes = sorted({s for x in limits for s in (x - 1, x, x + 1) if 0 <= s <= 9000} | {0, 1, 31, 32, 33})
     rng = np.random.default_rng(k)
     sets = [rng.integers(0, g.n, s) if s > g.n else rng.choice(g.n, s, replace=False) for s in sizes]
