@@ -193,43 +193,92 @@ __global__ void k_gather_bits(const uint32_t *__restrict__ rec_val, const uint64
         rbits[r] = hvals[2ull * rec_val[r]];
 }
 
+// ---- a SKIM step ------------------------------------------------------------------
+//
+// Everything between two residual searches: lanes whose source the last search
+// covered leave the batch, the scan for the next stop, the commit of the lanes up
+// to it.  One launch with four grid barriers (one block of 1024 threads per SM: a
+// barrier costs 2-3 us) instead of ten kernels and clears; with few records the
+// launches were the cost.  The residual search takes the seed from ctl->step, so it
+// is queued behind the step at once and the host's wait runs beside it.  50 seeds,
+// l = 64: R-MAT 18 wc 11.0 -> 9.6 ms (steps 2.0 -> 1.4 ms), R-MAT 20 p = 0.01, whose
+// batches have up to 2 M records, 30 -> 27 ms (12 -> 10 ms).  Two blocks of 512 or
+// 1024 threads per SM and other back-offs are within 1 %, one of 512 is 20 % slower
+// there.
+constexpr int kStepThreads = 1024;
+
+// Grid barrier number i of the launch: false once the wait limit has passed.  Its
+// counter is zero again when the next barrier has been passed.
+SKIM_DEV bool step_barrier(DevCtl *ctl, int i, uint64_t timeout_ns) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(&ctl->step.bar[i], 1u);
+        const uint64_t t0 = globaltimer();
+        int ok = 1;
+        while (*reinterpret_cast<volatile unsigned *>(&ctl->step.bar[i]) < gridDim.x) {
+            if (globaltimer() - t0 > timeout_ns) {
+                atomicOr(&ctl->err, kErrTimeout);
+                ok = 0;
+                break;
+            }
+            __nanosleep(40);
+        }
+        __threadfence();
+        if (blockIdx.x == 0) ctl->step.bar[(i + 3) & 3] = 0;
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+// Lanes from lo on whose source was covered are no longer alive.
+SKIM_DEV void step_refilter(const StepArgs &a) {
+    for (uint32_t j = a.lo + blockIdx.x * blockDim.x + threadIdx.x; j < a.B; j += gridDim.x * blockDim.x) {
+        const uint64_t bit = 1ull << (j & 63);
+        if (!(a.alive[j >> 6] & bit)) continue;
+        const uint32_t pr = a.lane_pair[j], u = pr / a.l, i = pr % a.l;
+        if ((a.covered[u] >> i) & 1ull) atomicAnd(reinterpret_cast<unsigned long long *>(&a.alive[j >> 6]), ~bit);
+    }
+}
+
 // SKIM's stop: per node v the lane at which size[v] reaches k, i.e. the
 // need = k - size[v]-th uncovered lane bit (from lane lo on) of v's records in
 // rank order (a node already at k stops at its first record).  Warps own the
 // runs that start in 32-record windows, as in the acceptance; a segmented
 // scan over the lanes counts each node's bits in order.
-__global__ void k_candidates(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                             const uint64_t *alive, uint32_t lo, const uint32_t *size, uint32_t k, DevCtl *ctl) {
+SKIM_DEV void step_candidates(const StepArgs &a) {
     const uint32_t lane = threadIdx.x & 31;
-    const uint64_t tmask = (1ull << tbits) - 1;
+    const uint64_t tmask = (1ull << a.tbits) - 1;
     const uint64_t warps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;
-    const uint64_t nwin = (R + 31) / 32;
+    const uint64_t nwin = (a.R + 31) / 32;
     for (uint64_t w = (blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x) >> 5; w < nwin; w += warps) {
-        const uint64_t W0 = w * 32, W1 = min(R, W0 + 32);
+        const uint64_t W0 = w * 32, W1 = min(a.R, W0 + 32);
         bool st = false;
-        if (W0 + lane < W1) st = run_start(rec_key, W0 + lane, tbits);
+        if (W0 + lane < W1) st = run_start(a.rec_key, W0 + lane, a.tbits);
         const unsigned sb = __ballot_sync(kFull, st);
         if (!sb) continue;
         const uint64_t s0 = W0 + __ffs(sb) - 1;
-        const uint64_t last = rec_key[W1 - 1] >> tbits;
+        const uint64_t last = a.rec_key[W1 - 1] >> a.tbits;
         uint64_t cv = ~0ull;  // node that continues from the previous chunk, and its count so far
         uint32_t ccum = 0;
         for (uint64_t c0 = s0;; c0 += 32) {
             const uint64_t rr = c0 + lane;
             uint64_t key = 0, m = 0;
             bool act = false;
-            if (rr < R) {
-                key = rec_key[rr];
-                act = rr < W1 || (key >> tbits) == last;
+            if (rr < a.R) {
+                key = a.rec_key[rr];
+                act = rr < W1 || (key >> a.tbits) == last;
             }
             const unsigned actb = __ballot_sync(kFull, act);
             if (!actb) break;
-            const uint64_t v = key >> tbits, t = key & tmask;
+            const uint64_t v = key >> a.tbits, t = key & tmask;
             // lanes of the record's word from lo on; its lane bits only when
             // some are left
             if (act) {
-                m = range_mask(t, lo, 0xffffffffu);
-                if (m) m &= rbits[rr] & alive[t];
+                m = range_mask(t, a.lo, 0xffffffffu);
+                if (m) m &= a.rbits[rr] & __ldcg(&a.alive[t]);
             }
             const uint32_t c = __popcll(m);
             // inclusive count of v's bits up to this record (runs are contiguous)
@@ -242,11 +291,11 @@ __global__ void k_candidates(const uint64_t *rec_key, const uint64_t *rbits, uin
             }
             if (v == cv) incl += ccum;
             if (act) {
-                const uint32_t excl = incl - c, need = k - size[v];
-                const bool hit = need == 0 ? run_start(rec_key, rr, tbits) : (excl < need && incl >= need);
+                const uint32_t excl = incl - c, need = a.k - a.size[v];
+                const bool hit = need == 0 ? run_start(a.rec_key, rr, a.tbits) : (excl < need && incl >= need);
                 if (hit) {
                     const uint64_t p = t * 64 + nth_set_bit(m, static_cast<int>(need - excl - 1));
-                    atomicMin(&ctl->best, (p << 32) | v);
+                    atomicMin(&a.ctl->step.best, (p << 32) | v);
                 }
             }
             const int ll = 31 - __clz(actb);
@@ -257,93 +306,98 @@ __global__ void k_candidates(const uint64_t *rec_key, const uint64_t *rbits, uin
     }
 }
 
-// Commit of lanes [lo, hi]: size[v] += the committed uncovered lane bits of
-// v's records, and per lane the number of nodes it reaches (the index
-// segment lengths).  Additive, so one thread per record.
-__global__ void k_commit_count(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                               const uint64_t *alive, uint32_t lo, uint32_t hi, uint32_t *size,
-                               unsigned long long *lane_cnt, DevCtl *ctl) {
-    const uint64_t tmask = (1ull << tbits) - 1;
-    unsigned long long ins = 0;
-    for (uint64_t r = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; r < R;
+// Calls f(node, lane bits, word) for the records with uncovered lanes in [lo, hi].
+template <class F>
+SKIM_DEV void step_records(const StepArgs &a, uint32_t hi, const F &f) {
+    const uint64_t tmask = (1ull << a.tbits) - 1;
+    for (uint64_t r = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; r < a.R;
          r += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const uint64_t key = rec_key[r];
-        const uint64_t t = key & tmask;
-        uint64_t m = range_mask(t, lo, hi);
-        if (!m) continue;
-        m &= rbits[r] & alive[t];
-        if (!m) continue;
-        const uint32_t c = __popcll(m);
-        atomicAdd(&size[key >> tbits], c);
-        ins += c;
-        while (m) {
-            const int j = __ffsll(m) - 1;
-            m &= m - 1;
-            atomicAdd(&lane_cnt[t * 64 + j], 1ull);
-        }
-    }
-    warp_add(&ctl->stats[kStInsert], ins);
-}
-
-__global__ void k_commit_scatter(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                                 const uint64_t *alive, uint32_t lo, uint32_t hi, const uint64_t *lane_off,
-                                 uint32_t *lane_fill, const uint64_t *idx_ctr, uint32_t *idx_nodes) {
-    const uint64_t tmask = (1ull << tbits) - 1;
-    const uint64_t idx_base = idx_ctr[0];
-    for (uint64_t r = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; r < R;
-         r += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        const uint64_t v = rec_key[r] >> tbits;
-        const uint64_t t = rec_key[r] & tmask;
-        uint64_t m = range_mask(t, lo, hi);
-        if (m) m &= rbits[r] & alive[t];
-        while (m) {
-            int j = __ffsll(m) - 1;
-            m &= m - 1;
-            const uint64_t lane = t * 64 + j;
-            uint32_t pos = atomicAdd(&lane_fill[lane], 1u);
-            idx_nodes[idx_base + lane_off[lane] + pos] = static_cast<uint32_t>(v);
-        }
+        const uint64_t key = a.rec_key[r], t = key & tmask;
+        uint64_t m = range_mask(t, a.lo, hi);
+        if (m) m &= a.rbits[r] & __ldcg(&a.alive[t]);
+        if (m) f(static_cast<uint32_t>(key >> a.tbits), m, t);
     }
 }
 
-__global__ void k_commit_segments(const uint32_t *lane_pair, uint32_t lo, uint32_t hi, const uint64_t *lane_cnt,
-                                  const uint64_t *lane_off, const uint64_t *idx_ctr, uint64_t *seg_start,
-                                  uint32_t *seg_len) {
-    const uint64_t idx_base = idx_ctr[0];
-    for (uint64_t j = lo + blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; j <= hi;
-         j += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
-        uint64_t c = lane_cnt[j];
+// Index space for the lanes [lo, hi] from their counts, which are zero again
+// after; lane_pos = where the next entry of a lane goes.
+SKIM_DEV void step_segments(const StepArgs &a, uint32_t hi) {
+    __shared__ unsigned long long s_warp[kStepThreads / 32], s_base;
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint64_t j0 = a.lo + static_cast<uint64_t>(blockIdx.x) * kStepThreads; j0 <= hi;
+         j0 += static_cast<uint64_t>(gridDim.x) * kStepThreads) {
+        const uint64_t j = j0 + threadIdx.x;
+        uint32_t c = 0;
+        if (j <= hi) c = __ldcg(&a.lane_cnt[j]);
+        unsigned long long tot;
+        const unsigned long long ex = warp_excl_scan(c, &tot);
+        if (lane == 0) s_warp[warp] = tot;
+        __syncthreads();
+        if (warp == 0) {
+            const unsigned long long w = warp_excl_scan(s_warp[lane], &tot);
+            s_warp[lane] = w;
+            if (lane == 0) s_base = tot ? atomicAdd(reinterpret_cast<unsigned long long *>(a.idx_ctr), tot) : 0;
+        }
+        __syncthreads();
         if (c) {
-            uint32_t pr = lane_pair[j];
-            seg_start[pr] = idx_base + lane_off[j];
-            seg_len[pr] = static_cast<uint32_t>(c);
+            const uint64_t at = s_base + s_warp[warp] + ex;
+            const uint32_t pr = a.lane_pair[j];
+            a.lane_pos[j] = at;
+            a.lane_cnt[j] = 0;
+            a.seg_start[pr] = at;
+            a.seg_len[pr] = c;
         }
+        __syncthreads();
     }
 }
 
-// After a commit of `total` index entries: idx_ctr[1] = the commit's first
-// entry, idx_ctr[0] = the next free one.
-__global__ void k_idx_advance(uint64_t *idx_ctr, const unsigned long long *total) {
-    idx_ctr[1] = idx_ctr[0];
-    idx_ctr[0] += *total;
-}
-
-__global__ void k_refilter(const uint32_t *lane_pair, uint32_t lo, uint32_t B, uint32_t l, const uint64_t *covered,
-                           uint64_t *alive) {
-    for (uint32_t j = lo + blockIdx.x * blockDim.x + threadIdx.x; j < B; j += gridDim.x * blockDim.x) {
-        const uint64_t bit = 1ull << (j & 63);
-        if (!(alive[j >> 6] & bit)) continue;
-        uint32_t pr = lane_pair[j];
-        uint32_t u = pr / l, i = pr % l;
-        if ((covered[u] >> i) & 1ull) atomicAnd(reinterpret_cast<unsigned long long *>(&alive[j >> 6]), ~bit);
+__global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant__ StepArgs a) {
+    DevCtl *C = a.ctl;
+    const bool first = blockIdx.x == 0 && threadIdx.x == 0;
+    // the last search is not finished: the host ends it and launches the step again
+    if (*reinterpret_cast<volatile unsigned *>(&C->spill) | *reinterpret_cast<volatile unsigned *>(&C->err)) {
+        if (first) {
+            C->step.best = ~0ull;
+            C->step.stalled = 1;
+        }
+        return;
+    }
+    if (first) C->step.best = ~0ull;
+    if (a.refilter) step_refilter(a);
+    if (!step_barrier(C, 0, a.timeout_ns)) return;
+    if (a.scan) step_candidates(a);
+    if (!step_barrier(C, 1, a.timeout_ns)) return;
+    const uint64_t best = ld_volatile(&C->step.best);
+    const uint32_t hi = best == ~0ull ? a.B - 1 : static_cast<uint32_t>(best >> 32);
+    // additive, so a thread per record
+    unsigned long long ins = 0;
+    step_records(a, hi, [&](uint32_t v, uint64_t m, uint64_t t) {
+        const uint32_t c = __popcll(m);
+        atomicAdd(&a.size[v], c);
+        ins += c;
+        for (; m; m &= m - 1) atomicAdd(&a.lane_cnt[t * 64 + __ffsll(m) - 1], 1u);
+    });
+    __syncwarp();
+    warp_add(&C->stats[kStInsert], ins);
+    if (!step_barrier(C, 2, a.timeout_ns)) return;
+    step_segments(a, hi);
+    if (!step_barrier(C, 3, a.timeout_ns)) return;
+    step_records(a, hi, [&](uint32_t v, uint64_t m, uint64_t t) {
+        for (; m; m &= m - 1)
+            a.idx_nodes[atomicAdd(reinterpret_cast<unsigned long long *>(&a.lane_pos[t * 64 + __ffsll(m) - 1]), 1ull)] = v;
+    });
+    if (first) {  // what the host takes, and the count of the next search from zero
+        C->step.cov = C->ix_cov;
+        C->ix_cov = 0;
+        C->step.stalled = 0;
     }
 }
 
 // Section 4.3.2: add delta to the size of every node in the committed index
-// list of lane p (each node appears once in a lane's list).
-__global__ void k_lane_size_add(const uint32_t *idx_nodes, const uint64_t *idx_base, const uint64_t *lane_off,
-                                const uint64_t *lane_cnt, uint32_t p, uint32_t *size, int delta) {
-    const uint64_t off = *idx_base + lane_off[p], cnt = lane_cnt[p];
+// list of a lane (each node appears once in a lane's list).
+__global__ void k_lane_size_add(const uint32_t *idx_nodes, const uint64_t *seg_start, const uint32_t *seg_len,
+                                const uint32_t *lane_pair, uint32_t *size, int delta) {
+    const uint64_t off = seg_start[*lane_pair], cnt = seg_len[*lane_pair];
     for (uint64_t j = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; j < cnt;
          j += static_cast<uint64_t>(gridDim.x) * blockDim.x)
         size[idx_nodes[off + j]] += static_cast<uint32_t>(delta);
@@ -404,68 +458,34 @@ cudaError_t launch_gather_bits(const uint32_t *rec_val, const uint64_t *hvals, u
     k_gather_bits<<<grid_for(R, 256), 256, 0, s>>>(rec_val, hvals, R, rbits);
     return cudaGetLastError();
 }
-cudaError_t launch_candidates(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                              const uint64_t *alive, uint32_t lo, const uint32_t *size, uint32_t k, DevCtl *ctl,
-                              cudaStream_t s) {
-    if (R == 0) return cudaSuccess;
+cudaError_t launch_step(const StepArgs &a, cudaStream_t s) {
+    int dev = 0, sms = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_step, kStepThreads, 0);
+    if (e != cudaSuccess) return e;
+    const uint64_t work = std::max<uint64_t>(a.R, a.B - std::min(a.lo, a.B));
+    const unsigned grid = std::min<unsigned>(grid_for(work, kStepThreads), static_cast<unsigned>(sms) * std::min(per, 1));
     note_launch();
-    k_candidates<<<grid_for(R, 256), 256, 0, s>>>(rec_key, rbits, R, tbits, alive, lo, size, k, ctl);
-    return cudaGetLastError();
-}
-cudaError_t launch_commit_count(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                                const uint64_t *alive, uint32_t lo, uint32_t hi, uint32_t *size, uint64_t *lane_cnt,
-                                DevCtl *ctl, cudaStream_t s) {
-    if (R == 0) return cudaSuccess;
-    note_launch();
-    k_commit_count<<<grid_for(R, 256), 256, 0, s>>>(rec_key, rbits, R, tbits, alive, lo, hi, size,
-                                                    reinterpret_cast<unsigned long long *>(lane_cnt), ctl);
-    return cudaGetLastError();
-}
-cudaError_t launch_commit_scatter(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                                  const uint64_t *alive, uint32_t lo, uint32_t hi, const uint64_t *lane_off,
-                                  uint32_t *lane_fill, const uint64_t *idx_ctr, uint32_t *idx_nodes, cudaStream_t s) {
-    if (R == 0) return cudaSuccess;
-    note_launch();
-    k_commit_scatter<<<grid_for(R, 256), 256, 0, s>>>(rec_key, rbits, R, tbits, alive, lo, hi, lane_off, lane_fill,
-                                                      idx_ctr, idx_nodes);
-    return cudaGetLastError();
-}
-cudaError_t launch_commit_segments(const uint32_t *lane_pair, uint32_t lo, uint32_t hi, const uint64_t *lane_cnt,
-                                   const uint64_t *lane_off, const uint64_t *idx_ctr, uint64_t *seg_start,
-                                   uint32_t *seg_len, cudaStream_t s) {
-    note_launch();
-    k_commit_segments<<<grid_for(hi - lo + 1, 256), 256, 0, s>>>(lane_pair, lo, hi, lane_cnt, lane_off, idx_ctr,
-                                                                 seg_start, seg_len);
-    return cudaGetLastError();
-}
-cudaError_t launch_refilter(const uint32_t *lane_pair, uint32_t lo, uint32_t B, uint32_t l, const uint64_t *covered,
-                            uint64_t *alive, cudaStream_t s) {
-    if (lo >= B) return cudaSuccess;
-    note_launch();
-    k_refilter<<<grid_for(B - lo, 256), 256, 0, s>>>(lane_pair, lo, B, l, covered, alive);
-    return cudaGetLastError();
+    void *args[] = {const_cast<StepArgs *>(&a)};
+    return cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_step), dim3(grid), dim3(kStepThreads), args, 0, s);
 }
 cudaError_t launch_argmax_size(const uint32_t *size, uint32_t n, DevCtl *ctl, cudaStream_t s) {
     note_launch();
     k_argmax_size<<<grid_for(n, 256), 256, 0, s>>>(size, n, ctl);
     return cudaGetLastError();
 }
-cudaError_t launch_second_size(const uint32_t *idx_nodes, const uint64_t *idx_base, const uint64_t *lane_off,
-                               const uint64_t *lane_cnt, uint32_t p, uint32_t *size, uint32_t n, uint32_t x,
-                               uint32_t *out, cudaStream_t s) {
+cudaError_t launch_second_size(const uint32_t *idx_nodes, const uint64_t *seg_start, const uint32_t *seg_len,
+                               const uint32_t *lane_pair, uint32_t *size, uint32_t n, uint32_t x, uint32_t *out,
+                               cudaStream_t s) {
     // the stop lane's list holds at most n nodes (its length is on the device)
     const unsigned g = grid_for(n, 256, 1024);
     note_launch();
-    k_lane_size_add<<<g, 256, 0, s>>>(idx_nodes, idx_base, lane_off, lane_cnt, p, size, -1);
+    k_lane_size_add<<<g, 256, 0, s>>>(idx_nodes, seg_start, seg_len, lane_pair, size, -1);
     note_launch();
     k_max_size_except<<<grid_for(n, 256), 256, 0, s>>>(size, n, x, out);
     note_launch();
-    k_lane_size_add<<<g, 256, 0, s>>>(idx_nodes, idx_base, lane_off, lane_cnt, p, size, 1);
-    return cudaGetLastError();
-}
-cudaError_t launch_idx_advance(uint64_t *idx_ctr, const unsigned long long *total, cudaStream_t s) {
-    note_launch();
-    k_idx_advance<<<1, 1, 0, s>>>(idx_ctr, total);
+    k_lane_size_add<<<g, 256, 0, s>>>(idx_nodes, seg_start, seg_len, lane_pair, size, 1);
     return cudaGetLastError();
 }
 cudaError_t launch_min_unchosen(const uint8_t *chosen, uint32_t n, DevCtl *ctl, cudaStream_t s) {

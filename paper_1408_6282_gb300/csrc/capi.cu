@@ -85,7 +85,7 @@ struct skim_ctx {
     size_t ws_bytes = 0;
     uint8_t *lane_inst = nullptr;
     uint64_t *lane_g = nullptr;
-    uint64_t *alive = nullptr, *lane_cnt = nullptr, *lane_off = nullptr;
+    uint64_t *alive = nullptr, *lane_off = nullptr;
     uint32_t *lane_fill = nullptr;
     uint32_t lane_cap = 0;
     int grid_rev = 0, grid_coin = 0, grid_fwd = 0, grid_ring = 0;
@@ -138,6 +138,9 @@ struct skim_ctx {
     // newly covered pairs at *pend_cov
     bool pend_res = false;
     uint64_t *pend_cov = nullptr;
+    bool refilter = false;          // a search ran since the active batch's lanes were last filtered
+    bool pend_queue = false;        // it used the work queue
+    cudaEvent_t step_done = nullptr;  // of the last step's read-back
     // queries
     uint32_t *qseeds = nullptr;
     uint64_t qseeds_cap = 0;
@@ -492,7 +495,10 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
     RC(reset_ctl(c));
     CK(c, launch_lane_inst(c->spair + p0, c->rank_mode == SKIM_RANKS_IC_MODEL ? c->srank + p0 : nullptr, B, c->l,
                            c->lane_inst, c->lane_g, c->st));
-    if (!mode_build) CK(c, cudaMemsetAsync(c->alive, 0, T * sizeof(uint64_t), c->st));
+    if (!mode_build) {
+        CK(c, cudaMemsetAsync(c->alive, 0, T * sizeof(uint64_t), c->st));
+        CK(c, cudaMemsetAsync(c->lane_fill, 0, B * sizeof(uint32_t), c->st));
+    }
     TravArgs a = base_args(c, false);
     a.tbits = tbits;
     a.hnode = T <= kNodeHashWords ? 1 : 0;
@@ -684,6 +690,7 @@ int skim_state_init(skim_ctx *c) {
     c->last_gap = 0;
     c->vpl_est = 0;
     c->last_B = 0;
+    c->refilter = false;
     c->sk_init = true;
     return SKIM_OK;
 }
@@ -703,30 +710,9 @@ int ensure_idx(skim_ctx *c, uint64_t need) {
     return SKIM_OK;
 }
 
-// Commit lanes [lo, hi] of the active batch: sizes and the inverted index.
-// The index was sized for the whole batch when it was searched, and its fill
-// offset stays on the device, so a commit needs no read-back.
-int commit_lanes(skim_ctx *c, uint32_t lo, uint32_t hi) {
-    if (lo > hi) return SKIM_OK;
-    const uint32_t cnt = hi - lo + 1;
-    CK(c, cudaMemsetAsync(c->lane_cnt + lo, 0, cnt * sizeof(uint64_t), c->st));
-    CK(c, cudaMemsetAsync(c->lane_fill + lo, 0, cnt * sizeof(uint32_t), c->st));
-    KTimer kt(c, SKIM_K_STEP);
-    CK(c, launch_commit_count(c->rkey, c->rbits, c->bR, c->btbits, c->alive, lo, hi, c->size, c->lane_cnt,
-                              c->ctl, c->st));
-    CK(c, exclusive_scan_u64(c->lane_cnt + lo, c->lane_off + lo, cnt, reinterpret_cast<uint64_t *>(&c->ctl->total),
-                             c->ws, c->st));
-    CK(c, launch_commit_scatter(c->rkey, c->rbits, c->bR, c->btbits, c->alive, lo, hi, c->lane_off,
-                                c->lane_fill, c->idx_ctr, c->idx, c->st));
-    CK(c, launch_commit_segments(c->spair + c->bp0, lo, hi, c->lane_cnt, c->lane_off, c->idx_ctr, c->seg_start,
-                                 c->seg_len, c->st));
-    CK(c, launch_idx_advance(c->idx_ctr, &c->ctl->total, c->st));
-    return SKIM_OK;
-}
-
 // Finish the pending residual search, after a read of the control block that
 // followed it.  A search that parked work (its queue overflowed) resumes until
-// the queue drains; the lane filter launched after it then runs again, and
+// the queue drains, and
 // *again tells the caller that what it read back (stop candidate, argmax) was
 // computed before the search had finished.  Then the search's count of newly
 // covered pairs goes out and the queue is emptied.
@@ -749,11 +735,10 @@ int finish_residual(skim_ctx *c, bool *again) {
             CK(c, launch_respill_fwd(a, c->n, c->st));
         }
         RC(run_traversal(c, a, true, nullptr));
-        if (c->batch_active)
-            CK(c, launch_refilter(c->spair + c->bp0, c->blo, c->bB, c->l, c->covered, c->alive, c->st));
+        c->pend_queue = true;
     }
     *c->pend_cov = c->hctl->ix_cov;
-    RC(reset_queue(c, c->hctl->q_tail.v));
+    if (c->pend_queue) RC(reset_queue(c, c->hctl->q_tail.v));
     return SKIM_OK;
 }
 
@@ -763,6 +748,23 @@ int settle_residual(skim_ctx *c) {
     RC(sync_ctl(c));
     bool again = false;
     return finish_residual(c, &again);
+}
+
+bool by_blocks(const skim_ctx *c) {
+    return c->mat && (c->l >= kReachInst || c->live_total <= kReachPairs * c->l);
+}
+
+int residual_blocks(skim_ctx *c, uint32_t x) {
+    KTimer kt(c, SKIM_K_FWD);
+    ReachArgs r = reach_args(c, c->covered, 1);
+    r.pend_trav = c->pend_trav;
+    r.seg_start = c->seg_start;
+    r.seg_len = c->seg_len;
+    r.size = c->size;
+    r.idx_nodes = c->idx;
+    r.chosen = c->chosen;
+    CK(c, launch_reach(r, x, c->st));
+    return SKIM_OK;
 }
 
 // Residual problem for seed x: forward search in every instance.  The search
@@ -779,16 +781,9 @@ int residual(skim_ctx *c, uint32_t x, uint64_t *cov) {
         cudaEventCreate(&t1);
         cudaEventRecord(t0, c->st);
     }
-    if (c->mat && (c->l >= kReachInst || c->live_total <= kReachPairs * c->l)) {
-        KTimer kt(c, SKIM_K_FWD);
-        ReachArgs r = reach_args(c, c->covered, 1);
-        r.pend_trav = c->pend_trav;
-        r.seg_start = c->seg_start;
-        r.seg_len = c->seg_len;
-        r.size = c->size;
-        r.idx_nodes = c->idx;
-        r.chosen = c->chosen;
-        CK(c, launch_reach(r, x, c->st));
+    c->pend_queue = !by_blocks(c);
+    if (by_blocks(c)) {
+        RC(residual_blocks(c, x));
     } else {
         CK(c, launch_fwd_source(a, x, c->st));
         {
@@ -815,44 +810,69 @@ int residual(skim_ctx *c, uint32_t x, uint64_t *cov) {
     return SKIM_OK;
 }
 
+// A step over what is left of the active batch; scan false: commit all of it.
+StepArgs step_args(const skim_ctx *c, bool scan) {
+    return StepArgs{c->rkey, c->rbits, c->bR, c->btbits, c->blo, c->bB, c->l, c->k, c->refilter ? 1u : 0u, scan ? 1u : 0u,
+                    c->spair + c->bp0, c->covered, c->alive, c->size, c->lane_fill, c->lane_off, c->idx_ctr, c->idx,
+                    c->seg_start, c->seg_len, c->ctl, c->timeout_ns};
+}
+
 int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
     for (;;) {
         if (c->batch_active) {
-            CK(c, cudaMemsetAsync(&c->ctl->best, 0xff, sizeof(unsigned long long), c->st));
             {
                 KTimer kt(c, SKIM_K_STEP);
-                CK(c, launch_candidates(c->rkey, c->rbits, c->bR, c->btbits, c->alive, c->blo, c->size,
-                                        c->k, c->ctl, c->st));
+                CK(c, launch_step(step_args(c, true), c->st));
             }
-            RC(sync_ctl(c));
+            // the search of the seed it finds goes behind it at once, unless
+            // something has to come between or each is timed alone
+            const bool ahead = by_blocks(c) && !c->rec_tau && !c->timing && !trace_batches();
+            if (ahead) {
+                CK(c, cudaMemcpyAsync(c->hctl, c->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, c->st));
+                CK(c, cudaEventRecord(c->step_done, c->st));
+                RC(residual_blocks(c, kSeedOfStep));
+                CK(c, cudaEventSynchronize(c->step_done));
+            } else {
+                RC(sync_ctl(c));
+            }
             {
+                if (c->hctl->err & kErrTimeout) {  // of the search before or of the step
+                    c->broken = true;
+                    return SKIM_ETIMEOUT;
+                }
                 bool again = false;
+                if (!c->hctl->step.stalled) c->hctl->ix_cov = c->hctl->step.cov;
                 RC(finish_residual(c, &again));
-                if (again) continue;  // the scan ran before the last seed's search had finished
+                if (again) continue;  // the step found the last seed's search unfinished and did nothing
             }
-            const uint64_t best = c->hctl->best;
+            c->refilter = false;
+            const uint64_t best = c->hctl->step.best;
             if (best != ~0ull) {
                 const uint32_t p = static_cast<uint32_t>(best >> 32);
                 const uint32_t x = static_cast<uint32_t>(best & 0xffffffffu);
-                RC(commit_lanes(c, c->blo, p));
                 if (c->rec_tau) {
                     CK(c, cudaMemcpyAsync(c->rec_tau + c->rec_j, c->srank + c->bp0 + p, sizeof(uint64_t),
                                           cudaMemcpyDeviceToDevice, c->st));
-                    CK(c, launch_second_size(c->idx, c->idx_ctr + 1, c->lane_off, c->lane_cnt, p, c->size, c->n, x,
+                    CK(c, launch_second_size(c->idx, c->seg_start, c->seg_len, c->spair + c->bp0 + p, c->size, c->n, x,
                                              c->rec_kp + c->rec_j, c->st));
                 }
-                RC(residual(c, x, cov_out));
+                if (ahead) {
+                    c->pend_res = true;
+                    c->pend_queue = false;
+                    c->pend_cov = cov_out;
+                } else {
+                    RC(residual(c, x, cov_out));
+                }
                 {
                     const uint64_t after = c->bB - 1 - p;  // batch lanes not yet consumed
                     c->last_gap = c->since_stop - after;
                     c->since_stop = after;
                 }
                 c->blo = p + 1;
-                CK(c, launch_refilter(c->spair + c->bp0, c->blo, c->bB, c->l, c->covered, c->alive, c->st));
+                c->refilter = true;
                 *x_out = x;
                 return SKIM_OK;
             }
-            RC(commit_lanes(c, c->blo, c->bB - 1));
             RC(clear_batch(c));
             c->batch_active = false;
             continue;
@@ -894,6 +914,7 @@ int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
             c->bp0 = c->cursor;
             c->bB = B;
             c->blo = 0;
+            c->refilter = false;
             c->cursor += B;
             c->hstats[SKIM_STAT_RANKS] += B;
             c->since_stop += B;
@@ -1069,12 +1090,13 @@ int skim_destroy(skim_ctx *c) {
     dfree(c, c->rbase); dfree(c, c->rtm1); dfree(c, c->ftm1);
     dfree(c, c->ctl); dfree(c, c->dflag);
     if (c->hctl) cudaFreeHost(c->hctl);
+    if (c->step_done) cudaEventDestroy(c->step_done);
     dfree(c, c->q); dfree(c, c->hkeys); dfree(c, c->pend);
     c->hvals = nullptr;
     dfree(c, c->rkey); dfree(c, c->rkey2); dfree(c, c->rval); dfree(c, c->rval2);
     dfree(c, c->ncnt); dfree(c, c->noff); dfree(c, c->nlist); dfree(c, c->nlist_cnt);
     dfree(c, c->ws);
-    dfree(c, c->lane_inst); dfree(c, c->lane_g); dfree(c, c->alive); dfree(c, c->lane_cnt); dfree(c, c->lane_off); dfree(c, c->lane_fill);
+    dfree(c, c->lane_inst); dfree(c, c->lane_g); dfree(c, c->alive); dfree(c, c->lane_off); dfree(c, c->lane_fill);
     dfree(c, c->nonempty); dfree(c, c->need); dfree(c, c->comp); dfree(c, c->comp_up);
     dfree(c, c->over_seg); dfree(c, c->over_buf); dfree(c, c->full_list); dfree(c, c->hitbits); dfree(c, c->defbits); dfree(c, c->defpair);
     dfree(c, c->node_off); dfree(c, c->comp_ws); dfree(c, c->need_ws);
@@ -1167,6 +1189,7 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
     {
         TRY(dalloc(c, &c->ctl, 1));
         TRYC(cudaMallocHost(reinterpret_cast<void **>(&c->hctl), sizeof(DevCtl) + sizeof(double)));
+        TRYC(cudaEventCreateWithFlags(&c->step_done, cudaEventDisableTiming));
         c->hq = reinterpret_cast<double *>(c->hctl + 1);
         TRYC(cudaMemsetAsync(c->ctl, 0, sizeof(DevCtl), c->st));
         TRY(dalloc(c, &c->dflag, 1));
@@ -1284,7 +1307,6 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
         TRYC(cudaMemsetAsync(c->lane_inst, 0, c->lane_cap, c->st));
         TRY(dalloc(c, &c->lane_g, c->lane_cap));
         TRY(dalloc(c, &c->alive, c->lane_cap / 64 + 1));
-        TRY(dalloc(c, &c->lane_cnt, c->lane_cap));
         TRY(dalloc(c, &c->lane_off, c->lane_cap));
         TRY(dalloc(c, &c->lane_fill, c->lane_cap));
         c->grid_rev = traverse_grid(false, true);
@@ -1932,7 +1954,7 @@ int skim_build_sketches(skim_ctx *c) {
         RC(dalloc(c, &c->X, static_cast<size_t>(c->n) * c->k));
     }
     if (c->batch_active) {  // a SKIM batch holds the visited table: release it
-        RC(commit_lanes(c, c->blo, c->bB - 1));
+        CK(c, launch_step(step_args(c, false), c->st));
         RC(clear_batch(c));
         c->batch_active = false;
     }
@@ -1987,7 +2009,6 @@ int skim_set_live_rows(skim_ctx *c, int on) {
     if (!c) return SKIM_EINVAL;
     if (c->broken) return SKIM_ECUDA;
     if (c->batch_active) {
-        RC(commit_lanes(c, c->blo, c->bB - 1));
         RC(clear_batch(c));
         c->batch_active = false;
     }

@@ -129,6 +129,13 @@ struct BuildCtl {
     unsigned failed;                // a need pass ran into the wait limit
 };
 
+// Of the SKIM steps (batch.cu): barrier counters; the stop (lane << 32) | node, or
+// ~0; pairs covered by the search before; that search is unfinished.
+struct StepCtl {
+    unsigned long long best, cov;
+    unsigned bar[4], stalled;
+};
+
 // Device control block: queue cursors, counters, flags, reductions.
 // src_next, busy and beat serve the reverse searches with per-warp queues:
 // the next unclaimed source lane of the batch, the warps that hold work, and
@@ -136,15 +143,15 @@ struct BuildCtl {
 struct DevCtl {
     HotCounter q_head, q_tail, q_done, rec_count;
     HotCounter src_next, busy, beat;
-    unsigned long long best;        // SKIM stop candidate: (lane << 32) | node
+    unsigned long long best;        // smallest node not chosen
     unsigned long long ix_cov;      // pairs newly covered by the residual search
     unsigned long long argmax;      // (size << 32) | ~node
-    unsigned long long total;       // generic total (lane commits)
     unsigned long long stats[8];
     unsigned int err;
     unsigned int spill;   // some work was parked in pending masks
     unsigned int pad[2];
     BuildCtl b;
+    StepCtl step;
 };
 
 enum Stat { kStRevVisits = 0, kStRevCoins, kStInsert, kStFwdVisits, kStFwdCoins, kStRevEdges, kStFwdEdges };

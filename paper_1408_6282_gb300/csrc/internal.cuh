@@ -177,6 +177,7 @@ struct ReachArgs {
     DevCtl *ctl;
     uint64_t timeout_ns;
 };
+constexpr uint32_t kSeedOfStep = 0xffffffffu;  // as x: the seed in ctl->step.best, nothing if there is none
 cudaError_t launch_reach(const ReachArgs &a, uint32_t x, cudaStream_t s);
 // What the nodes pivot[64 * q + i], q < starts, reach in instance i, for every
 // instance: its bit in mask
@@ -279,32 +280,36 @@ cudaError_t launch_node_sort(uint64_t *rec_key, uint32_t *rec_val, uint64_t R, u
                              uint64_t *cnt, uint64_t *off, uint64_t *tmp, uint32_t *list, unsigned *nlist,
                              void *scan_ws, cudaStream_t s);
 // SKIM batch: the records' lane bits gathered from the visited table into
-// rbits (R words), read by the three kernels below.
+// rbits (R words), read by the steps.
 cudaError_t launch_gather_bits(const uint32_t *rec_val, const uint64_t *hvals, uint64_t R, uint64_t *rbits,
                                cudaStream_t s);
-cudaError_t launch_candidates(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                              const uint64_t *alive, uint32_t lo, const uint32_t *size, uint32_t k, DevCtl *ctl,
-                              cudaStream_t s);
-cudaError_t launch_commit_count(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                                const uint64_t *alive, uint32_t lo, uint32_t hi, uint32_t *size, uint64_t *lane_cnt,
-                                DevCtl *ctl, cudaStream_t s);
-cudaError_t launch_commit_scatter(const uint64_t *rec_key, const uint64_t *rbits, uint64_t R, uint32_t tbits,
-                                  const uint64_t *alive, uint32_t lo, uint32_t hi, const uint64_t *lane_off,
-                                  uint32_t *lane_fill, const uint64_t *idx_ctr, uint32_t *idx_nodes, cudaStream_t s);
-cudaError_t launch_commit_segments(const uint32_t *lane_pair, uint32_t lo, uint32_t hi, const uint64_t *lane_cnt,
-                                   const uint64_t *lane_off, const uint64_t *idx_ctr, uint64_t *seg_start,
-                                   uint32_t *seg_len, cudaStream_t s);
-// idx_ctr[1] = idx_ctr[0]; idx_ctr[0] += *total (the index entries a commit added)
-cudaError_t launch_idx_advance(uint64_t *idx_ctr, const unsigned long long *total, cudaStream_t s);
-cudaError_t launch_refilter(const uint32_t *lane_pair, uint32_t lo, uint32_t B, uint32_t l, const uint64_t *covered,
-                            uint64_t *alive, cudaStream_t s);
+// A step over the active batch's R records: the lanes [lo, B) of covered sources
+// dropped (refilter), the next stop (scan) into ctl->step.best ((lane << 32) | node, ~0 if
+// there is none), the lanes up to it (or all) committed.  ctl->step.cov = the last
+// search's count; nothing is done and ctl->step.stalled set if it is unfinished.
+struct StepArgs {
+    const uint64_t *rec_key, *rbits;
+    uint64_t R;
+    uint32_t tbits, lo, B, l, k, refilter, scan;
+    const uint32_t *lane_pair;
+    const uint64_t *covered;
+    uint64_t *alive;
+    uint32_t *size, *lane_cnt;  // lane_cnt: zero on entry and on return
+    uint64_t *lane_pos, *idx_ctr;
+    uint32_t *idx_nodes;
+    uint64_t *seg_start;
+    uint32_t *seg_len;
+    DevCtl *ctl;
+    uint64_t timeout_ns;
+};
+cudaError_t launch_step(const StepArgs &a, cudaStream_t s);
 cudaError_t launch_argmax_size(const uint32_t *size, uint32_t n, DevCtl *ctl, cudaStream_t s);
 cudaError_t launch_min_unchosen(const uint8_t *chosen, uint32_t n, DevCtl *ctl, cudaStream_t s);
-// Section 4.3.2: k' = max size over v != x with the stop lane p taken out
-// (sizes are restored); atomicMax into *out, which the caller zeroes.
-cudaError_t launch_second_size(const uint32_t *idx_nodes, const uint64_t *idx_base, const uint64_t *lane_off,
-                               const uint64_t *lane_cnt, uint32_t p, uint32_t *size, uint32_t n, uint32_t x,
-                               uint32_t *out, cudaStream_t s);
+// Section 4.3.2: k' = max size over v != x with the stop lane (of *lane_pair)
+// taken out (sizes are restored); atomicMax into *out, which the caller zeroes.
+cudaError_t launch_second_size(const uint32_t *idx_nodes, const uint64_t *seg_start, const uint32_t *seg_len,
+                               const uint32_t *lane_pair, uint32_t *size, uint32_t n, uint32_t x, uint32_t *out,
+                               cudaStream_t s);
 
 // query.cu
 // Scratch of the queries: per-block partial sums, counters of the larger queries'

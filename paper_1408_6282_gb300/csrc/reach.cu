@@ -220,7 +220,8 @@ struct Reach {
 };
 
 // Block i searches instance i, from node x (RES: the residual search of seed
-// x) or from the pivots of instance i (blocks from l on: against the edges).  The wait of a level's barrier is bounded like every
+// x, or of the seed the step before it found, if any) or from the pivots of instance i
+// (blocks from l on: against the edges).  The wait of a level's barrier is bounded like every
 // other wait: a level that takes longer than the limit ends the search with
 // the error flag.
 template <bool RES>
@@ -228,6 +229,10 @@ __global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_
                                                             uint32_t starts, uint32_t *count) {
     extern __shared__ char s_raw[];
     ReachShared &sh = *reinterpret_cast<ReachShared *>(s_raw);
+    if (RES && x == kSeedOfStep) {
+        if (A.ctl->step.best == ~0ull) return;
+        x = static_cast<uint32_t>(A.ctl->step.best);
+    }
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool back = !RES && blockIdx.x >= A.l;
     const uint32_t inst = back ? blockIdx.x - A.l : blockIdx.x;

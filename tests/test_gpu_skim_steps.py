@@ -1,0 +1,44 @@
+"""SKIM steps (batch.cu) where they can go wrong: the search queued behind the step
+and the search that waits for it, batches of one lane word, of a word and a bit
+and of all ranks, stops at a batch's last lane, searches that park work and make
+the step wait, ranks that run out, a run in pieces with a sketch build between.
+Seeds and coverages are whole numbers and must equal the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+GRAPHS = {
+    "rmat10": lambda: synth.rmat(10, 8, 3),
+    "er2003": lambda: synth.erdos_renyi(2003, 9000, 4),
+    "clique": lambda: synth.clique(70),
+}
+
+
+@pytest.mark.parametrize("items", [None, 128])
+@pytest.mark.parametrize("name", list(GRAPHS))
+@pytest.mark.parametrize("l,k,p,bl", [(64, 16, 0.2, 0), (33, 2, 0.1, 64), (64, 5, 0.05, 65), (1, 3, 0.4, 128),
+                                      (40, 64, 0.3, 1000)])
+def test_steps_match_oracle(monkeypatch, name, l, k, p, bl, items):
+    import paper_1408_6282_gb300 as pkg
+    g = GRAPHS[name]()
+    ks = synth.Keys.from_seed(l + k)
+    if items:
+        monkeypatch.setenv("SKIM_QUEUE_ITEMS", str(items))
+    pb = oracle.Problem(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
+    seeds, cov, tau, kp, _ = oracle.skim_stops(pb, 40)
+    with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, batch_lanes=bl) as sk:
+        a, b = sk.greedy(40)
+        assert np.array_equal(a, seeds) and np.array_equal(b, cov)
+        sk.greedy_reset()
+        parts = [sk.greedy(1), sk.greedy_stops(20)[:2], sk.greedy(19)]
+        assert np.array_equal(np.concatenate([x[0] for x in parts]), seeds)
+        assert np.array_equal(np.concatenate([x[1] for x in parts]), cov)
+        sk.greedy_reset()
+        sk.greedy(7)
+        sk.build_sketches()  # commits the active batch unscanned
+        x, ln = sk.sketches()
+        ox, oln, _ = oracle.build_sketches(pb)
+        assert np.array_equal(ln, oln) and np.array_equal(x, ox)
