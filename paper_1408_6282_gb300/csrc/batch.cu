@@ -233,11 +233,12 @@ SKIM_DEV bool step_barrier(DevCtl *ctl, int i, uint64_t timeout_ns) {
     return s_ok != 0;
 }
 
-// Lanes from lo on whose source was covered are no longer alive.
+// Lanes from lo on whose source was covered are no longer alive.  (Leaf lanes are
+// looked at when they are committed.)
 SKIM_DEV void step_refilter(const StepArgs &a) {
     for (uint32_t j = a.lo + blockIdx.x * blockDim.x + threadIdx.x; j < a.B; j += gridDim.x * blockDim.x) {
         const uint64_t bit = 1ull << (j & 63);
-        if (!(a.alive[j >> 6] & bit)) continue;
+        if (!(a.alive[j >> 6] & ~a.leaf[j >> 6] & bit)) continue;
         const uint32_t pr = a.lane_pair[j], u = pr / a.l, i = pr % a.l;
         if ((a.covered[u] >> i) & 1ull) atomicAnd(reinterpret_cast<unsigned long long *>(&a.alive[j >> 6]), ~bit);
     }
@@ -351,6 +352,30 @@ SKIM_DEV void step_segments(const StepArgs &a, uint32_t hi) {
     }
 }
 
+// The leaf lanes of [lo, hi]; returns their number.
+SKIM_DEV uint32_t step_leafs(const StepArgs &a, uint32_t hi) {
+    uint32_t n = 0;
+    for (uint64_t j = a.lo + blockIdx.x * blockDim.x + threadIdx.x; j <= hi; j += gridDim.x * blockDim.x) {
+        if (!((a.leaf[j >> 6] & __ldcg(&a.alive[j >> 6])) >> (j & 63) & 1u)) continue;
+        const uint32_t pr = a.lane_pair[j], u = pr / a.l;
+        if (a.covered[u] >> (pr - u * a.l) & 1u) continue;
+        atomicAdd(&a.size[u], 1u);
+        a.seg_len[pr] = kLeafSegment;
+        n++;
+    }
+    return n;
+}
+
+// k' of Section 4.3.2: the largest size among the nodes other than x.
+SKIM_DEV void step_second(const StepArgs &a, uint32_t x) {
+    uint32_t best = 0;
+    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < a.n; v += gridDim.x * blockDim.x)
+        if (v != x) best = max(best, __ldcg(&a.size[v]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_down_sync(kFull, best, o));
+    if ((threadIdx.x & 31) == 0 && best) atomicMax(a.kprime, best);
+}
+
 __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant__ StepArgs a) {
     DevCtl *C = a.ctl;
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
@@ -369,11 +394,13 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant_
     if (!step_barrier(C, 1, a.timeout_ns)) return;
     const uint64_t best = ld_volatile(&C->step.best);
     const uint32_t hi = best == ~0ull ? a.B - 1 : static_cast<uint32_t>(best >> 32);
-    // additive, so a thread per record
-    unsigned long long ins = 0;
+    // Additive, so a thread per record.  The stop lane's own part of the sizes
+    // follows in the last phase: k' is counted without it.
+    const uint64_t stop = best == ~0ull ? ~0ull : hi;
+    unsigned long long ins = step_leafs(a, hi);
     step_records(a, hi, [&](uint32_t v, uint64_t m, uint64_t t) {
-        const uint32_t c = __popcll(m);
-        atomicAdd(&a.size[v], c);
+        const uint32_t c = __popcll(m), d = t == stop >> 6 ? static_cast<uint32_t>(m >> (stop & 63)) & 1u : 0;
+        if (c > d) atomicAdd(&a.size[v], c - d);
         ins += c;
         for (; m; m &= m - 1) atomicAdd(&a.lane_cnt[t * 64 + __ffsll(m) - 1], 1u);
     });
@@ -381,8 +408,13 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant_
     warp_add(&C->stats[kStInsert], ins);
     if (!step_barrier(C, 2, a.timeout_ns)) return;
     step_segments(a, hi);
+    if (a.kprime && best != ~0ull) {
+        step_second(a, static_cast<uint32_t>(best));
+        if (first) *a.tau = a.lane_rank[hi];
+    }
     if (!step_barrier(C, 3, a.timeout_ns)) return;
     step_records(a, hi, [&](uint32_t v, uint64_t m, uint64_t t) {
+        if (t == stop >> 6 && (m >> (stop & 63) & 1u)) atomicAdd(&a.size[v], 1u);
         for (; m; m &= m - 1)
             a.idx_nodes[atomicAdd(reinterpret_cast<unsigned long long *>(&a.lane_pos[t * 64 + __ffsll(m) - 1]), 1ull)] = v;
     });
@@ -391,26 +423,6 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant_
         C->ix_cov = 0;
         C->step.stalled = 0;
     }
-}
-
-// Section 4.3.2: add delta to the size of every node in the committed index
-// list of a lane (each node appears once in a lane's list).
-__global__ void k_lane_size_add(const uint32_t *idx_nodes, const uint64_t *seg_start, const uint32_t *seg_len,
-                                const uint32_t *lane_pair, uint32_t *size, int delta) {
-    const uint64_t off = seg_start[*lane_pair], cnt = seg_len[*lane_pair];
-    for (uint64_t j = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; j < cnt;
-         j += static_cast<uint64_t>(gridDim.x) * blockDim.x)
-        size[idx_nodes[off + j]] += static_cast<uint32_t>(delta);
-}
-
-// k' of Section 4.3.2: the largest size among nodes other than x.
-__global__ void k_max_size_except(const uint32_t *size, uint32_t n, uint32_t x, uint32_t *out) {
-    uint32_t best = 0;
-    for (uint32_t v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x)
-        if (v != x) best = max(best, size[v]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_down_sync(kFull, best, o));
-    if ((threadIdx.x & 31) == 0 && best) atomicMax(out, best);
 }
 
 __global__ void k_argmax_size(const uint32_t *size, uint32_t n, DevCtl *ctl) {
@@ -473,19 +485,6 @@ cudaError_t launch_step(const StepArgs &a, cudaStream_t s) {
 cudaError_t launch_argmax_size(const uint32_t *size, uint32_t n, DevCtl *ctl, cudaStream_t s) {
     note_launch();
     k_argmax_size<<<grid_for(n, 256), 256, 0, s>>>(size, n, ctl);
-    return cudaGetLastError();
-}
-cudaError_t launch_second_size(const uint32_t *idx_nodes, const uint64_t *seg_start, const uint32_t *seg_len,
-                               const uint32_t *lane_pair, uint32_t *size, uint32_t n, uint32_t x, uint32_t *out,
-                               cudaStream_t s) {
-    // the stop lane's list holds at most n nodes (its length is on the device)
-    const unsigned g = grid_for(n, 256, 1024);
-    note_launch();
-    k_lane_size_add<<<g, 256, 0, s>>>(idx_nodes, seg_start, seg_len, lane_pair, size, -1);
-    note_launch();
-    k_max_size_except<<<grid_for(n, 256), 256, 0, s>>>(size, n, x, out);
-    note_launch();
-    k_lane_size_add<<<g, 256, 0, s>>>(idx_nodes, seg_start, seg_len, lane_pair, size, 1);
     return cudaGetLastError();
 }
 cudaError_t launch_min_unchosen(const uint8_t *chosen, uint32_t n, DevCtl *ctl, cudaStream_t s) {

@@ -85,7 +85,7 @@ struct skim_ctx {
     size_t ws_bytes = 0;
     uint8_t *lane_inst = nullptr;
     uint64_t *lane_g = nullptr;
-    uint64_t *alive = nullptr, *lane_off = nullptr;
+    uint64_t *alive = nullptr, *leaf = nullptr, *lane_off = nullptr;
     uint32_t *lane_fill = nullptr;
     uint32_t lane_cap = 0;
     int grid_rev = 0, grid_coin = 0, grid_fwd = 0, grid_ring = 0;
@@ -107,7 +107,7 @@ struct skim_ctx {
     // SKIM
     bool sk_init = false;
     uint64_t *covered = nullptr, *seg_start = nullptr, *pend_trav = nullptr, *pend_erase = nullptr;
-    uint32_t *size = nullptr, *seg_len = nullptr, *idx = nullptr;
+    uint32_t *size = nullptr, *seg_len = nullptr, *idx = nullptr, *ncount = nullptr;
     uint8_t *chosen = nullptr;
     uint64_t idx_cap = 0;
     // inverted index fill: on the device [0] entries used, [1] first entry of
@@ -385,7 +385,7 @@ struct RevSources {
     const uint32_t *lane_pair;
     uint32_t B;
     const uint64_t *covered;
-    uint64_t *alive;
+    uint64_t *alive, *leaf;
 };
 
 // Run traversal rounds until the queue drains with nothing spilled.  With
@@ -396,10 +396,14 @@ int run_traversal(skim_ctx *c, TravArgs &a, bool forward, uint64_t *R_out, const
         {
             KTimer kt(c, forward ? SKIM_K_FWD : SKIM_K_REV);
             if (rs)
-                CK(c, launch_rev_ring(a, rs->lane_pair, rs->B, c->l, rs->covered, rs->alive, first, c->grid_ring,
-                                      c->st));
+                CK(c, launch_rev_ring(a, rs->lane_pair, rs->B, c->l, rs->covered, rs->alive, rs->leaf, first,
+                                      c->grid_ring, c->st));
             else
                 CK(c, launch_traverse(a, forward, forward ? c->grid_fwd : c->mat ? c->grid_rev : c->grid_coin, c->st));
+        }
+        if (rs && rs->leaf) {
+            KTimer kt(c, SKIM_K_SOURCES);
+            CK(c, launch_leaf_records(a, rs->lane_pair, rs->B, c->l, rs->leaf, c->k, c->st));
         }
         RC(sync_ctl(c));
         const DevCtl &h = *c->hctl;
@@ -437,6 +441,12 @@ constexpr uint32_t kPlaceBits = SKIM_PLACE_BITS;
 // visited-table slots per expected visit record of a batch, and per lane when
 // the records per lane are not known yet
 constexpr double kTableSlots = SKIM_TABLE_SLOTS;
+// SKIM batches of at least this many lanes leave the lanes of sources without a
+// live in-neighbour out of the search (traverse.cu: k_leaf_records): two clears and a
+// launch more, 15 us.  50 seeds of R-MAT 18 wc, whose batches have up to 38 K lanes:
+// 9.6 ms without, 9.8 with; R-MAT 20 p = 0.01, up to 2 M lanes: 27 and 20 ms.
+constexpr uint32_t kLeafLanes = 1 << 16;
+constexpr double kTableLeast = 0.25;  // records per lane a table is sized for at least (leaf lanes may become records)
 #ifndef SKIM_RING_RECORDS_PER_LANE
 #define SKIM_RING_RECORDS_PER_LANE 8
 #endif
@@ -497,6 +507,7 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
                            c->lane_inst, c->lane_g, c->st));
     if (!mode_build) {
         CK(c, cudaMemsetAsync(c->alive, 0, T * sizeof(uint64_t), c->st));
+        CK(c, cudaMemsetAsync(c->leaf, 0, T * sizeof(uint64_t), c->st));
         CK(c, cudaMemsetAsync(c->lane_fill, 0, B * sizeof(uint32_t), c->st));
     }
     TravArgs a = base_args(c, false);
@@ -505,7 +516,7 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
     {
         uint64_t want = c->hcap;
         if (est_per_lane > 0)
-            want = static_cast<uint64_t>(kTableSlots * est_per_lane * static_cast<double>(B));
+            want = static_cast<uint64_t>(kTableSlots * std::max(est_per_lane, kTableLeast) * static_cast<double>(B));
         want = pow2_at_least(std::max<uint64_t>(1ull << 16, want));
         a.hmask = std::min(want, c->hcap) - 1;
         CK(c, clear_table(c, a.hmask + 1));
@@ -529,7 +540,13 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
     }
     const bool use_ring = c->mat && SKIM_REV_RING && est_per_lane > 0 && est_per_lane <= c->ring_rpl;
     if (use_ring) {
-        const RevSources rs{c->spair + p0, B, mode_build ? nullptr : c->covered, mode_build ? nullptr : c->alive};
+        const bool leafs = !mode_build && B >= kLeafLanes;
+        const RevSources rs{c->spair + p0, B, mode_build ? nullptr : c->covered, mode_build ? nullptr : c->alive,
+                            leafs ? c->leaf : nullptr};
+        if (leafs) {
+            a.cnt = c->ncount;
+            CK(c, cudaMemsetAsync(c->ncount, 0, c->n * sizeof(uint32_t), c->st));
+        }
         RC(run_traversal(c, a, false, &R, &rs));
     } else {
         {
@@ -613,7 +630,7 @@ int clear_batch(skim_ctx *c) {
 
 int pull_stats(skim_ctx *c) {
     RC(sync_ctl(c));
-    c->hstats[SKIM_STAT_REV_VISITS] = c->hctl->stats[kStRevVisits];
+    c->hstats[SKIM_STAT_REV_VISITS] = c->hctl->stats[kStRevVisits] + c->hctl->stats[kStLeafs];
     c->hstats[SKIM_STAT_REV_COINS] = c->hctl->stats[kStRevCoins];
     c->hstats[SKIM_STAT_INSERTIONS] = c->hctl->stats[kStInsert];
     c->hstats[SKIM_STAT_FWD_VISITS] = c->hctl->stats[kStFwdVisits];
@@ -660,12 +677,24 @@ uint32_t default_lanes(skim_ctx *c) {
     return static_cast<uint32_t>(std::max<uint64_t>(64, b));
 }
 
+// Lanes of a SKIM batch when the caller sets none.  A batch is sized by its
+// visits (next_seed), and most lanes of a sparse one are leaf lanes: 50 seeds of
+// R-MAT 20 p = 0.01 take 20, 19, 17.8, 17.0 ms with at most 2, 4, 8, 16 M.
+#ifndef SKIM_SL
+#define SKIM_SL 24
+#endif
+uint32_t skim_lanes(skim_ctx *c) {
+    return c->batch_cfg ? default_lanes(c) : static_cast<uint32_t>(std::min<uint64_t>(1ull << SKIM_SL, c->lane_cap));
+}
+
 // ---- SKIM steps ------------------------------------------------------------
 
 int skim_state_init(skim_ctx *c) {
     if (!c->covered) {
         RC(dalloc(c, &c->covered, c->n));
         RC(dalloc(c, &c->size, c->n));
+        RC(dalloc(c, &c->ncount, c->n));
+        RC(dalloc(c, &c->leaf, c->lane_cap / 64 + 1));
         RC(dalloc(c, &c->seg_start, c->nl));
         RC(dalloc(c, &c->seg_len, c->nl));
         RC(dalloc(c, &c->chosen, c->n));
@@ -813,8 +842,9 @@ int residual(skim_ctx *c, uint32_t x, uint64_t *cov) {
 // A step over what is left of the active batch; scan false: commit all of it.
 StepArgs step_args(const skim_ctx *c, bool scan) {
     return StepArgs{c->rkey, c->rbits, c->bR, c->btbits, c->blo, c->bB, c->l, c->k, c->refilter ? 1u : 0u, scan ? 1u : 0u,
-                    c->spair + c->bp0, c->covered, c->alive, c->size, c->lane_fill, c->lane_off, c->idx_ctr, c->idx,
-                    c->seg_start, c->seg_len, c->ctl, c->timeout_ns};
+                    c->spair + c->bp0, c->covered, c->alive, c->leaf, c->size, c->lane_fill, c->lane_off, c->idx_ctr, c->idx,
+                    c->seg_start, c->seg_len, c->ctl, c->timeout_ns, c->n, c->rec_tau && scan ? c->rec_kp + c->rec_j : nullptr,
+                    c->rec_tau ? c->rec_tau + c->rec_j : nullptr, c->srank + c->bp0};
 }
 
 int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
@@ -825,8 +855,8 @@ int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
                 CK(c, launch_step(step_args(c, true), c->st));
             }
             // the search of the seed it finds goes behind it at once, unless
-            // something has to come between or each is timed alone
-            const bool ahead = by_blocks(c) && !c->rec_tau && !c->timing && !trace_batches();
+            // each is timed alone
+            const bool ahead = by_blocks(c) && !c->timing && !trace_batches();
             if (ahead) {
                 CK(c, cudaMemcpyAsync(c->hctl, c->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, c->st));
                 CK(c, cudaEventRecord(c->step_done, c->st));
@@ -850,12 +880,6 @@ int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
             if (best != ~0ull) {
                 const uint32_t p = static_cast<uint32_t>(best >> 32);
                 const uint32_t x = static_cast<uint32_t>(best & 0xffffffffu);
-                if (c->rec_tau) {
-                    CK(c, cudaMemcpyAsync(c->rec_tau + c->rec_j, c->srank + c->bp0 + p, sizeof(uint64_t),
-                                          cudaMemcpyDeviceToDevice, c->st));
-                    CK(c, launch_second_size(c->idx, c->seg_start, c->seg_len, c->spair + c->bp0 + p, c->size, c->n, x,
-                                             c->rec_kp + c->rec_j, c->st));
-                }
                 if (ahead) {
                     c->pend_res = true;
                     c->pend_queue = false;
@@ -896,7 +920,7 @@ int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
                 want = std::max<uint64_t>(want, 64);
             }
             if (c->skim_B && c->skim_B < want) want = c->skim_B;  // shrunk after an overflow
-            want = std::min<uint64_t>(want, default_lanes(c));
+            want = std::min<uint64_t>(want, skim_lanes(c));
             uint32_t B = static_cast<uint32_t>(std::min<uint64_t>(want, c->nl - c->cursor));
             bool retry = false;
             RC(rev_batch(c, c->cursor, B, false, &retry, c->vpl_est));
@@ -1096,13 +1120,13 @@ int skim_destroy(skim_ctx *c) {
     dfree(c, c->rkey); dfree(c, c->rkey2); dfree(c, c->rval); dfree(c, c->rval2);
     dfree(c, c->ncnt); dfree(c, c->noff); dfree(c, c->nlist); dfree(c, c->nlist_cnt);
     dfree(c, c->ws);
-    dfree(c, c->lane_inst); dfree(c, c->lane_g); dfree(c, c->alive); dfree(c, c->lane_off); dfree(c, c->lane_fill);
+    dfree(c, c->lane_inst); dfree(c, c->lane_g); dfree(c, c->alive); dfree(c, c->leaf); dfree(c, c->lane_off); dfree(c, c->lane_fill);
     dfree(c, c->nonempty); dfree(c, c->need); dfree(c, c->comp); dfree(c, c->comp_up);
     dfree(c, c->over_seg); dfree(c, c->over_buf); dfree(c, c->full_list); dfree(c, c->hitbits); dfree(c, c->defbits); dfree(c, c->defpair);
     dfree(c, c->node_off); dfree(c, c->comp_ws); dfree(c, c->need_ws);
     dfree(c, c->lcnt); dfree(c, c->full); dfree(c, c->X); dfree(c, c->xlen);
     dfree(c, c->covered); dfree(c, c->seg_start); dfree(c, c->pend_trav); dfree(c, c->pend_erase);
-    dfree(c, c->size); dfree(c, c->seg_len); dfree(c, c->idx); dfree(c, c->chosen);
+    dfree(c, c->size); dfree(c, c->ncount); dfree(c, c->seg_len); dfree(c, c->idx); dfree(c, c->chosen);
     dfree(c, c->rec_tau); dfree(c, c->rec_kp); dfree(c, c->idx_ctr);
     dfree(c, c->rmask); dfree(c, c->fmask); dfree(c, c->loff); dfree(c, c->rlive); dfree(c, c->rrow); dfree(c, c->rev2fwd);
     dfree(c, c->foff); dfree(c, c->flive);
@@ -1688,7 +1712,7 @@ int search_deferred(skim_ctx *c, uint64_t p0, uint32_t D, uint64_t R0, const Bui
         CK(c, cudaMemsetAsync(&c->ctl->src_next, 0, 3 * sizeof(HotCounter), c->st));  // src_next, busy, beat
         const uint64_t v0 = c->hctl->stats[kStRevVisits];
         if (*vpl > 0 && *vpl <= c->ring_rpl) {
-            const RevSources rs{c->defpair, D, nullptr, nullptr};
+            const RevSources rs{c->defpair, D, nullptr, nullptr, nullptr};
             RC(run_traversal(c, a, false, R, &rs));
         } else {
             {

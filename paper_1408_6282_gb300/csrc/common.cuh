@@ -154,7 +154,12 @@ struct DevCtl {
     StepCtl step;
 };
 
-enum Stat { kStRevVisits = 0, kStRevCoins, kStInsert, kStFwdVisits, kStFwdCoins, kStRevEdges, kStFwdEdges };
+// kStLeafs: visits of source lanes that take no part in the search (kLeafSegment)
+enum Stat { kStRevVisits = 0, kStRevCoins, kStInsert, kStFwdVisits, kStFwdCoins, kStRevEdges, kStFwdEdges, kStLeafs };
+
+// Length of the index segment of a pair whose rank only its own node has: no
+// entries are stored for it.
+constexpr uint32_t kLeafSegment = 0xffffffffu;
 
 SKIM_DEV uint64_t ld_acquire(const uint64_t *p) {
     uint64_t v;

@@ -71,6 +71,7 @@ struct TravArgs {
     const uint32_t *lane_of;
     uint32_t lbits;
     int own, words;
+    uint32_t *cnt;              // SKIM: per node, the batch's visits (null: not counted)
 };
 
 // graph.cu
@@ -154,7 +155,12 @@ int traverse_grid(bool forward, bool mat);  // resident blocks for the persisten
 // before the first launch of a batch.
 int rev_ring_grid();
 cudaError_t launch_rev_ring(const TravArgs &a, const uint32_t *lane_pair, uint32_t B, uint32_t l,
-                            const uint64_t *covered, uint64_t *alive, bool sources, int grid, cudaStream_t s);
+                            const uint64_t *covered, uint64_t *alive, uint64_t *leaf, bool sources, int grid,
+                            cudaStream_t s);
+// Behind a search with leaf lanes (traverse.cu): those of nodes whose sketch can fill
+// up in this batch become records.
+cudaError_t launch_leaf_records(const TravArgs &a, const uint32_t *lane_pair, uint32_t B, uint32_t l, uint64_t *leaf,
+                                uint32_t k, cudaStream_t s);
 
 // reach.cu: the residual search of seed x over materialised rows, one block per
 // instance (the seed is marked chosen)
@@ -294,6 +300,7 @@ struct StepArgs {
     const uint32_t *lane_pair;
     const uint64_t *covered;
     uint64_t *alive;
+    const uint64_t *leaf;       // lanes committed without a record
     uint32_t *size, *lane_cnt;  // lane_cnt: zero on entry and on return
     uint64_t *lane_pos, *idx_ctr;
     uint32_t *idx_nodes;
@@ -301,16 +308,16 @@ struct StepArgs {
     uint32_t *seg_len;
     DevCtl *ctl;
     uint64_t timeout_ns;
+    // of the stop, if there is one and kprime is not null: its rank to *tau, and k'
+    // of Section 4.3.2 to *kprime (zero before): the largest size over the other
+    // nodes without the stop lane's own part
+    uint32_t n, *kprime;
+    uint64_t *tau;
+    const uint64_t *lane_rank;
 };
 cudaError_t launch_step(const StepArgs &a, cudaStream_t s);
 cudaError_t launch_argmax_size(const uint32_t *size, uint32_t n, DevCtl *ctl, cudaStream_t s);
 cudaError_t launch_min_unchosen(const uint8_t *chosen, uint32_t n, DevCtl *ctl, cudaStream_t s);
-// Section 4.3.2: k' = max size over v != x with the stop lane (of *lane_pair)
-// taken out (sizes are restored); atomicMax into *out, which the caller zeroes.
-cudaError_t launch_second_size(const uint32_t *idx_nodes, const uint64_t *seg_start, const uint32_t *seg_len,
-                               const uint32_t *lane_pair, uint32_t *size, uint32_t n, uint32_t x, uint32_t *out,
-                               cudaStream_t s);
-
 // query.cu
 // Scratch of the queries: per-block partial sums, counters of the larger queries'
 // finished blocks (zero between calls), an error flag.

@@ -102,7 +102,10 @@ struct Reach {
                 }
             }
         }
-        if (RES && fresh && sl) {
+        if (RES && fresh && sl == kLeafSegment) {  // only x has this rank
+            atomicSub(&A.size[x], 1u);
+            A.seg_len[r] = 0;
+        } else if (RES && fresh && sl) {
             const uint32_t at = atomicAdd(&sh.n_erase, 1u);
             if (at < kEraseCap)
                 sh.erase[at] = make_uint2(static_cast<uint32_t>(r), sl);

@@ -42,3 +42,31 @@ def test_steps_match_oracle(monkeypatch, name, l, k, p, bl, items):
         x, ln = sk.sketches()
         ox, oln, _ = oracle.build_sketches(pb)
         assert np.array_equal(ln, oln) and np.array_equal(x, ox)
+
+
+SPARSE = {
+    "rmat12": lambda: synth.rmat(12, 8, 5),
+    "empty": lambda: synth.empty_graph(3001),
+    "cycle": lambda: synth.cycle(4099),
+}
+
+
+@pytest.mark.parametrize("hook", [None, ("SKIM_RECORD_ITEMS", "2048"), ("SKIM_QUEUE_ITEMS", "64")])
+@pytest.mark.parametrize("name", list(SPARSE))
+@pytest.mark.parametrize("l,k,p,mode", [(64, 16, 0.01, 0), (64, 64, 0.03, 0), (64, 3, 0.02, 1), (33, 32, 0.01, 0)])
+def test_lanes_that_reach_their_source_only(monkeypatch, name, l, k, p, mode, hook):
+    """Batches of 2^16 lanes and more: leaf lanes, and those of nodes that fill up."""
+    import paper_1408_6282_gb300 as pkg
+    g = SPARSE[name]()
+    ks = synth.Keys.from_seed(l + k)
+    if hook:
+        monkeypatch.setenv(*hook)
+    pb = oracle.Problem(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
+    seeds, cov, tau, kp, _ = oracle.skim_stops(pb, 60, rank_mode=mode)
+    with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, rank_mode=mode) as sk:
+        got = sk.greedy_stops(60)
+        for a, b in zip(got, (seeds, cov, tau, kp)):
+            assert np.array_equal(a, b)
+        sk.greedy_reset()
+        a, b = sk.greedy(60)
+        assert np.array_equal(a, seeds) and np.array_equal(b, cov)
