@@ -121,6 +121,7 @@ struct skim_ctx {
     uint64_t bp0 = 0;
     uint32_t bB = 0, btbits = 0, blo = 0;
     uint64_t bR = 0;
+    uint64_t bentries = 0;  // visited-table entries of the batch (its records, and those of full nodes)
     uint32_t skim_B = 0;
     uint32_t retry_run = 0;  // consecutive SKIM batch re-runs
     // SKIM batch sizing: ranks consumed since the last seed, and the gap (in
@@ -523,6 +524,8 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
     }
     // IC-model searches are never pruned: every lane is its own instance
     a.prune = mode_build && c->rank_mode != SKIM_RANKS_IC_MODEL ? 1 : 0;
+    if (mode_build && !a.prune) a.xlen = c->xlen;
+    a.k = c->k;
     uint64_t R = 0;
 #ifndef SKIM_REV_RING
 #define SKIM_REV_RING 1
@@ -614,6 +617,7 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
         CK(c, launch_gather_bits(c->rval, c->hvals, R, c->rbits, c->st));
     }
     c->bR = R;
+    c->bentries = R + (a.xlen ? c->hctl->beat.v : 0);
     c->btbits = tbits;
     c->hstats[SKIM_STAT_BATCHES]++;
     trace_line();
@@ -1919,7 +1923,7 @@ int build_coins(skim_ctx *c) {
     // hub-heavy graphs), and the next batch is sized from this one.
     uint32_t B = std::min<uint32_t>(Bmax, kBuildFirst);
     uint64_t p0 = 0;
-    double rpl = 0;  // records per lane of the last batch (0: unknown)
+    double rpl = 0;  // table entries per lane of the last batch (0: unknown)
     while (p0 < c->nbuild) {
         uint32_t b = static_cast<uint32_t>(std::min<uint64_t>(B, c->nbuild - p0));
         bool retry = false;
@@ -1950,7 +1954,7 @@ int build_coins(skim_ctx *c) {
                 cudaEventDestroy(t1);
             }
         }
-        const uint64_t recs = c->bR;
+        const uint64_t recs = c->bentries;
         RC(clear_batch(c));
         p0 += b;
         c->hstats[SKIM_STAT_RANKS] += b;

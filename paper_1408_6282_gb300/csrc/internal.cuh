@@ -72,6 +72,8 @@ struct TravArgs {
     uint32_t lbits;
     int own, words;
     uint32_t *cnt;              // SKIM: per node, the batch's visits (null: not counted)
+    const uint32_t *xlen;       // Algorithm 2 in the IC model: ranks of every sketch before the batch, of at most k
+    uint32_t k;
 };
 
 // graph.cu

@@ -467,8 +467,15 @@ SKIM_DEV void emit_rev(const TravArgs &A, Acc &acc, bool act, uint32_t u, uint32
             atomicOr(&A.ctl->err, kErrHash);
         }
     }
-    // record of the (node, word) entry, written once by its creator
+    // record of the (node, word) entry, written once by its creator; none for a
+    // node whose sketch is full (its ranks are lower), which is only counted
     {
+        if (A.xlen) {
+            const bool done = first && A.xlen[u] >= A.k;
+            const unsigned db = __ballot_sync(kFull, done);
+            if ((threadIdx.x & 31) == 0 && db) atomicAdd(&A.ctl->beat.v, static_cast<unsigned long long>(__popc(db)));
+            first &= !done;
+        }
         unsigned ball = __ballot_sync(kFull, first);
         if (ball) {
             unsigned long long base = 0;
@@ -791,7 +798,7 @@ SKIM_DEV Desc shfl_desc(const Desc &d, int src) {
 #define SKIM_TRAV_MIN_BLOCKS 3
 #endif
 #ifndef SKIM_COIN_MIN_BLOCKS
-#define SKIM_COIN_MIN_BLOCKS 3
+#define SKIM_COIN_MIN_BLOCKS 4
 #endif
 constexpr int kUnroll = SKIM_UNROLL;  // edges per lane per step: independent hash chains
 
@@ -842,7 +849,7 @@ SKIM_DEV uint64_t edge_live(const TravArgs &A, const Desc &d, uint32_t idx, uint
 }
 
 // Algorithm 2: drop lanes whose instance-local sketch at u already holds k ranks.
-SKIM_DEV uint64_t prune_full(const TravArgs &A, uint32_t t, uint32_t u, uint64_t live) {
+__device__ __noinline__ uint64_t prune_full(const TravArgs &A, uint32_t t, uint32_t u, uint64_t live) {
     const uint64_t fu = A.full[u];
     if (!fu) return live;
     const uint8_t *li = A.lane_inst + static_cast<size_t>(t) * 64;
@@ -856,18 +863,22 @@ SKIM_DEV uint64_t prune_full(const TravArgs &A, uint32_t t, uint32_t u, uint64_t
 // ---- reverse items with coins drawn in the search ------------------------------
 //
 // A visit of a hub draws thousands of coins of which a few are live, so the live
-// edges are collected in shared memory and visited 32 at a time: visiting after
-// every 32 edges kept one lane of the warp busy (R-MAT 15, IC model, p = 0.01:
-// 22 G coins, 190 ms of search; 97 ms so, and 139 with the visits inlined four
-// times).  Rows of 32 edges and more are swept by
-// the warp, 128 edges a step (four independent hash chains per lane; an edge's
-// other end is read only where it is live), the edges of the others are spread
-// over the lanes.
-constexpr uint32_t kCoinStage = 32 + 4 * 32;  // live edges a warp holds
+// edges are collected in shared memory and visited 32 at a time (visiting after
+// every 32 edges kept one lane of the warp busy).  Rows of 32 edges and more are
+// swept by the warp, 128 edges a step: four independent loads and hash chains per
+// lane (an edge's other end is read only where it is live); the edges of the others
+// are spread over the lanes.  What is rarely needed (visits, thresholds per edge,
+// items of several lanes, pruning) is not inlined and the steps' live edges are put
+// away by one copy of the code, because the warps waited for instructions most of
+// all.  R-MAT 15, IC model, p = 0.01, 22 G coins, time of the searches: 190 ms with
+// the visits in place, 97 ms collected, 139 with the visits inlined four times, 79 ms
+// with the rare parts out of line and four blocks per SM (three: 85; 1, 2, 3, 5, 8 steps
+// in flight: 100, 91, 81, 82, 89).
+constexpr uint32_t kCoinSteps = 4;  // steps of 32 coins of a row in flight
+constexpr uint32_t kCoinStage = 32 + kCoinSteps * 32;  // live edges a warp holds
 
 // Warp-collective: visit the first min(n, 32) of the n live edges in st ({other
 // end | word << 32, lanes}) and move the others up; returns the lane's new visits.
-// (Not inlined: the loops that draw coins have to fit the instruction cache.)
 __device__ __noinline__ uint32_t coin_visit(const TravArgs &A, ulonglong2 *st, uint32_t n) {
     const uint32_t lane = threadIdx.x & 31, c = min(n, 32u), rest = n - c;
     __syncwarp();
@@ -900,6 +911,13 @@ struct CoinStage {
     }
 };
 
+__device__ __noinline__ uint64_t coin_tm1(const TravArgs &A, uint32_t idx, uint32_t v) {
+    return edge_tm1_rev(A, idx, A.col[idx], v, 0);
+}
+__device__ __noinline__ uint64_t coin_lanes(const TravArgs &A, uint32_t idx, uint64_t mask, uint64_t tm1, uint32_t t) {
+    return live_lanes(A.he[idx], mask, tm1, A.lane_g + static_cast<size_t>(t) * 64);
+}
+
 SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have, const Item &it) {
     const uint32_t lane = threadIdx.x & 31;
     Desc d = describe<false, false>(A, have, it);
@@ -921,18 +939,28 @@ SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have
         if (b.single) {
             const uint64_t *he = A.he + b.begin;
             const uint32_t steps = (b.cnt + 31) / 32;
-            for (uint32_t s0 = 0; s0 < steps; s0 += 4) {
-                uint64_t h[4];
+            for (uint32_t s0 = 0; s0 < steps; s0 += kCoinSteps) {
+                uint64_t h[kCoinSteps];
 #pragma unroll
-                for (uint32_t q = 0; q < 4; q++) h[q] = he[min((s0 + q) * 32 + lane, b.cnt - 1)];
+                for (uint32_t q = 0; q < kCoinSteps; q++) h[q] = he[min((s0 + q) * 32 + lane, b.cnt - 1)];
+                uint32_t live = 0;  // bit q: edge (s0 + q) * 32 + lane
+                if (plain) {
 #pragma unroll
-                for (uint32_t q = 0; q < 4; q++) {
-                    if (s0 + q >= steps) break;
-                    const uint32_t k = (s0 + q) * 32 + lane;
-                    uint64_t t1 = b.tm1;
-                    if (!plain && k < b.cnt) t1 = edge_tm1_rev(A, b.begin + k, A.col[b.begin + k], b.v, 0);
-                    const bool live = fmix_le(h[q] + b.g1, t1) && k < b.cnt;
-                    if (__any_sync(kFull, live)) S.put(A, live ? b.mask : 0, live ? A.col[b.begin + k] : 0, t);
+                    for (uint32_t q = 0; q < kCoinSteps; q++) live |= static_cast<uint32_t>(fmix_le(h[q] + b.g1, b.tm1)) << q;
+                } else {
+#pragma unroll 1
+                    for (uint32_t q = 0; q < kCoinSteps; q++) {
+                        const uint32_t k = min((s0 + q) * 32 + lane, b.cnt - 1);
+                        const uint64_t t1 = coin_tm1(A, b.begin + k, b.v);
+                        live |= static_cast<uint32_t>(fmix_le(he[k] + b.g1, t1)) << q;
+                    }
+                }
+                const uint32_t left = b.cnt - s0 * 32;
+                live &= lane < left ? (1u << min(kCoinSteps, (left - lane + 31) / 32)) - 1 : 0;
+#pragma unroll 1
+                for (uint32_t q = 0; q < kCoinSteps; q++) {
+                    const bool l = live >> q & 1u;
+                    if (__any_sync(kFull, l)) S.put(A, l ? b.mask : 0, l ? A.col[b.begin + (s0 + q) * 32 + lane] : 0, t);
                 }
                 while (S.n >= 32) S.visit(A, acc);
             }
@@ -943,8 +971,7 @@ SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have
                 uint32_t x = 0;
                 if (k < b.cnt) {
                     x = A.col[idx];
-                    live = live_lanes(A.he[idx], b.mask, edge_tm1_rev(A, idx, x, b.v, b.tm1),
-                                      A.lane_g + static_cast<size_t>(t) * 64);
+                    live = coin_lanes(A, idx, b.mask, plain ? b.tm1 : coin_tm1(A, idx, b.v), t);
                 }
                 S.put(A, live, x, t);
                 if (S.n >= 32) S.visit(A, acc);
@@ -975,9 +1002,8 @@ SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have
         uint32_t x = 0;
         if (o < total) {
             x = A.col[idx];
-            const uint64_t t1 = edge_tm1_rev(A, idx, x, v, tm1), he = A.he[idx];
-            live = (mask & (mask - 1)) == 0 ? (fmix_le(he + g1, t1) ? mask : 0)
-                                            : live_lanes(he, mask, t1, A.lane_g + static_cast<size_t>(t) * 64);
+            const uint64_t t1 = plain ? tm1 : coin_tm1(A, idx, v);
+            live = (mask & (mask - 1)) == 0 ? (fmix_le(A.he[idx] + g1, t1) ? mask : 0) : coin_lanes(A, idx, mask, t1, t);
         }
         S.put(A, live, x, t);
         if (S.n >= 32) S.visit(A, acc);
