@@ -18,7 +18,11 @@
 // R-MAT 20 p = 0.01 3.4 -> 1.2 ms; 30 seeds of R-MAT 20 wc 9.8 -> 5.3 ms.  An
 // index segment erased by one warp (a rank that hit a giant component lists
 // 160 K nodes) cost R-MAT 20 p = 0.05 2.5 ms a search: the block erases such a
-// segment together.  One barrier per level instead of five: 5.6 -> 5.3 ms.
+// segment together.  One barrier per level instead of five: 5.6 -> 5.3 ms.  A level
+// waits for the warp with the longest row, so rows of 128 entries and more are swept
+// by the block (50 seeds of R-MAT 18 wc: from 512 entries 4.24 ms, 256 4.0, 128 3.94, 64
+// 3.86, but R-MAT 20 p = 0.01 1.27, 1.26, 1.28, 1.33).  Two to four entries of a lane in
+// flight: 4.7 to 5.2 ms (registers; most rounds have one).
 #include "internal.cuh"
 
 namespace skim {
@@ -30,7 +34,7 @@ constexpr uint32_t kReachWarps = kReachThreads / 32;
 constexpr uint32_t kFrontCap = 1024;  // frontier rows kept in shared memory, per level parity
 constexpr uint32_t kEraseCap = 1024;  // index segments kept for erasing
 constexpr uint32_t kLongCap = 64;     // rows swept by the whole block, per level
-constexpr uint32_t kLongRow = 512;    // entries from which a row is swept by the block
+constexpr uint32_t kLongRow = 128;    // entries from which a row is swept by the block
 constexpr uint32_t kSeen = 4096;      // nodes remembered as reached (direct-mapped)
 
 struct ReachShared {
