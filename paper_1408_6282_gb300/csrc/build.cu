@@ -1197,17 +1197,6 @@ __global__ void __launch_bounds__(kMergeWarps * 32) k_merge(BuildNode g, const u
     warp_add(&ctl->stats[kStInsert], ins);
 }
 
-// Per node the instances in which its row of live in-neighbours is not empty.
-__global__ void k_nonempty(const uint32_t *loff, uint32_t n, uint32_t l, uint64_t *nonempty) {
-    const uint32_t lane = threadIdx.x & 31;
-    for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += (gridDim.x * blockDim.x) >> 5) {
-        const uint64_t r = static_cast<uint64_t>(v) * l + lane;
-        const unsigned lo = __ballot_sync(kFull, lane < l && loff[r + 1] > loff[r]);
-        const unsigned hi = __ballot_sync(kFull, lane + 32 < l && loff[r + 33] > loff[r + 32]);
-        if (lane == 0) nonempty[v] = static_cast<uint64_t>(hi) << 32 | lo;
-    }
-}
-
 template <class KT, bool SCC>
 cudaError_t search_launch(const BuildArgs &a, cudaStream_t s) {
     const size_t smem = sizeof(WarpMem<KT>) * (kSearchThreads / 32);
@@ -1239,12 +1228,6 @@ cudaError_t launch_deferred_lanes(uint32_t *deflist, uint32_t D, bool all, const
                                   uint32_t *defpair, uint8_t *lane_inst, cudaStream_t s) {
     note_launch();
     k_deferred_lanes<<<grid_for(D, 256), 256, 0, s>>>(deflist, D, all, pair, l, defpair, lane_inst);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_nonempty(const uint32_t *loff, uint32_t n, uint32_t l, uint64_t *nonempty, cudaStream_t s) {
-    note_launch();
-    k_nonempty<<<grid_for(static_cast<size_t>(n) * 32, 256), 256, 0, s>>>(loff, n, l, nonempty);
     return cudaGetLastError();
 }
 

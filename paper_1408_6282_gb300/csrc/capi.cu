@@ -995,18 +995,17 @@ int make_instances(skim_ctx *c) {
         RC(dalloc(c, &c->nonempty, c->n));
         RC(dalloc_bytes(c, &c->pieces, live_pieces_bytes(c->m)));
     }
-    // counts per (v, i) scanned into 64-bit offsets, kept as 32-bit offsets
-    uint64_t *off = nullptr;
-    RC(dalloc(c, &off, c->nl + 1));
+    uint64_t *first = nullptr;  // of every node: its live pairs, then those of the nodes before it
+    RC(dalloc(c, &first, static_cast<size_t>(c->n) + 1));
     CK(c, launch_live_masks(c->rrow, c->rcol, c->rhe, c->rtm1, c->rev2fwd, c->cm, c->m, c->l, c->rmask, c->fmask,
                             c->st));
-    CK(c, launch_live_count(c->rptr, c->rmask, c->n, c->m, c->l, off, c->pieces, c->st));
-    CK(c, cudaMemsetAsync(off + c->nl, 0, sizeof(uint64_t), c->st));
-    CK(c, exclusive_scan_u64(off, off, c->nl + 1, nullptr, c->ws, c->st));
-    CK(c, cudaMemcpyAsync(&c->live_total, off + c->nl, sizeof(uint64_t), cudaMemcpyDeviceToHost, c->st));
+    CK(c, launch_live_count(c->rptr, c->rmask, c->n, c->m, c->l, first, c->loff, c->pieces, c->st));
+    CK(c, cudaMemsetAsync(first + c->n, 0, sizeof(uint64_t), c->st));
+    CK(c, exclusive_scan_u64(first, first, static_cast<size_t>(c->n) + 1, nullptr, c->ws, c->st));
+    CK(c, cudaMemcpyAsync(&c->live_total, first + c->n, sizeof(uint64_t), cudaMemcpyDeviceToHost, c->st));
     CK(c, cudaStreamSynchronize(c->st));
     if (c->live_total > kMaxLive) {  // offsets would not fit 31 bits: coins are drawn in the searches
-        dfree(c, off);
+        dfree(c, first);
         return SKIM_OK;
     }
     if (c->live_total > c->rlive_cap) {
@@ -1017,16 +1016,15 @@ int make_instances(skim_ctx *c) {
         RC(dalloc(c, &c->flive, c->live_total));
         c->rlive_cap = c->live_total;
     }
-    CK(c, launch_live_fill(c->rptr, c->rcol, c->rmask, c->n, c->m, c->l, off, c->rlive, c->pieces, c->st));
-    CK(c, launch_offsets_u32(off, c->nl, c->loff, c->st));
-    CK(c, launch_nonempty(c->loff, c->n, c->l, c->nonempty, c->st));
+    CK(c, launch_live_fill(c->rptr, c->rcol, c->rmask, c->n, c->m, c->l, first, c->loff, c->nonempty, c->rlive,
+                           c->pieces, c->st));
     // the same live pairs by tail: rows of live out-neighbours for the residual
-    CK(c, launch_live_count(c->fptr, c->fmask, c->n, c->m, c->l, off, c->pieces, c->st));
-    CK(c, cudaMemsetAsync(off + c->nl, 0, sizeof(uint64_t), c->st));
-    CK(c, exclusive_scan_u64(off, off, c->nl + 1, nullptr, c->ws, c->st));
-    CK(c, launch_live_fill(c->fptr, c->fcol, c->fmask, c->n, c->m, c->l, off, c->flive, c->pieces, c->st));
-    CK(c, launch_offsets_u32(off, c->nl, c->foff, c->st));
-    dfree(c, off);
+    CK(c, launch_live_count(c->fptr, c->fmask, c->n, c->m, c->l, first, c->foff, c->pieces, c->st));
+    CK(c, cudaMemsetAsync(first + c->n, 0, sizeof(uint64_t), c->st));
+    CK(c, exclusive_scan_u64(first, first, static_cast<size_t>(c->n) + 1, nullptr, c->ws, c->st));
+    CK(c, launch_live_fill(c->fptr, c->fcol, c->fmask, c->n, c->m, c->l, first, c->foff, nullptr, c->flive, c->pieces,
+                           c->st));
+    dfree(c, first);
     c->live_ready = true;
     c->mat = c->mat_wanted;
     return SKIM_OK;

@@ -176,7 +176,23 @@ SKIM_DEV void warp_count(const uint64_t *mask, uint32_t e0, uint32_t e1, uint64_
 }
 
 // Writes the tile's live edges of instances lane and lane + 32 at p0 and p1,
-// in edge order; the warp loops as often as the fullest instance needs.
+// in edge order (lane q holds the other end w of edge q); the warp loops as often as
+// the fullest instance needs.
+SKIM_DEV void warp_fill_tile(uint32_t m0, uint32_t m1, uint32_t w, uint64_t &p0, uint64_t &p1, uint32_t *live) {
+    while (__any_sync(kFull, (m0 | m1) != 0)) {
+        const uint32_t x0 = __shfl_sync(kFull, w, m0 ? __ffs(m0) - 1 : 0);
+        const uint32_t x1 = __shfl_sync(kFull, w, m1 ? __ffs(m1) - 1 : 0);
+        if (m0) {
+            live[p0++] = x0;
+            m0 &= m0 - 1;
+        }
+        if (m1) {
+            live[p1++] = x1;
+            m1 &= m1 - 1;
+        }
+    }
+}
+
 SKIM_DEV void warp_fill(const uint64_t *mask, const uint32_t *col, uint32_t e0, uint32_t e1, uint64_t &p0,
                         uint64_t &p1, uint32_t *live) {
     const uint32_t lane = threadIdx.x & 31;
@@ -184,26 +200,18 @@ SKIM_DEV void warp_fill(const uint64_t *mask, const uint32_t *col, uint32_t e0, 
         const bool in = e0 + lane < e1;
         const uint64_t mk = in ? mask[e0 + lane] : 0;
         const uint32_t w = in ? col[e0 + lane] : 0;
-        uint32_t m0 = warp_transpose32(static_cast<uint32_t>(mk));
-        uint32_t m1 = warp_transpose32(static_cast<uint32_t>(mk >> 32));
-        while (__any_sync(kFull, (m0 | m1) != 0)) {
-            const uint32_t x0 = __shfl_sync(kFull, w, m0 ? __ffs(m0) - 1 : 0);
-            const uint32_t x1 = __shfl_sync(kFull, w, m1 ? __ffs(m1) - 1 : 0);
-            if (m0) {
-                live[p0++] = x0;
-                m0 &= m0 - 1;
-            }
-            if (m1) {
-                live[p1++] = x1;
-                m1 &= m1 - 1;
-            }
-        }
+        const uint32_t m0 = warp_transpose32(static_cast<uint32_t>(mk));
+        const uint32_t m1 = warp_transpose32(static_cast<uint32_t>(mk >> 32));
+        warp_fill_tile(m0, m1, w, p0, p1, live);
     }
 }
 
-// counts of live edges per (node, instance) into off[v*l + i], rows up to kBigRow
-__global__ void k_live_count(const uint32_t *ptr, const uint64_t *mask, uint32_t n, uint32_t l, uint64_t *off,
-                             Pieces P) {
+// Live pairs per node, rows up to kBigRow.  Only a node's total has to be known
+// before its row: the counts of its instances are taken again in the fill pass, where
+// the masks are in registers or close by, and scanned across the warp.  (Counts of
+// every pair, scanned as 64-bit offsets and cut to 32 bits: 3.7 GB of traffic per
+// direction at R-MAT 20, l = 64, so 0.6 GB; both directions 3.7 -> 2.5 ms.)
+__global__ void k_live_count(const uint32_t *ptr, const uint64_t *mask, uint32_t n, uint64_t *tot, Pieces P) {
     const uint32_t lane = threadIdx.x & 31;
     for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += (gridDim.x * blockDim.x) >> 5) {
         const uint32_t e0 = ptr[v], e1 = ptr[v + 1];
@@ -211,24 +219,73 @@ __global__ void k_live_count(const uint32_t *ptr, const uint64_t *mask, uint32_t
             if (lane == 0) claim_pieces(P, v, e0, e1);
             continue;
         }
-        uint64_t c0 = 0, c1 = 0;
-        warp_count(mask, e0, e1, c0, c1);
-        const uint64_t base = static_cast<uint64_t>(v) * l;
-        if (lane < l) off[base + lane] = c0;
-        if (lane + 32 < l) off[base + lane + 32] = c1;
+        uint32_t c = 0;
+        for (uint32_t e = e0 + lane; e < e1; e += 32) c += __popcll(mask[e]);
+        c = __reduce_add_sync(kFull, c);
+        if (lane == 0) tot[v] = c;
     }
 }
 
-// the live edges of (v, i) written in row order from off[v*l + i], rows up to kBigRow
-__global__ void k_live_fill(const uint32_t *ptr, const uint32_t *col, const uint64_t *mask, uint32_t n, uint32_t l,
-                            const uint64_t *off, uint32_t *live) {
+// Offsets of the instances of node v (lane: instances lane and lane + 32, with c0
+// and c1 live pairs) from the node's first on: to off, and p0, p1.
+// TILE: a row of one tile, whose counts of up to 32 are scanned two in a word.
+template <bool TILE>
+SKIM_DEV void warp_offsets(uint32_t v, uint32_t l, uint64_t first, uint32_t c0, uint32_t c1, uint32_t *off,
+                           uint64_t *nonempty, uint64_t &p0, uint64_t &p1) {
     const uint32_t lane = threadIdx.x & 31;
+    uint32_t i0 = TILE ? c1 << 16 | c0 : c0, i1 = c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y0 = __shfl_up_sync(kFull, i0, o), y1 = TILE ? 0 : __shfl_up_sync(kFull, i1, o);
+        if (lane >= static_cast<uint32_t>(o)) {
+            i0 += y0;
+            i1 += y1;
+        }
+    }
+    if (TILE) {
+        i1 = i0 >> 16;
+        i0 &= 0xffffu;
+    }
+    p0 = first + (i0 - c0);
+    p1 = first + __shfl_sync(kFull, i0, 31) + (i1 - c1);
+    const uint64_t base = static_cast<uint64_t>(v) * l;
+    if (lane < l) off[base + lane] = static_cast<uint32_t>(p0);
+    if (lane + 32 < l) off[base + lane + 32] = static_cast<uint32_t>(p1);
+    const unsigned b0 = __ballot_sync(kFull, c0 != 0), b1 = __ballot_sync(kFull, c1 != 0);
+    if (nonempty && lane == 0) nonempty[v] = static_cast<uint64_t>(b1) << 32 | b0;
+}
+
+// Rows up to kBigRow: the offsets of (v, i) and its live edges in row order.
+__global__ void k_live_fill(const uint32_t *ptr, const uint32_t *col, const uint64_t *mask, uint32_t n, uint32_t l,
+                            const uint64_t *first, uint32_t *off, uint64_t *nonempty, uint32_t *live) {
+    const uint32_t lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && threadIdx.x == 0) off[static_cast<uint64_t>(n) * l] = static_cast<uint32_t>(first[n]);
     for (uint32_t v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < n; v += (gridDim.x * blockDim.x) >> 5) {
         const uint32_t e0 = ptr[v], e1 = ptr[v + 1];
         if (e1 - e0 > kBigRow) continue;
-        const uint64_t base = static_cast<uint64_t>(v) * l;
-        uint64_t p0 = lane < l ? off[base + lane] : 0, p1 = lane + 32 < l ? off[base + lane + 32] : 0;
-        warp_fill(mask, col, e0, e1, p0, p1, live);
+        uint64_t p0, p1;
+        if (e1 - e0 <= 32) {  // (most rows)
+            const bool in = e0 + lane < e1;
+            const uint64_t mk = in ? mask[e0 + lane] : 0;
+            const uint32_t w = in ? col[e0 + lane] : 0;
+            if (!__any_sync(kFull, mk != 0)) {  // nothing to place
+                const uint64_t base = static_cast<uint64_t>(v) * l;
+                const uint32_t f = static_cast<uint32_t>(first[v]);
+                if (lane < l) off[base + lane] = f;
+                if (lane + 32 < l) off[base + lane + 32] = f;
+                if (nonempty && lane == 0) nonempty[v] = 0;
+                continue;
+            }
+            const uint32_t m0 = warp_transpose32(static_cast<uint32_t>(mk));
+            const uint32_t m1 = warp_transpose32(static_cast<uint32_t>(mk >> 32));
+            warp_offsets<true>(v, l, first[v], __popc(m0), __popc(m1), off, nonempty, p0, p1);
+            warp_fill_tile(m0, m1, w, p0, p1, live);
+        } else {
+            uint64_t c0 = 0, c1 = 0;
+            warp_count(mask, e0, e1, c0, c1);
+            warp_offsets<false>(v, l, first[v], static_cast<uint32_t>(c0), static_cast<uint32_t>(c1), off, nonempty, p0, p1);
+            warp_fill(mask, col, e0, e1, p0, p1, live);
+        }
     }
 }
 
@@ -244,9 +301,10 @@ __global__ void k_piece_count(const uint32_t *ptr, const uint64_t *mask, Pieces 
     }
 }
 
-// one warp per row (its first piece): per instance, the row's total into off
-// and each piece's count replaced by the sum over the row's earlier pieces
-__global__ void k_piece_rows(const uint32_t *ptr, uint32_t l, uint64_t *off, Pieces P) {
+// one warp per row (its first piece): per instance, the row's count into off (for
+// k_piece_offsets) and each piece's count replaced by the sum over the row's
+// earlier pieces; the node's total
+__global__ void k_piece_rows(const uint32_t *ptr, uint32_t l, uint64_t *tot, uint32_t *off, Pieces P) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t np = min(*P.count, P.cap);
     for (uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < np; p += (gridDim.x * blockDim.x) >> 5) {
@@ -262,13 +320,31 @@ __global__ void k_piece_rows(const uint32_t *ptr, uint32_t l, uint64_t *off, Pie
             r1 += a1;
         }
         const uint64_t base = static_cast<uint64_t>(v) * l;
-        if (lane < l) off[base + lane] = r0;
-        if (lane + 32 < l) off[base + lane + 32] = r1;
+        if (lane < l) off[base + lane] = static_cast<uint32_t>(r0);
+        if (lane + 32 < l) off[base + lane + 32] = static_cast<uint32_t>(r1);
+        uint64_t t = r0 + r1;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(kFull, t, o);
+        if (lane == 0) tot[v] = t;
+    }
+}
+
+__global__ void k_piece_offsets(const uint32_t *ptr, uint32_t l, const uint64_t *first, uint32_t *off,
+                                uint64_t *nonempty, Pieces P) {
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t np = min(*P.count, P.cap);
+    for (uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < np; p += (gridDim.x * blockDim.x) >> 5) {
+        const uint32_t v = P.row[p];
+        if (P.e0[p] != ptr[v]) continue;  // not the row's first piece
+        const uint64_t base = static_cast<uint64_t>(v) * l;
+        uint64_t p0, p1;
+        warp_offsets<false>(v, l, first[v], lane < l ? off[base + lane] : 0, lane + 32 < l ? off[base + lane + 32] : 0, off,
+                     nonempty, p0, p1);
     }
 }
 
 __global__ void k_piece_fill(const uint32_t *ptr, const uint32_t *col, const uint64_t *mask, uint32_t l,
-                             const uint64_t *off, uint32_t *live, Pieces P) {
+                             const uint32_t *off, uint32_t *live, Pieces P) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t np = min(*P.count, P.cap);
     for (uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < np; p += (gridDim.x * blockDim.x) >> 5) {
@@ -587,39 +663,28 @@ unsigned piece_grid(uint64_t m) { return grid_for((2 * (m / kBigRow) + 2) * 32, 
 }  // namespace
 
 cudaError_t launch_live_count(const uint32_t *ptr, const uint64_t *mask, uint32_t n, uint64_t m, uint32_t l,
-                              uint64_t *off, void *pieces_ws, cudaStream_t s) {
+                              uint64_t *tot, uint32_t *off, void *pieces_ws, cudaStream_t s) {
     const Pieces P = carve_pieces(pieces_ws, m);
     cudaError_t e = cudaMemsetAsync(P.count, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
     note_launch();
-    k_live_count<<<grid_for(static_cast<size_t>(n) * 32, 256), 256, 0, s>>>(ptr, mask, n, l, off, P);
+    k_live_count<<<grid_for(static_cast<size_t>(n) * 32, 256), 256, 0, s>>>(ptr, mask, n, tot, P);
     note_launch();
     k_piece_count<<<piece_grid(m), 256, 0, s>>>(ptr, mask, P);
     note_launch();
-    k_piece_rows<<<piece_grid(m), 256, 0, s>>>(ptr, l, off, P);
+    k_piece_rows<<<piece_grid(m), 256, 0, s>>>(ptr, l, tot, off, P);
     return cudaGetLastError();
 }
 cudaError_t launch_live_fill(const uint32_t *ptr, const uint32_t *col, const uint64_t *mask, uint32_t n, uint64_t m,
-                             uint32_t l, const uint64_t *off, uint32_t *live, void *pieces_ws, cudaStream_t s) {
+                             uint32_t l, const uint64_t *first, uint32_t *off, uint64_t *nonempty, uint32_t *live,
+                             void *pieces_ws, cudaStream_t s) {
     const Pieces P = carve_pieces(pieces_ws, m);
     note_launch();
-    k_live_fill<<<grid_for(static_cast<size_t>(n) * 32, 256), 256, 0, s>>>(ptr, col, mask, n, l, off, live);
+    k_live_fill<<<grid_for(static_cast<size_t>(n) * 32, 256), 256, 0, s>>>(ptr, col, mask, n, l, first, off, nonempty, live);
+    note_launch();
+    k_piece_offsets<<<piece_grid(m), 256, 0, s>>>(ptr, l, first, off, nonempty, P);
     note_launch();
     k_piece_fill<<<piece_grid(m), 256, 0, s>>>(ptr, col, mask, l, off, live, P);
-    return cudaGetLastError();
-}
-
-namespace {
-__global__ void k_offsets_u32(const uint64_t *off, uint64_t count, uint32_t *off32) {
-    for (uint64_t r = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; r <= count;
-         r += static_cast<uint64_t>(gridDim.x) * blockDim.x)
-        off32[r] = static_cast<uint32_t>(off[r]);
-}
-}  // namespace
-
-cudaError_t launch_offsets_u32(const uint64_t *off, uint64_t count, uint32_t *off32, cudaStream_t s) {
-    note_launch();
-    k_offsets_u32<<<grid_for(count + 1, 256), 256, 0, s>>>(off, count, off32);
     return cudaGetLastError();
 }
 

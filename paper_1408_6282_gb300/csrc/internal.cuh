@@ -92,9 +92,10 @@ cudaError_t launch_wc_thresholds(const uint32_t *rptr, uint32_t n, uint64_t *thr
 // Per-edge coin-stream states of a CSR: he[e] for edge (row node, col[e]);
 // reverse = 1 when rows are heads (edge col[e] -> row).
 // Materialised instances (Section 2: the l live-edge graphs): live masks of
-// every CSR edge (bit i = coin of instance i), and the node-major lists of live
-// in-neighbours: counts per (v, i) into off[v*l + i], then (after an exclusive
-// scan of off) the sources themselves.
+// every CSR edge (bit i = coin of instance i), the nodes' live pairs (tot), and after
+// an exclusive scan of those (first; n + 1 of them) the offsets off[v*l + i] of the
+// node-major lists of live neighbours, which rows are not empty (nonempty, may be
+// null) and the lists.
 cudaError_t launch_live_masks(const uint32_t *rrow, const uint32_t *rcol, const uint64_t *rhe, const uint64_t *rtm1,
                               const uint32_t *rev2fwd, const CoinModel &cm, uint64_t m, uint32_t l, uint64_t *rmask,
                               uint64_t *fmask, cudaStream_t s);
@@ -103,11 +104,10 @@ cudaError_t launch_live_masks(const uint32_t *rrow, const uint32_t *rcol, const 
 // precede its fill pass with the same workspace.
 size_t live_pieces_bytes(uint64_t m);
 cudaError_t launch_live_count(const uint32_t *ptr, const uint64_t *mask, uint32_t n, uint64_t m, uint32_t l,
-                              uint64_t *off, void *pieces_ws, cudaStream_t s);
+                              uint64_t *tot, uint32_t *off, void *pieces_ws, cudaStream_t s);
 cudaError_t launch_live_fill(const uint32_t *ptr, const uint32_t *col, const uint64_t *mask, uint32_t n, uint64_t m,
-                             uint32_t l, const uint64_t *off, uint32_t *live, void *pieces_ws, cudaStream_t s);
-// off32[r] = off[r] for r <= count (offsets below 2^31)
-cudaError_t launch_offsets_u32(const uint64_t *off, uint64_t count, uint32_t *off32, cudaStream_t s);
+                             uint32_t l, const uint64_t *first, uint32_t *off, uint64_t *nonempty, uint32_t *live,
+                             void *pieces_ws, cudaStream_t s);
 
 // Rank order of all pairs: bucket by the top bits, then sort each bucket.
 // rank of pair x = v*l+i is fmix(rank_key + G*x), or fmix(rbase[v] + G*i)
@@ -254,7 +254,6 @@ cudaError_t launch_append_words(const uint64_t *rec, const uint32_t *rec_val, ui
 cudaError_t launch_overflow(uint64_t R, uint32_t lbits, const uint64_t *lane_rank, uint32_t k, uint32_t *len,
                             uint64_t *X, bool done, const BuildScratch &b, DevCtl *ctl, cudaStream_t s);
 cudaError_t launch_need_start(uint64_t *need, uint32_t n, uint64_t lmask, cudaStream_t s);
-cudaError_t launch_nonempty(const uint32_t *loff, uint32_t n, uint32_t l, uint64_t *nonempty, cudaStream_t s);
 // *next (device): the first rank not yet processed; full_list: n entries kept
 // from pass to pass
 cudaError_t launch_need(const BuildNode &g, const uint64_t *next, uint64_t *need, uint32_t *full_list, void *scratch,

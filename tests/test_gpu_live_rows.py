@@ -1,0 +1,48 @@
+"""Stored instances (graph.cu) at the row sizes where they can go wrong: none, one
+tile of 32 edges, more, rows cut into pieces; one instance to 64, no coin live and
+all of them.  Seeds and coverages walk the rows of out-neighbours, sketches those of
+in-neighbours; both are whole numbers and must equal the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+pytestmark = pytest.mark.gpu
+DEGREES = [1, 31, 32, 33, 64, 65, 2047, 2048, 2049, 4097, 6000]
+
+
+def _graph(reverse):
+    """Nodes with DEGREES in-neighbours (reverse: out-neighbours) among 6100 nodes, the rest without."""
+    rng = np.random.default_rng(4)
+    n = 6100
+    a, b = [], []
+    for i, d in enumerate(DEGREES):
+        v = 3 + 50 * i
+        a.append(rng.choice(np.setdiff1d(np.arange(n), [v]), d, replace=False).astype(np.uint32))
+        b.append(np.full(d, v, np.uint32))
+    src, dst = (np.concatenate(b), np.concatenate(a)) if reverse else (np.concatenate(a), np.concatenate(b))
+    order = np.lexsort((dst, src))
+    return n, src[order], dst[order]
+
+
+@pytest.mark.parametrize("reverse", [False, True])
+@pytest.mark.parametrize("l", [1, 31, 32, 33, 64])
+@pytest.mark.parametrize("model,p", [(0, 1e-9), (0, 0.01), (0, 1.0), (1, 0.0)])
+def test_row_sizes(model, p, l, reverse):
+    import paper_1408_6282_gb300 as pkg
+    n, src, dst = _graph(reverse)
+    ks = synth.Keys.from_seed(21)
+    k = 16
+    pb = oracle.Problem(n, src, dst, l, k, model, p, ks.coin, ks.rank, ks.prob)
+    ox, oln, _ = oracle.build_sketches(pb)
+    seeds, cov, tau, kp, _ = oracle.skim_stops(pb, 15)
+    with pkg.Skim(n, src, dst, l, k, model, p, ks.coin, ks.rank, ks.prob) as sk:
+        for _ in range(2):
+            sk.build_sketches()
+            x, ln = sk.sketches()
+            assert np.array_equal(ln, oln) and np.array_equal(x, ox)
+            sk.greedy_reset()
+            got = sk.greedy_stops(15)
+            for a, b in zip(got, (seeds, cov, tau, kp)):
+                assert np.array_equal(a, b)
