@@ -83,3 +83,15 @@ def test_node_ids_past_24_bits():
         sk.build_sketches()
         y, lm = sk.sketches()
         assert np.array_equal(ln, lm) and np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("n", [510, 511, 512, 513, 514, 1500])
+@pytest.mark.parametrize("width", [1, 31, 32, 33])
+def test_long_narrow_components(n, width):
+    """Rings of n layers: walks of more levels than a narrow component is followed."""
+    a = np.arange(n * width, dtype=np.uint32)
+    layer, pos = a // width, a % width
+    src = np.concatenate([a, a])
+    dst = np.concatenate([((layer + 1) % n) * width + pos, ((layer + 1) % n) * width + (pos + 1) % width])
+    key = np.unique(src.astype(np.uint64) << np.uint64(32) | dst.astype(np.uint64))
+    _check(n * width, (key >> np.uint64(32)).astype(np.uint32), (key & np.uint64(0xffffffff)).astype(np.uint32), 3, 8, 0, 1.0)
