@@ -135,7 +135,7 @@ def traffic_record(kernel: str, workload: str):
     return None
 
 
-def kernel_roofline(kname, kt, gold, m, l, steps, sm_max, hbm_peak, total_ms, workload, gather=None):
+def kernel_roofline(kname, kt, gold, m, l, steps, sm_max, hbm_peak, total_ms, workload, gather=None, done=None):
     """Roofline of one kernel group of the step, from its CUDA-event time and
     the algorithmic work of one step (the oracle's counts, so redundant GPU
     work is not credited).
@@ -146,6 +146,8 @@ def kernel_roofline(kname, kt, gold, m, l, steps, sm_max, hbm_peak, total_ms, wo
                 pruning flag) and reads and writes its 8 B visited word (16 B);
                 every expansion also writes its 12 B visit record.  Sources are
                 taken inside the search kernel, so their lanes count here.
+                (The searches skip what no node needs any more and contract
+                giant components; `done` is what they did visit and walk.)
     fwd_search  (memory): 16 B per forward expansion (the two row bounds of
                 (v, i)) + 20 B per live out-edge (4 B neighbour id, covered word
                 read and write) + 8 B per index entry erased (node id, size).
@@ -173,14 +175,15 @@ def kernel_roofline(kname, kt, gold, m, l, steps, sm_max, hbm_peak, total_ms, wo
         units = (f"{cand} candidate visits ({lanes} source lanes + {L} live in-edges) x 28 B + {E} expansions "
                  "x 12 B per step")
         key = "rev_search"
-        if gather:
-            # each candidate costs at least two independent random accesses
-            # (its row entry and its visited slot) and each live in-edge's id
-            # is a third: the count a random-access ceiling applies to
-            acc = 2 * cand + L
+        if gather and done:
+            # each visit costs at least two independent random accesses (its
+            # row entry and its visited slot) and each live in-edge walked a
+            # third: the count a random-access ceiling applies to
+            acc = 2 * done["rev_visits"] + done["rev_edges"]
             extra["random_access"] = {"achieved": acc / sec / 1e9, "peak": gather / 1e9, "unit": "G accesses/s",
                                       "frac": acc / sec / gather,
-                                      "basis": "2 random accesses per candidate visit + 1 per live in-edge; peak = "
+                                      "visits": done["rev_visits"], "live_in_edges_walked": done["rev_edges"],
+                                      "basis": "2 random accesses per visit made + 1 per live in-edge walked; peak = "
                                                "random 8-byte gathers over a 4 GiB array (torch index_select) "
                                                "timed in this run"}
     else:
@@ -676,6 +679,12 @@ def main():
     e2e_t = max_over_ranks(statistics.median(e2e_times), dist, device="cuda")
     e2e_value = job_value(world, 1, t_alg, e2e_t)
 
+    # what the searches of one step do
+    done = {"rev_visits": 0, "rev_edges": 0}
+    sk.build_sketches()
+    for stats in (sk.stats(), (sk.greedy_reset(), sk.greedy(w.seeds), sk.stats())[2]):
+        for key in done:
+            done[key] += stats[key]
     sk.close()
     # large plain SKIM (config 5) on the same GPU, after the step's context is gone
     config5 = config5_object(pkg, stream, local) if args.config5 else None
@@ -689,7 +698,7 @@ def main():
     total_ms = sum(v[0] for v in kt.values())
     dominant = max(("rev_search", "fwd_search", "instances"), key=lambda kname: kt[kname][0])
     roofline = kernel_roofline(dominant, kt, gold, g.m, w.l, args.steps, sm_max, hbm_peak, total_ms, w.name,
-                               gather)
+                               gather, done)
     sk_c, sm_c = gold["sketches"]["counters"], gold["skim"]["counters"]
     step_s = elapsed / args.steps
 
