@@ -136,11 +136,15 @@ SKIM_DEV double fixed_to_double(const U192 &a) {
 // what it would wait for, so a larger one takes a cluster of 16 blocks whose
 // warps share the seeds and put a rank into the table of the block that has its
 // hash, through distributed shared memory: 64 ranks per sketch, 445 seeds 61 -> 32
-// us, 1000 seeds 66 -> 40 us (clusters of 8: 66 us, of 4: 118 us; parts: 85 us).  A batch fills the
-// chip with parts and is slower with clusters (1000 queries, with copies: 0.52 ms;
-// clusters of 4, 8, 16: 0.63, 0.76, 1.07 ms), so clusters are for two queries, or
-// four of few parts (4 of 1000 seeds, 16 ranks per sketch: 67 us, in parts 91 us;
-// 64 ranks per sketch: 91 and 82 us; 8 of 200 seeds: 80 and 66 us).  Both
+// us, 1000 seeds 66 -> 40 us (clusters of 8: 66 us, of 4: 118 us; parts: 85 us).  So do the
+// larger ones of a call with few of them, the small ones beside them in the same launch; a
+// cluster of 4 does where it holds the whole query, and the chip has room for more of
+// those.  Calls of 10, 32, 64, 128 queries of 1 to 1000 seeds, 16 ranks per sketch: parts
+// 100, 110, 125, 130 us, clusters 55, 70, 74, 92 us (a table in global memory, four launches:
+// 67, 75, 85, 102 us); 64 ranks, 10, 16, 32, 64 queries: parts 75, 84, 90, 95 us, clusters of 16 59, 69,
+// then parts (four launches: 76, 86, 96, 126 us).  A batch fills the chip with parts and is
+// slower with clusters (1000 queries, with copies: 0.52 ms; clusters of 4, 8, 16: 0.63,
+// 0.76, 1.07 ms).  Both
 // read a query once per part or round of clusters: from kBlockMost ranks on the
 // table is in global memory (64 ranks per sketch, 30000 seeds: 264 us, clusters
 // 555 us, parts 1100 us; 9000 seeds, clusters: 107 us).
@@ -153,8 +157,12 @@ constexpr uint32_t kPartEntries = 8000, kPartSlots = 12287;  // 192 KB
 constexpr int kPartThreads = 1024;
 constexpr uint32_t kStage = 64;  // pairs a warp collects
 constexpr uint32_t kOneEntries = 1500;
-constexpr uint32_t kCluster = 16, kClusterSlots = kPartSlots, kClusterEntries = kCluster * 7800;
-constexpr uint32_t kClusterQueries = 4, kClusterParts = 8;
+constexpr uint32_t kCluster = 16, kClusterSlots = kPartSlots, kBlockEntries = 7800, kClusterEntries = kCluster * kBlockEntries;
+constexpr uint32_t kClusterFour = 4;
+// larger queries of a call that take clusters of 16, the same if some do not fit four
+// blocks, and those that take clusters of 4 if all do
+constexpr uint32_t kFewLarge = 8, kFewLargest = 16, kMoreLarge = 64;
+constexpr uint32_t kClusterParts = 8;
 constexpr uint64_t kBlockMost = 1 << 20;  // ranks, above that the table is in global memory
 constexpr uint32_t kTableBlocks = 152 * 2;
 
@@ -331,15 +339,16 @@ SKIM_DEV U192 query_block(const uint64_t *X, const uint32_t *xlen, uint32_t n, u
 // part `part` of `parts`, in the tables of the cluster's blocks (H + 1 slots each; a
 // block has a range of the hashes), in `cut` pieces or more.  Thread 0 of block 0
 // has the total; *bad: the ranks of some hash are more than fit.
+template <uint32_t CL>
 SKIM_DEV U192 query_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                             const uint32_t *seeds, uint32_t s, uint64_t part, uint64_t parts, uint64_t cut,
                             uint64_t *tab, uint32_t H, unsigned *err, bool *bad) {
-    __shared__ U192 sums[kCluster];
+    __shared__ U192 sums[CL];
     __shared__ int s_full;
     namespace cg = cooperative_groups;
     const cg::cluster_group cl = cg::this_cluster();
     const uint32_t rank = cl.block_rank(), lane = threadIdx.x & 31;
-    const uint32_t w = rank * (blockDim.x >> 5) + (threadIdx.x >> 5), ways = kCluster * (blockDim.x >> 5);
+    const uint32_t w = rank * (blockDim.x >> 5) + (threadIdx.x >> 5), ways = CL * (blockDim.x >> 5);
     uint64_t *keys = tab, *val = tab + H + 1;
     U192 acc{{0, 0, 0}};
     *bad = false;
@@ -347,7 +356,7 @@ SKIM_DEV U192 query_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n,
         const uint64_t pieces = parts * cut, piece = part * cut + c;
         const uint64_t lo = (piece << 32) / pieces, hi = ((piece + 1) << 32) / pieces;  // of the 32-bit hash
         const uint32_t lo32 = static_cast<uint32_t>(lo), last = static_cast<uint32_t>(hi - lo - 1);
-        const uint64_t scale = (static_cast<uint64_t>(kCluster * H) << 32) / (hi - lo);
+        const uint64_t scale = (static_cast<uint64_t>(CL * H) << 32) / (hi - lo);
         for (uint32_t i = threadIdx.x; i <= H; i += blockDim.x) keys[i] = val[i] = kEmptyKey;
         if (threadIdx.x == 0) s_full = 0;
         cl.sync();
@@ -370,7 +379,7 @@ SKIM_DEV U192 query_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n,
                     const uint32_t h = rank_hash(z) - lo32;
                     if (h > last) continue;
                     const uint32_t at = static_cast<uint32_t>(__umul64hi(static_cast<uint64_t>(h) << 32, scale));
-                    const uint32_t g = min(kCluster * H - 1, at), b = g / H;
+                    const uint32_t g = min(CL * H - 1, at), b = g / H;
                     over |= !table_put_remote(cl.map_shared_rank(keys, b), cl.map_shared_rank(val, b), H, g - b * H, z, t);
                 }
             }
@@ -395,10 +404,16 @@ SKIM_DEV U192 query_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n,
     if (threadIdx.x == 0) *cl.map_shared_rank(&sums[rank], 0) = acc;
     cl.sync();  // (a block leaves when nobody needs its memory any more)
     if (rank == 0 && threadIdx.x == 0)
-        for (uint32_t r = 1; r < kCluster; r++) add192(acc, sums[r]);
+        for (uint32_t r = 1; r < CL; r++) add192(acc, sums[r]);
     return acc;
 }
 
+// slots of each block of a cluster
+template <uint32_t CL>
+SKIM_HD uint32_t cluster_slots(uint64_t entries) {
+    const uint64_t h = entries * 2 / CL + 64;
+    return h < kClusterSlots ? static_cast<uint32_t>(h) : kClusterSlots;
+}
 constexpr SKIM_HD uint32_t small_slots(uint64_t entries) { return static_cast<uint32_t>(entries + entries / 2 + 32); }
 
 // One query whose seeds are kernel arguments; the estimate goes to host memory.
@@ -422,7 +437,7 @@ __global__ void __launch_bounds__(1024)
                     const __grid_constant__ SeedArgs<CAP> a, uint32_t H, double *out) {
     extern __shared__ ulonglong2 s_tab[];
     bool full;
-    const U192 e = query_cluster(X, xlen, n, k, terms, a.seeds, a.s, 0, 1, 1, reinterpret_cast<uint64_t *>(s_tab), H, nullptr, &full);
+    const U192 e = query_cluster<kCluster>(X, xlen, n, k, terms, a.seeds, a.s, 0, 1, 1, reinterpret_cast<uint64_t *>(s_tab), H, nullptr, &full);
     if (blockIdx.x == 0 && threadIdx.x == 0) *out = full ? -1.0 : fixed_to_double(e) / terms.div;
 }
 
@@ -512,23 +527,36 @@ __global__ void __launch_bounds__(kPartThreads) k_q_part(const uint64_t *X, cons
     add_parts(e, c, first, end, partial, &done[qi], &out[qi], terms.div);
 }
 
-// The same by clusters, `ways` for each query.
-__global__ void __launch_bounds__(kPartThreads) k_q_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n,
-                                                            uint32_t k, QueryTerms terms, const uint32_t *seeds,
-                                                            const uint64_t *offsets, const uint64_t *block_off,
-                                                            uint32_t ways, U192 *partial, unsigned *done, double *out,
-                                                            unsigned *err) {
+// A few queries: `ways` clusters for each of the larger ones, then a block for each
+// of the small ones.
+struct FewArgs {
+    uint32_t q, n_large, ways, large[kMoreLarge];
+};
+template <uint32_t CL>
+__global__ void __launch_bounds__(kPartThreads) k_q_few(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k,
+                                                        QueryTerms terms, const uint32_t *seeds,
+                                                        const uint64_t *offsets, const FewArgs f, U192 *partial,
+                                                        unsigned *done, double *out, unsigned *err) {
     extern __shared__ ulonglong2 s_tab[];
-    const uint32_t c = blockIdx.x / kCluster, qi = c / ways;
-    if (block_off[qi + 1] == block_off[qi]) return;
-    const uint64_t s0 = offsets[qi], s = offsets[qi + 1] - s0, room = static_cast<uint64_t>(kClusterEntries) * ways;
+    uint64_t *tab = reinterpret_cast<uint64_t *>(s_tab);
+    const uint32_t c = blockIdx.x / CL, ways = f.ways;
+    const uint32_t qi = c < f.n_large * ways ? f.large[c / ways] : blockIdx.x - f.n_large * ways * CL;
+    if (qi >= f.q) return;
+    const uint64_t s0 = offsets[qi], s = offsets[qi + 1] - s0, entries = s * (k - 1);
+    if (c >= f.n_large * ways) {
+        if (entries > kSmallEntries) return;
+        const U192 e = query_block<false>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(s), 0, 1, tab,
+                                          small_slots(entries), err);
+        if (threadIdx.x == 0) out[qi] = fixed_to_double(e) / terms.div;
+        return;
+    }
+    const uint64_t room = static_cast<uint64_t>((CL * kBlockEntries)) * ways, cut = (entries + room - 1) / room;
     bool bad;
-    const U192 e = query_cluster(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(s), c % ways, ways,
-                                 (s * (k - 1) + room - 1) / room, reinterpret_cast<uint64_t *>(s_tab), kClusterSlots, err,
-                                 &bad);
-    if (blockIdx.x % kCluster) return;
+    const U192 e = query_cluster<CL>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(s), c % ways, ways, cut, tab,
+                                 cluster_slots<CL>(entries / (ways * cut)), err, &bad);
+    if (blockIdx.x % CL) return;
     if (bad && threadIdx.x == 0) atomicOr(err, 2u);
-    add_parts(e, c, qi * ways, (qi + 1) * ways, partial, &done[qi], &out[qi], terms.div);
+    add_parts(e, c, c / ways * ways, (c / ways + 1) * ways, partial, &done[qi], &out[qi], terms.div);
 }
 
 // Single-node influence estimates from each node's own sketch: the bottom-k
@@ -583,7 +611,7 @@ bool query_fits_args(uint64_t seeds, uint32_t k) {
 
 namespace {
 
-template <class K, class... Args>
+template <uint32_t CL, class K, class... Args>
 cudaError_t cluster_launch(K kernel, unsigned clusters, uint32_t H, cudaStream_t st, const Args &...args) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (kClusterSlots + 1) * sizeof(ulonglong2));
@@ -591,10 +619,10 @@ cudaError_t cluster_launch(K kernel, unsigned clusters, uint32_t H, cudaStream_t
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = kCluster;
+    at.val.clusterDim.x = CL;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(clusters * kCluster);
+    cfg.gridDim = dim3(clusters * CL);
     cfg.blockDim = dim3(kPartThreads);
     cfg.dynamicSmemBytes = (H + 1) * sizeof(ulonglong2);
     cfg.stream = st;
@@ -619,8 +647,8 @@ cudaError_t one_launch(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint
         return cudaGetLastError();
     }
     if constexpr (CAP > 60) {
-        const uint32_t H = static_cast<uint32_t>(std::min<uint64_t>(kClusterSlots, entries * 2 / kCluster + 64));
-        return cluster_launch(k_q_one_cluster<CAP>, 1, H, st, X, xlen, n, k, terms, a, H, out_host);
+        const uint32_t H = cluster_slots<kCluster>(entries);
+        return cluster_launch<kCluster>(k_q_one_cluster<CAP>, 1, H, st, X, xlen, n, k, terms, a, H, out_host);
     }
     return cudaErrorInvalidValue;
 }
@@ -659,11 +687,27 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
             e = cudaGetLastError();
         }
     }
-    if (e == cudaSuccess && blocks && (q <= 2 || (q <= kClusterQueries && blocks <= kCluster))) {
-        const uint32_t ways = std::max(1u, std::min(kClusterParts / q, (blocks * kPartEntries - 1) / kClusterEntries + 1));
-        e = cluster_launch(k_q_cluster, q * ways, kClusterSlots, s, X, xlen, n, k, terms, seeds, offsets, block_off, ways,
-                           partial, qs.done, out, qs.err);
-    } else if (e == cudaSuccess && blocks) {
+    FewArgs f{q, 0, 0, {}};
+    uint64_t most = 0;
+    for (uint32_t i = 0; blocks && i < q && f.n_large <= kMoreLarge; i++) {
+        const uint64_t cnt = h_offsets[i + 1] - h_offsets[i];
+        if (!query_blocks(cnt, k)) continue;
+        if (f.n_large < kMoreLarge) f.large[f.n_large] = i;
+        f.n_large++;
+        most = std::max(most, cnt * (k - 1));
+    }
+    const bool fits_four = most <= kClusterFour * kBlockEntries;
+    if (e == cudaSuccess && f.n_large && f.n_large <= (fits_four ? kMoreLarge : kFewLargest)) {
+        const bool few = f.n_large <= kFewLarge || !fits_four;
+        const uint32_t cl = few ? kCluster : kClusterFour;
+        f.ways = few ? std::max(1u, std::min(kClusterParts / f.n_large, (blocks * kPartEntries - 1) / kClusterEntries + 1)) : 1;
+        const uint32_t clusters = f.n_large * f.ways + (q > f.n_large + tables ? (q + cl - 1) / cl : 0);
+        return few ? cluster_launch<kCluster>(k_q_few<kCluster>, clusters, kClusterSlots, s, X, xlen, n, k, terms, seeds,
+                                              offsets, f, partial, qs.done, out, qs.err)
+                   : cluster_launch<kClusterFour>(k_q_few<kClusterFour>, clusters, kClusterSlots, s, X, xlen, n, k, terms,
+                                                  seeds, offsets, f, partial, qs.done, out, qs.err);
+    }
+    if (e == cudaSuccess && blocks) {
         const int smem = (kPartSlots + 1 + kPartThreads / 32 * kStage) * sizeof(ulonglong2);
         e = cudaFuncSetAttribute(k_q_part, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
@@ -672,7 +716,7 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
                                                     out, qs.err);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess && (q > 1 || (!blocks && !tables))) {
+    if (e == cudaSuccess && q > tables) {
         const int smem = (kSmallSlots + 1) * sizeof(ulonglong2);
         e = cudaFuncSetAttribute(k_q_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;

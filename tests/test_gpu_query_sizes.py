@@ -34,3 +34,20 @@ def test_sizes_around_the_limits(k, mode):
             assert a == b
             ref = oracle.union_estimate(ox, oln, l, s, rank_mode=mode)
             assert abs(a - ref) <= REL * abs(ref)
+
+
+@pytest.mark.parametrize("large", [1, 8, 9, 16, 17, 64, 65])
+@pytest.mark.parametrize("k,seeds", [(16, 181), (16, 2000), (64, 400), (64, 600), (64, 2200)])
+def test_calls_with_some_larger_queries(large, k, seeds):
+    """Clusters of 16 and of 4, parts; small queries and empty ones beside them."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.erdos_renyi(3001, 15000, 47)
+    ks = synth.Keys.from_seed(47)
+    rng = np.random.default_rng(large)
+    sets = [rng.choice(g.n, seeds if i < large else rng.integers(0, 30), replace=False) for i in range(large + 21)]
+    sets = [sets[i] for i in rng.permutation(len(sets))]
+    with pkg.Skim(g.n, g.src, g.dst, 16, k, 0, 0.15, ks.coin, ks.rank, ks.prob) as sk:
+        sk.build_sketches()
+        want = [sk.query(s) for s in sets]
+        for _ in range(2):
+            assert np.array_equal(sk.query_batch(sets), want)
