@@ -487,8 +487,9 @@ int node_buffers(skim_ctx *c) {
     return SKIM_OK;
 }
 
-// Reverse search of the batch of ranks [p0, p0+B).  mode_build: Algorithm 2
-// (pruned by local counts); otherwise SKIM (covered sources skipped).
+// Reverse search of the batch of ranks [p0, p0+B).  mode_build: Algorithm 2 with
+// coins drawn in the searches
+// (pruned by local counts; not in the IC model); otherwise SKIM (covered sources skipped).
 // est_per_lane: expected visit records per lane (0 or negative = unknown, or
 // a re-run after an overflow: the whole table).  The visited table used is a
 // power of two of about 4 slots per expected record, zeroed before the batch
@@ -527,9 +528,6 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
     if (mode_build && !a.prune) a.xlen = c->xlen;
     a.k = c->k;
     uint64_t R = 0;
-#ifndef SKIM_REV_RING
-#define SKIM_REV_RING 1
-#endif
     // SKIM_TRACE_BATCHES=1 in the environment: one line per batch on stderr
     // (search kernel, lanes, records, visits, device time of its searches and
     // of its record sort)
@@ -541,11 +539,11 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
         cudaEventCreate(&tr2);
         cudaEventRecord(tr0, c->st);
     }
-    const bool use_ring = c->mat && SKIM_REV_RING && est_per_lane > 0 && est_per_lane <= c->ring_rpl;
+    const bool use_ring = c->mat && est_per_lane > 0 && est_per_lane <= c->ring_rpl;
     if (use_ring) {
-        const bool leafs = !mode_build && B >= kLeafLanes;
-        const RevSources rs{c->spair + p0, B, mode_build ? nullptr : c->covered, mode_build ? nullptr : c->alive,
-                            leafs ? c->leaf : nullptr};
+        // (only SKIM's batches come here: Algorithm 2 over rows is build_rows)
+        const bool leafs = B >= kLeafLanes;
+        const RevSources rs{c->spair + p0, B, c->covered, c->alive, leafs ? c->leaf : nullptr};
         if (leafs) {
             a.cnt = c->ncount;
             CK(c, cudaMemsetAsync(c->ncount, 0, c->n * sizeof(uint32_t), c->st));
@@ -684,11 +682,8 @@ uint32_t default_lanes(skim_ctx *c) {
 // Lanes of a SKIM batch when the caller sets none.  A batch is sized by its
 // visits (next_seed), and most lanes of a sparse one are leaf lanes: 50 seeds of
 // R-MAT 20 p = 0.01 take 20, 19, 17.8, 17.0 ms with at most 2, 4, 8, 16 M.
-#ifndef SKIM_SL
-#define SKIM_SL 24
-#endif
 uint32_t skim_lanes(skim_ctx *c) {
-    return c->batch_cfg ? default_lanes(c) : static_cast<uint32_t>(std::min<uint64_t>(1ull << SKIM_SL, c->lane_cap));
+    return c->batch_cfg ? default_lanes(c) : static_cast<uint32_t>(std::min<uint64_t>(1ull << 24, c->lane_cap));
 }
 
 // ---- SKIM steps ------------------------------------------------------------

@@ -532,11 +532,6 @@ struct GlobalSink {
     }
 };
 
-// Where a residual search puts its new items: the block's ring (null: none)
-// while it has room, else the global queue.
-struct FwdSink {
-    FwdRing *ring;
-};
 
 // Warp-collective, materialised reverse searches: lanes with `act` reach node
 // u for lane j of word t (instance inst).  The row bounds of (u, inst) are
@@ -791,61 +786,19 @@ SKIM_DEV Desc shfl_desc(const Desc &d, int src) {
     return o;
 }
 
-#ifndef SKIM_UNROLL
-#define SKIM_UNROLL 1
-#endif
 #ifndef SKIM_TRAV_MIN_BLOCKS
 #define SKIM_TRAV_MIN_BLOCKS 3
 #endif
 #ifndef SKIM_COIN_MIN_BLOCKS
 #define SKIM_COIN_MIN_BLOCKS 4
 #endif
-constexpr int kUnroll = SKIM_UNROLL;  // edges per lane per step: independent hash chains
 
-// Coin test of CSR edge idx for item d: the lanes (reverse) or instances
-// (forward) for which the edge is live; *tgt = the edge's other end.
-#ifndef SKIM_HE_TABLE
-#define SKIM_HE_TABLE 1
-#endif
-#ifndef SKIM_PREFETCH
-#define SKIM_PREFETCH 1
-#endif
-
-// Per-edge value the live test needs: the coin-stream state of CSR edge idx
-// (other end x), or with materialised instances its live mask (forward; the
-// reverse live rows need nothing).
-template <bool FWD, bool MAT>
-SKIM_DEV uint64_t edge_key(const TravArgs &A, const Desc &d, uint32_t idx, uint32_t x) {
-    if (MAT) return 0;  // materialised rows hold live edges only
-#if SKIM_HE_TABLE
-    return A.he[idx];
-#else
-    return FWD ? edge_state(A.cm.coin_key, d.v, x) : edge_state(A.cm.coin_key, x, d.v);
-#endif
-}
-
-// Live lanes (reverse) or instances (forward) of an edge with other end x
-// and coin-stream state he.
-template <bool FWD, bool MAT>
-SKIM_DEV uint64_t edge_live_xh(const TravArgs &A, const Desc &d, uint32_t idx, uint32_t x, uint64_t he,
-                               const uint64_t *ginst) {
-    if (MAT) return d.mask;
-    if (FWD) return live_lanes(he, d.mask, edge_tm1_fwd(A, idx, d.v, x), ginst);
-    const uint64_t t1 = edge_tm1_rev(A, idx, x, d.v, d.tm1);
-    if (d.single) return fmix_le(he + d.g1, t1) ? d.mask : 0;
-    return live_lanes(he, d.mask, t1, A.lane_g + static_cast<size_t>(d.w >> kChunkBits) * 64);
-}
-
-template <bool FWD, bool MAT>
-SKIM_DEV uint64_t edge_live(const TravArgs &A, const Desc &d, uint32_t idx, uint32_t *tgt, const uint64_t *ginst) {
-    const uint32_t x = A.col[idx];
-    const uint64_t he = edge_key<FWD, MAT>(A, d, idx, x);
-    *tgt = x;
-    if (MAT) return d.mask;
-    if (FWD) return live_lanes(he, d.mask, edge_tm1_fwd(A, idx, d.v, x), ginst);
-    const uint64_t t1 = edge_tm1_rev(A, idx, x, d.v, d.tm1);
-    if (d.single) return fmix_le(he + d.g1, t1) ? d.mask : 0;
-    return live_lanes(he, d.mask, t1, A.lane_g + static_cast<size_t>(d.w >> kChunkBits) * 64);
+// Residual searches: the instances in which CSR edge idx to x is live, of item
+// d's (with materialised instances rows hold live edges only).
+template <bool MAT>
+SKIM_DEV uint64_t fwd_live(const TravArgs &A, const Desc &d, uint32_t idx, uint32_t x, uint64_t he,
+                           const uint64_t *ginst) {
+    return MAT ? d.mask : live_lanes(he, d.mask, edge_tm1_fwd(A, idx, d.v, x), ginst);
 }
 
 // Algorithm 2: drop lanes whose instance-local sketch at u already holds k ranks.
@@ -1011,105 +964,71 @@ SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have
     while (S.n) S.visit(A, acc);  // before the items count as done
 }
 
-// Hand the live results of one step to the emitters (warp-collective).
-template <bool FWD, bool MAT, class SK>
-SKIM_DEV void emit_step(const TravArgs &A, Acc &acc, SK &sk, const Desc &d, const uint64_t *lv, const uint32_t *tg) {
-#pragma unroll
-    for (int q = 0; q < kUnroll; q++) {
-        uint64_t live = lv[q];
-        if constexpr (FWD) {
-            emit_fwd<MAT>(A, acc, live != 0, tg[q], live, sk.ring);
-        }
-    }
-}
-
-// Expand entries [k0, k0 + kUnroll*stride) of item d, entry k at index
-// begin + k for k < cnt (stride = 32 when the warp shares the item, 1 when
-// the lane owns it).  Warp-collective.
-template <bool FWD, bool MAT, class SK>
-SKIM_DEV void expand_step(const TravArgs &A, Acc &acc, SK &sk, const Desc &d, uint32_t k0, uint32_t stride, bool own,
+// ---- items of residual searches ----------------------------------------------------
+//
+// Warp-collective: edge (or index entry) k of item d, of the lanes that own one.
+template <bool MAT>
+SKIM_DEV void expand_step(const TravArgs &A, Acc &acc, FwdRing *ring, const Desc &d, uint32_t k, bool own,
                           const uint64_t *ginst) {
-    uint64_t lv[kUnroll];
-    uint32_t tg[kUnroll];
-#pragma unroll
-    for (int q = 0; q < kUnroll; q++) {
-        const uint32_t k = k0 + q * stride;
-        lv[q] = 0;
-        tg[q] = 0;
-        if (own && k < d.cnt) {
-            if (FWD && d.erase)
-                atomicSub(&A.size[A.idx_nodes[(d.mask - 1) + d.begin + k]], 1u);
-            else
-                lv[q] = edge_live<FWD, MAT>(A, d, d.begin + k, &tg[q], ginst);
+    uint64_t live = 0;
+    uint32_t x = 0;
+    if (own && k < d.cnt) {
+        const uint32_t idx = d.begin + k;
+        if (d.erase) {
+            atomicSub(&A.size[A.idx_nodes[(d.mask - 1) + idx]], 1u);
+        } else {
+            x = A.col[idx];
+            live = fwd_live<MAT>(A, d, idx, x, MAT ? 0 : A.he[idx], ginst);
         }
     }
-    uint64_t anyl = 0;
-#pragma unroll
-    for (int q = 0; q < kUnroll; q++) anyl |= lv[q];
-    if (__any_sync(kFull, anyl != 0)) emit_step<FWD, MAT>(A, acc, sk, d, lv, tg);
+    if (__any_sync(kFull, live != 0)) emit_fwd<MAT>(A, acc, live != 0, x, live, ring);
 }
 
-// Expand the items held by the lanes with `have`: an item of 32 or more
-// entries is swept by the whole warp (lane = entry), smaller items by their
-// own lane.
-template <bool FWD, bool MAT, class SK>
-SKIM_DEV void process_items(const TravArgs &A, Acc &acc, SK &sk, bool have, const Item &it, const uint64_t *ginst) {
-    const int lane = threadIdx.x & 31;
-    Desc d = describe<FWD, MAT>(A, have, it);
+// Warp-collective: the items the lanes hold.  The warp sweeps an item of 32 edges and
+// more, the others are taken an edge of each lane's own at a step.  New items go to
+// the block's ring (null: none) while it has room, else to the global queue.
+template <bool MAT>
+SKIM_DEV void fwd_expand(const TravArgs &A, Acc &acc, FwdRing *ring, bool have, const Item &it, const uint64_t *ginst) {
+    const uint32_t lane = threadIdx.x & 31;
+    const Desc d = describe<true, MAT>(A, have, it);
     if (d.cnt && !d.erase) {
         acc.edges += d.cnt;
         if (!MAT) acc.coins += static_cast<unsigned long long>(d.cnt) * __popcll(d.mask);
-        if (!FWD && !MAT) {
-            d.tm1 = A.cm.model == 1 ? A.cm.thr_wc[d.v] : A.cm.tm1_uniform;
-            d.single = (d.mask & (d.mask - 1)) == 0;
-            if (d.single) d.g1 = A.lane_g[static_cast<size_t>(d.w >> kChunkBits) * 64 + (__ffsll(d.mask) - 1)];
-        }
     }
     unsigned big = __ballot_sync(kFull, d.cnt >= 32);
     while (big) {
         const int src = __ffs(big) - 1;
         big &= big - 1;
         const Desc b = shfl_desc(d, src);
-#if SKIM_PREFETCH
-        if (FWD && b.erase) {  // index-erase items
-            for (uint32_t k0 = 0; k0 < b.cnt; k0 += 32 * kUnroll) expand_step<FWD, MAT>(A, acc, sk, b, k0 + lane, 32, true, ginst);
-        } else {
-            // one step ahead: the next edge's column and key are in flight
-            // while the current coin is computed
-            uint32_t x = 0;
-            uint64_t h = 0;
-            if (lane < b.cnt) {
-                x = A.col[b.begin + lane];
-                h = edge_key<FWD, MAT>(A, b, b.begin + lane, x);
-            }
-            for (uint32_t k0 = 0; k0 < b.cnt; k0 += 32) {
-                const uint32_t k = k0 + lane;
-                uint32_t xn = 0;
-                uint64_t hn = 0;
-                if (k + 32 < b.cnt) {
-                    xn = A.col[b.begin + k + 32];
-                    hn = edge_key<FWD, MAT>(A, b, b.begin + k + 32, xn);
-                }
-                uint64_t lv[kUnroll] = {0};
-                uint32_t tg[kUnroll] = {0};
-                if (k < b.cnt) {
-                    lv[0] = edge_live_xh<FWD, MAT>(A, b, b.begin + k, x, h, ginst);
-                    tg[0] = x;
-                }
-                if (__any_sync(kFull, lv[0] != 0)) emit_step<FWD, MAT>(A, acc, sk, b, lv, tg);
-                x = xn;
-                h = hn;
-            }
+        if (b.erase) {  // index-erase items
+            for (uint32_t k0 = 0; k0 < b.cnt; k0 += 32) expand_step<MAT>(A, acc, ring, b, k0 + lane, true, ginst);
+            continue;
         }
-#else
-        for (uint32_t k0 = 0; k0 < b.cnt; k0 += 32 * kUnroll) expand_step<FWD, MAT>(A, acc, sk, b, k0 + lane, 32, true, ginst);
-#endif
+        // one step ahead: the next edge's other end and coin stream are in
+        // flight while the current coin is computed
+        uint32_t x = 0;
+        uint64_t h = 0;
+        if (lane < b.cnt) {
+            x = A.col[b.begin + lane];
+            if (!MAT) h = A.he[b.begin + lane];
+        }
+        for (uint32_t k0 = 0; k0 < b.cnt; k0 += 32) {
+            const uint32_t k = k0 + lane;
+            uint32_t xn = 0;
+            uint64_t hn = 0;
+            if (k + 32 < b.cnt) {
+                xn = A.col[b.begin + k + 32];
+                if (!MAT) hn = A.he[b.begin + k + 32];
+            }
+            const uint64_t live = k < b.cnt ? fwd_live<MAT>(A, b, b.begin + k, x, h, ginst) : 0;
+            if (__any_sync(kFull, live != 0)) emit_fwd<MAT>(A, acc, live != 0, x, live, ring);
+            x = xn;
+            h = hn;
+        }
     }
     const uint32_t mine = d.cnt < 32 ? d.cnt : 0;
-    uint32_t steps = (mine + kUnroll - 1) / kUnroll;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) steps = max(steps, __shfl_xor_sync(kFull, steps, o));
-    for (uint32_t st = 0; st < steps; st++) expand_step<FWD, MAT>(A, acc, sk, d, st * kUnroll, 1, mine != 0, ginst);
+    const uint32_t steps = __reduce_max_sync(kFull, mine);
+    for (uint32_t st = 0; st < steps; st++) expand_step<MAT>(A, acc, ring, d, st, mine != 0, ginst);
 }
 
 // ---- Reverse searches over materialised live rows, with per-warp queues ----
@@ -1538,7 +1457,6 @@ __global__ void __launch_bounds__(kTravThreads, FWD ? 1 : MAT ? SKIM_TRAV_MIN_BL
     const int lane = threadIdx.x & 31;
     DevCtl *C = A.ctl;
     Acc acc;
-    FwdSink fsink{ring};
     const uint32_t wib = kStaged ? threadIdx.x >> 5 : 0;
     RingSink ssink{nullptr, s_rk[wib], s_rs[wib], 0, 0, 0, 0};
     uint64_t t_progress = globaltimer();
@@ -1578,7 +1496,7 @@ __global__ void __launch_bounds__(kTravThreads, FWD ? 1 : MAT ? SKIM_TRAV_MIN_BL
                 if constexpr (kStaged)
                     ring_expand(A, acc, ssink, have, it);
                 else if constexpr (FWD)
-                    process_items<FWD, MAT>(A, acc, fsink, have, it, ginst);
+                    fwd_expand<MAT>(A, acc, ring, have, it, ginst);
                 else
                     coin_expand(A, acc, s_coin[threadIdx.x >> 5], have, it);
                 if constexpr (kLocal) {
@@ -1698,7 +1616,7 @@ __global__ void __launch_bounds__(kTravThreads, FWD ? 1 : MAT ? SKIM_TRAV_MIN_BL
                 continue;
             }
             t_last = globaltimer();
-            process_items<FWD, MAT>(A, acc, fsink, have, it, ginst);
+            fwd_expand<MAT>(A, acc, ring, have, it, ginst);
             __syncwarp();
             if (lane == 0) ring_finish(A, ring, __popc(lb));
         }
