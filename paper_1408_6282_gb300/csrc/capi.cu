@@ -1875,9 +1875,10 @@ int build_rows(skim_ctx *c) {
         const double recs = static_cast<double>(std::max<uint64_t>(R, 1)) / b;
         const double defs = static_cast<double>(std::max<uint64_t>(v2 - v1, 1)) / b;
         uint64_t fit = static_cast<uint64_t>(std::min(c->rcap / 4.0 / recs, c->hcap / 8.0 / defs));
-        // ... or twice that, if it is the last batch (n = 4096, 32768 edges, l = 16:
+        // ... or more than that, if it is the last batch (n = 4096, 32768 edges, l = 16:
         // two batches of mostly waiting instead of three, 615 -> 430 us)
-        if (c->nbuild - p0 <= 2 * fit) fit = c->nbuild - p0;
+        const double rest = static_cast<double>(c->nbuild - p0);
+        if (rest * recs <= 0.6 * c->rcap && rest * defs <= c->hcap / 3.0) fit = c->nbuild - p0;
         // (visits per lane as measured, unless a component has just been contracted)
         per = static_cast<double>(std::max<uint64_t>(v2 - v0, 1)) / b;
         uint64_t next = kRowsGrowth * static_cast<uint64_t>(b);
