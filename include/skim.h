@@ -71,7 +71,7 @@ typedef struct {
  *              a real in [0,1) after scaling by 2^-64 (ranks never tie);
  *   prob_key   trivalency class of edge (u,v): fmix(prob_key ^ (u<<32|v)) % 3;
  *   batch_lanes  ranks per batched search, 0 = automatic (sketch builds over
- *              materialised instances: up to 16M; otherwise 2M, and 4M on
+ *              materialised instances and SKIM: up to 16M; otherwise 2M, and 4M on
  *              graphs of 2^23 nodes or more);
  *   rank_mode  SKIM_RANKS_*: how the pairs are ordered and what a sketch holds.
  *     SKIM_RANKS_UNIFORM (0): the uniform 64-bit ranks above.
