@@ -873,6 +873,7 @@ int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
                 if (!c->hctl->step.stalled) c->hctl->ix_cov = c->hctl->step.cov;
                 RC(finish_residual(c, &again));
                 if (again) continue;  // the step found the last seed's search unfinished and did nothing
+                if (c->hctl->step.stalled) return fail_cuda(c, cudaErrorIllegalState);  // (no search was pending)
             }
             c->refilter = false;
             const uint64_t best = c->hctl->step.best;
