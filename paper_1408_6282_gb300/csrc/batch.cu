@@ -376,7 +376,15 @@ SKIM_DEV void step_second(const StepArgs &a, uint32_t x) {
     if ((threadIdx.x & 31) == 0 && best) atomicMax(a.kprime, best);
 }
 
+// Lanes of a commit up to which a block counts them in shared memory, and takes its
+// places in their segments at once: the first batches have few lanes that reach up to
+// every node, and their records' atomics would meet on as few counters (50 seeds of R-MAT
+// 18 trivalency: steps 10.1 -> 9.4 ms; R-MAT 20 p = 0.01: 5.6 -> 4.6 ms).
+constexpr uint32_t kDenseLanes = 3072;
+
 __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant__ StepArgs a) {
+    __shared__ uint32_t s_cnt[kDenseLanes];
+    __shared__ unsigned long long s_pos[kDenseLanes];
     DevCtl *C = a.ctl;
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
     // the last search is not finished: the host ends it and launches the step again
@@ -397,14 +405,23 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant_
     // Additive, so a thread per record.  The stop lane's own part of the sizes
     // follows in the last phase: k' is counted without it.
     const uint64_t stop = best == ~0ull ? ~0ull : hi;
+    const uint32_t range = hi >= a.lo && a.lo < a.B ? hi - a.lo + 1 : 0;
+    const bool dense = range <= kDenseLanes;
+    for (uint32_t i = threadIdx.x; dense && i < range; i += kStepThreads) s_cnt[i] = 0;
+    __syncthreads();
     unsigned long long ins = step_leafs(a, hi);
     step_records(a, hi, [&](uint32_t v, uint64_t m, uint64_t t) {
         const uint32_t c = __popcll(m), d = t == stop >> 6 ? static_cast<uint32_t>(m >> (stop & 63)) & 1u : 0;
         if (c > d) atomicAdd(&a.size[v], c - d);
         ins += c;
-        for (; m; m &= m - 1) atomicAdd(&a.lane_cnt[t * 64 + __ffsll(m) - 1], 1u);
+        for (; m; m &= m - 1) {
+            const uint64_t j = t * 64 + __ffsll(m) - 1;
+            atomicAdd(dense ? &s_cnt[j - a.lo] : &a.lane_cnt[j], 1u);
+        }
     });
-    __syncwarp();
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; dense && i < range; i += kStepThreads)
+        if (s_cnt[i]) atomicAdd(&a.lane_cnt[a.lo + i], s_cnt[i]);
     warp_add(&C->stats[kStInsert], ins);
     if (!step_barrier(C, 2, a.timeout_ns)) return;
     step_segments(a, hi);
@@ -413,10 +430,19 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant_
         if (first) *a.tau = a.lane_rank[hi];
     }
     if (!step_barrier(C, 3, a.timeout_ns)) return;
+    // (the block's records are those it counted)
+    for (uint32_t i = threadIdx.x; dense && i < range; i += kStepThreads)
+        if (s_cnt[i]) s_pos[i] = atomicAdd(reinterpret_cast<unsigned long long *>(&a.lane_pos[a.lo + i]), s_cnt[i]);
+    __syncthreads();
     step_records(a, hi, [&](uint32_t v, uint64_t m, uint64_t t) {
         if (t == stop >> 6 && (m >> (stop & 63) & 1u)) atomicAdd(&a.size[v], 1u);
-        for (; m; m &= m - 1)
-            a.idx_nodes[atomicAdd(reinterpret_cast<unsigned long long *>(&a.lane_pos[t * 64 + __ffsll(m) - 1]), 1ull)] = v;
+        for (; m; m &= m - 1) {
+            const uint64_t j = t * 64 + __ffsll(m) - 1;
+            const uint64_t at =
+                dense ? s_pos[j - a.lo] + atomicSub(&s_cnt[j - a.lo], 1u) - 1
+                      : atomicAdd(reinterpret_cast<unsigned long long *>(&a.lane_pos[j]), 1ull);
+            a.idx_nodes[at] = v;
+        }
     });
     if (first) {  // what the host takes, and the count of the next search from zero
         C->step.cov = C->ix_cov;

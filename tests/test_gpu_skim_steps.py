@@ -70,3 +70,18 @@ def test_lanes_that_reach_their_source_only(monkeypatch, name, l, k, p, mode, ho
         sk.greedy_reset()
         a, b = sk.greedy(60)
         assert np.array_equal(a, seeds) and np.array_equal(b, cov)
+
+
+@pytest.mark.parametrize("bl", [3071, 3072, 3073, 6200])
+@pytest.mark.parametrize("name", ["rmat10", "clique"])
+def test_commits_of_few_and_many_lanes(name, bl):
+    """Lanes counted in a block's shared memory up to 3072 of a commit, globally above."""
+    import paper_1408_6282_gb300 as pkg
+    g = GRAPHS[name]()
+    ks = synth.Keys.from_seed(bl)
+    l, k, p = 64, 64, 0.02
+    pb = oracle.Problem(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
+    seeds, cov, tau, kp, _ = oracle.skim_stops(pb, 30)
+    with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, batch_lanes=bl) as sk:
+        for a, b in zip(sk.greedy_stops(30), (seeds, cov, tau, kp)):
+            assert np.array_equal(a, b)
