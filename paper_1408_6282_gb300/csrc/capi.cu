@@ -1332,7 +1332,7 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
         TRY(dalloc(c, &c->lane_off, c->lane_cap));
         TRY(dalloc(c, &c->lane_fill, c->lane_cap));
         c->grid_rev = traverse_grid(false, true);
-        c->grid_coin = traverse_grid(false, false);
+        c->grid_coin = traverse_grid(false, false, c->rank_mode == SKIM_RANKS_IC_MODEL);
         c->grid_ring = rev_ring_grid();
         c->grid_fwd = traverse_grid(true, true);
         TRYC(cudaStreamSynchronize(c->st));

@@ -789,9 +789,11 @@ SKIM_DEV Desc shfl_desc(const Desc &d, int src) {
 #ifndef SKIM_TRAV_MIN_BLOCKS
 #define SKIM_TRAV_MIN_BLOCKS 3
 #endif
-#ifndef SKIM_COIN_MIN_BLOCKS
-#define SKIM_COIN_MIN_BLOCKS 4
-#endif
+// Blocks per SM of a search that draws coins: four in the IC model, whose batches
+// fill the chip (R-MAT 15: 84 ms, three 91 ms), three else, where a small graph's search is
+// a chain of hops and spilled registers and idle warps cost (R-MAT 12, p = 0.01, l = 16: 0.80 and
+// 0.95 ms, R-MAT 14 1.87 and 2.14 ms; R-MAT 17 wc, l = 64: 26.0 and 25.7 ms).
+constexpr int kCoinBlocks = 3, kCoinBlocksIc = 4;
 
 // Residual searches: the instances in which CSR edge idx to x is live, of item
 // d's (with materialised instances rows hold live edges only).
@@ -825,7 +827,7 @@ __device__ __noinline__ uint64_t prune_full(const TravArgs &A, uint32_t t, uint3
 // away by one copy of the code, because the warps waited for instructions most of
 // all.  R-MAT 15, IC model, p = 0.01, 22 G coins, time of the searches: 190 ms with
 // the visits in place, 97 ms collected, 139 with the visits inlined four times, 79 ms
-// with the rare parts out of line and four blocks per SM (three: 85; 1, 2, 3, 5, 8 steps
+// with the rare parts out of line and four blocks per SM (three: 86; 1, 2, 3, 5, 8 steps
 // in flight: 100, 91, 81, 82, 89).
 constexpr uint32_t kCoinSteps = 4;  // steps of 32 coins of a row in flight
 constexpr uint32_t kCoinStage = 32 + kCoinSteps * 32;  // live edges a warp holds
@@ -1436,8 +1438,8 @@ constexpr unsigned long long kDoneBatch = 64;
 // materialised rows keep items in the block's ring (FwdRing) while it has
 // room; a warp takes ring items into its lanes that hold no queue item.
 struct NoRing {};
-template <bool FWD, bool MAT>
-__global__ void __launch_bounds__(kTravThreads, FWD ? 1 : MAT ? SKIM_TRAV_MIN_BLOCKS : SKIM_COIN_MIN_BLOCKS)
+template <bool FWD, bool MAT, int BLOCKS = FWD ? 1 : MAT ? SKIM_TRAV_MIN_BLOCKS : kCoinBlocks>
+__global__ void __launch_bounds__(kTravThreads, BLOCKS)
     k_traverse(const __grid_constant__ TravArgs A) {
     constexpr bool kStaged = !FWD && MAT;
     constexpr bool kLocal = FWD && MAT && kFwdKeep > 0;
@@ -1639,7 +1641,7 @@ __global__ void __launch_bounds__(kTravThreads, FWD ? 1 : MAT ? SKIM_TRAV_MIN_BL
 // occupies SMs at the same time (another stream of this process, another
 // context) can break it the same way.  The reverse searches over materialised
 // rows (k_rev_ring) have no such requirement.
-int traverse_grid(bool forward, bool mat) {
+int traverse_grid(bool forward, bool mat, bool ic) {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1648,6 +1650,7 @@ int traverse_grid(bool forward, bool mat) {
     // fill the machine: as many blocks as fit.
     if (forward) return sms;
     if (mat) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, true>, kTravThreads, 0);
+    else if (ic) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, false, kCoinBlocksIc>, kTravThreads, 0);
     else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, false>, kTravThreads, 0);
     if (per < 1) per = 1;
     return sms * per;
@@ -1682,7 +1685,8 @@ cudaError_t launch_traverse(const TravArgs &a, bool forward, int grid, cudaStrea
         if (a.mat)
             k_traverse<false, true><<<grid, kTravThreads, 0, s>>>(a);
         else
-            k_traverse<false, false><<<grid, kTravThreads, 0, s>>>(a);
+            a.xlen ? k_traverse<false, false, kCoinBlocksIc><<<grid, kTravThreads, 0, s>>>(a)
+                   : k_traverse<false, false><<<grid, kTravThreads, 0, s>>>(a);
     }
     return cudaGetLastError();
 }
