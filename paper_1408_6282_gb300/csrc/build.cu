@@ -236,7 +236,9 @@ struct WarpSearch {
                 const uint32_t k = k0 + lane;
                 const uint32_t xn = k + 32 < bc ? A.rlive[bb + k + 32] : 0;
                 visit(k < bc, x, bi);
-                if (deferred(bi)) break;
+                // one decision for the warp: the next visit may defer the search
+                // before every lane has looked
+                if (__any_sync(kFull, deferred(bi))) break;
                 x = xn;
             }
         }

@@ -95,3 +95,17 @@ def test_long_narrow_components(n, width):
     dst = np.concatenate([((layer + 1) % n) * width + pos, ((layer + 1) % n) * width + (pos + 1) % width])
     key = np.unique(src.astype(np.uint64) << np.uint64(32) | dst.astype(np.uint64))
     _check(n * width, (key >> np.uint64(32)).astype(np.uint32), (key & np.uint64(0xffffffff)).astype(np.uint32), 3, 8, 0, 1.0)
+
+
+@pytest.mark.parametrize("hubs,spokes", [(3, 640), (3, 735), (40, 1500), (1, 9000)])
+def test_searches_deferred_inside_a_long_row(hubs, spokes):
+    """Rows swept by a warp whose entries overflow the warp's reached set on the way
+    (704 of 1024 slots): the whole warp leaves the row at the same entry.  Few lanes
+    start at a hub, so batches stay with the warps' own searches."""
+    n = hubs * (spokes + 1) + 12000
+    h = np.arange(hubs, dtype=np.uint32)
+    src = (np.arange(hubs * spokes, dtype=np.uint32) + np.uint32(hubs))
+    dst = np.repeat(h, spokes)
+    order = np.lexsort((dst, src))
+    _check(n, src[order], dst[order], 16, 64, 0, 1.0)
+    _check(n, src[order], dst[order], 16, 64, 0, 0.9, mode=1)
