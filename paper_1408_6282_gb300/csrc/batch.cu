@@ -388,7 +388,9 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant_
     DevCtl *C = a.ctl;
     const bool first = blockIdx.x == 0 && threadIdx.x == 0;
     // the last search is not finished: the host ends it and launches the step again
-    if (*reinterpret_cast<volatile unsigned *>(&C->spill) | *reinterpret_cast<volatile unsigned *>(&C->err)) {
+    // (a block that gives up at a barrier sets err: one decision for the block)
+    if (__syncthreads_or(*reinterpret_cast<volatile unsigned *>(&C->spill) |
+                         *reinterpret_cast<volatile unsigned *>(&C->err))) {
         if (first) {
             C->step.best = ~0ull;
             C->step.stalled = 1;

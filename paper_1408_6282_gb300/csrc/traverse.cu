@@ -1776,7 +1776,9 @@ __global__ void k_respill_fwd(TravArgs A, uint32_t n) {
 // committed.  50 seeds of R-MAT 20 p = 0.01, l = 64: 27 -> LL ms.
 __global__ void __launch_bounds__(256) k_leaf_records(TravArgs A, const uint32_t *lane_pair, uint32_t B, uint32_t l,
                                                       uint64_t *leaf, uint32_t k) {
-    if (A.ctl->spill | A.ctl->err) return;  // the search goes on, or is run again
+    // the search goes on, or is run again (other blocks may be setting err: one
+    // decision for the warp)
+    if (__any_sync(kFull, (A.ctl->spill | A.ctl->err) != 0)) return;
     const uint32_t lane = threadIdx.x & 31, step = gridDim.x * blockDim.x;
     unsigned long long put = 0;
     for (uint64_t j0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; j0 < B; j0 += step) {
