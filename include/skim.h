@@ -217,7 +217,8 @@ int skim_get_sketch(skim_ctx *ctx, uint32_t v, uint64_t *out_k, uint32_t *out_le
 int skim_sketch_pointers(skim_ctx *ctx, const uint64_t **x_dev, const uint32_t **len_dev);
 
 /* SKIM, Algorithm 1 (Section 4): select n_seeds more seeds.  Continues the
- * sequence on repeated calls (resume after tau_v, Section 4).  Outputs (host):
+ * sequence on repeated calls (resume after tau_v, Section 4), also when sketches
+ * are built in between.  Outputs (host):
  * seeds_out[j] the j-th new seed, cov_out[j] its marginal coverage in
  * node-instance pairs, i.e. l * I_j (integer).  Tie rules: the seed is the
  * smallest node id among nodes whose partial sketch reaches k on the same

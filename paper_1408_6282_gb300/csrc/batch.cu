@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(kStepThreads, 1) k_step(const __grid_constant_
     if (first) C->step.best = ~0ull;
     if (a.refilter) step_refilter(a);
     if (!step_barrier(C, 0, a.timeout_ns)) return;
-    if (a.scan) step_candidates(a);
+    step_candidates(a);
     if (!step_barrier(C, 1, a.timeout_ns)) return;
     const uint64_t best = ld_volatile(&C->step.best);
     const uint32_t hi = best == ~0ull ? a.B - 1 : static_cast<uint32_t>(best >> 32);

@@ -838,12 +838,30 @@ int residual(skim_ctx *c, uint32_t x, uint64_t *cov) {
     return SKIM_OK;
 }
 
-// A step over what is left of the active batch; scan false: commit all of it.
-StepArgs step_args(const skim_ctx *c, bool scan) {
-    return StepArgs{c->rkey, c->rbits, c->bR, c->btbits, c->blo, c->bB, c->l, c->k, c->refilter ? 1u : 0u, scan ? 1u : 0u,
-                    c->spair + c->bp0, c->covered, c->alive, c->leaf, c->size, c->lane_fill, c->lane_off, c->idx_ctr, c->idx,
-                    c->seg_start, c->seg_len, c->ctl, c->timeout_ns, c->n, c->rec_tau && scan ? c->rec_kp + c->rec_j : nullptr,
-                    c->rec_tau ? c->rec_tau + c->rec_j : nullptr, c->srank + c->bp0};
+// A step over what is left of the active batch.
+StepArgs step_args(const skim_ctx *c) {
+    return StepArgs{c->rkey, c->rbits, c->bR, c->btbits, c->blo, c->bB, c->l, c->k, c->refilter ? 1u : 0u,
+                    c->spair + c->bp0, c->covered, c->alive, c->leaf, c->size, c->lane_fill, c->lane_off, c->idx_ctr,
+                    c->idx, c->seg_start, c->seg_len, c->ctl, c->timeout_ns, c->n,
+                    c->rec_tau ? c->rec_kp + c->rec_j : nullptr, c->rec_tau ? c->rec_tau + c->rec_j : nullptr,
+                    c->srank + c->bp0};
+}
+
+// Between two seeds: the active batch goes, and the lanes past the last stop are
+// searched again by the next one (they hold stops that have not been looked for, so
+// committing them would lose seeds).
+int drop_batch(skim_ctx *c) {
+    if (!c->batch_active) return SKIM_OK;
+    uint64_t used = 0;  // the dropped lanes take no room in the index
+    CK(c, cudaMemcpyAsync(&used, c->idx_ctr, sizeof(uint64_t), cudaMemcpyDeviceToHost, c->st));
+    CK(c, cudaStreamSynchronize(c->st));
+    const uint64_t left = c->bB - c->blo;
+    c->idx_bound = used;
+    c->cursor = c->bp0 + c->blo;
+    c->since_stop -= std::min(c->since_stop, left);
+    c->batch_active = false;
+    c->refilter = false;
+    return clear_batch(c);
 }
 
 int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
@@ -851,7 +869,7 @@ int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
         if (c->batch_active) {
             {
                 KTimer kt(c, SKIM_K_STEP);
-                CK(c, launch_step(step_args(c, true), c->st));
+                CK(c, launch_step(step_args(c), c->st));
             }
             // the search of the seed it finds goes behind it at once, unless
             // each is timed alone
@@ -1979,11 +1997,7 @@ int skim_build_sketches(skim_ctx *c) {
         RC(dalloc(c, &c->xlen, c->n));
         RC(dalloc(c, &c->X, static_cast<size_t>(c->n) * c->k));
     }
-    if (c->batch_active) {  // a SKIM batch holds the visited table: release it
-        CK(c, launch_step(step_args(c, false), c->st));
-        RC(clear_batch(c));
-        c->batch_active = false;
-    }
+    RC(drop_batch(c));  // (a SKIM batch holds the records and the visited table)
     RC(reset_stats(c));
     c->built = false;
     RC(c->mat ? build_rows(c) : build_coins(c));

@@ -291,13 +291,13 @@ cudaError_t launch_node_sort(uint64_t *rec_key, uint32_t *rec_val, uint64_t R, u
 cudaError_t launch_gather_bits(const uint32_t *rec_val, const uint64_t *hvals, uint64_t R, uint64_t *rbits,
                                cudaStream_t s);
 // A step over the active batch's R records: the lanes [lo, B) of covered sources
-// dropped (refilter), the next stop (scan) into ctl->step.best ((lane << 32) | node, ~0 if
+// dropped (refilter), the next stop into ctl->step.best ((lane << 32) | node, ~0 if
 // there is none), the lanes up to it (or all) committed.  ctl->step.cov = the last
 // search's count; nothing is done and ctl->step.stalled set if it is unfinished.
 struct StepArgs {
     const uint64_t *rec_key, *rbits;
     uint64_t R;
-    uint32_t tbits, lo, B, l, k, refilter, scan;
+    uint32_t tbits, lo, B, l, k, refilter;
     const uint32_t *lane_pair;
     const uint64_t *covered;
     uint64_t *alive;

@@ -85,3 +85,22 @@ def test_commits_of_few_and_many_lanes(name, bl):
     with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, batch_lanes=bl) as sk:
         for a, b in zip(sk.greedy_stops(30), (seeds, cov, tau, kp)):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("name", list(GRAPHS) + ["sparse"])
+@pytest.mark.parametrize("l,k,p,bl", [(64, 16, 0.2, 0), (33, 2, 0.1, 64), (64, 5, 0.01, 0), (1, 3, 0.4, 128)])
+def test_builds_between_seeds_lose_no_stop(name, l, k, p, bl):
+    """Sketches built between two calls: the sequence goes on where it stopped, with the
+    ranks of the batch that was active then."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.rmat(12, 8, 5) if name == "sparse" else GRAPHS[name]()
+    ks = synth.Keys.from_seed(l + k)
+    pb = oracle.Problem(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
+    seeds, cov, tau, kp, _ = oracle.skim_stops(pb, 40)
+    with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, batch_lanes=bl) as sk:
+        got = []
+        for c in (7, 1, 2, 30):
+            got.append(sk.greedy_stops(c))
+            sk.build_sketches()
+        for q, want in enumerate((seeds, cov, tau, kp)):
+            assert np.array_equal(np.concatenate([x[q] for x in got]), want)
