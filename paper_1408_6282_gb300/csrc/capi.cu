@@ -481,7 +481,7 @@ int node_buffers(skim_ctx *c) {
     if (c->ncnt) return SKIM_OK;
     RC(dalloc(c, &c->ncnt, static_cast<size_t>(c->n) + 1));
     RC(dalloc(c, &c->noff, static_cast<size_t>(c->n) + 1));
-    RC(dalloc(c, &c->nlist, c->n));
+    if (!c->nlist) RC(dalloc(c, &c->nlist, c->n));  // (a sketch build has it too)
     RC(dalloc(c, &c->nlist_cnt, 2));
     CK(c, cudaMemsetAsync(c->ncnt, 0, (static_cast<size_t>(c->n) + 1) * sizeof(uint64_t), c->st));
     return SKIM_OK;
