@@ -154,6 +154,7 @@ struct skim_ctx {
     uint64_t qpart_cap = 0;
     uint64_t *qtab = nullptr;  // table of the largest queries (16 bytes per slot)
     uint64_t qtab_slots = 0;
+    uint64_t refuse = 0;  // test hook: allocations until one is refused (0: none)
     // counters of the last build/greedy call
     uint64_t hstats[SKIM_STAT_COUNT] = {0};
     // kernel timing (CUDA events on the context stream)
@@ -220,6 +221,7 @@ cudaError_t device_pool(cudaMemPool_t *out) {
 
 int dalloc_bytes(skim_ctx *c, void **p, size_t bytes) {
     *p = nullptr;
+    if (c->refuse && --c->refuse == 0) return SKIM_ENOMEM;
     cudaMemPool_t pool;
     cudaError_t e = device_pool(&pool);
     if (e == cudaSuccess) e = cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, c->st);
@@ -241,6 +243,26 @@ void dfree(skim_ctx *c, T *&p) {
     if (p) cudaFreeAsync(p, c->st);
     p = nullptr;
 }
+
+// A buffer that the context keeps: allocated unless it is there already.  A group
+// of them of which one was refused is completed by the next call that needs it.
+template <class T>
+int dkeep(skim_ctx *c, T **p, size_t count) {
+    return *p ? SKIM_OK : dalloc(c, p, count);
+}
+
+// Device memory of a scope, freed on every way out.
+template <class T>
+struct Scratch {
+    skim_ctx *c;
+    T *p = nullptr;
+    explicit Scratch(skim_ctx *ctx) : c(ctx) {}
+    Scratch(const Scratch &) = delete;
+    ~Scratch() { free(); }
+    int alloc(size_t count) { return dalloc(c, &p, count); }
+    void free() { dfree(c, p); }
+    operator T *() const { return p; }
+};
 
 int bitlen(uint64_t x) {  // bits needed to hold values 0..x
     int b = 0;
@@ -478,11 +500,11 @@ bool trace_batches() {
 
 // Buffers of the per-node record placement; the counters start at zero.
 int node_buffers(skim_ctx *c) {
+    RC(dkeep(c, &c->noff, static_cast<size_t>(c->n) + 1));
+    RC(dkeep(c, &c->nlist, c->n));  // (a sketch build has it too)
+    RC(dkeep(c, &c->nlist_cnt, 2));
     if (c->ncnt) return SKIM_OK;
     RC(dalloc(c, &c->ncnt, static_cast<size_t>(c->n) + 1));
-    RC(dalloc(c, &c->noff, static_cast<size_t>(c->n) + 1));
-    if (!c->nlist) RC(dalloc(c, &c->nlist, c->n));  // (a sketch build has it too)
-    RC(dalloc(c, &c->nlist_cnt, 2));
     CK(c, cudaMemsetAsync(c->ncnt, 0, (static_cast<size_t>(c->n) + 1) * sizeof(uint64_t), c->st));
     return SKIM_OK;
 }
@@ -689,18 +711,16 @@ uint32_t skim_lanes(skim_ctx *c) {
 // ---- SKIM steps ------------------------------------------------------------
 
 int skim_state_init(skim_ctx *c) {
-    if (!c->covered) {
-        RC(dalloc(c, &c->covered, c->n));
-        RC(dalloc(c, &c->size, c->n));
-        RC(dalloc(c, &c->ncount, c->n));
-        RC(dalloc(c, &c->leaf, c->lane_cap / 64 + 1));
-        RC(dalloc(c, &c->seg_start, c->nl));
-        RC(dalloc(c, &c->seg_len, c->nl));
-        RC(dalloc(c, &c->chosen, c->n));
-        RC(dalloc(c, &c->pend_trav, c->n));
-        RC(dalloc(c, &c->pend_erase, c->n));
-        RC(dalloc(c, &c->idx_ctr, 2));
-    }
+    RC(dkeep(c, &c->covered, c->n));
+    RC(dkeep(c, &c->size, c->n));
+    RC(dkeep(c, &c->ncount, c->n));
+    RC(dkeep(c, &c->leaf, c->lane_cap / 64 + 1));
+    RC(dkeep(c, &c->seg_start, c->nl));
+    RC(dkeep(c, &c->seg_len, c->nl));
+    RC(dkeep(c, &c->chosen, c->n));
+    RC(dkeep(c, &c->pend_trav, c->n));
+    RC(dkeep(c, &c->pend_erase, c->n));
+    RC(dkeep(c, &c->idx_ctr, 2));
     CK(c, cudaMemsetAsync(c->covered, 0, c->n * sizeof(uint64_t), c->st));
     CK(c, cudaMemsetAsync(c->size, 0, c->n * sizeof(uint32_t), c->st));
     CK(c, cudaMemsetAsync(c->seg_len, 0, c->nl * sizeof(uint32_t), c->st));
@@ -1009,8 +1029,8 @@ int make_instances(skim_ctx *c) {
         RC(dalloc(c, &c->nonempty, c->n));
         RC(dalloc_bytes(c, &c->pieces, live_pieces_bytes(c->m)));
     }
-    uint64_t *first = nullptr;  // of every node: its live pairs, then those of the nodes before it
-    RC(dalloc(c, &first, static_cast<size_t>(c->n) + 1));
+    Scratch<uint64_t> first(c);  // of every node: its live pairs, then those of the nodes before it
+    RC(first.alloc(static_cast<size_t>(c->n) + 1));
     CK(c, launch_live_masks(c->rrow, c->rcol, c->rhe, c->rtm1, c->rev2fwd, c->cm, c->m, c->l, c->rmask, c->fmask,
                             c->st));
     CK(c, launch_live_count(c->rptr, c->rmask, c->n, c->m, c->l, first, c->loff, c->pieces, c->st));
@@ -1018,10 +1038,7 @@ int make_instances(skim_ctx *c) {
     CK(c, exclusive_scan_u64(first, first, static_cast<size_t>(c->n) + 1, nullptr, c->ws, c->st));
     CK(c, cudaMemcpyAsync(&c->live_total, first + c->n, sizeof(uint64_t), cudaMemcpyDeviceToHost, c->st));
     CK(c, cudaStreamSynchronize(c->st));
-    if (c->live_total > kMaxLive) {  // offsets would not fit 31 bits: coins are drawn in the searches
-        dfree(c, first);
-        return SKIM_OK;
-    }
+    if (c->live_total > kMaxLive) return SKIM_OK;  // offsets would not fit 31 bits: coins are drawn in the searches
     if (c->live_total > c->rlive_cap) {
         dfree(c, c->rlive);
         dfree(c, c->flive);
@@ -1038,7 +1055,6 @@ int make_instances(skim_ctx *c) {
     CK(c, exclusive_scan_u64(first, first, static_cast<size_t>(c->n) + 1, nullptr, c->ws, c->st));
     CK(c, launch_live_fill(c->fptr, c->fcol, c->fmask, c->n, c->m, c->l, first, c->foff, nullptr, c->flive, c->pieces,
                            c->st));
-    dfree(c, first);
     c->live_ready = true;
     c->mat = c->mat_wanted;
     return SKIM_OK;
@@ -1203,6 +1219,9 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
     c->batch_cfg = prm->batch_lanes;
     c->ring_rpl = kRingRecordsPerLane;
     c->node_density = static_cast<uint32_t>(kNodeSortDensity);
+    // SKIM_REFUSE_ALLOC in the environment (a test hook): that allocation of the
+    // context, counted from its creation, is refused
+    if (const char *ra = getenv("SKIM_REFUSE_ALLOC")) c->refuse = strtoull(ra, nullptr, 10);
     c->cm.model = prm->prob_model;
     c->cm.tm1_uniform = prm->prob_model == 0 ? tm1_of(prm->p) : 0;
     c->cm.tm1_class[0] = tm1_of(0.1);
@@ -1234,18 +1253,17 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
         TRYC(cudaMemsetAsync(c->ctl, 0, sizeof(DevCtl), c->st));
         TRY(dalloc(c, &c->dflag, 1));
         // edges on the device
-        uint32_t *dsrc = nullptr, *ddst = nullptr;
-        bool own_edges = !g->on_device;
-        if (own_edges) {
-            TRY(dalloc(c, &dsrc, m));
-            TRY(dalloc(c, &ddst, m));
+        Scratch<uint32_t> own_src(c), own_dst(c);
+        const uint32_t *dsrc = g->src, *ddst = g->dst;
+        if (!g->on_device) {
+            TRY(own_src.alloc(m));
+            TRY(own_dst.alloc(m));
             if (m) {
-                TRYC(cudaMemcpyAsync(dsrc, g->src, m * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st));
-                TRYC(cudaMemcpyAsync(ddst, g->dst, m * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st));
+                TRYC(cudaMemcpyAsync(own_src, g->src, m * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st));
+                TRYC(cudaMemcpyAsync(own_dst, g->dst, m * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st));
             }
-        } else {
-            dsrc = const_cast<uint32_t *>(g->src);
-            ddst = const_cast<uint32_t *>(g->dst);
+            dsrc = own_src;
+            ddst = own_dst;
         }
         TRYC(cudaMemsetAsync(c->dflag, 0, sizeof(unsigned), c->st));
         TRYC(launch_check_edges(dsrc, ddst, m, n, c->dflag, c->st));
@@ -1253,7 +1271,6 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
         TRYC(cudaMemcpyAsync(&bad, c->dflag, sizeof(unsigned), cudaMemcpyDeviceToHost, c->st));
         TRYC(cudaStreamSynchronize(c->st));
         if (bad) {
-            if (own_edges) { dfree(c, dsrc); dfree(c, ddst); }
             rc = SKIM_EGRAPH;
             goto fail;
         }
@@ -1287,19 +1304,19 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
         if (m) TRYC(cudaMemcpyAsync(c->fcol, ddst, m * sizeof(uint32_t), cudaMemcpyDeviceToDevice, c->st));
         // reverse CSR: (dst, src) order, by a stable sort on the dst bits
         if (m) {
-            uint64_t *k1 = nullptr, *k2 = nullptr;
-            uint32_t *v1 = nullptr, *v2 = nullptr;
-            TRY(dalloc(c, &k1, m));
-            TRY(dalloc(c, &k2, m));
-            TRY(dalloc(c, &v1, m));
-            TRY(dalloc(c, &v2, m));
+            Scratch<uint64_t> k1(c), k2(c);
+            Scratch<uint32_t> v1(c), v2(c);
+            TRY(k1.alloc(m));
+            TRY(k2.alloc(m));
+            TRY(v1.alloc(m));
+            TRY(v2.alloc(m));
             TRYC(launch_make_rev_keys(dsrc, ddst, m, k1, v1, c->st));
             TRYC(radix_sort_pairs(k1, v1, k2, v2, m, std::max(1, bitlen(n - 1)), c->ws, c->st));
             TRYC(launch_split_rev(k1, v1, m, c->rcol, c->rrow, c->rev2fwd, c->st));
-            dfree(c, k1); dfree(c, k2); dfree(c, v1); dfree(c, v2);  // (stream-ordered)
         }
         TRYC(launch_row_ptr(c->rrow, m, n, c->rptr, c->st));
-        if (own_edges) { dfree(c, dsrc); dfree(c, ddst); }
+        own_src.free();  // (stream-ordered)
+        own_dst.free();
         TRYC(cudaMemsetAsync(c->ctl, 0, sizeof(DevCtl), c->st));
         TRY(dalloc(c, &c->rhe, m));
         TRY(dalloc(c, &c->fhe, m));
@@ -1364,6 +1381,43 @@ fail:
     return rc;
 }
 
+}  // extern "C"
+
+namespace {
+
+// What the graphs of a batch have each of their own, on the device.  keys: coin, rank
+// and probability keys and uniform thresholds, `count` of each.
+int batch_tables(skim_ctx *c, uint32_t count, const std::vector<uint32_t> &node_off, const std::vector<uint64_t> &keys,
+                 const std::vector<int> &model) {
+    Scratch<uint32_t> graph(c);  // of every node
+    Scratch<uint64_t> key(c);
+    Scratch<int> mod(c);
+    RC(dalloc(c, &c->node_off, count + 1));
+    RC(graph.alloc(c->n));
+    RC(key.alloc(keys.size()));
+    RC(mod.alloc(count));
+    RC(dalloc(c, &c->rbase, c->n));
+    RC(dalloc(c, &c->rtm1, c->m));
+    RC(dalloc(c, &c->ftm1, c->m));
+    const BatchDesc b{count, graph, c->node_off, key, key + count, key + 2 * count, key + 3 * count, mod,
+                      {tm1_of(0.1), tm1_of(0.01), tm1_of(0.001)}};
+    CK(c, cudaMemcpyAsync(c->node_off, node_off.data(), (count + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st));
+    CK(c, cudaMemcpyAsync(key, keys.data(), keys.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, c->st));
+    CK(c, cudaMemcpyAsync(mod, model.data(), count * sizeof(int), cudaMemcpyHostToDevice, c->st));
+    CK(c, launch_node_graph(c->node_off, count, graph, c->st));
+    CK(c, launch_edge_states_batch(c->rptr, c->rcol, c->n, b, 1, c->rhe, c->st));
+    CK(c, launch_edge_states_batch(c->fptr, c->fcol, c->n, b, 0, c->fhe, c->st));
+    CK(c, launch_edge_tm1_batch(c->rptr, c->rcol, c->n, b, c->thr_wc, 1, c->rtm1, c->st));
+    CK(c, launch_edge_tm1_batch(c->fptr, c->fcol, c->n, b, c->thr_wc, 0, c->ftm1, c->st));
+    CK(c, launch_rank_bases(b, c->n, c->l, c->rbase, c->st));
+    CK(c, cudaStreamSynchronize(c->st));
+    return SKIM_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 int skim_create_batch(const skim_graph *graphs, const skim_params *prm, uint32_t count, void *stream,
                       skim_ctx **out) {
     if (!graphs || !prm || !out || count == 0) return SKIM_EINVAL;
@@ -1413,41 +1467,12 @@ int skim_create_batch(const skim_graph *graphs, const skim_params *prm, uint32_t
         skim_destroy(c);
         return r;
     };
-    // per-graph tables on the device
-    uint32_t *d_off = nullptr, *d_ng = nullptr;
-    uint64_t *d_keys = nullptr;
-    int *d_model = nullptr;
-    if ((rc = dalloc(c, &d_off, count + 1)) || (rc = dalloc(c, &d_ng, n_tot)) || (rc = dalloc(c, &d_keys, 4ull * count)) ||
-        (rc = dalloc(c, &d_model, count)))
-        return fail(rc);
     std::vector<uint64_t> keys;
     keys.insert(keys.end(), ck.begin(), ck.end());
     keys.insert(keys.end(), rk.begin(), rk.end());
     keys.insert(keys.end(), pk.begin(), pk.end());
     keys.insert(keys.end(), tu.begin(), tu.end());
-    BatchDesc b{count, d_ng, d_off, d_keys, d_keys + count, d_keys + 2 * count, d_keys + 3 * count, d_model,
-                {tm1_of(0.1), tm1_of(0.01), tm1_of(0.001)}};
-    bool ok = cudaMemcpyAsync(d_off, node_off.data(), (count + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st) ==
-                  cudaSuccess &&
-              cudaMemcpyAsync(d_keys, keys.data(), keys.size() * sizeof(uint64_t), cudaMemcpyHostToDevice, c->st) ==
-                  cudaSuccess &&
-              cudaMemcpyAsync(d_model, model.data(), count * sizeof(int), cudaMemcpyHostToDevice, c->st) == cudaSuccess &&
-              launch_node_graph(d_off, count, d_ng, c->st) == cudaSuccess;
-    if (ok) {
-        if ((rc = dalloc(c, &c->rbase, n_tot)) || (rc = dalloc(c, &c->rtm1, m_tot)) || (rc = dalloc(c, &c->ftm1, m_tot)))
-            return fail(rc);
-        ok = launch_edge_states_batch(c->rptr, c->rcol, c->n, b, 1, c->rhe, c->st) == cudaSuccess &&
-             launch_edge_states_batch(c->fptr, c->fcol, c->n, b, 0, c->fhe, c->st) == cudaSuccess &&
-             launch_edge_tm1_batch(c->rptr, c->rcol, c->n, b, c->thr_wc, 1, c->rtm1, c->st) == cudaSuccess &&
-             launch_edge_tm1_batch(c->fptr, c->fcol, c->n, b, c->thr_wc, 0, c->ftm1, c->st) == cudaSuccess &&
-             launch_rank_bases(b, c->n, c->l, c->rbase, c->st) == cudaSuccess;
-    }
-    if (ok) ok = cudaStreamSynchronize(c->st) == cudaSuccess;
-    c->node_off = d_off;
-    dfree(c, d_ng);
-    dfree(c, d_keys);
-    dfree(c, d_model);
-    if (!ok) return fail(fail_cuda(c, cudaGetLastError()));
+    if ((rc = batch_tables(c, count, node_off, keys, model))) return fail(rc);
     c->cm.model = 3;
     c->batch_count = count;
     if ((rc = make_instances(c))) return fail(rc);
@@ -1555,9 +1580,8 @@ int skim_instances(skim_ctx *c) {
         RC(clear_batch(c));
         c->batch_active = false;
     }
-    RC(make_instances(c));
     c->sk_init = false;
-    return SKIM_OK;
+    return make_instances(c);
 }
 
 int skim_instance_stats(skim_ctx *c, uint64_t *live_pairs, int *materialised) {
@@ -1614,16 +1638,16 @@ constexpr double kGiantMean = 64.0;
 
 int rows_buffers(skim_ctx *c) {
     if (c->need) return SKIM_OK;
-    RC(dalloc(c, &c->over_seg, c->n));
-    RC(dalloc(c, &c->over_buf, c->rcap));
-    RC(dalloc(c, &c->full_list, c->n));
-    RC(dalloc(c, &c->hitbits, c->lane_cap / 32 + 1));
-    RC(dalloc(c, &c->defbits, c->lane_cap / 32 + 1));
-    RC(dalloc(c, &c->defpair, c->lane_cap));
-    if (!c->nlist) RC(dalloc(c, &c->nlist, c->n));
+    RC(dkeep(c, &c->over_seg, c->n));
+    RC(dkeep(c, &c->over_buf, c->rcap));
+    RC(dkeep(c, &c->full_list, c->n));
+    RC(dkeep(c, &c->hitbits, c->lane_cap / 32 + 1));
+    RC(dkeep(c, &c->defbits, c->lane_cap / 32 + 1));
+    RC(dkeep(c, &c->defpair, c->lane_cap));
+    RC(dkeep(c, &c->nlist, c->n));
     // a task is 24 bytes; about a third of the pairs can be one
     const uint64_t tasks = std::min<uint64_t>(8 * c->nl, 4ull << 30);
-    if (tasks > c->hcap * 2 * sizeof(uint64_t)) {
+    if (!c->need_ws && tasks > c->hcap * 2 * sizeof(uint64_t)) {
         RC(dalloc_bytes(c, &c->need_ws, tasks));
         c->need_ws_bytes = tasks;
     }
@@ -1662,11 +1686,9 @@ size_t comp_space(uint32_t graphs, uint32_t l, uint32_t k, void *ws, CompSpace *
 // false if none is worth it.
 int contract_components(skim_ctx *c, BuildNode &g, CompSpace *sp, bool *on) {
     *on = false;
-    if (!c->comp) {
-        RC(dalloc(c, &c->comp_up, c->n));
-        RC(dalloc_bytes(c, &c->comp_ws, comp_space(g.graphs, c->l, c->k, nullptr, sp)));
-        RC(dalloc(c, &c->comp, c->n));
-    }
+    RC(dkeep(c, &c->comp, c->n));
+    RC(dkeep(c, &c->comp_up, c->n));
+    if (!c->comp_ws) RC(dalloc_bytes(c, &c->comp_ws, comp_space(g.graphs, c->l, c->k, nullptr, sp)));
     comp_space(g.graphs, c->l, c->k, c->comp_ws, sp);
     g.tlen = sp->tlen;
     g.topen = sp->topen;
@@ -1680,13 +1702,12 @@ int contract_components(skim_ctx *c, BuildNode &g, CompSpace *sp, bool *on) {
         r.back_off = c->loff;
         r.back_rows = c->rlive;
         r.back_mask = c->comp_up;
-        uint64_t *pend = nullptr;
-        RC(dalloc(c, &pend, 2ull * c->n));
+        Scratch<uint64_t> pend(c);
+        RC(pend.alloc(2ull * c->n));
         CK(c, cudaMemsetAsync(pend, 0, 2ull * c->n * sizeof(uint64_t), c->st));
         r.pend_trav = pend;
         r.back_pend = pend + c->n;
         CK(c, launch_reach_from(r, sp->pivot, g.graphs, sp->count, c->st));
-        dfree(c, pend);
         CK(c, launch_components(g, c->comp, c->comp_up, sp->count, sp->count + 64, c->ctl, c->st));
     }
     RC(sync_ctl(c));
@@ -1922,10 +1943,8 @@ int build_rows(skim_ctx *c) {
 
 // Algorithm 2 with coins drawn in the searches.
 int build_coins(skim_ctx *c) {
-    if (!c->lcnt) {
-        RC(dalloc(c, &c->full, c->n));
-        RC(dalloc(c, &c->lcnt, c->nl));
-    }
+    RC(dkeep(c, &c->full, c->n));
+    RC(dkeep(c, &c->lcnt, c->nl));
     CK(c, cudaMemsetAsync(c->lcnt, 0, c->nl, c->st));
     CK(c, cudaMemsetAsync(c->full, 0, c->n * sizeof(uint64_t), c->st));
     CK(c, cudaMemsetAsync(c->X, 0, static_cast<size_t>(c->n) * c->k * sizeof(uint64_t), c->st));
@@ -1993,10 +2012,8 @@ extern "C" {
 int skim_build_sketches(skim_ctx *c) {
     if (!c) return SKIM_EINVAL;
     if (c->broken) return SKIM_ECUDA;
-    if (!c->X) {
-        RC(dalloc(c, &c->xlen, c->n));
-        RC(dalloc(c, &c->X, static_cast<size_t>(c->n) * c->k));
-    }
+    RC(dkeep(c, &c->xlen, c->n));
+    RC(dkeep(c, &c->X, static_cast<size_t>(c->n) * c->k));
     RC(drop_batch(c));  // (a SKIM batch holds the records and the visited table)
     RC(reset_stats(c));
     c->built = false;

@@ -36,3 +36,52 @@ def test_build_and_seeds_leave_no_memory_behind(build_first):
     before = _free()
     once()
     assert _free() >= before - (1 << 20)
+
+
+def test_a_refused_allocation_costs_one_call(monkeypatch):
+    """Every device allocation of a context refused in turn (SKIM_REFUSE_ALLOC): the call
+    that wanted it reports SKIM_ENOMEM, the same call works when it is made again, and
+    nothing stays allocated."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.rmat(11, 12, 8)
+    ks = synth.Keys.from_seed(2)
+    pb = oracle.Problem(g.n, g.src, g.dst, 8, 8, 0, 0.3, ks.coin, ks.rank, ks.prob)
+    ox, oln, _ = oracle.build_sketches(pb)
+    want = oracle.skim_stops(pb, 6)[:4]
+    q = [np.arange(a, dtype=np.uint32) for a in (3, 2000)]
+    ref = [oracle.union_estimate(ox, oln, 8, s) for s in q]
+
+    def create():
+        return pkg.Skim(g.n, g.src, g.dst, 8, 8, 0, 0.3, ks.coin, ks.rank, ks.prob)
+
+    create().close()
+    before = _free()
+    refused = []
+    for at in range(1, 111):
+        monkeypatch.setenv("SKIM_REFUSE_ALLOC", str(at))
+        hit = []
+
+        def twice(f, between=lambda: None):
+            try:
+                return f()
+            except pkg.SkimError as e:
+                assert e.code == -2 and not hit
+                hit.append(f)
+                monkeypatch.delenv("SKIM_REFUSE_ALLOC")
+                between()
+                return f()
+
+        with twice(create) as sk:
+            for rows in (True, False):
+                sk.set_live_rows(rows)
+                twice(sk.build_sketches)
+                x, ln = sk.sketches()
+                assert np.array_equal(ln, oln) and np.array_equal(x, ox), at
+                for a, b in zip(twice(lambda: sk.greedy_stops(6), sk.greedy_reset), want):
+                    assert np.array_equal(a, b), at
+            for a, b in zip(twice(lambda: sk.query_batch(q)), ref):
+                assert abs(a - b) <= 1e-12 * b
+            twice(sk.node_estimates)
+        refused.append(len(hit))
+    assert sum(refused) >= 60 and not any(refused[-5:])  # past the last allocation
+    assert _free() >= before - (1 << 20)
