@@ -831,29 +831,32 @@ __global__ void k_need_open(uint32_t k, uint32_t graphs, uint32_t *tlen, uint64_
 
 // Per graph and instance the node with the largest product of live in- and
 // out-degree (a member of the largest component where there is a large one).
-// blockIdx.y: graph.
-__global__ void __launch_bounds__(256) k_pivots(BuildNode g, unsigned long long *best) {
-    const uint32_t lane = threadIdx.x & 31;
-    const uint32_t v0 = g.graphs == 1 ? 0 : g.node_off[blockIdx.y], v1 = g.graphs == 1 ? g.n : g.node_off[blockIdx.y + 1];
-    unsigned long long b[2] = {0, 0};
-    for (uint32_t v = v0 + ((blockIdx.x * blockDim.x + threadIdx.x) >> 5); v < v1; v += (gridDim.x * blockDim.x) >> 5) {
-        const uint64_t ne = g.nonempty[v];
+// `per` blocks a graph, the graphs in steps of the grid (a batch may have more than
+// any grid dimension holds).
+__global__ void __launch_bounds__(256) k_pivots(BuildNode g, uint32_t per, unsigned long long *best) {
+    const uint32_t lane = threadIdx.x & 31, part = blockIdx.x % per;
+    for (uint32_t q = blockIdx.x / per; q < g.graphs; q += gridDim.x / per) {
+        const uint32_t v0 = g.graphs == 1 ? 0 : g.node_off[q], v1 = g.graphs == 1 ? g.n : g.node_off[q + 1];
+        unsigned long long b[2] = {0, 0};
+        for (uint32_t v = v0 + ((part * blockDim.x + threadIdx.x) >> 5); v < v1; v += (per * blockDim.x) >> 5) {
+            const uint64_t ne = g.nonempty[v];
 #pragma unroll
-        for (uint32_t h = 0; h < 2; h++) {
-            const uint32_t i = lane + 32 * h;
-            uint64_t d = 0;
-            if ((ne >> i) & 1ull) {
-                const uint64_t r = static_cast<uint64_t>(v) * g.l + i;
-                d = static_cast<uint64_t>(g.loff[r + 1] - g.loff[r]) * (g.foff[r + 1] - g.foff[r]);
+            for (uint32_t h = 0; h < 2; h++) {
+                const uint32_t i = lane + 32 * h;
+                uint64_t d = 0;
+                if ((ne >> i) & 1ull) {
+                    const uint64_t r = static_cast<uint64_t>(v) * g.l + i;
+                    d = static_cast<uint64_t>(g.loff[r + 1] - g.loff[r]) * (g.foff[r + 1] - g.foff[r]);
+                }
+                const unsigned long long x =
+                    static_cast<unsigned long long>(d < 0xFFFFFFFFu ? d : 0xFFFFFFFFu) << 32 | (0xFFFFFFFFu - v);
+                b[h] = max(b[h], x);
             }
-            const unsigned long long x =
-                static_cast<unsigned long long>(d < 0xFFFFFFFFu ? d : 0xFFFFFFFFu) << 32 | (0xFFFFFFFFu - v);
-            b[h] = max(b[h], x);
         }
-    }
 #pragma unroll
-    for (uint32_t h = 0; h < 2; h++)
-        if (lane + 32 * h < g.l && b[h]) atomicMax(&best[blockIdx.y * 64 + lane + 32 * h], b[h]);
+        for (uint32_t h = 0; h < 2; h++)
+            if (lane + 32 * h < g.l && b[h]) atomicMax(&best[q * 64ull + lane + 32 * h], b[h]);
+    }
 }
 
 __global__ void k_pivot_nodes(const unsigned long long *best, uint32_t count, uint32_t *pivot) {
@@ -917,38 +920,43 @@ __global__ void __launch_bounds__(128) k_hit_rows(uint32_t lists, uint32_t l, ui
     }
 }
 
-// Block (i, graph): places of list i's entries in the graph's rank order of
-// all hits, out[graph][place], and per instance the bitmap of its places.
-__global__ void k_hits_sort(const uint64_t *hits, const uint32_t *tlen, uint32_t l, uint32_t k, uint64_t *out,
-                            uint64_t *places, uint32_t *total) {
+// A block per list i of a graph, in steps of the grid: places of the list's entries in
+// the graph's rank order of all hits, out[graph][place], and per instance the bitmap
+// of its places.
+__global__ void k_hits_sort(const uint64_t *hits, const uint32_t *tlen, uint32_t graphs, uint32_t l, uint32_t k,
+                            uint64_t *out, uint64_t *places, uint32_t *total) {
     __shared__ uint32_t s_cnt[64];
-    const uint32_t i = blockIdx.x, g = blockIdx.y, words = (l * k + 63) / 64;
-    if (threadIdx.x < 64) s_cnt[threadIdx.x] = threadIdx.x < l ? min(tlen[g * 64 + threadIdx.x] & ~kRowDone, k) : 0;
-    __syncthreads();
-    const uint64_t *h = hits + static_cast<uint64_t>(g) * 64 * k;
-    uint64_t *bits = places + (static_cast<uint64_t>(g) * 64 + i) * words;
-    for (uint32_t w = threadIdx.x; w < words; w += blockDim.x) bits[w] = 0;
-    __syncthreads();
-    for (uint32_t q = threadIdx.x; q < s_cnt[i]; q += blockDim.x) {
-        const uint64_t x = h[static_cast<uint64_t>(i) * k + q];
-        uint32_t at = q;
-        for (uint32_t o = 0; o < l; o++) {  // entries of the other (ascending) lists below x
-            if (o == i) continue;
-            uint32_t lo = 0, hi = s_cnt[o];
-            while (lo < hi) {
-                const uint32_t mid = (lo + hi) >> 1;
-                if (h[static_cast<uint64_t>(o) * k + mid] < x) lo = mid + 1;
-                else hi = mid;
+    const uint32_t words = (l * k + 63) / 64;
+    for (uint64_t b = blockIdx.x; b < static_cast<uint64_t>(graphs) * l; b += gridDim.x) {
+        const uint64_t g = b / l;
+        const uint32_t i = static_cast<uint32_t>(b - g * l);
+        __syncthreads();  // (the counts of the list before have been used)
+        if (threadIdx.x < 64) s_cnt[threadIdx.x] = threadIdx.x < l ? min(tlen[g * 64 + threadIdx.x] & ~kRowDone, k) : 0;
+        const uint64_t *h = hits + g * 64 * k;
+        uint64_t *bits = places + (g * 64 + i) * words;
+        for (uint32_t w = threadIdx.x; w < words; w += blockDim.x) bits[w] = 0;
+        __syncthreads();
+        for (uint32_t q = threadIdx.x; q < s_cnt[i]; q += blockDim.x) {
+            const uint64_t x = h[static_cast<uint64_t>(i) * k + q];
+            uint32_t at = q;
+            for (uint32_t o = 0; o < l; o++) {  // entries of the other (ascending) lists below x
+                if (o == i) continue;
+                uint32_t lo = 0, hi = s_cnt[o];
+                while (lo < hi) {
+                    const uint32_t mid = (lo + hi) >> 1;
+                    if (h[static_cast<uint64_t>(o) * k + mid] < x) lo = mid + 1;
+                    else hi = mid;
+                }
+                at += lo;
             }
-            at += lo;
+            out[g * l * k + at] = x;
+            atomicOr(reinterpret_cast<unsigned long long *>(&bits[at >> 6]), 1ull << (at & 63));
         }
-        out[static_cast<uint64_t>(g) * l * k + at] = x;
-        atomicOr(reinterpret_cast<unsigned long long *>(&bits[at >> 6]), 1ull << (at & 63));
-    }
-    if (i == 0 && threadIdx.x == 0) {
-        uint32_t t = 0;
-        for (uint32_t o = 0; o < l; o++) t += s_cnt[o];
-        total[g] = t;
+        if (i == 0 && threadIdx.x == 0) {
+            uint32_t t = 0;
+            for (uint32_t o = 0; o < l; o++) t += s_cnt[o];
+            total[g] = t;
+        }
     }
 }
 
@@ -1299,9 +1307,9 @@ cudaError_t launch_need(const BuildNode &g, const uint64_t *next, uint64_t *need
 cudaError_t launch_pivots(const BuildNode &g, unsigned long long *best, uint32_t *pivot, cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(best, 0, g.graphs * 64ull * sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
-    const unsigned x = grid_for(static_cast<size_t>(g.n) * 32 / g.graphs + 1, 256, std::max(1u, 152 * 8 / g.graphs));
+    const unsigned per = grid_for(static_cast<size_t>(g.n) * 32 / g.graphs + 1, 256, std::max(1u, 152 * 8 / g.graphs));
     note_launch();
-    k_pivots<<<dim3(x, g.graphs), 256, 0, s>>>(g, best);
+    k_pivots<<<per * std::min(g.graphs, 152u * 32), 256, 0, s>>>(g, per, best);
     note_launch();
     k_pivot_nodes<<<grid_for(g.graphs * 64, 256), 256, 0, s>>>(best, g.graphs * 64, pivot);
     return cudaGetLastError();
@@ -1337,7 +1345,8 @@ cudaError_t launch_merge(const BuildNode &g, uint64_t *X, uint64_t *hits, uint64
         note_launch();
         k_hit_rows<<<grid_for(g.graphs * 64, 4), 128, 0, s>>>(g.graphs * 64, g.l, g.k, g.tlen, hits);
         note_launch();
-        k_hits_sort<<<dim3(g.l, g.graphs), 256, 0, s>>>(hits, g.tlen, g.l, g.k, hits_sorted, places, total);
+        k_hits_sort<<<grid_for(static_cast<size_t>(g.l) * g.graphs, 1), 256, 0, s>>>(hits, g.tlen, g.graphs, g.l, g.k,
+                                                                                     hits_sorted, places, total);
     }
     const unsigned grid = grid_for(static_cast<size_t>(g.n) * 32, kMergeWarps * 32, 152 * 64);
     note_launch();

@@ -109,3 +109,22 @@ def test_searches_deferred_inside_a_long_row(hubs, spokes):
     order = np.lexsort((dst, src))
     _check(n, src[order], dst[order], 16, 64, 0, 1.0)
     _check(n, src[order], dst[order], 16, 64, 0, 0.9, mode=1)
+
+
+def test_components_of_more_graphs_than_a_grid_dimension():
+    """66000 rings of 80 nodes, contracted: a list per graph and instance, against the
+    build with coins drawn in the searches."""
+    import paper_1408_6282_gb300 as pkg
+    count, size = 66000, 80
+    a = np.arange(size, dtype=np.uint32)
+    ring = (size, a, np.roll(a, -1))
+    keys = [synth.Keys.from_seed(g % 977) for g in range(count)]
+    with pkg.Skim.batch([ring] * count, 2, 3, [0] * count, [1.0] * count, [q.coin for q in keys],
+                        [q.rank + g for g, q in enumerate(keys)], [q.prob for q in keys]) as sk:
+        sk.build_sketches()
+        x, ln = sk.sketches()
+        sk.set_live_rows(False)
+        sk.build_sketches()
+        y, lm = sk.sketches()
+        assert np.array_equal(ln, lm) and np.array_equal(x, y)
+        assert np.all(ln == 3)
