@@ -1645,11 +1645,13 @@ int rows_buffers(skim_ctx *c) {
     RC(dkeep(c, &c->defbits, c->lane_cap / 32 + 1));
     RC(dkeep(c, &c->defpair, c->lane_cap));
     RC(dkeep(c, &c->nlist, c->n));
-    // a task is 24 bytes; about a third of the pairs can be one
+    // a task is 24 bytes; about a third of the pairs can be one (the visited table does
+    // with less, searched for longer, where there is no room)
     const uint64_t tasks = std::min<uint64_t>(8 * c->nl, 4ull << 30);
     if (!c->need_ws && tasks > c->hcap * 2 * sizeof(uint64_t)) {
-        RC(dalloc_bytes(c, &c->need_ws, tasks));
-        c->need_ws_bytes = tasks;
+        const int rc = dalloc_bytes(c, &c->need_ws, tasks);
+        if (rc == SKIM_OK) c->need_ws_bytes = tasks;
+        else if (rc != SKIM_ENOMEM) return rc;
     }
     return dalloc(c, &c->need, c->n);
 }
@@ -1683,12 +1685,23 @@ size_t comp_space(uint32_t graphs, uint32_t l, uint32_t k, void *ws, CompSpace *
 }
 
 // Contract the component around each instance's pivot (of every graph); *on =
-// false if none is worth it.
+// false if none is worth it or there is no room for the lists (64 k ranks a graph and
+// as much again for their order), where the searches go on as they are.
 int contract_components(skim_ctx *c, BuildNode &g, CompSpace *sp, bool *on) {
     *on = false;
-    RC(dkeep(c, &c->comp, c->n));
-    RC(dkeep(c, &c->comp_up, c->n));
-    if (!c->comp_ws) RC(dalloc_bytes(c, &c->comp_ws, comp_space(g.graphs, c->l, c->k, nullptr, sp)));
+    if (g.graphs > 0xFFFFFFFFu / 64) return SKIM_OK;  // (a list has a 32-bit number)
+    Scratch<uint64_t> pend(c);
+    int rc = dkeep(c, &c->comp, c->n);
+    if (rc == SKIM_OK) rc = dkeep(c, &c->comp_up, c->n);
+    if (rc == SKIM_OK && !c->comp_ws) rc = dalloc_bytes(c, &c->comp_ws, comp_space(g.graphs, c->l, c->k, nullptr, sp));
+    if (rc == SKIM_OK) rc = pend.alloc(2ull * c->n);
+    if (rc == SKIM_ENOMEM) {
+        dfree(c, c->comp);
+        dfree(c, c->comp_up);
+        dfree(c, c->comp_ws);
+        return SKIM_OK;
+    }
+    RC(rc);
     comp_space(g.graphs, c->l, c->k, c->comp_ws, sp);
     g.tlen = sp->tlen;
     g.topen = sp->topen;
@@ -1702,8 +1715,6 @@ int contract_components(skim_ctx *c, BuildNode &g, CompSpace *sp, bool *on) {
         r.back_off = c->loff;
         r.back_rows = c->rlive;
         r.back_mask = c->comp_up;
-        Scratch<uint64_t> pend(c);
-        RC(pend.alloc(2ull * c->n));
         CK(c, cudaMemsetAsync(pend, 0, 2ull * c->n * sizeof(uint64_t), c->st));
         r.pend_trav = pend;
         r.back_pend = pend + c->n;

@@ -85,3 +85,32 @@ def test_a_refused_allocation_costs_one_call(monkeypatch):
         refused.append(len(hit))
     assert sum(refused) >= 60 and not any(refused[-5:])  # past the last allocation
     assert _free() >= before - (1 << 20)
+
+
+def test_a_build_does_without_workspace_it_can_spare(monkeypatch):
+    """Contraction is a shortcut: a refused allocation of its workspace leaves the build
+    as it would be without it, so a graph with components wants no more than one without."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.rmat(11, 12, 8)
+    refused = {}
+    for p in (1e-6, 0.3):
+        pb = oracle.Problem(g.n, g.src, g.dst, 8, 8, 0, p, 5, 6, 7)
+        ox, oln, _ = oracle.build_sketches(pb)
+        refused[p] = 0
+        for at in range(30, 80):
+            monkeypatch.setenv("SKIM_REFUSE_ALLOC", str(at))
+            try:
+                sk = pkg.Skim(g.n, g.src, g.dst, 8, 8, 0, p, 5, 6, 7)
+            except pkg.SkimError as e:
+                assert e.code == -2
+                continue
+            with sk:
+                try:
+                    sk.build_sketches()
+                except pkg.SkimError as e:
+                    assert e.code == -2
+                    refused[p] += 1
+                    sk.build_sketches()
+                x, ln = sk.sketches()
+                assert np.array_equal(ln, oln) and np.array_equal(x, ox), (p, at)
+    assert refused[0.3] == refused[1e-6] > 5
