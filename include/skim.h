@@ -345,7 +345,10 @@ int skim_kernel_times(skim_ctx *ctx, double *ms_out, uint64_t *launches_out, uin
 /* Bound of every device-side wait of this context's searches: a warp that
  * sees no progress for `ns` nanoseconds (default 2e9) gives up, every warp of
  * the search then returns, and the call reports SKIM_ETIMEOUT (the context
- * is then unusable; destroy it).  A short limit makes the waits give up on
+ * is then unusable; destroy it).  What blocks of threads leave together (a level of
+ * a search by one block per instance, the phases of a SKIM step and of a build's need
+ * pass) makes progress in steps (a row, 32 records) and may take `ns` for each of
+ * them, up to 10 s or `ns` in all.  A short limit makes the waits give up on
  * purpose, which is how failure handling is tested.  Errors: SKIM_EINVAL
  * (null context, ns = 0). */
 int skim_set_wait_limit_ns(skim_ctx *ctx, uint64_t ns);

@@ -507,7 +507,10 @@ cudaError_t launch_step(const StepArgs &a, cudaStream_t s) {
     const uint64_t work = std::max<uint64_t>(a.R, a.B - std::min(a.lo, a.B));
     const unsigned grid = std::min<unsigned>(grid_for(work, kStepThreads), static_cast<unsigned>(sms) * std::min(per, 1));
     note_launch();
-    void *args[] = {const_cast<StepArgs *>(&a)};
+    // between two barriers a warp walks a node's records 32 at a time, a thread the lanes in steps of the grid
+    StepArgs b = a;
+    b.timeout_ns = phase_limit(a.timeout_ns, 1 + a.R / 32 + work / kStepThreads);
+    void *args[] = {&b};
     return cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_step), dim3(grid), dim3(kStepThreads), args, 0, s);
 }
 cudaError_t launch_argmax_size(const uint32_t *size, uint32_t n, DevCtl *ctl, cudaStream_t s) {

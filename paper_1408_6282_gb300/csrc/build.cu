@@ -1299,6 +1299,8 @@ cudaError_t launch_need(const BuildNode &g, const uint64_t *next, uint64_t *need
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_need_sweep, kSweepThreads, 0);  // all blocks resident at once
     if (e != cudaSuccess) return e;
     const unsigned grid = std::min<unsigned>(grid_for(g.n, 64), static_cast<unsigned>(sms) * std::min(per, 1));
+    // between two barriers a warp walks a row 32 entries at a time, a thread the tasks in steps of the grid
+    timeout_ns = phase_limit(timeout_ns, 1 + g.n / 32 + static_cast<uint64_t>(g.n) * g.l / kSweepThreads);
     note_launch();
     void *args[] = {const_cast<BuildNode *>(&g), &need, &tasks, &wl0, &wl1, &task_cap, &ctl, &timeout_ns};
     return cudaLaunchCooperativeKernel(reinterpret_cast<void *>(k_need_sweep), dim3(grid), dim3(kSweepThreads), args, 0, s);

@@ -73,6 +73,14 @@ SKIM_DEV bool fmix_le(uint64_t z, uint64_t t) {
     z *= 0x94D049BB133111EBull;
     return (z ^ (z >> 31)) <= t;
 }
+// Wait limit of a phase that threads leave together and that makes progress in up to
+// `steps` steps one after the other: each may take the limit, the phase ten seconds.
+SKIM_HD uint64_t phase_limit(uint64_t ns, uint64_t steps) {
+    constexpr uint64_t most = 10000000000ull;
+    if (ns >= most) return ns;
+    const uint64_t all = ns * (steps < (1u << 29) ? steps : 1u << 29);
+    return all < ns ? ns : all < most ? all : most;
+}
 SKIM_HD bool coin_live(uint64_t he, uint32_t inst, uint64_t tm1) {
     return fmix(he + kGolden * static_cast<uint64_t>(inst + 1)) <= tm1;
 }

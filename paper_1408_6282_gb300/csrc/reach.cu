@@ -234,9 +234,9 @@ struct Reach {
 
 // Block i searches instance i, from node x (RES: the residual search of seed
 // x, or of the seed the step before it found, if any) or from the pivots of instance i
-// (blocks from l on: against the edges).  The wait of a level's barrier is bounded like every
-// other wait: a level that takes longer than the limit ends the search with
-// the error flag.
+// (blocks from l on: against the edges).  A level that makes no progress ends the search
+// with the error flag: each of its rows may take the wait limit (phase_limit; what the
+// block sweeps and erases together always ends).
 template <bool RES>
 __global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_t x, const uint32_t *pivot,
                                                             uint32_t starts, uint32_t *count) {
@@ -276,7 +276,10 @@ __global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_
     bool narrow = false;
     for (uint32_t t = 0;; t++) {
         uint32_t m = min(sh.n_rows[t % 3], kFrontCap + A.cap);
-        if (!RES && m == 0 && sh.parked) m = R.unpark(t);
+        if (!RES && m == 0 && sh.parked) {
+            m = R.unpark(t);
+            t_level = globaltimer();
+        }
         if (m == 0) break;
         if (!RES) {
             walked += m;
@@ -296,7 +299,7 @@ __global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_
         int late = 0;
         if (threadIdx.x == 0) {
             const uint64_t now = globaltimer();
-            late = now - t_level > A.timeout_ns;
+            late = now - t_level > phase_limit(A.timeout_ns, m);
             if (late) atomicOr(&A.ctl->err, kErrTimeout);
             t_level = now;
         }
@@ -307,6 +310,7 @@ __global__ void __launch_bounds__(kReachThreads, 1) k_reach(ReachArgs A, uint32_
             __syncthreads();
             if (threadIdx.x == 0) sh.n_long = 0;
             R.erase_all();
+            if (threadIdx.x == 0) t_level = globaltimer();
         }
     }
     __syncthreads();
