@@ -155,6 +155,7 @@ struct skim_ctx {
     uint64_t *qtab = nullptr;  // table of the largest queries (16 bytes per slot)
     uint64_t qtab_slots = 0;
     uint64_t refuse = 0;  // test hook: allocations until one is refused (0: none)
+    bool clusters = true;  // false, a test hook: launches of query clusters are refused
     // counters of the last build/greedy call
     uint64_t hstats[SKIM_STAT_COUNT] = {0};
     // kernel timing (CUDA events on the context stream)
@@ -1113,6 +1114,8 @@ int ensure_query_space(skim_ctx *c, uint64_t seeds, uint64_t q, uint64_t blocks,
 
 }  // namespace
 
+bool skim::query_clusters_of(const skim_ctx *c) { return c->clusters; }
+
 QueryTerms skim::query_terms_of(const skim_ctx *c) {
     if (c->rank_mode == SKIM_RANKS_PERMUTATION)
         return QueryTerms{1, static_cast<double>(c->nl - 1), static_cast<double>(c->l)};
@@ -1219,8 +1222,10 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
     c->batch_cfg = prm->batch_lanes;
     c->ring_rpl = kRingRecordsPerLane;
     c->node_density = static_cast<uint32_t>(kNodeSortDensity);
-    // SKIM_REFUSE_ALLOC in the environment (a test hook): that allocation of the
-    // context, counted from its creation, is refused
+    // Test hooks in the environment.  SKIM_REFUSE_ALLOC: that allocation of the
+    // context, counted from its creation, is refused; SKIM_REFUSE_CLUSTERS: so are
+    // launches of query clusters
+    c->clusters = getenv("SKIM_REFUSE_CLUSTERS") == nullptr;
     if (const char *ra = getenv("SKIM_REFUSE_ALLOC")) c->refuse = strtoull(ra, nullptr, 10);
     c->cm.model = prm->prob_model;
     c->cm.tm1_uniform = prm->prob_model == 0 ? tm1_of(prm->p) : 0;
@@ -2207,7 +2212,7 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
     double *dout = on_device ? est_out : c->qout;
     {
         KTimer kt(c, SKIM_K_QUERY);
-        QueryScratch qs{c->qpart, c->qdone, flag, c->qtab, c->qtab_slots};
+        QueryScratch qs{c->qpart, c->qdone, flag, c->qtab, c->qtab_slots, c->clusters};
         CK(c, launch_query_multi(c->X, c->xlen, c->n, c->k, query_terms_of(c), dseeds, d_off, d_boff, q, offsets,
                                  static_cast<uint32_t>(boff[q]), qs, dout, c->st));
     }
@@ -2231,13 +2236,16 @@ int skim_oracle_query(skim_ctx *c, const uint32_t *seeds, uint32_t n_seeds, doub
     }
     for (uint32_t i = 0; i < n_seeds; i++)
         if (seeds[i] >= c->n) return SKIM_EINVAL;
+    cudaError_t e = cudaSuccess;
     {
         KTimer kt(c, SKIM_K_QUERY);
-        CK(c, launch_query_one(c->X, c->xlen, c->n, c->k, query_terms_of(c), seeds, n_seeds, c->hq, c->st));
+        e = launch_query_one(c->X, c->xlen, c->n, c->k, query_terms_of(c), seeds, n_seeds, c->hq, c->clusters, c->st);
     }
-    CK(c, cudaStreamSynchronize(c->st));
-    resolve_timers(c);
-    if (*c->hq < 0) {  // a block's table was full
+    if (e == cudaSuccess) {
+        CK(c, cudaStreamSynchronize(c->st));
+        resolve_timers(c);
+    }
+    if (e != cudaSuccess || *c->hq < 0) {  // no cluster to be had, or a block's table was full
         uint64_t off[2] = {0, n_seeds};
         return skim_oracle_query_batch(c, off, 1, seeds, est_out, 0);
     }

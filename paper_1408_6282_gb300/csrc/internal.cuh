@@ -328,6 +328,7 @@ struct QueryScratch {
     unsigned *err;
     void *table;            // for the largest queries, 16 bytes per slot
     uint64_t table_slots;
+    bool clusters;          // may be launched (else every larger query is taken in parts)
 };
 uint32_t query_blocks(uint64_t seeds, uint32_t k);  // parts of a larger query, 0 for a small one and for the largest
 uint64_t query_table_slots(uint64_t seeds, uint32_t k);  // of the largest ones' table in global memory, else 0
@@ -345,6 +346,7 @@ struct QueryTerms {
     double div;
 };
 QueryTerms query_terms_of(const skim_ctx *c);
+bool query_clusters_of(const skim_ctx *c);
 cudaError_t launch_node_estimates(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, uint32_t l,
                                   int mode, double *out, cudaStream_t s);
 // block_off: prefix sums of query_blocks; blocks: their total; h_offsets: offsets, on the host
@@ -352,10 +354,11 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
                                const uint32_t *seeds, const uint64_t *offsets, const uint64_t *block_off, uint32_t q,
                                const uint64_t *h_offsets, uint32_t blocks, const QueryScratch &qs, double *out,
                                cudaStream_t s);
-// One query with few enough seeds (host) to be kernel arguments; out_host: pinned.
+// One query with few enough seeds (host) to be kernel arguments; out_host: pinned.  An
+// error: it takes a cluster, which the device refuses (or clusters is false); the batch form does without.
 constexpr uint32_t kQueryArgSeeds = 8000;
 bool query_fits_args(uint64_t seeds, uint32_t k);
 cudaError_t launch_query_one(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
-                             const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st);
+                             const uint32_t *seeds, uint32_t s, double *out_host, bool clusters, cudaStream_t st);
 
 }  // namespace skim

@@ -611,8 +611,11 @@ bool query_fits_args(uint64_t seeds, uint32_t k) {
 
 namespace {
 
+// An error: the device would not take clusters of this size (another program's
+// partition of it, for instance); nothing has been launched.
 template <uint32_t CL, class K, class... Args>
-cudaError_t cluster_launch(K kernel, unsigned clusters, uint32_t H, cudaStream_t st, const Args &...args) {
+cudaError_t cluster_launch(bool allowed, K kernel, unsigned clusters, uint32_t H, cudaStream_t st, const Args &...args) {
+    if (!allowed) return cudaErrorInvalidClusterSize;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (kClusterSlots + 1) * sizeof(ulonglong2));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -628,13 +631,15 @@ cudaError_t cluster_launch(K kernel, unsigned clusters, uint32_t H, cudaStream_t
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    note_launch();
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (e == cudaSuccess) note_launch();
+    else cudaGetLastError();
+    return e;
 }
 
 template <uint32_t CAP>
 cudaError_t one_launch(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
-                       const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st) {
+                       const uint32_t *seeds, uint32_t s, double *out_host, bool clusters, cudaStream_t st) {
     SeedArgs<CAP> a;
     a.s = s;
     std::copy(seeds, seeds + s, a.seeds);
@@ -648,17 +653,17 @@ cudaError_t one_launch(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint
     }
     if constexpr (CAP > 60) {
         const uint32_t H = cluster_slots<kCluster>(entries);
-        return cluster_launch<kCluster>(k_q_one_cluster<CAP>, 1, H, st, X, xlen, n, k, terms, a, H, out_host);
+        return cluster_launch<kCluster>(clusters, k_q_one_cluster<CAP>, 1, H, st, X, xlen, n, k, terms, a, H, out_host);
     }
     return cudaErrorInvalidValue;
 }
 }  // namespace
 
 cudaError_t launch_query_one(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
-                             const uint32_t *seeds, uint32_t s, double *out_host, cudaStream_t st) {
-    if (s <= 60 && s * (k - 1) <= kOneEntries) return one_launch<60>(X, xlen, n, k, terms, seeds, s, out_host, st);
-    return s <= 960 ? one_launch<960>(X, xlen, n, k, terms, seeds, s, out_host, st)
-                    : one_launch<kQueryArgSeeds>(X, xlen, n, k, terms, seeds, s, out_host, st);
+                             const uint32_t *seeds, uint32_t s, double *out_host, bool clusters, cudaStream_t st) {
+    if (s <= 60 && s * (k - 1) <= kOneEntries) return one_launch<60>(X, xlen, n, k, terms, seeds, s, out_host, clusters, st);
+    return s <= 960 ? one_launch<960>(X, xlen, n, k, terms, seeds, s, out_host, clusters, st)
+                    : one_launch<kQueryArgSeeds>(X, xlen, n, k, terms, seeds, s, out_host, clusters, st);
 }
 
 cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
@@ -702,10 +707,12 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
         const uint32_t cl = few ? kCluster : kClusterFour;
         f.ways = few ? std::max(1u, std::min(kClusterParts / f.n_large, (blocks * kPartEntries - 1) / kClusterEntries + 1)) : 1;
         const uint32_t clusters = f.n_large * f.ways + (q > f.n_large + tables ? (q + cl - 1) / cl : 0);
-        return few ? cluster_launch<kCluster>(k_q_few<kCluster>, clusters, kClusterSlots, s, X, xlen, n, k, terms, seeds,
-                                              offsets, f, partial, qs.done, out, qs.err)
-                   : cluster_launch<kClusterFour>(k_q_few<kClusterFour>, clusters, kClusterSlots, s, X, xlen, n, k, terms,
-                                                  seeds, offsets, f, partial, qs.done, out, qs.err);
+        const cudaError_t ce =
+            few ? cluster_launch<kCluster>(qs.clusters, k_q_few<kCluster>, clusters, kClusterSlots, s, X, xlen, n, k,
+                                           terms, seeds, offsets, f, partial, qs.done, out, qs.err)
+                : cluster_launch<kClusterFour>(qs.clusters, k_q_few<kClusterFour>, clusters, kClusterSlots, s, X, xlen, n,
+                                               k, terms, seeds, offsets, f, partial, qs.done, out, qs.err);
+        if (ce == cudaSuccess) return ce;  // (refused: parts need no clusters)
     }
     if (e == cudaSuccess && blocks) {
         const int smem = (kPartSlots + 1 + kPartThreads / 32 * kStage) * sizeof(ulonglong2);

@@ -78,6 +78,7 @@ struct skim_server {
     const uint32_t *xlen = nullptr;
     uint32_t n = 0, k = 0, l = 0;
     QueryTerms terms{0, 0.0, 1.0};
+    bool clusters = true;
     uint32_t max_inflight = 0;
     std::vector<Lane> lanes;
     std::mutex mu;
@@ -183,7 +184,7 @@ bool admit(skim_server *s, std::unique_lock<std::mutex> &lock) {
     std::copy(ln->boff.begin(), ln->boff.end(), ln->h_meta + g1);
     ok &= cudaMemcpyAsync(ln->d_meta, ln->h_meta, 2 * g1 * sizeof(uint64_t), cudaMemcpyHostToDevice, ln->st) ==
           cudaSuccess;
-    QueryScratch qs{ln->d_part, ln->d_done, ln->d_err, ln->d_table, ln->d_table ? ln->arena_slots : 0};
+    QueryScratch qs{ln->d_part, ln->d_done, ln->d_err, ln->d_table, ln->d_table ? ln->arena_slots : 0, s->clusters};
     ok &= launch_query_multi(s->X, s->xlen, s->n, s->k, s->terms, ln->d_seeds, ln->d_meta, ln->d_meta + g1, cnt, ln->h_meta,
                              static_cast<uint32_t>(ln->boff.back()), qs, ln->d_out, ln->st) == cudaSuccess;
     ok &= cudaMemcpyAsync(ln->h_out, ln->d_out, cnt * sizeof(double), cudaMemcpyDeviceToHost, ln->st) == cudaSuccess;
@@ -258,6 +259,7 @@ int skim_server_start(skim_ctx *ctx, uint32_t max_inflight, uint64_t scratch_slo
     s->k = k;
     s->l = l;
     s->terms = query_terms_of(ctx);
+    s->clusters = query_clusters_of(ctx);
     s->max_inflight = max_inflight;
     s->lanes.resize(streams);
     const uint64_t arena = std::max<uint64_t>(scratch_slots / streams, 64);

@@ -51,3 +51,27 @@ def test_calls_with_some_larger_queries(large, k, seeds):
         want = [sk.query(s) for s in sets]
         for _ in range(2):
             assert np.array_equal(sk.query_batch(sets), want)
+
+
+@pytest.mark.parametrize("k", [16, 64])
+def test_without_clusters(monkeypatch, k):
+    """A device that refuses clusters (SKIM_REFUSE_CLUSTERS): parts answer every query that
+    would have taken one, alone, in a batch and served, with the same bits."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.erdos_renyi(3001, 15000, 53)
+    rng = np.random.default_rng(k)
+    sets = [rng.choice(g.n, s, replace=False).astype(np.uint32) for s in (0, 5, 95, 110, 200, 700, 1000, 3000)]
+    sets.append(np.tile(sets[-1], 2))
+    got = []
+    for refuse in (False, True):
+        if refuse:
+            monkeypatch.setenv("SKIM_REFUSE_CLUSTERS", "1")
+        with pkg.Skim(g.n, g.src, g.dst, 16, k, 0, 0.15, 3, 4, 5) as sk:
+            sk.build_sketches()
+            alone = [sk.query(s) for s in sets]
+            few = [sk.query_batch(sets[i:i + 2]) for i in range(len(sets) - 1)]
+            with sk.server(max_inflight=8, scratch_slots=1 << 21, streams=2) as srv:
+                served = [srv.wait(t, 60000) for t in [srv.submit(s) for s in sets]]
+            assert served == alone and all(np.array_equal(f, alone[i:i + 2]) for i, f in enumerate(few))
+            got.append(alone)
+    assert got[0] == got[1]
