@@ -152,7 +152,20 @@ SKIM_DEV double fixed_to_double(const U192 &a) {
 // kOneEntries (100 seeds of 16 ranks: 28 us both; 43 seeds of 64: 30 and 29 us).
 
 constexpr uint32_t kSmallEntries = 2700, kSmallSlots = 4095;  // 64 KB: three blocks per SM
-constexpr int kSmallThreads = 256;
+// Threads of a small query's block: many while a call leaves room for them (host to host,
+// 64 ranks per sketch, 1 to 42 seeds; 256, 512, 1024 threads: 10 queries 66, 57, 53 us, 152
+// 69, 68, 62, 304 71, 71, 82, 608 91, 97, 114, 2000 174, 196, 273).
+constexpr uint32_t kSmsUsual = 152;
+constexpr int small_threads(uint32_t queries) {
+    return queries <= kSmsUsual ? 1024 : queries <= 3 * kSmsUsual ? 512 : 256;
+}
+// Small queries go in one launch with the clusters of a few larger ones, in a block of
+// 1024 threads each and one per SM, while they are few: with clusters of 4 up to
+// kFewSmall, with clusters of 16, of which 8 are resident at once, up to kFewClusters of
+// them in all.  Else they take a launch of their own (as above, beside one larger query
+// 152, 304, 608, 2000 small ones: 81, 108, 174, 438 us together, 96, 111, 116, 208 us
+// apart; 152 beside 6: 97 and 89 us).
+constexpr uint32_t kFewSmall = 2 * kSmsUsual, kFewClusters = 14;
 constexpr uint32_t kPartEntries = 8000, kPartSlots = 12287;  // 192 KB
 constexpr int kPartThreads = 1024;
 constexpr uint32_t kStage = 64;  // pairs a warp collects
@@ -442,9 +455,9 @@ __global__ void __launch_bounds__(1024)
 }
 
 // Block q: query q, if it is small.
-__global__ void __launch_bounds__(kSmallThreads) k_q_small(const uint64_t *X, const uint32_t *xlen, uint32_t n,
-                                                           uint32_t k, QueryTerms terms, const uint32_t *seeds,
-                                                           const uint64_t *offsets, double *out, unsigned *err) {
+__global__ void __launch_bounds__(1024) k_q_small(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k,
+                                                  QueryTerms terms, const uint32_t *seeds, const uint64_t *offsets,
+                                                  double *out, unsigned *err) {
     extern __shared__ ulonglong2 s_tab[];
     const uint32_t q = blockIdx.x;
     const uint64_t s0 = offsets[q];
@@ -706,13 +719,17 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
         const bool few = f.n_large <= kFewLarge || !fits_four;
         const uint32_t cl = few ? kCluster : kClusterFour;
         f.ways = few ? std::max(1u, std::min(kClusterParts / f.n_large, (blocks * kPartEntries - 1) / kClusterEntries + 1)) : 1;
-        const uint32_t clusters = f.n_large * f.ways + (q > f.n_large + tables ? (q + cl - 1) / cl : 0);
+        const uint32_t small = q - f.n_large - tables;
+        const uint32_t with_small = f.n_large * f.ways + (q + cl - 1) / cl;
+        const bool together = small == 0 || (small <= kFewSmall && (!few || with_small <= kFewClusters));
+        const uint32_t clusters = small && together ? with_small : f.n_large * f.ways;
         const cudaError_t ce =
             few ? cluster_launch<kCluster>(qs.clusters, k_q_few<kCluster>, clusters, kClusterSlots, s, X, xlen, n, k,
                                            terms, seeds, offsets, f, partial, qs.done, out, qs.err)
                 : cluster_launch<kClusterFour>(qs.clusters, k_q_few<kClusterFour>, clusters, kClusterSlots, s, X, xlen, n,
                                                k, terms, seeds, offsets, f, partial, qs.done, out, qs.err);
-        if (ce == cudaSuccess) return ce;  // (refused: parts need no clusters)
+        if (ce == cudaSuccess && together) return ce;
+        if (ce == cudaSuccess) blocks = 0;  // (refused: parts need no clusters)
     }
     if (e == cudaSuccess && blocks) {
         const int smem = (kPartSlots + 1 + kPartThreads / 32 * kStage) * sizeof(ulonglong2);
@@ -728,7 +745,7 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
         e = cudaFuncSetAttribute(k_q_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         note_launch();
-        k_q_small<<<q, kSmallThreads, smem, s>>>(X, xlen, n, k, terms, seeds, offsets, out, qs.err);
+        k_q_small<<<q, small_threads(q), smem, s>>>(X, xlen, n, k, terms, seeds, offsets, out, qs.err);
         e = cudaGetLastError();
     }
     return e;

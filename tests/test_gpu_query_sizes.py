@@ -75,3 +75,24 @@ def test_without_clusters(monkeypatch, k):
             assert served == alone and all(np.array_equal(f, alone[i:i + 2]) for i, f in enumerate(few))
             got.append(alone)
     assert got[0] == got[1]
+
+
+@pytest.mark.parametrize("large,small,launches", [(0, 152, 1), (0, 153, 1), (0, 456, 1), (0, 457, 1), (1, 207, 1),
+                                                  (1, 208, 2), (8, 88, 1), (8, 89, 2), (20, 304, 1), (20, 305, 2),
+                                                  (70, 300, 2), (1, 5000, 2)])
+def test_calls_with_many_small_queries(large, small, launches):
+    """Blocks of 1024, 512 and 256 threads for small queries; beside larger ones in their
+    launch while they are few, else in one of their own."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.erdos_renyi(3001, 15000, 59)
+    rng = np.random.default_rng(large + small)
+    sets = [rng.choice(g.n, 70 if i < large else rng.integers(0, 43), replace=False).astype(np.uint32)
+            for i in range(large + small)]
+    sets = [sets[i] for i in rng.permutation(len(sets))]
+    with pkg.Skim(g.n, g.src, g.dst, 16, 64, 0, 0.15, 3, 4, 5) as sk:
+        sk.build_sketches()
+        want = [sk.query(s) for s in sets]
+        sk.query_batch(sets)
+        before = pkg.skim_kernel_launches()
+        assert np.array_equal(sk.query_batch(sets), want)
+        assert pkg.skim_kernel_launches() - before == launches
