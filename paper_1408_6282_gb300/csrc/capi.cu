@@ -703,10 +703,12 @@ uint32_t default_lanes(skim_ctx *c) {
 }
 
 // Lanes of a SKIM batch when the caller sets none.  A batch is sized by its
-// visits (next_seed), and most lanes of a sparse one are leaf lanes: 50 seeds of
-// R-MAT 20 p = 0.01 take 20, 19, 17.8, 17.0 ms with at most 2, 4, 8, 16 M.
+// visits (next_seed), and over stored rows most lanes of a sparse one are leaf lanes: 50
+// seeds of R-MAT 20 p = 0.01 take 20, 19, 17.8, 17.0 ms with at most 2, 4, 8, 16 M.  With
+// coins every lane is a table entry and a record: 50 seeds of R-MAT 18 p = 0.01 27.1 ms
+// with at most 16 M, 24.8 with 2 M, 30 of R-MAT 17 trivalency 17.9 and 15.7.
 uint32_t skim_lanes(skim_ctx *c) {
-    return c->batch_cfg ? default_lanes(c) : static_cast<uint32_t>(std::min<uint64_t>(1ull << 24, c->lane_cap));
+    return c->batch_cfg || !c->mat ? default_lanes(c) : static_cast<uint32_t>(std::min<uint64_t>(1ull << 24, c->lane_cap));
 }
 
 // ---- SKIM steps ------------------------------------------------------------

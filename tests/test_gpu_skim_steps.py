@@ -104,3 +104,17 @@ def test_builds_between_seeds_lose_no_stop(name, l, k, p, bl):
             sk.build_sketches()
         for q, want in enumerate((seeds, cov, tau, kp)):
             assert np.array_equal(np.concatenate([x[q] for x in got]), want)
+
+
+def test_coin_batches_keep_to_their_lanes():
+    """With coins drawn in the searches no batch has more than 2M lanes (over stored rows
+    16M, where most have no record); ranks that run out."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.empty_graph(300_000)
+    with pkg.Skim(g.n, g.src, g.dst, 64, 255, 0, 0.1, 1, 2, 3) as sk:
+        for rows, most in ((True, 1 << 24), (False, 1 << 21)):
+            sk.set_live_rows(rows)
+            seeds, cov = sk.greedy(3)
+            assert seeds.tolist() == [0, 1, 2] and cov.tolist() == [64] * 3
+            st = sk.stats()
+            assert st["ranks"] == 64 * g.n and st["batches"] >= -(-st["ranks"] // most)
