@@ -88,7 +88,8 @@ struct skim_ctx {
     uint64_t *alive = nullptr, *leaf = nullptr, *lane_off = nullptr;
     uint32_t *lane_fill = nullptr;
     uint32_t lane_cap = 0;
-    int grid_rev = 0, grid_coin = 0, grid_fwd = 0, grid_ring = 0;
+    int grid_rev = 0, grid_coin[2] = {0, 0}, grid_fwd = 0, grid_ring = 0;  // grid_coin: few visits, many
+    double coin_vpl = 0;  // visits per lane of the last batch with coins (0: unknown)
     uint64_t timeout_ns = 2000000000ull;
     // sketches
     uint8_t *lcnt = nullptr;
@@ -423,7 +424,7 @@ int run_traversal(skim_ctx *c, TravArgs &a, bool forward, uint64_t *R_out, const
                 CK(c, launch_rev_ring(a, rs->lane_pair, rs->B, c->l, rs->covered, rs->alive, rs->leaf, first,
                                       c->grid_ring, c->st));
             else
-                CK(c, launch_traverse(a, forward, forward ? c->grid_fwd : c->mat ? c->grid_rev : c->grid_coin, c->st));
+                CK(c, launch_traverse(a, forward, forward ? c->grid_fwd : c->mat ? c->grid_rev : c->grid_coin[a.many], c->st));
         }
         if (rs && rs->leaf) {
             KTimer kt(c, SKIM_K_SOURCES);
@@ -481,6 +482,8 @@ constexpr double kRingRecordsPerLane = SKIM_RING_RECORDS_PER_LANE;
 // batches of at most this many lane words place a node's visited-table
 // entries side by side (traverse.cu: table_slot)
 constexpr uint32_t kNodeHashWords = SKIM_NODE_HASH_WORDS;
+// visits from which a batch with coins fills the chip (traverse.cu: kCoinBlocksMany)
+constexpr double kCoinMany = 1 << 20;
 
 // Residual searches over materialised rows run as one block per instance
 // (reach.cu) except where few instances are large: a block then walks alone
@@ -550,6 +553,8 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
     a.prune = mode_build && c->rank_mode != SKIM_RANKS_IC_MODEL ? 1 : 0;
     if (mode_build && !a.prune) a.xlen = c->xlen;
     a.k = c->k;
+    a.many = !c->mat && c->coin_vpl * B >= kCoinMany ? 1 : 0;
+    const uint64_t v0 = c->hctl->stats[kStRevVisits];
     uint64_t R = 0;
     // SKIM_TRACE_BATCHES=1 in the environment: one line per batch on stderr
     // (search kernel, lanes, records, visits, device time of its searches and
@@ -606,6 +611,7 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
         return SKIM_OK;
     }
     RC(reset_queue(c, h.q_tail.v));
+    if (!c->mat) c->coin_vpl = static_cast<double>(h.stats[kStRevVisits] - v0) / B;
     if (!mode_build) {  // SKIM: the batch's commits add at most its visit bits to the index
         const uint64_t vis = h.stats[kStRevVisits] - c->vis_seen;
         c->vis_seen = h.stats[kStRevVisits];
@@ -741,6 +747,7 @@ int skim_state_init(skim_ctx *c) {
     c->last_gap = 0;
     c->vpl_est = 0;
     c->last_B = 0;
+    c->coin_vpl = 0;
     c->refilter = false;
     c->sk_init = true;
     return SKIM_OK;
@@ -1374,7 +1381,7 @@ int skim_create(const skim_graph *g, const skim_params *prm, void *stream, skim_
         TRY(dalloc(c, &c->lane_off, c->lane_cap));
         TRY(dalloc(c, &c->lane_fill, c->lane_cap));
         c->grid_rev = traverse_grid(false, true);
-        c->grid_coin = traverse_grid(false, false, c->rank_mode == SKIM_RANKS_IC_MODEL);
+        for (int many = 0; many < 2; many++) c->grid_coin[many] = traverse_grid(false, false, many != 0);
         c->grid_ring = rev_ring_grid();
         c->grid_fwd = traverse_grid(true, true);
         TRYC(cudaStreamSynchronize(c->st));
@@ -1974,6 +1981,7 @@ int build_coins(skim_ctx *c) {
     uint32_t B = std::min<uint32_t>(Bmax, kBuildFirst);
     uint64_t p0 = 0;
     double rpl = 0;  // table entries per lane of the last batch (0: unknown)
+    c->coin_vpl = 0;
     while (p0 < c->nbuild) {
         uint32_t b = static_cast<uint32_t>(std::min<uint64_t>(B, c->nbuild - p0));
         bool retry = false;

@@ -74,6 +74,7 @@ struct TravArgs {
     uint32_t *cnt;              // SKIM: per node, the batch's visits (null: not counted)
     const uint32_t *xlen;       // Algorithm 2 in the IC model: ranks of every sketch before the batch, of at most k
     uint32_t k;
+    int many;                   // coins drawn in the search: the batch is expected to fill the chip
 };
 
 // graph.cu
@@ -149,7 +150,7 @@ cudaError_t launch_traverse(const TravArgs &a, bool forward, int grid, cudaStrea
 // reverse searches find it by their table slots.
 cudaError_t launch_respill_rev(const TravArgs &a, cudaStream_t s);
 cudaError_t launch_respill_fwd(const TravArgs &a, uint32_t n, cudaStream_t s);
-int traverse_grid(bool forward, bool mat, bool ic = false);  // resident blocks for the persistent traversal
+int traverse_grid(bool forward, bool mat, bool many = false);  // resident blocks for the persistent traversal
 // Reverse searches over materialised live rows with per-warp queues in shared
 // memory (Algorithms 1 and 2): the batch's source lanes are taken by the
 // kernel itself (sources = false: an earlier launch took them; covered/alive

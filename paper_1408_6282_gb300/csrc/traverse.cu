@@ -801,11 +801,13 @@ SKIM_DEV Desc shfl_desc(const Desc &d, int src) {
 #ifndef SKIM_TRAV_MIN_BLOCKS
 #define SKIM_TRAV_MIN_BLOCKS 3
 #endif
-// Blocks per SM of a search that draws coins: four in the IC model, whose batches
-// fill the chip (R-MAT 15: 84 ms, three 91 ms), three else, where a small graph's search is
-// a chain of hops and spilled registers and idle warps cost (R-MAT 12, p = 0.01, l = 16: 0.80 and
-// 0.95 ms, R-MAT 14 1.87 and 2.14 ms; R-MAT 17 wc, l = 64: 26.0 and 25.7 ms).
-constexpr int kCoinBlocks = 3, kCoinBlocksIc = 4;
+// Blocks per SM of a search that draws coins: four where its batch fills the chip, two
+// where it is a chain of hops and spilled registers and idle warps that poll cost more
+// than they bring.  One batch each with 2, 3, 4 blocks: 10 K visits (R-MAT 13, p = 0.01)
+// 0.20, 0.23, 0.29 ms; 68 K (R-MAT 13 wc) 0.28, 0.33, 0.40; 0.35 M 0.32, 0.39, 0.39; 1.3 M (R-MAT
+// 14 wc, IC model) 1.04, 1.01, 1.07; 2 M (R-MAT 15, p = 0.01, IC model) 1.45, 1.31, 1.38; 8.8 M 5.0, 4.1,
+// 3.8; 21 M (R-MAT 17 trivalency) 23.7, 17.2, 14.8.
+constexpr int kCoinBlocksFew = 2, kCoinBlocksMany = 4;
 
 // Residual searches: the instances in which CSR edge idx to x is live, of item
 // d's (with materialised instances rows hold live edges only).
@@ -1450,7 +1452,7 @@ constexpr unsigned long long kDoneBatch = 64;
 // materialised rows keep items in the block's ring (FwdRing) while it has
 // room; a warp takes ring items into its lanes that hold no queue item.
 struct NoRing {};
-template <bool FWD, bool MAT, int BLOCKS = FWD ? 1 : MAT ? SKIM_TRAV_MIN_BLOCKS : kCoinBlocks>
+template <bool FWD, bool MAT, int BLOCKS = FWD ? 1 : MAT ? SKIM_TRAV_MIN_BLOCKS : kCoinBlocksFew>
 __global__ void __launch_bounds__(kTravThreads, BLOCKS)
     k_traverse(const __grid_constant__ TravArgs A) {
     constexpr bool kStaged = !FWD && MAT;
@@ -1653,7 +1655,7 @@ __global__ void __launch_bounds__(kTravThreads, BLOCKS)
 // occupies SMs at the same time (another stream of this process, another
 // context) can break it the same way.  The reverse searches over materialised
 // rows (k_rev_ring) have no such requirement.
-int traverse_grid(bool forward, bool mat, bool ic) {
+int traverse_grid(bool forward, bool mat, bool many) {
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1662,7 +1664,7 @@ int traverse_grid(bool forward, bool mat, bool ic) {
     // fill the machine: as many blocks as fit.
     if (forward) return sms;
     if (mat) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, true>, kTravThreads, 0);
-    else if (ic) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, false, kCoinBlocksIc>, kTravThreads, 0);
+    else if (many) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, false, kCoinBlocksMany>, kTravThreads, 0);
     else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_traverse<false, false>, kTravThreads, 0);
     if (per < 1) per = 1;
     return sms * per;
@@ -1697,7 +1699,7 @@ cudaError_t launch_traverse(const TravArgs &a, bool forward, int grid, cudaStrea
         if (a.mat)
             k_traverse<false, true><<<grid, kTravThreads, 0, s>>>(a);
         else
-            a.xlen ? k_traverse<false, false, kCoinBlocksIc><<<grid, kTravThreads, 0, s>>>(a)
+            a.many ? k_traverse<false, false, kCoinBlocksMany><<<grid, kTravThreads, 0, s>>>(a)
                    : k_traverse<false, false><<<grid, kTravThreads, 0, s>>>(a);
     }
     return cudaGetLastError();

@@ -43,3 +43,27 @@ def test_row_sizes(model, p, mode, l, bl):
             sk.build_sketches()
             x, ln = sk.sketches()
             assert np.array_equal(ln, oln) and np.array_equal(x, ox)
+
+
+@pytest.mark.parametrize("p", [0.01, 0.3])
+@pytest.mark.parametrize("mode,l", [(2, 1), (0, 64), (1, 64)])
+def test_batches_of_few_and_many_visits(p, mode, l):
+    """Batches expected to make fewer and more than 2^20 visits take different launches."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.rmat(11, 16, 21)
+    ks = synth.Keys.from_seed(18)
+    k = 40
+    pb = oracle.Problem(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
+    ox, oln, _ = oracle.build_ic_sketches(pb) if mode == 2 else oracle.build_sketches(pb, rank_mode=mode)
+    with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, rank_mode=mode) as sk:
+        sk.set_live_rows(False)
+        for _ in range(2):
+            sk.build_sketches()
+            x, ln = sk.sketches()
+            assert np.array_equal(ln, oln) and np.array_equal(x, ox)
+        if p == 0.3:
+            assert sk.stats()["rev_visits"] > 20 * 2**20 or mode != 2
+        if mode != 2:
+            want = oracle.skim_stops(pb, 15, rank_mode=mode)
+            for a, b in zip(sk.greedy_stops(15), want):
+                assert np.array_equal(a, b)
