@@ -1649,6 +1649,8 @@ constexpr uint32_t kRowsLanes = SKIM_ROWS_LANES;    // lanes of a batch unless t
 // They are far apart: 11-22 on weighted cascades (R-MAT 18 to 20) and near-critical
 // Erdos-Renyi graphs, hundreds to tens of thousands above the threshold.
 constexpr double kGiantMean = 64.0;
+// and visits that the remaining lanes would make like them: what contraction costs
+constexpr double kGiantVisitsLeft = 1 << 20;
 
 int rows_buffers(skim_ctx *c) {
     if (c->need) return SKIM_OK;
@@ -1924,7 +1926,17 @@ int build_rows(skim_ctx *c) {
                 CK(c, launch_hits(g, c->hitbits, a.pair, ranks, b, a.lbits, c->rkey, cs.hits, hs, c->ctl, c->st));
             }
         }
-        if (p0 == 0 && static_cast<double>(v2 - v0) >= kGiantMean * b) {
+        // Contraction is left out where its cost is not in what remains (kGiantVisitsLeft),
+        // and where few instances and small k let the first batch give the visited nodes
+        // all the ranks that they can use: about k of every instance where they are
+        // reached in one, k in all where they are reached in every one (R counts a node
+        // once per word of 64 lanes).  Whole builds of one instance with and without: R-MAT 10,
+        // p = 0.1, k = 16 0.37 and 0.27 ms (0.27 with searches pruned per instance), R-MAT 12
+        // trivalency 0.41 and 0.29 (0.29).
+        const double seen = static_cast<double>(v2 - v0);
+        const bool closed = kBuildFirst >= 2ull * c->k * c->l &&
+                            2.0 * seen * ((b + 63) / 64) >= static_cast<double>(R) * c->k * (c->l + 1.0);
+        if (p0 == 0 && seen >= kGiantMean * b && (c->nbuild - b) * (seen / b) >= kGiantVisitsLeft && !closed) {
             RC(contract_components(c, g, &cs, &giant));
             if (giant) {
                 a.scc = g.scc = c->comp;

@@ -128,3 +128,11 @@ def test_components_of_more_graphs_than_a_grid_dimension():
         y, lm = sk.sketches()
         assert np.array_equal(ln, lm) and np.array_equal(x, y)
         assert np.all(ln == 3)
+
+
+@pytest.mark.parametrize("l,k,p", [(1, 16, 0.1), (1, 64, 0.3), (4, 16, 0.1), (4, 32, 0.1), (2, 64, 0.05)])
+def test_few_instances(l, k, p):
+    """Where the first batch gives components all their ranks, and where it does not."""
+    for scale in (10, 13):
+        g = synth.rmat(scale, 16, 3)
+        _check(g.n, g.src, g.dst, l, k, 0, p)
