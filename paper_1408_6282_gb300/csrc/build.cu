@@ -421,6 +421,21 @@ __global__ void k_append_words(const uint64_t *__restrict__ rec, const uint32_t 
     }
 }
 
+// Lanes of the records of each chunk.
+__global__ void __launch_bounds__(kWordChunk) k_count_words(const uint32_t *__restrict__ rec_val, uint64_t R,
+                                                            const uint64_t *__restrict__ hvals, uint32_t *cnt) {
+    __shared__ uint32_t s_n;
+    for (uint64_t q = blockIdx.x; q * kWordChunk < R; q += gridDim.x) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const uint64_t r = q * kWordChunk + threadIdx.x;
+        const uint32_t n = __reduce_add_sync(kFull, r < R ? __popcll(hvals[2ull * rec_val[r]]) : 0);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&s_n, n);
+        __syncthreads();
+        if (threadIdx.x == 0) cnt[q] = s_n;
+    }
+}
+
 // space of each listed node's overflow
 __global__ void k_over_alloc(const uint32_t *list, const uint32_t *len, uint32_t k, uint32_t *seg, DevCtl *ctl) {
     const uint32_t n = ctl->b.n_list;
@@ -1248,6 +1263,12 @@ cudaError_t launch_append(const uint64_t *rec, uint64_t r0, uint64_t r1, uint32_
     note_launch();
     k_append<<<grid_for(r1 - r0, 256), 256, 0, s>>>(rec, r0, r1, lbits, defbits, lane_rank, k, len, X, b.over_key,
                                                     b.over_pos, b.list, ctl, nullptr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_count_words(const uint32_t *rec_val, uint64_t R, const uint64_t *hvals, uint32_t *cnt, cudaStream_t s) {
+    note_launch();
+    k_count_words<<<grid_for(R, kWordChunk, 152 * 4), kWordChunk, 0, s>>>(rec_val, R, hvals, cnt);
     return cudaGetLastError();
 }
 

@@ -1644,6 +1644,8 @@ constexpr double kRowsCheap = SKIM_ROWS_CHEAP;      // visits that a batch may m
 #ifndef SKIM_ROWS_LAST
 #define SKIM_ROWS_LAST 0.5
 #endif
+// Visits per table entry of a batch from which the next one too has a record per entry.
+constexpr double kRowsDense = 4.0;
 constexpr uint32_t kRowsLanes = SKIM_ROWS_LANES;    // lanes of a batch unless the caller says otherwise
 // Visits per lane of the first batch from which components are contracted.
 // They are far apart: 11-22 on weighted cascades (R-MAT 18 to 20) and near-critical
@@ -1807,6 +1809,33 @@ int search_deferred(skim_ctx *c, uint64_t p0, uint32_t D, uint64_t R0, const Bui
     }
 }
 
+// Ends of the parts in which R records per table entry are appended: those of a part
+// have at most rcap lanes, all of which may overflow their rows.  visits: lanes of all of
+// them.
+int word_parts(skim_ctx *c, uint64_t R, uint64_t visits, std::vector<uint64_t> *ends) {
+    uint64_t part = R;
+    if (visits > c->rcap) {
+        part = std::max<uint64_t>(1, c->rcap / 64);
+        if (part >= kWordChunk) {  // by count, in chunks of records
+            std::vector<uint32_t> cnt((R + kWordChunk - 1) / kWordChunk);
+            CK(c, launch_count_words(c->rval, R, c->hvals, c->rval2, c->st));
+            CK(c, cudaMemcpyAsync(cnt.data(), c->rval2, cnt.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->st));
+            CK(c, cudaStreamSynchronize(c->st));
+            uint64_t sum = 0;
+            for (uint64_t q = 0; q < cnt.size(); q++) {
+                if (sum + cnt[q] > c->rcap) {
+                    ends->push_back(q * kWordChunk);
+                    sum = 0;
+                }
+                sum += cnt[q];
+            }
+            part = R;
+        }
+    }
+    for (uint64_t r = ends->empty() ? 0 : ends->back(); r < R; r += part) ends->push_back(std::min(R, r + part));
+    return SKIM_OK;
+}
+
 int build_rows(skim_ctx *c) {
     RC(rows_buffers(c));
     const bool own_rec = c->rank_mode != SKIM_RANKS_UNIFORM;  // positions: not recomputable from the pair
@@ -1852,6 +1881,7 @@ int build_rows(skim_ctx *c) {
     double per = 1e9;  // visits per lane of the last batch
     double vpl = 0, vpl_def = 0;  // visits per lane of the last batch searched whole, of the last deferred lanes
     bool giant = false;
+    bool dense = false;  // the next batch too has a record per table entry
     bool force = false;  // after an overflow: a global table with a record per entry, which needs the least room
     while (p0 < c->nbuild) {
         const uint32_t b = static_cast<uint32_t>(std::min<uint64_t>(B, c->nbuild - p0));
@@ -1868,7 +1898,7 @@ int build_rows(skim_ctx *c) {
         uint64_t R0 = 0, v1 = v0;
         uint32_t D = b;
         const bool direct = force || (b <= kRowsDirect && per >= kRowsDirectVisits);
-        const bool words = force || (direct && p0 == 0);
+        const bool words = force || (direct && (p0 == 0 || dense));
         if (!direct) {
             {
                 KTimer kt(c, SKIM_K_REV);
@@ -1907,15 +1937,14 @@ int build_rows(skim_ctx *c) {
             CK(c, launch_append(c->rkey, 0, R0, a.lbits, D ? c->defbits : nullptr, ranks, c->k, c->xlen, c->X, sc,
                                 c->ctl, c->st));
             if (words) {
-                // a record appends at most k ranks, and a part of the records
-                // as many as there is room for should all of them overflow
-                const uint64_t part = std::max<uint64_t>(1, c->rcap / std::min(c->k, 64u));
-                for (uint64_t r = 0; r < R; r += part) {
-                    const uint64_t m = std::min(part, R - r);
+                std::vector<uint64_t> ends;
+                RC(word_parts(c, R, v2 - v0, &ends));
+                for (uint64_t r = 0, i = 0; i < ends.size(); r = ends[i++]) {
+                    const uint64_t m = ends[i] - r;
                     if (r) CK(c, cudaMemsetAsync(&c->ctl->b.n_over, 0, 3 * sizeof(unsigned), c->st));
                     CK(c, launch_append_words(c->rkey + r, c->rval + r, m, bitlen((b + 63) / 64 - 1), c->hvals, a.pair,
                                               c->l, a.own, a.lbits, ranks, c->k, c->xlen, c->X, sc, c->ctl, c->st));
-                    CK(c, launch_overflow(m, a.lbits, ranks, c->k, c->xlen, c->X, R <= part, sc, c->ctl, c->st));
+                    CK(c, launch_overflow(m, a.lbits, ranks, c->k, c->xlen, c->X, ends.size() == 1, sc, c->ctl, c->st));
                 }
             } else {
                 CK(c, launch_append(c->rkey, R0, R, a.lbits, nullptr, ranks, c->k, c->xlen, c->X, sc, c->ctl, c->st));
@@ -1960,6 +1989,16 @@ int build_rows(skim_ctx *c) {
         per = static_cast<double>(std::max<uint64_t>(v2 - v0, 1)) / b;
         uint64_t next = kRowsGrowth * static_cast<uint64_t>(b);
         if (per >= kRowsDirectVisits && !(giant && p0 == b)) next = std::max(next, static_cast<uint64_t>(kRowsCheap / per));
+        // Where a record per visit would keep the next batch small, and the last one had
+        // several visits per table entry, it has a record per entry as well, and of those
+        // at most n for every 64 lanes.  (Not behind a contraction if an instance need not
+        // give a node several ranks or the visited nodes have k already: few searches are
+        // left then.)  Erdos-Renyi 5003, p = 0.15, l = 16, k = 128: 3.2 and 2.0 ms (2.2 with
+        // searches pruned per instance), R-MAT 12, p = 0.1, l = 1, k = 16 0.38 and 0.32 (0.31).
+        dense = words && seen >= kRowsDense * static_cast<double>(R) &&
+                fit < std::min<uint64_t>({bmax, next, c->nbuild - p0}) &&
+                !(giant && (c->k < 4 * c->l || seen * ((b + 63) / 64) >= static_cast<double>(R) * c->k));
+        if (dense) fit = std::max(static_cast<uint64_t>(c->rcap / 4.0 / recs), c->rcap / c->n * 64);
         B = std::max<uint64_t>(64, std::min<uint64_t>({bmax, next, fit}));
         since += v2 - v0;
         if (p0 < c->nbuild && ((static_cast<double>(p0) < SKIM_ROWS_LAST * static_cast<double>(c->nbuild) &&

@@ -247,6 +247,9 @@ cudaError_t launch_append(const uint64_t *rec, uint64_t r0, uint64_t r1, uint32_
 // records node << tbits | word of a search of all lanes of a batch (slots
 // rec_val, lane bits hvals): the ranks of each one's lanes, without the node's
 // own unless `own`
+// Lanes of every kWordChunk of R such records, to cnt.
+constexpr uint32_t kWordChunk = 1024;
+cudaError_t launch_count_words(const uint32_t *rec_val, uint64_t R, const uint64_t *hvals, uint32_t *cnt, cudaStream_t s);
 cudaError_t launch_append_words(const uint64_t *rec, const uint32_t *rec_val, uint64_t R, uint32_t tbits,
                                 const uint64_t *hvals, const uint32_t *pair, uint32_t l, int own, uint32_t lbits, const uint64_t *lane_rank, uint32_t k, uint32_t *len,
                                 uint64_t *X, const BuildScratch &b, DevCtl *ctl, cudaStream_t s);

@@ -136,3 +136,15 @@ def test_few_instances(l, k, p):
     for scale in (10, 13):
         g = synth.rmat(scale, 16, 3)
         _check(g.n, g.src, g.dst, l, k, 0, p)
+
+
+@pytest.mark.parametrize("records", [None, "70000", "6000"])
+@pytest.mark.parametrize("l,k,p", [(1, 255, 0.15), (16, 128, 0.15), (1, 16, 0.4)])
+def test_batches_of_many_visits_per_entry(monkeypatch, records, l, k, p):
+    """Later batches with a record per table entry, appended in parts of as many lanes as
+    the record table holds, by count and (a small table, that of 64 lanes) by the most
+    there can be."""
+    if records:
+        monkeypatch.setenv("SKIM_RECORD_ITEMS", records)
+    g = synth.erdos_renyi(5003, 40009, 6)
+    _check(g.n, g.src, g.dst, l, k, 0, p)
