@@ -246,6 +246,17 @@ SKIM_DEV SeedRow seed_row(const uint64_t *X, const uint32_t *xlen, uint32_t k, c
     return SeedRow{u, ln == k ? k - 1 : ln, static_cast<uint64_t>(__double_as_longlong(term_of(terms, tau)))};
 }
 
+// How a warp reads rows of up to `most` ranks: `rows` of them at a step, lane's share
+// is rank `pos` (and every 32nd after it) of row `row`.  (One row at a step left 31 lanes
+// idle with k = 2: 100000 seeds in 396 us.)
+struct RowShare {
+    uint32_t rows, row, pos;
+};
+SKIM_DEV RowShare row_share(uint32_t most) {
+    const uint32_t lane = threadIdx.x & 31, w = most > 16 ? 32 : most <= 1 ? 1 : 1u << (32 - __clz(most - 1));
+    return RowShare{32 / w, lane / w, lane & (w - 1)};
+}
+
 SKIM_DEV U192 warp_sum192(U192 a) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -284,6 +295,7 @@ SKIM_DEV U192 query_block(const uint64_t *X, const uint32_t *xlen, uint32_t n, u
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5, lane = threadIdx.x & 31;
     uint64_t *keys = tab, *val = tab + H + 1;
     ulonglong2 *st = reinterpret_cast<ulonglong2 *>(val + H + 1) + warp * kStage;
+    const RowShare sh = row_share(k - 1);
     U192 acc{{0, 0, 0}};
     for (uint64_t cut = 1, c = 0; c < cut;) {  // one piece, unless the table overflows
         const uint64_t pieces = parts * cut, piece = part * cut + c;
@@ -304,13 +316,14 @@ SKIM_DEV U192 query_block(const uint64_t *X, const uint32_t *xlen, uint32_t n, u
                 else atomicOr(err, 1u);
             }
             const uint32_t cnt = min(32u, (s - j0 - warp + warps - 1) / warps);
-            for (uint32_t i = 0; i < cnt; i++) {
-                const uint32_t u = __shfl_sync(kFull, r.u, i), body = __shfl_sync(kFull, r.body, i);
-                const uint64_t t = __shfl_sync(kFull, r.term, i);
+            for (uint32_t i = 0; i < cnt; i += sh.rows) {  // (rows past cnt have no ranks)
+                const uint32_t u = __shfl_sync(kFull, r.u, i + sh.row), body = __shfl_sync(kFull, r.body, i + sh.row);
+                const uint64_t t = __shfl_sync(kFull, r.term, i + sh.row);
                 const uint64_t *row = X + static_cast<uint64_t>(u) * k;
-                for (uint32_t p0 = 0; p0 < body; p0 += 32) {
-                    const bool in = p0 + lane < body;
-                    const uint64_t z = in ? row[p0 + lane] : 0;
+                const uint32_t end = sh.rows > 1 ? 1 : body;  // (the same for the warp)
+                for (uint32_t p0 = 0; p0 < end; p0 += 32) {
+                    const bool in = p0 + sh.pos < body;
+                    const uint64_t z = in ? row[p0 + sh.pos] : 0;
                     const uint32_t h = rank_hash(z);
                     const bool mine = in && h - lo32 <= last;
                     if (!PART) {
@@ -363,6 +376,7 @@ SKIM_DEV U192 query_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n,
     const uint32_t rank = cl.block_rank(), lane = threadIdx.x & 31;
     const uint32_t w = rank * (blockDim.x >> 5) + (threadIdx.x >> 5), ways = CL * (blockDim.x >> 5);
     uint64_t *keys = tab, *val = tab + H + 1;
+    const RowShare sh = row_share(k - 1);
     U192 acc{{0, 0, 0}};
     *bad = false;
     for (uint64_t c = 0; c < cut;) {
@@ -383,11 +397,11 @@ SKIM_DEV U192 query_cluster(const uint64_t *X, const uint32_t *xlen, uint32_t n,
                 else atomicOr(err, 1u);
             }
             const uint32_t cnt = min(32u, (s - j0 + ways - 1) / ways);
-            for (uint32_t i = 0; i < cnt; i++) {
-                const uint32_t u = __shfl_sync(kFull, r.u, i), body = __shfl_sync(kFull, r.body, i);
-                const uint64_t t = __shfl_sync(kFull, r.term, i);
+            for (uint32_t i = 0; i < cnt; i += sh.rows) {  // (rows past cnt have no ranks)
+                const uint32_t u = __shfl_sync(kFull, r.u, i + sh.row), body = __shfl_sync(kFull, r.body, i + sh.row);
+                const uint64_t t = __shfl_sync(kFull, r.term, i + sh.row);
                 const uint64_t *row = X + static_cast<uint64_t>(u) * k;
-                for (uint32_t p = lane; p < body; p += 32) {
+                for (uint32_t p = sh.pos; p < body; p += 32) {
                     const uint64_t z = row[p];
                     const uint32_t h = rank_hash(z) - lo32;
                     if (h > last) continue;
@@ -501,6 +515,7 @@ __global__ void __launch_bounds__(512) k_q_table(const uint64_t *X, const uint32
                                                  uint32_t H, unsigned *err) {
     const uint32_t lane = threadIdx.x & 31, ways = gridDim.x * (blockDim.x >> 5);
     const uint32_t w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const RowShare sh = row_share(k - 1);
     for (uint64_t j0 = static_cast<uint64_t>(w) * 32; j0 < s; j0 += static_cast<uint64_t>(ways) * 32) {
         SeedRow r{0, 0, 0};
         if (j0 + lane < s) {
@@ -508,10 +523,10 @@ __global__ void __launch_bounds__(512) k_q_table(const uint64_t *X, const uint32
             if (u < n) r = seed_row(X, xlen, k, terms, u);
             else atomicOr(err, 1u);
         }
-        for (int i = 0; i < 32; i++) {
-            const uint32_t u = __shfl_sync(kFull, r.u, i), body = __shfl_sync(kFull, r.body, i);
-            const uint64_t t = __shfl_sync(kFull, r.term, i);
-            for (uint32_t p = lane; p < body; p += 32) {
+        for (uint32_t i = 0; i < 32; i += sh.rows) {
+            const uint32_t u = __shfl_sync(kFull, r.u, i + sh.row), body = __shfl_sync(kFull, r.body, i + sh.row);
+            const uint64_t t = __shfl_sync(kFull, r.term, i + sh.row);
+            for (uint32_t p = sh.pos; p < body; p += 32) {
                 const uint64_t z = X[static_cast<uint64_t>(u) * k + p];
                 if (!table_put(tab, tab + H + 1, H, __umulhi(rank_hash(z), H), z, t)) atomicOr(err, 2u);
             }

@@ -96,3 +96,26 @@ def test_calls_with_many_small_queries(large, small, launches):
         before = pkg.skim_kernel_launches()
         assert np.array_equal(sk.query_batch(sets), want)
         assert pkg.skim_kernel_launches() - before == launches
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("k", [2, 3, 4, 5, 9, 10, 17, 18, 33, 34])
+def test_rows_read_by_a_warp_at_a_step(k, mode):
+    """Rows of 1, 2, up to 4, 8 and 16 ranks share a warp's step, longer ones have it alone;
+    sketches that are not full, counts of seeds that leave lanes over."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.erdos_renyi(3001, 5000, 67)
+    ks = synth.Keys.from_seed(67)
+    l, p = 16, 0.3
+    pb = oracle.Problem(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
+    ox, oln, _ = oracle.build_sketches(pb, rank_mode=mode)
+    rng = np.random.default_rng(k)
+    sets = [rng.choice(g.n, s, replace=False) for s in (1, 2, 7, 31, 33, 65, 500, 1023, 3001)]
+    with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, rank_mode=mode) as sk:
+        sk.build_sketches()
+        few, many = sk.query_batch(sets), sk.query_batch(sets * 20)
+        assert np.array_equal(np.tile(few, 20), many)
+        for s, b in zip(sets, few):
+            assert sk.query(s) == b
+            ref = oracle.union_estimate(ox, oln, l, s, rank_mode=mode)
+            assert abs(b - ref) <= REL * abs(ref)
