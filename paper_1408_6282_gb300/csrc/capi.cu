@@ -2250,8 +2250,8 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
     for (uint32_t i = 0; i < q; i++) {
         if (offsets[i + 1] < offsets[i]) return SKIM_EINVAL;
         const uint64_t cnt = offsets[i + 1] - offsets[i];
-        boff[i + 1] = boff[i] + query_blocks(cnt, c->k);
-        table_slots = std::max(table_slots, query_table_slots(cnt, c->k));
+        boff[i + 1] = boff[i] + query_blocks(cnt, c->k, q == 1);
+        table_slots = std::max(table_slots, query_table_slots(cnt, c->k, q == 1));
     }
     std::copy(offsets, offsets + q1, meta.data());
     const uint64_t total = offsets[q];
@@ -2275,7 +2275,7 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
         KTimer kt(c, SKIM_K_QUERY);
         QueryScratch qs{c->qpart, c->qdone, flag, c->qtab, c->qtab_slots, c->clusters};
         CK(c, launch_query_multi(c->X, c->xlen, c->n, c->k, query_terms_of(c), dseeds, d_off, d_boff, q, offsets,
-                                 static_cast<uint32_t>(boff[q]), qs, dout, c->st));
+                                 static_cast<uint32_t>(boff[q]), q == 1, qs, dout, c->st));
     }
     unsigned bad = 0;
     CK(c, cudaMemcpyAsync(&bad, flag, sizeof(unsigned), cudaMemcpyDeviceToHost, c->st));

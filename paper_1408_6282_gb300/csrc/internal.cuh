@@ -334,8 +334,8 @@ struct QueryScratch {
     uint64_t table_slots;
     bool clusters;          // may be launched (else every larger query is taken in parts)
 };
-uint32_t query_blocks(uint64_t seeds, uint32_t k);  // parts of a larger query, 0 for a small one and for the largest
-uint64_t query_table_slots(uint64_t seeds, uint32_t k);  // of the largest ones' table in global memory, else 0
+uint32_t query_blocks(uint64_t seeds, uint32_t k, bool alone);  // parts of a larger query, 0 for a small one and for the largest
+uint64_t query_table_slots(uint64_t seeds, uint32_t k, bool alone);  // of the largest ones' table in global memory, else 0
 uint32_t query_partials(uint32_t blocks, uint64_t table_slots);  // places of `partial`
 size_t query_partial_bytes();
 // How a threshold becomes a term of Eq. unionest, and the final divisor:
@@ -356,8 +356,8 @@ cudaError_t launch_node_estimates(const uint64_t *X, const uint32_t *xlen, uint3
 // block_off: prefix sums of query_blocks; blocks: their total; h_offsets: offsets, on the host
 cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                                const uint32_t *seeds, const uint64_t *offsets, const uint64_t *block_off, uint32_t q,
-                               const uint64_t *h_offsets, uint32_t blocks, const QueryScratch &qs, double *out,
-                               cudaStream_t s);
+                               const uint64_t *h_offsets, uint32_t blocks, bool alone, const QueryScratch &qs,
+                               double *out, cudaStream_t s);
 // One query with few enough seeds (host) to be kernel arguments; out_host: pinned.  An
 // error: it takes a cluster, which the device refuses (or clusters is false); the batch form does without.
 constexpr uint32_t kQueryArgSeeds = 8000;

@@ -145,7 +145,7 @@ SKIM_DEV double fixed_to_double(const U192 &a) {
 // then parts (four launches: 76, 86, 96, 126 us).  A batch fills the chip with parts and is
 // slower with clusters (1000 queries, with copies: 0.52 ms; clusters of 4, 8, 16: 0.63,
 // 0.76, 1.07 ms).  Both
-// read a query once per part or round of clusters: from kBlockMost ranks on the
+// read a query once per part or round of clusters: where in_memory says so the
 // table is in global memory (64 ranks per sketch, 30000 seeds: 264 us, clusters
 // 555 us, parts 1100 us; 9000 seeds, clusters: 107 us).
 // One block is as fast as the cluster up to
@@ -161,8 +161,8 @@ constexpr int small_threads(uint32_t queries) {
 }
 // Small queries go in one launch with the clusters of a few larger ones, in a block of
 // 1024 threads each and one per SM, while they are few: with clusters of 4 up to
-// kFewSmall, with clusters of 16, of which 8 are resident at once, up to kFewClusters of
-// them in all.  Else they take a launch of their own (as above, beside one larger query
+// kFewSmall, with clusters of 16, of which kClusterParts are resident at once, up to
+// kFewClusters of them in all.  Else they take a launch of their own (as above, beside one larger query
 // 152, 304, 608, 2000 small ones: 81, 108, 174, 438 us together, 96, 111, 116, 208 us
 // apart; 152 beside 6: 97 and 89 us).
 constexpr uint32_t kFewSmall = 2 * kSmsUsual, kFewClusters = 14;
@@ -175,9 +175,26 @@ constexpr uint32_t kClusterFour = 4;
 // larger queries of a call that take clusters of 16, the same if some do not fit four
 // blocks, and those that take clusters of 4 if all do
 constexpr uint32_t kFewLarge = 8, kFewLargest = 16, kMoreLarge = 64;
-constexpr uint32_t kClusterParts = 8;
-constexpr uint64_t kBlockMost = 1 << 20;  // ranks, above that the table is in global memory
+// Clusters of 16 that are resident at once (an eighth waits for another to end: 60000 seeds
+// of 16 ranks 243 us with 8, 147 us with 7), and ranks per block that they take in a round,
+// all distinct (0.8 of the slots).
+constexpr uint32_t kClusterParts = 7, kBlockFill = 9800;
+// Ranks above which the table is in global memory: what the resident clusters take in a
+// round, or with long rows a little more, whose ranks meet on as few slots (20000 seeds of 64
+// ranks, table 418 us, two rounds 329; 100000 of 16 191 and 398; 60000 of 32 265 and 497).
+constexpr uint64_t kBlockMost = kClusterParts * kCluster * kBlockFill, kBlockMostLong = 1500000;
+constexpr uint32_t kLongRanks = 64;
+// Seeds above which a query alone has its table there too, with short rows and others:
+// reading them is what a cluster waits for, and each reads all (k = 2, 100000 seeds 138 and
+// 104 us, k = 4, 60000 122 and 105, k = 16, 60000 209 and 178).
+constexpr uint32_t kTableSeedsShort = 25000, kTableSeeds = 50000, kShortRanks = 8;
 constexpr uint32_t kTableBlocks = 152 * 2;
+
+// (alone: the only query of its call)
+bool in_memory(uint64_t seeds, uint32_t k, bool alone) {
+    return seeds * (k - 1) > (k >= kLongRanks ? kBlockMostLong : kBlockMost) ||
+           (alone && seeds > (k <= kShortRanks ? kTableSeedsShort : kTableSeeds));
+}
 
 SKIM_DEV uint32_t upper_bound_u64(const uint64_t *a, uint32_t n, uint64_t x) {  // first i with a[i] > x
     uint32_t lo = 0, hi = n;
@@ -196,14 +213,17 @@ SKIM_DEV uint32_t rank_hash(uint64_t z) {
     h = (h ^ (h >> 15)) * 0x85EBCA77u;
     return h ^ (h >> 13);
 }
+// GLOBAL: a table in global memory, looked at through the first-level cache (a key
+// stays once it is there and a term only falls, so an old value costs a trip more).
+template <bool GLOBAL = false>
 SKIM_DEV bool table_put(uint64_t *keys, uint64_t *terms, uint32_t H, uint32_t at, uint64_t z, uint64_t t) {
     if (z == kEmptyKey) at = H;  // a place of its own
     for (uint32_t p = 0; p < H; p++) {
-        uint64_t k = *reinterpret_cast<volatile uint64_t *>(&keys[at]);
+        uint64_t k = GLOBAL ? __ldca(&keys[at]) : *reinterpret_cast<volatile uint64_t *>(&keys[at]);
         if (k == kEmptyKey && at != H)
             k = atomicCAS(reinterpret_cast<unsigned long long *>(&keys[at]), kEmptyKey, z);
         if (k == kEmptyKey || k == z) {
-            if (*reinterpret_cast<volatile uint64_t *>(&terms[at]) > t)
+            if ((GLOBAL ? __ldca(&terms[at]) : *reinterpret_cast<volatile uint64_t *>(&terms[at])) > t)
                 atomicMin(reinterpret_cast<unsigned long long *>(&terms[at]), t);
             return true;
         }
@@ -508,7 +528,7 @@ SKIM_DEV void add_parts(const U192 &e, uint64_t c, uint64_t first, uint64_t end,
     }
 }
 
-// A query of more than kBlockMost ranks: into a table of H + 1 slots in global
+// A query for in_memory: into a table of H + 1 slots in global
 // memory, then the sum over it.
 __global__ void __launch_bounds__(512) k_q_table(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k,
                                                  QueryTerms terms, const uint32_t *seeds, uint64_t s, uint64_t *tab,
@@ -528,7 +548,7 @@ __global__ void __launch_bounds__(512) k_q_table(const uint64_t *X, const uint32
             const uint64_t t = __shfl_sync(kFull, r.term, i + sh.row);
             for (uint32_t p = sh.pos; p < body; p += 32) {
                 const uint64_t z = X[static_cast<uint64_t>(u) * k + p];
-                if (!table_put(tab, tab + H + 1, H, __umulhi(rank_hash(z), H), z, t)) atomicOr(err, 2u);
+                if (!table_put<true>(tab, tab + H + 1, H, __umulhi(rank_hash(z), H), z, t)) atomicOr(err, 2u);
             }
         }
     }
@@ -578,7 +598,7 @@ __global__ void __launch_bounds__(kPartThreads) k_q_few(const uint64_t *X, const
         if (threadIdx.x == 0) out[qi] = fixed_to_double(e) / terms.div;
         return;
     }
-    const uint64_t room = static_cast<uint64_t>((CL * kBlockEntries)) * ways, cut = (entries + room - 1) / room;
+    const uint64_t room = static_cast<uint64_t>(CL * (CL == kCluster ? kBlockFill : kBlockEntries)) * ways, cut = (entries + room - 1) / room;
     bool bad;
     const U192 e = query_cluster<CL>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(s), c % ways, ways, cut, tab,
                                  cluster_slots<CL>(entries / (ways * cut)), err, &bad);
@@ -612,14 +632,14 @@ __global__ void k_node_estimates(const uint64_t *X, const uint32_t *xlen, uint32
 
 }  // namespace
 
-uint32_t query_blocks(uint64_t seeds, uint32_t k) {
+uint32_t query_blocks(uint64_t seeds, uint32_t k, bool alone) {
     const uint64_t e = seeds * (k - 1);
-    return e <= kSmallEntries || e > kBlockMost ? 0 : static_cast<uint32_t>((e + kPartEntries - 1) / kPartEntries);
+    return e <= kSmallEntries || in_memory(seeds, k, alone) ? 0 : static_cast<uint32_t>((e + kPartEntries - 1) / kPartEntries);
 }
 
-uint64_t query_table_slots(uint64_t seeds, uint32_t k) {
+uint64_t query_table_slots(uint64_t seeds, uint32_t k, bool alone) {
     const uint64_t e = seeds * (k - 1);
-    return e <= kBlockMost ? 0 : std::min<uint64_t>(e + e / 2, 0xfffffffeu) + 1;
+    return e <= kSmallEntries || !in_memory(seeds, k, alone) ? 0 : std::min<uint64_t>(e + e / 2, 0xfffffffeu) + 1;
 }
 
 size_t query_partial_bytes() { return sizeof(U192); }
@@ -696,16 +716,16 @@ cudaError_t launch_query_one(const uint64_t *X, const uint32_t *xlen, uint32_t n
 
 cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                                const uint32_t *seeds, const uint64_t *offsets, const uint64_t *block_off, uint32_t q,
-                               const uint64_t *h_offsets, uint32_t blocks, const QueryScratch &qs, double *out,
-                               cudaStream_t s) {
+                               const uint64_t *h_offsets, uint32_t blocks, bool alone, const QueryScratch &qs,
+                               double *out, cudaStream_t s) {
     if (q == 0) return cudaSuccess;
     static_assert(kSmallSlots >= kSmallEntries + kSmallEntries / 2 + 32, "a small query's table");
     U192 *partial = static_cast<U192 *>(qs.partial);
     cudaError_t e = cudaSuccess;
     uint32_t tables = 0;
-    if (h_offsets[q] * (k - 1) > kBlockMost) {  // some query may be one of those
+    if (in_memory(h_offsets[q], k, alone)) {  // some query may be one of those
         for (uint32_t i = 0; i < q && e == cudaSuccess; i++) {
-            const uint64_t cnt = h_offsets[i + 1] - h_offsets[i], slots = query_table_slots(cnt, k);
+            const uint64_t cnt = h_offsets[i + 1] - h_offsets[i], slots = query_table_slots(cnt, k, alone);
             if (!slots) continue;
             if (slots > qs.table_slots) return cudaErrorInvalidValue;
             tables++;
@@ -724,7 +744,7 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
     uint64_t most = 0;
     for (uint32_t i = 0; blocks && i < q && f.n_large <= kMoreLarge; i++) {
         const uint64_t cnt = h_offsets[i + 1] - h_offsets[i];
-        if (!query_blocks(cnt, k)) continue;
+        if (!query_blocks(cnt, k, alone)) continue;
         if (f.n_large < kMoreLarge) f.large[f.n_large] = i;
         f.n_large++;
         most = std::max(most, cnt * (k - 1));

@@ -154,7 +154,7 @@ bool admit(skim_server *s, std::unique_lock<std::mutex> &lock) {
         nseeds += r.count;
         used += r.slots;
         h_off[cnt + 1] = nseeds;
-        ln->boff.push_back(ln->boff.back() + query_blocks(r.count, s->k));
+        ln->boff.push_back(ln->boff.back() + query_blocks(r.count, s->k, false));
         ln->tickets.push_back(r.ticket);
         cnt++;
         s->pending.pop_front();
@@ -186,7 +186,7 @@ bool admit(skim_server *s, std::unique_lock<std::mutex> &lock) {
           cudaSuccess;
     QueryScratch qs{ln->d_part, ln->d_done, ln->d_err, ln->d_table, ln->d_table ? ln->arena_slots : 0, s->clusters};
     ok &= launch_query_multi(s->X, s->xlen, s->n, s->k, s->terms, ln->d_seeds, ln->d_meta, ln->d_meta + g1, cnt, ln->h_meta,
-                             static_cast<uint32_t>(ln->boff.back()), qs, ln->d_out, ln->st) == cudaSuccess;
+                             static_cast<uint32_t>(ln->boff.back()), false, qs, ln->d_out, ln->st) == cudaSuccess;
     ok &= cudaMemcpyAsync(ln->h_out, ln->d_out, cnt * sizeof(double), cudaMemcpyDeviceToHost, ln->st) == cudaSuccess;
     ok &= cudaEventRecord(ln->done, ln->st) == cudaSuccess;
     lock.lock();
@@ -273,7 +273,7 @@ int skim_server_start(skim_ctx *ctx, uint32_t max_inflight, uint64_t scratch_slo
         ok &= cudaEventCreateWithFlags(&ln.done, cudaEventDisableTiming) == cudaSuccess;
         ok &= cudaMalloc(&ln.d_seeds, ln.seed_cap * sizeof(uint32_t)) == cudaSuccess;
         // a block per 8000 ranks, for which a query is charged 16000 slots
-        const uint64_t table = query_table_slots(arena / 2 / (k - 1), k);  // the largest query's
+        const uint64_t table = query_table_slots(arena / 2 / (k - 1), k, false);  // the largest query's
         ln.part_cap = query_partials(static_cast<uint32_t>(arena / 2048 + gcap), table);
         if (table) ok &= cudaMalloc(&ln.d_table, arena * 2 * sizeof(uint64_t)) == cudaSuccess;
         ok &= cudaMalloc(&ln.d_meta, 2 * (gcap + 1) * sizeof(uint64_t)) == cudaSuccess;
