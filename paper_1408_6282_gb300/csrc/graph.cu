@@ -122,28 +122,33 @@ __global__ void k_live_masks(const uint32_t *rrow, const uint32_t *rcol, const u
 // Live rows from the masks.  A warp walks edges [e0, e1) of a row in tiles of
 // 32 (one per lane); for instance b the tile holds popc(ballot(bit b)) live
 // edges.  Lane b % 32 keeps the counts (or write cursors) of instances b < 32
-// (c0) and b >= 32 (c1).  Rows of up to kBigRow edges take one warp; longer
-// rows take a block of 8 warps on contiguous slices (kernels *_big).
-constexpr uint32_t kBigRow = 2048;
+// (c0) and b >= 32 (c1).  Rows of up to kBigRow edges take one warp, which is
+// what a small graph waits for (context creation, R-MAT 14 p = 0.01, l = 16; 2048, 1024, 512, 256
+// edges: 808, 729, 669, 642 us; R-MAT 20 wc, l = 64: 8.42, 7.44, 6.97, 7.00 ms).
+constexpr uint32_t kBigRow = 256;
 
-// Rows longer than kBigRow are cut into pieces of kBigRow edges, one warp per
+// Rows longer than kBigRow are cut into pieces of as many edges, or of more so that
+// a row has at most kRowPieces (a warp adds them up one by one), one warp per
 // piece: the row's pieces get consecutive ids (in edge order) when the count
 // pass meets the row; each piece's per-instance counts are summed per row into
 // off, with the exclusive prefix of every piece kept for the fill pass.
 struct Pieces {
     uint32_t *row;      // node of each piece
     uint32_t *e0;       // first edge of each piece
-    uint64_t *cnt;      // 64 per piece: live edges of each instance, then the prefix within the row
+    uint32_t *cnt;      // 64 per piece: live edges of each instance, then the prefix within the row
     unsigned *count;    // pieces in use
     uint32_t cap;
 };
 
+constexpr uint32_t kRowPieces = 1024;
+SKIM_DEV uint32_t piece_edges(uint32_t row) { return max(kBigRow, (row / kRowPieces + 32) & ~31u); }
+
 SKIM_DEV void claim_pieces(const Pieces &P, uint32_t v, uint32_t e0, uint32_t e1) {
-    const uint32_t np = (e1 - e0 + kBigRow - 1) / kBigRow;
+    const uint32_t step = piece_edges(e1 - e0), np = (e1 - e0 - 1) / step + 1;
     const unsigned base = atomicAdd(P.count, np);
     for (uint32_t q = 0; q < np && base + q < P.cap; q++) {
         P.row[base + q] = v;
-        P.e0[base + q] = e0 + q * kBigRow;
+        P.e0[base + q] = e0 + q * step;
     }
 }
 
@@ -293,11 +298,11 @@ __global__ void k_piece_count(const uint32_t *ptr, const uint64_t *mask, Pieces 
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t np = min(*P.count, P.cap);
     for (uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < np; p += (gridDim.x * blockDim.x) >> 5) {
-        const uint32_t v = P.row[p], e0 = P.e0[p], e1 = min(ptr[v + 1], e0 + kBigRow);
+        const uint32_t v = P.row[p], e0 = P.e0[p], end = ptr[v + 1], e1 = e0 + min(end - e0, piece_edges(end - ptr[v]));
         uint64_t c0 = 0, c1 = 0;
         warp_count(mask, e0, e1, c0, c1);
-        P.cnt[static_cast<uint64_t>(p) * 64 + lane] = c0;
-        P.cnt[static_cast<uint64_t>(p) * 64 + lane + 32] = c1;
+        P.cnt[static_cast<uint64_t>(p) * 64 + lane] = static_cast<uint32_t>(c0);
+        P.cnt[static_cast<uint64_t>(p) * 64 + lane + 32] = static_cast<uint32_t>(c1);
     }
 }
 
@@ -312,10 +317,10 @@ __global__ void k_piece_rows(const uint32_t *ptr, uint32_t l, uint64_t *tot, uin
         if (P.e0[p] != ptr[v]) continue;  // not the row's first piece
         uint64_t r0 = 0, r1 = 0;
         for (uint32_t q = p; q < np && P.row[q] == v; q++) {
-            uint64_t *c = P.cnt + static_cast<uint64_t>(q) * 64;
-            const uint64_t a0 = c[lane], a1 = c[lane + 32];
-            c[lane] = r0;
-            c[lane + 32] = r1;
+            uint32_t *c = P.cnt + static_cast<uint64_t>(q) * 64;
+            const uint32_t a0 = c[lane], a1 = c[lane + 32];
+            c[lane] = static_cast<uint32_t>(r0);  // (at most the row's edges)
+            c[lane + 32] = static_cast<uint32_t>(r1);
             r0 += a0;
             r1 += a1;
         }
@@ -348,11 +353,11 @@ __global__ void k_piece_fill(const uint32_t *ptr, const uint32_t *col, const uin
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t np = min(*P.count, P.cap);
     for (uint32_t p = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; p < np; p += (gridDim.x * blockDim.x) >> 5) {
-        const uint32_t v = P.row[p], e0 = P.e0[p], e1 = min(ptr[v + 1], e0 + kBigRow);
+        const uint32_t v = P.row[p], e0 = P.e0[p], end = ptr[v + 1], e1 = e0 + min(end - e0, piece_edges(end - ptr[v]));
         const uint64_t base = static_cast<uint64_t>(v) * l;
-        const uint64_t *c = P.cnt + static_cast<uint64_t>(p) * 64;
-        uint64_t p0 = lane < l ? off[base + lane] + c[lane] : 0;
-        uint64_t p1 = lane + 32 < l ? off[base + lane + 32] + c[lane + 32] : 0;
+        const uint32_t *c = P.cnt + static_cast<uint64_t>(p) * 64;
+        uint64_t p0 = lane < l ? static_cast<uint64_t>(off[base + lane]) + c[lane] : 0;
+        uint64_t p1 = lane + 32 < l ? static_cast<uint64_t>(off[base + lane + 32]) + c[lane + 32] : 0;
         warp_fill(mask, col, e0, e1, p0, p1, live);
     }
 }
@@ -644,7 +649,7 @@ cudaError_t launch_live_masks(const uint32_t *rrow, const uint32_t *rcol, const 
 }
 size_t live_pieces_bytes(uint64_t m) {
     const uint64_t cap = 2 * (m / kBigRow) + 2;
-    return cap * (4 + 4 + 64 * 8) + 256;
+    return cap * (4 + 4 + 64 * 4) + 256;
 }
 
 namespace {
@@ -652,7 +657,7 @@ Pieces carve_pieces(void *ws, uint64_t m) {
     Pieces P;
     const uint64_t cap = 2 * (m / kBigRow) + 2;
     char *p = static_cast<char *>(ws);
-    P.cnt = reinterpret_cast<uint64_t *>(p); p += cap * 64 * 8;
+    P.cnt = reinterpret_cast<uint32_t *>(p); p += cap * 64 * 4;
     P.row = reinterpret_cast<uint32_t *>(p); p += cap * 4;
     P.e0 = reinterpret_cast<uint32_t *>(p); p += cap * 4;
     P.count = reinterpret_cast<unsigned *>((reinterpret_cast<uintptr_t>(p) + 15) & ~static_cast<uintptr_t>(15));

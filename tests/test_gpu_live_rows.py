@@ -46,3 +46,29 @@ def test_row_sizes(model, p, l, reverse):
             got = sk.greedy_stops(15)
             for a, b in zip(got, (seeds, cov, tau, kp)):
                 assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("l", [1, 33, 64])
+@pytest.mark.parametrize("p", [0.004, 0.7])
+def test_rows_cut_into_pieces(l, p):
+    """Rows of one, two and many pieces of 256 edges, and rows whose pieces are longer so that
+    there are at most 1024 of them; both directions, against coins drawn in the searches."""
+    import paper_1408_6282_gb300 as pkg
+    degrees = [255, 256, 257, 511, 512, 513, 3001, 1024 * 256 - 1, 1024 * 256, 1024 * 256 + 1, 299_999]
+    n = 300_000
+    rng = np.random.default_rng(l)
+    a = [rng.choice(np.setdiff1d(np.arange(n), [7 * i]), d, replace=False) for i, d in enumerate(degrees)]
+    b = [np.full(d, 7 * i) for i, d in enumerate(degrees)]
+    u, v = np.concatenate(a), np.concatenate(b)
+    key = np.unique(np.concatenate([u << 32 | v, (v + 100) << 32 | u]).astype(np.uint64))
+    src, dst = (key >> np.uint64(32)).astype(np.uint32), (key & np.uint64(0xffffffff)).astype(np.uint32)
+    keep = src != dst
+    with pkg.Skim(n, src[keep], dst[keep], l, 8, 0, p, 3, 4, 5) as sk:
+        got = []
+        for rows in (True, False):
+            sk.set_live_rows(rows)
+            assert sk.instance_stats()[1] == rows
+            sk.build_sketches()
+            got.append((*sk.sketches(), *sk.greedy_stops(5)))
+        for x, y in zip(*got):
+            assert np.array_equal(x, y)
