@@ -140,6 +140,7 @@ struct skim_ctx {
     // newly covered pairs at *pend_cov
     bool pend_res = false;
     uint64_t *pend_cov = nullptr;
+    uint32_t bstops = 0, bfirst = 0;  // stops in the active batch, the lane behind its first
     bool refilter = false;          // a search ran since the active batch's lanes were last filtered
     bool pend_queue = false;        // it used the work queue
     cudaEvent_t step_done = nullptr;  // of the last step's read-back
@@ -877,9 +878,9 @@ StepArgs step_args(const skim_ctx *c) {
                     c->srank + c->bp0};
 }
 
-// Between two seeds: the active batch goes, and the lanes past the last stop are
-// searched again by the next one (they hold stops that have not been looked for, so
-// committing them would lose seeds).
+// Between two seeds, no search pending: the active batch goes, and the lanes past the last
+// stop are searched again by the next one (they hold stops that have not been looked
+// for, so committing them would lose seeds).
 int drop_batch(skim_ctx *c) {
     if (!c->batch_active) return SKIM_OK;
     uint64_t used = 0;  // the dropped lanes take no room in the index
@@ -889,12 +890,28 @@ int drop_batch(skim_ctx *c) {
     c->idx_bound = used;
     c->cursor = c->bp0 + c->blo;
     c->since_stop -= std::min(c->since_stop, left);
+    c->hstats[SKIM_STAT_RANKS] -= std::min(c->hstats[SKIM_STAT_RANKS], left);
     c->batch_active = false;
     c->refilter = false;
     return clear_batch(c);
 }
 
+// A step looks at all records of the batch, so a large batch whose stops follow each
+// other closely costs more than one searched again in pieces of the right size (next_seed):
+// it has made kDropStops steps, and at their pace kDropLeft more would not use it up.
+// R-MAT 18, l = 64, p = 0.1, 300 seeds: 58 ms, so 30; p = 0.03, 500 seeds: 86 and 39.
+constexpr uint64_t kDropRecords = 1 << 20;
+constexpr uint32_t kDropStops = 16, kDropLeft = 64;
+bool too_large(const skim_ctx *c) {
+    return c->batch_active && c->bR >= kDropRecords && c->bstops > kDropStops &&
+           static_cast<uint64_t>(c->bB - c->blo) * (c->bstops - 1) > static_cast<uint64_t>(c->blo - c->bfirst) * kDropLeft;
+}
+
 int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
+    if (too_large(c)) {
+        RC(settle_residual(c));
+        RC(drop_batch(c));
+    }
     for (;;) {
         if (c->batch_active) {
             {
@@ -941,6 +958,7 @@ int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
                     c->since_stop = after;
                 }
                 c->blo = p + 1;
+                if (c->bstops++ == 0) c->bfirst = c->blo;
                 c->refilter = true;
                 *x_out = x;
                 return SKIM_OK;
@@ -986,6 +1004,7 @@ int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
             c->bp0 = c->cursor;
             c->bB = B;
             c->blo = 0;
+            c->bstops = 0;
             c->refilter = false;
             c->cursor += B;
             c->hstats[SKIM_STAT_RANKS] += B;

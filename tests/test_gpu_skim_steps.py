@@ -118,3 +118,18 @@ def test_coin_batches_keep_to_their_lanes():
             assert seeds.tolist() == [0, 1, 2] and cov.tolist() == [64] * 3
             st = sk.stats()
             assert st["ranks"] == 64 * g.n and st["batches"] >= -(-st["ranks"] // most)
+
+
+@pytest.mark.parametrize("scale,p,k", [(16, 0.1, 16), (17, 0.03, 32)])
+def test_batches_too_large_for_their_stops(scale, p, k):
+    """Batches of a million records and more whose stops follow closely are left for smaller
+    ones: the same sequence as with batches that are small from the start."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.rmat(scale, 16, 3)
+    got = []
+    for bl in (0, 1 << 15):
+        with pkg.Skim(g.n, g.src, g.dst, 64, k, 0, p, 5, 6, 7, batch_lanes=bl) as sk:
+            parts = [sk.greedy_stops(c) for c in (300, 1, 99)]
+            got.append([np.concatenate([x[q] for x in parts]) for q in range(4)])
+    for a, b in zip(*got):
+        assert np.array_equal(a, b)
