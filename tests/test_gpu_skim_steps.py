@@ -133,3 +133,16 @@ def test_batches_too_large_for_their_stops(scale, p, k):
             got.append([np.concatenate([x[q] for x in parts]) for q in range(4)])
     for a, b in zip(*got):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("k", [20, 40, 100])
+@pytest.mark.parametrize("p", [0.02, 0.06, 0.2])
+def test_records_of_a_node_in_order(k, p):
+    """Nodes with up to 8, 32, 64, 128 and more records in a batch."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.rmat(11, 12, 9)
+    pb = oracle.Problem(g.n, g.src, g.dst, 64, k, 0, p, 7, 8, 9)
+    want = oracle.skim_stops(pb, 80)
+    with pkg.Skim(g.n, g.src, g.dst, 64, k, 0, p, 7, 8, 9) as sk:
+        for a, b in zip(sk.greedy_stops(80), want):
+            assert np.array_equal(a, b)
