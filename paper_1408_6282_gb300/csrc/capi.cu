@@ -713,9 +713,16 @@ uint32_t default_lanes(skim_ctx *c) {
 // visits (next_seed), and over stored rows most lanes of a sparse one are leaf lanes: 50
 // seeds of R-MAT 20 p = 0.01 take 20, 19, 17.8, 17.0 ms with at most 2, 4, 8, 16 M.  With
 // coins every lane is a table entry and a record: 50 seeds of R-MAT 18 p = 0.01 27.1 ms
-// with at most 16 M, 24.8 with 2 M, 30 of R-MAT 17 trivalency 17.9 and 15.7.
+// with at most 16 M, 24.8 with 2 M, 30 of R-MAT 17 trivalency 17.9 and 15.7.  So it is
+// over stored rows once nodes fill up with their own leaf lanes, which are records
+// then (k_leaf_records): from about k - 2 sqrt(k) lanes a node on (60 seeds of R-MAT 18
+// trivalency, k = 32, batches of up to 9.7 M lanes and so: 14.3 and 6.0 ms).
 uint32_t skim_lanes(skim_ctx *c) {
-    return c->batch_cfg || !c->mat ? default_lanes(c) : static_cast<uint32_t>(std::min<uint64_t>(1ull << 24, c->lane_cap));
+    if (c->batch_cfg || !c->mat) return default_lanes(c);
+    const double sparse = std::max(0.0, c->k - 2.0 * std::sqrt(static_cast<double>(c->k))) * c->n;
+    const uint64_t most =
+        std::max<uint64_t>(default_lanes(c), static_cast<uint64_t>(std::max(0.0, sparse - static_cast<double>(c->cursor))));
+    return static_cast<uint32_t>(std::min<uint64_t>({1ull << 24, most, c->lane_cap}));
 }
 
 // ---- SKIM steps ------------------------------------------------------------
