@@ -2272,12 +2272,12 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
     // one host block: seed offsets | block offsets
     const size_t q1 = static_cast<size_t>(q) + 1;
     std::vector<uint64_t> meta(2 * q1, 0);
-    uint64_t *boff = meta.data() + q1, table_slots = 0;
+    uint64_t *boff = meta.data() + q1, most = 0;
     for (uint32_t i = 0; i < q; i++) {
         if (offsets[i + 1] < offsets[i]) return SKIM_EINVAL;
         const uint64_t cnt = offsets[i + 1] - offsets[i];
         boff[i + 1] = boff[i] + query_blocks(cnt, c->k, q == 1);
-        table_slots = std::max(table_slots, query_table_slots(cnt, c->k, q == 1));
+        most = std::max(most, cnt);
     }
     std::copy(offsets, offsets + q1, meta.data());
     const uint64_t total = offsets[q];
@@ -2286,7 +2286,7 @@ int skim_oracle_query_batch(skim_ctx *c, const uint64_t *offsets, uint32_t q, co
         for (uint64_t i = 0; i < total; i++)
             if (seeds[i] >= c->n) return SKIM_EINVAL;
     }
-    RC(ensure_query_space(c, total, q, boff[q], table_slots));
+    RC(ensure_query_space(c, total, q, boff[q], query_table_slots(most, c->k, q == 1)));
     const uint32_t *dseeds = seeds;
     if (!on_device && total) {
         CK(c, cudaMemcpyAsync(c->qseeds, seeds, total * sizeof(uint32_t), cudaMemcpyHostToDevice, c->st));

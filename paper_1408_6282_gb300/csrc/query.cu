@@ -307,15 +307,16 @@ SKIM_DEV U192 block_sum192(U192 acc) {  // valid in thread 0
 // Block-collective: the exact sum over the ranks of a query whose hash lies in
 // part `part` of `parts` (thread 0's return value), table of H + 1 slots in tab.
 // PART: a row has few ranks of the part, so a warp collects 32 before it goes to
-// the table (kStage pairs per warp behind it).
-template <bool PART>
+// the table (kStage pairs per warp behind it).  LONG: rows are not shared (row_share; a
+// batch is bound by what it issues, 1000 queries of 64 ranks 504 and 520 us).
+template <bool PART, bool LONG = false>
 SKIM_DEV U192 query_block(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                           const uint32_t *seeds, uint32_t s, uint64_t part, uint64_t parts, uint64_t *tab, uint32_t H,
                           unsigned *err) {
     const uint32_t warp = threadIdx.x >> 5, warps = blockDim.x >> 5, lane = threadIdx.x & 31;
     uint64_t *keys = tab, *val = tab + H + 1;
     ulonglong2 *st = reinterpret_cast<ulonglong2 *>(val + H + 1) + warp * kStage;
-    const RowShare sh = row_share(k - 1);
+    const RowShare sh = LONG ? RowShare{1, 0, lane} : row_share(k - 1);
     U192 acc{{0, 0, 0}};
     for (uint64_t cut = 1, c = 0; c < cut;) {  // one piece, unless the table overflows
         const uint64_t pieces = parts * cut, piece = part * cut + c;
@@ -489,6 +490,7 @@ __global__ void __launch_bounds__(1024)
 }
 
 // Block q: query q, if it is small.
+template <bool LONG>
 __global__ void __launch_bounds__(1024) k_q_small(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k,
                                                   QueryTerms terms, const uint32_t *seeds, const uint64_t *offsets,
                                                   double *out, unsigned *err) {
@@ -497,7 +499,7 @@ __global__ void __launch_bounds__(1024) k_q_small(const uint64_t *X, const uint3
     const uint64_t s0 = offsets[q];
     const uint32_t s = static_cast<uint32_t>(offsets[q + 1] - s0);
     if (static_cast<uint64_t>(s) * (k - 1) > kSmallEntries) return;
-    const U192 e = query_block<false>(X, xlen, n, k, terms, seeds + s0, s, 0, 1, reinterpret_cast<uint64_t *>(s_tab),
+    const U192 e = query_block<false, LONG>(X, xlen, n, k, terms, seeds + s0, s, 0, 1, reinterpret_cast<uint64_t *>(s_tab),
                                small_slots(static_cast<uint64_t>(s) * (k - 1)), err);
     if (threadIdx.x == 0) out[q] = fixed_to_double(e) / terms.div;
 }
@@ -561,6 +563,7 @@ __global__ void __launch_bounds__(512) k_q_table_sum(const uint64_t *val, uint32
 }
 
 // One block per part of the larger queries.
+template <bool LONG>
 __global__ void __launch_bounds__(kPartThreads) k_q_part(const uint64_t *X, const uint32_t *xlen, uint32_t n,
                                                          uint32_t k, QueryTerms terms, const uint32_t *seeds,
                                                          const uint64_t *offsets, const uint64_t *block_off,
@@ -570,7 +573,7 @@ __global__ void __launch_bounds__(kPartThreads) k_q_part(const uint64_t *X, cons
     const uint32_t c = blockIdx.x;
     const uint32_t qi = upper_bound_u64(block_off + 1, q, c);
     const uint64_t first = block_off[qi], end = block_off[qi + 1], s0 = offsets[qi];
-    const U192 e = query_block<true>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(offsets[qi + 1] - s0), c - first,
+    const U192 e = query_block<true, LONG>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(offsets[qi + 1] - s0), c - first,
                                end - first, reinterpret_cast<uint64_t *>(s_tab), kPartSlots, err);
     add_parts(e, c, first, end, partial, &done[qi], &out[qi], terms.div);
 }
@@ -634,7 +637,8 @@ __global__ void k_node_estimates(const uint64_t *X, const uint32_t *xlen, uint32
 
 uint32_t query_blocks(uint64_t seeds, uint32_t k, bool alone) {
     const uint64_t e = seeds * (k - 1);
-    return e <= kSmallEntries || in_memory(seeds, k, alone) ? 0 : static_cast<uint32_t>((e + kPartEntries - 1) / kPartEntries);
+    if (e <= kSmallEntries) return 0;
+    return in_memory(seeds, k, alone) ? 0 : static_cast<uint32_t>((e + kPartEntries - 1) / kPartEntries);
 }
 
 uint64_t query_table_slots(uint64_t seeds, uint32_t k, bool alone) {
@@ -768,19 +772,21 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
     }
     if (e == cudaSuccess && blocks) {
         const int smem = (kPartSlots + 1 + kPartThreads / 32 * kStage) * sizeof(ulonglong2);
-        e = cudaFuncSetAttribute(k_q_part, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const auto kernel = k > 17 ? k_q_part<true> : k_q_part<false>;  // (row_share)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         note_launch();
-        k_q_part<<<blocks, kPartThreads, smem, s>>>(X, xlen, n, k, terms, seeds, offsets, block_off, q, partial, qs.done,
+        kernel<<<blocks, kPartThreads, smem, s>>>(X, xlen, n, k, terms, seeds, offsets, block_off, q, partial, qs.done,
                                                     out, qs.err);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && q > tables) {
         const int smem = (kSmallSlots + 1) * sizeof(ulonglong2);
-        e = cudaFuncSetAttribute(k_q_small, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const auto kernel = k > 17 ? k_q_small<true> : k_q_small<false>;  // (row_share)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         note_launch();
-        k_q_small<<<q, small_threads(q), smem, s>>>(X, xlen, n, k, terms, seeds, offsets, out, qs.err);
+        kernel<<<q, small_threads(q), smem, s>>>(X, xlen, n, k, terms, seeds, offsets, out, qs.err);
         e = cudaGetLastError();
     }
     return e;
