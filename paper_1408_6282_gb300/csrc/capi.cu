@@ -50,7 +50,7 @@ struct skim_ctx {
     bool mat_wanted = true;  // skim_set_live_rows: walk materialised live rows when they exist
     bool live_ready = false;  // the live rows of both directions are filled
     uint64_t *rmask = nullptr, *fmask = nullptr;
-    uint32_t *loff = nullptr, *foff = nullptr;  // live-row offsets (kRowFull flags on loff)
+    uint32_t *loff = nullptr, *foff = nullptr;  // live-row offsets
     uint32_t *rlive = nullptr, *flive = nullptr;  // live in- and out-neighbour rows
     uint32_t *rrow = nullptr, *rev2fwd = nullptr;  // per reverse CSR edge: head, forward position
     void *pieces = nullptr;                         // workspace of the long-row passes
@@ -80,7 +80,6 @@ struct skim_ctx {
     uint64_t *ncnt = nullptr, *noff = nullptr;
     uint32_t *nlist = nullptr;
     unsigned *nlist_cnt = nullptr;
-    bool bnode = false;  // the active batch's records were placed per node
     void *ws = nullptr;
     size_t ws_bytes = 0;
     uint8_t *lane_inst = nullptr;
@@ -111,9 +110,9 @@ struct skim_ctx {
     uint32_t *size = nullptr, *seg_len = nullptr, *idx = nullptr, *ncount = nullptr;
     uint8_t *chosen = nullptr;
     uint64_t idx_cap = 0;
-    // inverted index fill: on the device [0] entries used, [1] first entry of
-    // the last commit; on the host an upper bound of [0] (the visit bits of
-    // the SKIM batches so far), which sizes the index without a read-back
+    // inverted index fill: on the device the entries used; on the host an upper
+    // bound (the visit bits of the SKIM batches so far), which sizes the index
+    // without a read-back
     uint64_t *idx_ctr = nullptr;
     uint64_t idx_bound = 0, vis_seen = 0;
     uint64_t cursor = 0;
@@ -629,11 +628,11 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
     uint32_t sb = 0;
     while (sb + tbits < kPlaceBits && (static_cast<uint64_t>(c->n) >> sb) > std::max<uint64_t>(R, 1)) sb++;
     const uint32_t nb = static_cast<uint32_t>((static_cast<uint64_t>(c->n) + (1ull << sb) - 1) >> sb);
-    c->bnode = static_cast<uint64_t>(nb) <= static_cast<uint64_t>(c->node_density) * R;
-    if (c->bnode) RC(node_buffers(c));
+    const bool placed = static_cast<uint64_t>(nb) <= static_cast<uint64_t>(c->node_density) * R;
+    if (placed) RC(node_buffers(c));
     {
         KTimer kt(c, SKIM_K_SORT);
-        if (c->bnode)
+        if (placed)
             CK(c, launch_node_sort(c->rkey, c->rval, R, tbits + sb, nb, c->ncnt, c->noff, c->rkey2, c->nlist,
                                    c->nlist_cnt, c->ws, c->st));
         else
@@ -656,7 +655,6 @@ int rev_batch(skim_ctx *c, uint64_t p0, uint32_t B, bool mode_build, bool *retry
 // visited table it uses).
 int clear_batch(skim_ctx *c) {
     c->bR = 0;
-    c->bnode = false;
     return SKIM_OK;
 }
 
@@ -737,7 +735,7 @@ int skim_state_init(skim_ctx *c) {
     RC(dkeep(c, &c->chosen, c->n));
     RC(dkeep(c, &c->pend_trav, c->n));
     RC(dkeep(c, &c->pend_erase, c->n));
-    RC(dkeep(c, &c->idx_ctr, 2));
+    RC(dkeep(c, &c->idx_ctr, 1));
     CK(c, cudaMemsetAsync(c->covered, 0, c->n * sizeof(uint64_t), c->st));
     CK(c, cudaMemsetAsync(c->size, 0, c->n * sizeof(uint32_t), c->st));
     CK(c, cudaMemsetAsync(c->seg_len, 0, c->nl * sizeof(uint32_t), c->st));
@@ -745,7 +743,7 @@ int skim_state_init(skim_ctx *c) {
     CK(c, cudaMemsetAsync(c->pend_trav, 0, c->n * sizeof(uint64_t), c->st));
     CK(c, cudaMemsetAsync(c->pend_erase, 0, c->n * sizeof(uint64_t), c->st));
     if (c->batch_active) RC(clear_batch(c));
-    CK(c, cudaMemsetAsync(c->idx_ctr, 0, 2 * sizeof(uint64_t), c->st));
+    CK(c, cudaMemsetAsync(c->idx_ctr, 0, sizeof(uint64_t), c->st));
     c->idx_bound = 0;
     c->cursor = 0;
     c->nseeds = 0;

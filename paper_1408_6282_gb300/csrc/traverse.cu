@@ -451,8 +451,8 @@ SKIM_DEV void push_rev(const TravArgs &A, Acc &acc, uint32_t u, uint32_t t, uint
     }
 }
 
-// Warp-collective: lanes with `act` visit node u with lane bits `bits` in word t.
-template <bool MAT>
+// Warp-collective, coins drawn in the search: lanes with `act` visit node u with lane bits
+// `bits` in word t.
 SKIM_DEV void emit_rev(const TravArgs &A, Acc &acc, bool act, uint32_t u, uint32_t t, uint64_t bits) {
     if (!__any_sync(kFull, act && bits)) return;
     uint64_t nb = 0;
@@ -493,7 +493,7 @@ SKIM_DEV void emit_rev(const TravArgs &A, Acc &acc, bool act, uint32_t u, uint32
         }
     }
     acc.visits += __popcll(nb);
-    push_rev<MAT>(A, acc, u, t, nb, slot);
+    push_rev<false>(A, acc, u, t, nb, slot);
 }
 
 // Where a reverse search puts what it finds.  GlobalSink: visit records by
@@ -859,7 +859,7 @@ __device__ __noinline__ uint32_t coin_visit(const TravArgs &A, ulonglong2 *st, u
         __syncwarp();
     }
     Acc acc;
-    emit_rev<false>(A, acc, lane < c, static_cast<uint32_t>(e.x), static_cast<uint32_t>(e.x >> 32), e.y);
+    emit_rev(A, acc, lane < c, static_cast<uint32_t>(e.x), static_cast<uint32_t>(e.x >> 32), e.y);
     return static_cast<uint32_t>(acc.visits);
 }
 
@@ -1737,7 +1737,7 @@ __global__ void k_rev_sources(TravArgs A, const uint32_t *lane_pair, uint32_t B,
         if (A.mat)
             emit_rev_mat(A, acc, gsink, act, u, j >> 6, static_cast<int>(j & 63), i, true);
         else
-            emit_rev<false>(A, acc, act, u, j >> 6, 1ull << (j & 63));
+            emit_rev(A, acc, act, u, j >> 6, 1ull << (j & 63));
     }
     flush_acc(A, acc, false);
 }
