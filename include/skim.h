@@ -234,7 +234,7 @@ int skim_greedy(skim_ctx *ctx, uint32_t n_seeds, uint32_t *seeds_out, uint64_t *
  * size among all other nodes once that rank is taken out (k' <= k - 1).  When
  * the ranks have run out the seed comes from exact residual counts: then
  * tau_out[j] = 0 and kprime_out[j] = -1.  Either output may be NULL; with both
- * NULL this is skim_greedy.  Recording costs three small kernels per seed and
+ * NULL this is skim_greedy.  Recording costs a look at all sizes per seed and
  * device arrays of 12 * n_seeds bytes for the call.  Errors as skim_greedy. */
 int skim_greedy_ex(skim_ctx *ctx, uint32_t n_seeds, uint32_t *seeds_out, uint64_t *cov_out, uint64_t *tau_out,
                    int32_t *kprime_out);
@@ -367,7 +367,9 @@ int skim_context_shape(skim_ctx *ctx, uint32_t *n, uint32_t *k, uint32_t *l);
  * soon as slots and memory free up.  Each result is bitwise identical to
  * skim_oracle_query on the same seeds.  The context's sketches must stay
  * built, and the context must not be used by other calls, until
- * skim_server_stop() returns.  Submit, poll and wait may be called from any
+ * skim_server_stop() returns.  The server thread looks for finished groups and new
+ * requests without a pause while any group is in flight, so a loaded server keeps a
+ * host core busy; an idle one sleeps.  Submit, poll and wait may be called from any
  * host thread.  Errors: SKIM_EINVAL, SKIM_ENOTBUILT, SKIM_ENOMEM; submit
  * returns SKIM_ERANGE for a query larger than one stream's scratch. */
 typedef struct skim_server skim_server;

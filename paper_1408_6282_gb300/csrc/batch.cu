@@ -28,7 +28,6 @@ inline unsigned grid_for(size_t n, int threads, unsigned cap = 152 * 32) {
     return static_cast<unsigned>(g ? g : 1);
 }
 
-// Instance of every lane and the offset of its coin stream, (i + 1) * G.
 // Instance and coin-stream offset of every lane: instance i = pair % l, or in
 // the IC model (lane_rank given) a fresh instance numbered by the position.
 __global__ void k_lane_inst(const uint32_t *lane_pair, const uint64_t *lane_rank, uint32_t B, uint32_t l,

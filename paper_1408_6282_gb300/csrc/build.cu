@@ -389,7 +389,8 @@ __global__ void k_append(const uint64_t *__restrict__ rec, uint64_t r0, uint64_t
 // (R-MAT 20 wc with every batch of the first 400 K lanes in this form: 14.8 ms
 // instead of 13.2, for the look at every lane's source).
 __global__ void k_append_words(const uint64_t *__restrict__ rec, const uint32_t *__restrict__ rec_val, uint64_t R,
-                               uint32_t tbits, const uint64_t *__restrict__ hvals, const uint32_t *__restrict__ pair, uint32_t l, int own, uint32_t lbits,
+                               uint32_t tbits, const uint64_t *__restrict__ hvals, const uint32_t *__restrict__ pair,
+                               uint32_t l, int own, uint32_t lbits,
                                const uint64_t *__restrict__ lane_rank, uint32_t k, uint32_t *len, uint64_t *X,
                                uint64_t *over_key, uint32_t *over_pos, uint32_t *list, DevCtl *ctl) {
     const uint64_t tm = (1ull << tbits) - 1;
@@ -594,8 +595,8 @@ __global__ void k_need_full(BuildNode g, const uint64_t *next, uint32_t *list, D
 // says whether its hit list is open.  A row whose in-neighbours are all full
 // becomes a task {node, row (or its only entry), entries << 6 | instance} for
 // the sweeps, one of more than kTaskRow entries a task at the other end of the
-// space; one that finds no room sets its bit (searched for longer, same result).  Nothing to do while the full nodes and the open lists are those of
-// the last pass.
+// space; one that finds no room sets its bit (searched for longer, same result).
+// Nothing to do while the full nodes and the open lists are those of the last pass.
 constexpr uint32_t kTaskLook = 16;  // entries a lane looks at by itself
 constexpr uint32_t kTaskRow = 96;   // and the longest row of a short task
 __global__ void __launch_bounds__(256) k_need_tasks(BuildNode g, uint64_t *need, const uint32_t *__restrict__ list,
@@ -694,7 +695,8 @@ __global__ void __launch_bounds__(kSweepThreads) k_need_sweep(BuildNode g, uint6
                                                     uint32_t *wl1, uint32_t cap, DevCtl *ctl, uint64_t timeout_ns) {
     __shared__ uint4 s_long[kSweepLong];
     __shared__ uint32_t s_n;
-    const uint32_t nt = min(ctl->b.n_task, cap - cap / 16), nlong = min(ctl->b.n_long, cap / 16), lane = threadIdx.x & 31;
+    const uint32_t nt = min(ctl->b.n_task, cap - cap / 16), nlong = min(ctl->b.n_long, cap / 16);
+    const uint32_t lane = threadIdx.x & 31;
     if (threadIdx.x == 0) s_n = 0;
     if (blockIdx.x == 0 && threadIdx.x == 0) {  // what this pass has seen
         ctl->b.n_full_last = ctl->b.n_full;
@@ -790,7 +792,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_need_sweep(BuildNode g, uint6
                     if (q < kSweepLong && lane == 0) s_long[q] = make_uint4(ba, bn, bi, 0);
                 }
                 if (q >= kSweepLong)
-                    for (uint32_t z = 0; z < bn; z += 32) reach(z + lane < bn, z + lane < bn ? g.flive[ba + z + lane] : 0, bi);
+                    for (uint32_t z = lane; z < bn + lane; z += 32) reach(z < bn, z < bn ? g.flive[ba + z] : 0, bi);
             }
             const uint32_t c = len < 32 ? len : 0;
             uint32_t incl = c;
@@ -1266,15 +1268,17 @@ cudaError_t launch_append(const uint64_t *rec, uint64_t r0, uint64_t r1, uint32_
     return cudaGetLastError();
 }
 
-cudaError_t launch_count_words(const uint32_t *rec_val, uint64_t R, const uint64_t *hvals, uint32_t *cnt, cudaStream_t s) {
+cudaError_t launch_count_words(const uint32_t *rec_val, uint64_t R, const uint64_t *hvals, uint32_t *cnt,
+                               cudaStream_t s) {
     note_launch();
     k_count_words<<<grid_for(R, kWordChunk, 152 * 4), kWordChunk, 0, s>>>(rec_val, R, hvals, cnt);
     return cudaGetLastError();
 }
 
 cudaError_t launch_append_words(const uint64_t *rec, const uint32_t *rec_val, uint64_t R, uint32_t tbits,
-                                const uint64_t *hvals, const uint32_t *pair, uint32_t l, int own, uint32_t lbits, const uint64_t *lane_rank, uint32_t k, uint32_t *len,
-                                uint64_t *X, const BuildScratch &b, DevCtl *ctl, cudaStream_t s) {
+                                const uint64_t *hvals, const uint32_t *pair, uint32_t l, int own, uint32_t lbits,
+                                const uint64_t *lane_rank, uint32_t k, uint32_t *len, uint64_t *X,
+                                const BuildScratch &b, DevCtl *ctl, cudaStream_t s) {
     if (R == 0) return cudaSuccess;
     note_launch();
     k_append_words<<<grid_for(R, 128), 128, 0, s>>>(rec, rec_val, R, tbits, hvals, pair, l, own, lbits,

@@ -424,7 +424,8 @@ int run_traversal(skim_ctx *c, TravArgs &a, bool forward, uint64_t *R_out, const
                 CK(c, launch_rev_ring(a, rs->lane_pair, rs->B, c->l, rs->covered, rs->alive, rs->leaf, first,
                                       c->grid_ring, c->st));
             else
-                CK(c, launch_traverse(a, forward, forward ? c->grid_fwd : c->mat ? c->grid_rev : c->grid_coin[a.many], c->st));
+                CK(c, launch_traverse(a, forward, forward ? c->grid_fwd : c->mat ? c->grid_rev : c->grid_coin[a.many],
+                                      c->st));
         }
         if (rs && rs->leaf) {
             KTimer kt(c, SKIM_K_SOURCES);
@@ -514,8 +515,8 @@ int node_buffers(skim_ctx *c) {
 }
 
 // Reverse search of the batch of ranks [p0, p0+B).  mode_build: Algorithm 2 with
-// coins drawn in the searches
-// (pruned by local counts; not in the IC model); otherwise SKIM (covered sources skipped).
+// coins drawn in the searches (pruned by local counts; not in the IC model);
+// otherwise SKIM (covered sources skipped).
 // est_per_lane: expected visit records per lane (0 or negative = unknown, or
 // a re-run after an overflow: the whole table).  The visited table used is a
 // power of two of about 4 slots per expected record, zeroed before the batch
@@ -718,8 +719,8 @@ uint32_t default_lanes(skim_ctx *c) {
 uint32_t skim_lanes(skim_ctx *c) {
     if (c->batch_cfg || !c->mat) return default_lanes(c);
     const double sparse = std::max(0.0, c->k - 2.0 * std::sqrt(static_cast<double>(c->k))) * c->n;
-    const uint64_t most =
-        std::max<uint64_t>(default_lanes(c), static_cast<uint64_t>(std::max(0.0, sparse - static_cast<double>(c->cursor))));
+    const double left = std::max(0.0, sparse - static_cast<double>(c->cursor));
+    const uint64_t most = std::max<uint64_t>(default_lanes(c), static_cast<uint64_t>(left));
     return static_cast<uint32_t>(std::min<uint64_t>({1ull << 24, most, c->lane_cap}));
 }
 
@@ -776,10 +777,9 @@ int ensure_idx(skim_ctx *c, uint64_t need) {
 
 // Finish the pending residual search, after a read of the control block that
 // followed it.  A search that parked work (its queue overflowed) resumes until
-// the queue drains, and
-// *again tells the caller that what it read back (stop candidate, argmax) was
-// computed before the search had finished.  Then the search's count of newly
-// covered pairs goes out and the queue is emptied.
+// the queue drains, and *again tells the caller that what it read back (stop
+// candidate, argmax) was computed before the search had finished.  Then the
+// search's count of newly covered pairs goes out and the queue is emptied.
 int finish_residual(skim_ctx *c, bool *again) {
     *again = false;
     if (!c->pend_res) return SKIM_OK;
@@ -908,8 +908,9 @@ int drop_batch(skim_ctx *c) {
 constexpr uint64_t kDropRecords = 1 << 20;
 constexpr uint32_t kDropStops = 16, kDropLeft = 64;
 bool too_large(const skim_ctx *c) {
-    return c->batch_active && c->bR >= kDropRecords && c->bstops > kDropStops &&
-           static_cast<uint64_t>(c->bB - c->blo) * (c->bstops - 1) > static_cast<uint64_t>(c->blo - c->bfirst) * kDropLeft;
+    if (!c->batch_active || c->bR < kDropRecords || c->bstops <= kDropStops) return false;
+    const uint64_t left = c->bB - c->blo, used = c->blo - c->bfirst;
+    return left * (c->bstops - 1) > used * kDropLeft;
 }
 
 int next_seed(skim_ctx *c, uint32_t *x_out, uint64_t *cov_out) {
@@ -1188,9 +1189,11 @@ int skim_destroy(skim_ctx *c) {
     dfree(c, c->rkey); dfree(c, c->rkey2); dfree(c, c->rval); dfree(c, c->rval2);
     dfree(c, c->ncnt); dfree(c, c->noff); dfree(c, c->nlist); dfree(c, c->nlist_cnt);
     dfree(c, c->ws);
-    dfree(c, c->lane_inst); dfree(c, c->lane_g); dfree(c, c->alive); dfree(c, c->leaf); dfree(c, c->lane_off); dfree(c, c->lane_fill);
+    dfree(c, c->lane_inst); dfree(c, c->lane_g); dfree(c, c->alive); dfree(c, c->leaf);
+    dfree(c, c->lane_off); dfree(c, c->lane_fill);
     dfree(c, c->nonempty); dfree(c, c->need); dfree(c, c->comp); dfree(c, c->comp_up);
-    dfree(c, c->over_seg); dfree(c, c->over_buf); dfree(c, c->full_list); dfree(c, c->hitbits); dfree(c, c->defbits); dfree(c, c->defpair);
+    dfree(c, c->over_seg); dfree(c, c->over_buf); dfree(c, c->full_list);
+    dfree(c, c->hitbits); dfree(c, c->defbits); dfree(c, c->defpair);
     dfree(c, c->node_off); dfree(c, c->comp_ws); dfree(c, c->need_ws);
     dfree(c, c->lcnt); dfree(c, c->full); dfree(c, c->X); dfree(c, c->xlen);
     dfree(c, c->covered); dfree(c, c->seg_start); dfree(c, c->pend_trav); dfree(c, c->pend_erase);
@@ -1796,7 +1799,8 @@ int search_deferred(skim_ctx *c, uint64_t p0, uint32_t D, uint64_t R0, const Bui
     for (bool whole = *vpl <= 0;; whole = true) {
         uint64_t want = c->hcap;
         if (!whole)
-            want = static_cast<uint64_t>(std::min(std::max(65536.0, kTableSlots * *vpl * D), static_cast<double>(c->hcap)));
+            want = static_cast<uint64_t>(
+                std::min(std::max(65536.0, kTableSlots * *vpl * D), static_cast<double>(c->hcap)));
         a.hmask = pow2_at_least(std::min(want, c->hcap)) - 1;  // (hcap is a power of two)
         CK(c, clear_table(c, a.hmask + 1));
         CK(c, cudaMemsetAsync(&c->ctl->src_next, 0, 3 * sizeof(HotCounter), c->st));  // src_next, busy, beat
@@ -2012,7 +2016,8 @@ int build_rows(skim_ctx *c) {
         // (visits per lane as measured, unless a component has just been contracted)
         per = static_cast<double>(std::max<uint64_t>(v2 - v0, 1)) / b;
         uint64_t next = kRowsGrowth * static_cast<uint64_t>(b);
-        if (per >= kRowsDirectVisits && !(giant && p0 == b)) next = std::max(next, static_cast<uint64_t>(kRowsCheap / per));
+        if (per >= kRowsDirectVisits && !(giant && p0 == b))
+            next = std::max(next, static_cast<uint64_t>(kRowsCheap / per));
         // Where a record per visit would keep the next batch small, and the last one had
         // several visits per table entry, it has a record per entry as well, and of those
         // at most n for every 64 lanes.  (Not behind a contraction if an instance need not

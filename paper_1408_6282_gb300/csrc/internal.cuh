@@ -188,11 +188,12 @@ struct ReachArgs {
 };
 constexpr uint32_t kSeedOfStep = 0xffffffffu;  // as x: the seed in ctl->step.best, nothing if there is none
 cudaError_t launch_reach(const ReachArgs &a, uint32_t x, cudaStream_t s);
-// What the nodes pivot[64 * q + i], q < starts, reach in instance i, for every
-// instance: its bit in mask
-// (zero before), the number of nodes to count[i].  A walk that does not fit the
-// scratch sets its bit in BuildCtl::reach_fail.  Uses off, rows, l, mask, list,
-// cap, ctl and timeout_ns of a.
+// What the nodes pivot[64 * q + i], q < starts, reach in instance i along off and
+// rows, for every instance: its bit in mask (zero before), the number of nodes to count[i];
+// and what reaches them, along back_off and back_rows to back_mask and count[64 + i].
+// Rows that do not fit the scratch are parked in pend_trav and back_pend (zero before
+// and after) and taken up when the walk runs dry.  Uses l, n, list, cap, ctl and
+// timeout_ns of a too.
 cudaError_t launch_reach_from(const ReachArgs &a, const uint32_t *pivot, uint32_t starts, uint32_t *count,
                               cudaStream_t s);
 
@@ -244,15 +245,17 @@ cudaError_t launch_deferred_lanes(uint32_t *deflist, uint32_t D, bool all, const
 cudaError_t launch_append(const uint64_t *rec, uint64_t r0, uint64_t r1, uint32_t lbits, const uint32_t *defbits,
                           const uint64_t *lane_rank, uint32_t k, uint32_t *len, uint64_t *X, const BuildScratch &b,
                           DevCtl *ctl, cudaStream_t s);
-// records node << tbits | word of a search of all lanes of a batch (slots
-// rec_val, lane bits hvals): the ranks of each one's lanes, without the node's
-// own unless `own`
-// Lanes of every kWordChunk of R such records, to cnt.
+// lanes of every kWordChunk of R records node << tbits | word (slots rec_val, lane bits
+// hvals), to cnt
 constexpr uint32_t kWordChunk = 1024;
-cudaError_t launch_count_words(const uint32_t *rec_val, uint64_t R, const uint64_t *hvals, uint32_t *cnt, cudaStream_t s);
+cudaError_t launch_count_words(const uint32_t *rec_val, uint64_t R, const uint64_t *hvals, uint32_t *cnt,
+                               cudaStream_t s);
+// such records of a search of all lanes of a batch: the ranks of each one's lanes,
+// without the node's own unless `own`
 cudaError_t launch_append_words(const uint64_t *rec, const uint32_t *rec_val, uint64_t R, uint32_t tbits,
-                                const uint64_t *hvals, const uint32_t *pair, uint32_t l, int own, uint32_t lbits, const uint64_t *lane_rank, uint32_t k, uint32_t *len,
-                                uint64_t *X, const BuildScratch &b, DevCtl *ctl, cudaStream_t s);
+                                const uint64_t *hvals, const uint32_t *pair, uint32_t l, int own, uint32_t lbits,
+                                const uint64_t *lane_rank, uint32_t k, uint32_t *len, uint64_t *X,
+                                const BuildScratch &b, DevCtl *ctl, cudaStream_t s);
 // rows that received more than k ranks keep the k smallest (R: records appended;
 // done: and are full)
 cudaError_t launch_overflow(uint64_t R, uint32_t lbits, const uint64_t *lane_rank, uint32_t k, uint32_t *len,
@@ -334,8 +337,9 @@ struct QueryScratch {
     uint64_t table_slots;
     bool clusters;          // may be launched (else every larger query is taken in parts)
 };
-uint32_t query_blocks(uint64_t seeds, uint32_t k, bool alone);  // parts of a larger query, 0 for a small one and for the largest
-uint64_t query_table_slots(uint64_t seeds, uint32_t k, bool alone);  // of the largest ones' table in global memory, else 0
+// alone: the only query of its call
+uint32_t query_blocks(uint64_t seeds, uint32_t k, bool alone);  // parts of a larger query, 0 for a small or largest one
+uint64_t query_table_slots(uint64_t seeds, uint32_t k, bool alone);  // of a largest one's table in memory, else 0
 uint32_t query_partials(uint32_t blocks, uint64_t table_slots);  // places of `partial`
 size_t query_partial_bytes();
 // How a threshold becomes a term of Eq. unionest, and the final divisor:

@@ -170,7 +170,8 @@ constexpr uint32_t kPartEntries = 8000, kPartSlots = 12287;  // 192 KB
 constexpr int kPartThreads = 1024;
 constexpr uint32_t kStage = 64;  // pairs a warp collects
 constexpr uint32_t kOneEntries = 1500;
-constexpr uint32_t kCluster = 16, kClusterSlots = kPartSlots, kBlockEntries = 7800, kClusterEntries = kCluster * kBlockEntries;
+constexpr uint32_t kCluster = 16, kClusterSlots = kPartSlots, kBlockEntries = 7800;
+constexpr uint32_t kClusterEntries = kCluster * kBlockEntries;
 constexpr uint32_t kClusterFour = 4;
 // larger queries of a call that take clusters of 16, the same if some do not fit four
 // blocks, and those that take clusters of 4 if all do
@@ -485,7 +486,8 @@ __global__ void __launch_bounds__(1024)
                     const __grid_constant__ SeedArgs<CAP> a, uint32_t H, double *out) {
     extern __shared__ ulonglong2 s_tab[];
     bool full;
-    const U192 e = query_cluster<kCluster>(X, xlen, n, k, terms, a.seeds, a.s, 0, 1, 1, reinterpret_cast<uint64_t *>(s_tab), H, nullptr, &full);
+    const U192 e = query_cluster<kCluster>(X, xlen, n, k, terms, a.seeds, a.s, 0, 1, 1,
+                                           reinterpret_cast<uint64_t *>(s_tab), H, nullptr, &full);
     if (blockIdx.x == 0 && threadIdx.x == 0) *out = full ? -1.0 : fixed_to_double(e) / terms.div;
 }
 
@@ -573,8 +575,8 @@ __global__ void __launch_bounds__(kPartThreads) k_q_part(const uint64_t *X, cons
     const uint32_t c = blockIdx.x;
     const uint32_t qi = upper_bound_u64(block_off + 1, q, c);
     const uint64_t first = block_off[qi], end = block_off[qi + 1], s0 = offsets[qi];
-    const U192 e = query_block<true, LONG>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(offsets[qi + 1] - s0), c - first,
-                               end - first, reinterpret_cast<uint64_t *>(s_tab), kPartSlots, err);
+    const uint32_t s = static_cast<uint32_t>(offsets[qi + 1] - s0);
+    const U192 e = query_block<true, LONG>(X, xlen, n, k, terms, seeds + s0, s, c - first, end - first, reinterpret_cast<uint64_t *>(s_tab), kPartSlots, err);
     add_parts(e, c, first, end, partial, &done[qi], &out[qi], terms.div);
 }
 
@@ -601,7 +603,8 @@ __global__ void __launch_bounds__(kPartThreads) k_q_few(const uint64_t *X, const
         if (threadIdx.x == 0) out[qi] = fixed_to_double(e) / terms.div;
         return;
     }
-    const uint64_t room = static_cast<uint64_t>(CL * (CL == kCluster ? kBlockFill : kBlockEntries)) * ways, cut = (entries + room - 1) / room;
+    const uint64_t room = static_cast<uint64_t>(CL * (CL == kCluster ? kBlockFill : kBlockEntries)) * ways;
+    const uint64_t cut = (entries + room - 1) / room;
     bool bad;
     const U192 e = query_cluster<CL>(X, xlen, n, k, terms, seeds + s0, static_cast<uint32_t>(s), c % ways, ways, cut, tab,
                                  cluster_slots<CL>(entries / (ways * cut)), err, &bad);
@@ -713,7 +716,8 @@ cudaError_t one_launch(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint
 
 cudaError_t launch_query_one(const uint64_t *X, const uint32_t *xlen, uint32_t n, uint32_t k, const QueryTerms &terms,
                              const uint32_t *seeds, uint32_t s, double *out_host, bool clusters, cudaStream_t st) {
-    if (s <= 60 && s * (k - 1) <= kOneEntries) return one_launch<60>(X, xlen, n, k, terms, seeds, s, out_host, clusters, st);
+    if (s <= 60 && s * (k - 1) <= kOneEntries)
+        return one_launch<60>(X, xlen, n, k, terms, seeds, s, out_host, clusters, st);
     return s <= 960 ? one_launch<960>(X, xlen, n, k, terms, seeds, s, out_host, clusters, st)
                     : one_launch<kQueryArgSeeds>(X, xlen, n, k, terms, seeds, s, out_host, clusters, st);
 }
@@ -757,7 +761,8 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
     if (e == cudaSuccess && f.n_large && f.n_large <= (fits_four ? kMoreLarge : kFewLargest)) {
         const bool few = f.n_large <= kFewLarge || !fits_four;
         const uint32_t cl = few ? kCluster : kClusterFour;
-        f.ways = few ? std::max(1u, std::min(kClusterParts / f.n_large, (blocks * kPartEntries - 1) / kClusterEntries + 1)) : 1;
+        const uint32_t wanted = (blocks * kPartEntries - 1) / kClusterEntries + 1;
+        f.ways = few ? std::max(1u, std::min(kClusterParts / f.n_large, wanted)) : 1;
         const uint32_t small = q - f.n_large - tables;
         const uint32_t with_small = f.n_large * f.ways + (q + cl - 1) / cl;
         const bool together = small == 0 || (small <= kFewSmall && (!few || with_small <= kFewClusters));
@@ -777,7 +782,7 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
         if (e != cudaSuccess) return e;
         note_launch();
         kernel<<<blocks, kPartThreads, smem, s>>>(X, xlen, n, k, terms, seeds, offsets, block_off, q, partial, qs.done,
-                                                    out, qs.err);
+                                                  out, qs.err);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && q > tables) {

@@ -2,9 +2,10 @@
 // batching (queries of Section 5.1, Eq. unionest, over resident sketches).
 //
 // Requests are seed sets submitted from any host thread.  A server thread
-// admits pending requests into a launch group while in-flight slots and
-// scratch memory allow (each query needs a hash table of about 2|S|(k-1)
-// slots), copies the group's seeds to the device and launches the batched
+// admits pending requests into a launch group while in-flight slots and the
+// arena of hash-table slots allow (a query of |S| seeds counts as about
+// 2|S|(k-1); only the largest have a table there, the others theirs in shared
+// memory), copies the group's seeds to the device and launches the batched
 // query kernel on one of several streams.  Groups on different streams run
 // concurrently; when a group finishes, its slots and scratch return to the
 // pool and requests that arrived meanwhile are admitted into the next group.
