@@ -120,8 +120,8 @@ class Clocks:
 
 def traffic_record(kernel: str, workload: str):
     """DRAM bytes per launch of a kernel group on a workload, from the
-    committed ncu summaries (profiles/traffic.json), if the kernels' source
-    has not changed since they were taken."""
+    committed ncu summaries (profiles/traffic.json), if the source of the
+    kernels with most of the bytes has not changed since they were taken."""
     path = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(path):
         return None
@@ -142,8 +142,8 @@ def kernel_roofline(kname, kt, gold, m, l, steps, sm_max, hbm_peak, total_ms, wo
 
     rev_search  (memory): every candidate visit -- a batch's source lane or a
                 live in-edge walked -- reads a 4 B node or pair id, the 8 B
-                bounds of the live row of (v, i) (which carry Algorithm 2's
-                pruning flag) and reads and writes its 8 B visited word (16 B);
+                bounds of the live row of (v, i) and reads and writes its 8 B
+                visited word (16 B);
                 every expansion also writes its 12 B visit record.  Sources are
                 taken inside the search kernel, so their lanes count here.
                 (The searches skip what no node needs any more and contract

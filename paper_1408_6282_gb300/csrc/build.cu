@@ -385,9 +385,9 @@ __global__ void k_append(const uint64_t *__restrict__ rec, uint64_t r0, uint64_t
 // The same for records per table entry (node, lane word): a record's lanes are
 // the bits of its table slot, in rank order, so only the first k of them can
 // matter.  The node's own ranks are left out unless `own` (they are merged).
-// For a first batch, whose visits may be far more than the record table holds
-// (R-MAT 20 wc with every batch of the first 400 K lanes in this form: 14.8 ms
-// instead of 13.2, for the look at every lane's source).
+// For a first batch, whose visits may be far more than the record table holds, and for
+// dense ones behind it (R-MAT 20 wc with every batch of the first 400 K lanes in this
+// form: 14.8 ms instead of 13.2, for the look at every lane's source).
 __global__ void k_append_words(const uint64_t *__restrict__ rec, const uint32_t *__restrict__ rec_val, uint64_t R,
                                uint32_t tbits, const uint64_t *__restrict__ hvals, const uint32_t *__restrict__ pair,
                                uint32_t l, int own, uint32_t lbits,

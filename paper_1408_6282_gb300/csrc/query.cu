@@ -144,12 +144,10 @@ SKIM_DEV double fixed_to_double(const U192 &a) {
 // 67, 75, 85, 102 us); 64 ranks, 10, 16, 32, 64 queries: parts 75, 84, 90, 95 us, clusters of 16 59, 69,
 // then parts (four launches: 76, 86, 96, 126 us).  A batch fills the chip with parts and is
 // slower with clusters (1000 queries, with copies: 0.52 ms; clusters of 4, 8, 16: 0.63,
-// 0.76, 1.07 ms).  Both
-// read a query once per part or round of clusters: where in_memory says so the
-// table is in global memory (64 ranks per sketch, 30000 seeds: 264 us, clusters
-// 555 us, parts 1100 us; 9000 seeds, clusters: 107 us).
-// One block is as fast as the cluster up to
-// kOneEntries (100 seeds of 16 ranks: 28 us both; 43 seeds of 64: 30 and 29 us).
+// 0.76, 1.07 ms).  Both read a query once per part or round of clusters, so the
+// largest have their table in global memory (in_memory; 9000 seeds of 64 ranks, clusters:
+// 107 us).  One block is as fast as the cluster up to kOneEntries (100 seeds of 16 ranks:
+// 28 us both; 43 seeds of 64: 30 and 29 us).
 
 constexpr uint32_t kSmallEntries = 2700, kSmallSlots = 4095;  // 64 KB: three blocks per SM
 // Threads of a small query's block: many while a call leaves room for them (host to host,
