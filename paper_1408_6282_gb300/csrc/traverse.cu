@@ -469,33 +469,32 @@ SKIM_DEV void emit_rev(const TravArgs &A, Acc &acc, bool act, uint32_t u, uint32
             atomicOr(&A.ctl->err, kErrHash);
         }
     }
-    // record of the (node, word) entry, written once by its creator; none for a
-    // node whose sketch is full (its ranks are lower), which is only counted
-    {
-        if (A.xlen) {
-            const bool done = first && A.xlen[u] >= A.k;
-            const unsigned db = __ballot_sync(kFull, done);
-            if ((threadIdx.x & 31) == 0 && db) atomicAdd(&A.ctl->beat.v, static_cast<unsigned long long>(__popc(db)));
-            first &= !done;
-        }
-        unsigned ball = __ballot_sync(kFull, first);
-        if (ball) {
-            unsigned long long base = 0;
-            if ((threadIdx.x & 31) == 0) base = atomicAdd(&A.ctl->rec_count.v, static_cast<unsigned long long>(__popc(ball)));
-            base = __shfl_sync(kFull, base, 0);
-            if (first) {
-                unsigned long long r = base + __popc(ball & lanemask_lt());
-                if (r < A.rcap) {
-                    A.rec_key[r] = (static_cast<uint64_t>(u) << A.tbits) | t;
-                    A.rec_val[r] = static_cast<uint32_t>(slot);
-                } else {
-                    atomicOr(&A.ctl->err, kErrRecords);
-                }
-            }
-        }
-    }
     acc.visits += __popcll(nb);
     push_rev<false>(A, acc, u, t, nb, slot);
+    // record of the (node, word) entry, written once by its creator; none for a
+    // node whose sketch is full (its ranks are lower), which is only counted.  Behind
+    // the push, for which a chain of hops waits: a cycle of 3458 nodes, IC model, k = 8,
+    // batches of 64 lanes 7.82 s with the two round trips before it, 7.36 s so.
+    if (A.xlen) {
+        const bool done = first && A.xlen[u] >= A.k;
+        const unsigned db = __ballot_sync(kFull, done);
+        if ((threadIdx.x & 31) == 0 && db) atomicAdd(&A.ctl->beat.v, static_cast<unsigned long long>(__popc(db)));
+        first &= !done;
+    }
+    const unsigned ball = __ballot_sync(kFull, first);
+    if (!ball) return;
+    unsigned long long base = 0;
+    if ((threadIdx.x & 31) == 0) base = atomicAdd(&A.ctl->rec_count.v, static_cast<unsigned long long>(__popc(ball)));
+    base = __shfl_sync(kFull, base, 0);
+    if (first) {
+        const unsigned long long r = base + __popc(ball & lanemask_lt());
+        if (r < A.rcap) {
+            A.rec_key[r] = (static_cast<uint64_t>(u) << A.tbits) | t;
+            A.rec_val[r] = static_cast<uint32_t>(slot);
+        } else {
+            atomicOr(&A.ctl->err, kErrRecords);
+        }
+    }
 }
 
 // Where a reverse search puts what it finds.  GlobalSink: visit records by
@@ -889,6 +888,8 @@ __device__ __noinline__ uint64_t coin_lanes(const TravArgs &A, uint32_t idx, uin
     return live_lanes<true>(A.he[idx], mask, tm1, A.lane_g + static_cast<size_t>(t) * 64);
 }
 
+// FEW: the search of a batch of few visits (kCoinBlocksFew).
+template <bool FEW>
 SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have, const Item &it) {
     const uint32_t lane = threadIdx.x & 31;
     Desc d = describe<false, false>(A, have, it);
@@ -949,29 +950,43 @@ SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have
             }
         }
     }
-    const uint32_t c = d.cnt < 32 ? d.cnt : 0;
+    // each lane its own edges where that takes no more steps than spreading them, as in a
+    // chain (the cycle above: 7.36 and 6.95 s)
+    const uint32_t c = d.cnt < 32 ? d.cnt : 0, total = __reduce_add_sync(kFull, c);
+    const uint32_t most = __reduce_max_sync(kFull, c), spread = (total + 31) / 32;
+    const bool own = most <= spread;
     uint32_t incl = c;
+    if (!own) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= static_cast<uint32_t>(o)) incl += y;
-    }
-    const uint32_t total = __shfl_sync(kFull, incl, 31), first = d.begin - (incl - c);
-    for (uint32_t g = 0; g < total; g += 32) {
-        const uint32_t o = g + lane;
-        uint32_t sl = 0;  // owner: the first lane whose inclusive count exceeds o
-#pragma unroll
-        for (uint32_t step = 16; step > 0; step >>= 1) {
-            const uint32_t v = __shfl_sync(kFull, incl, sl + step - 1);
-            if (v <= o) sl += step;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(kFull, incl, o);
+            if (lane >= static_cast<uint32_t>(o)) incl += y;
         }
-        const uint32_t idx = __shfl_sync(kFull, first, sl) + o, v = __shfl_sync(kFull, d.v, sl);
-        const uint32_t t = __shfl_sync(kFull, d.w, sl) >> kChunkBits;
-        const uint64_t mask = __shfl_sync(kFull, d.mask, sl), tm1 = __shfl_sync(kFull, d.tm1, sl);
-        const uint64_t g1 = __shfl_sync(kFull, d.g1, sl);
+    }
+    const uint32_t first = d.begin - (incl - c);
+    for (uint32_t s = 0; s < (own ? most : spread); s++) {
+        uint32_t idx = d.begin + s, v = d.v, t = d.w >> kChunkBits;
+        uint64_t mask = d.mask, tm1 = d.tm1, g1 = d.g1;
+        bool act = s < c;
+        if (!own) {
+            const uint32_t o = s * 32 + lane;
+            uint32_t sl = 0;  // owner: the first lane whose inclusive count exceeds o
+#pragma unroll
+            for (uint32_t step = 16; step > 0; step >>= 1) {
+                const uint32_t y = __shfl_sync(kFull, incl, sl + step - 1);
+                if (y <= o) sl += step;
+            }
+            idx = __shfl_sync(kFull, first, sl) + o;
+            v = __shfl_sync(kFull, v, sl);
+            t = __shfl_sync(kFull, t, sl);
+            mask = __shfl_sync(kFull, mask, sl);
+            tm1 = __shfl_sync(kFull, tm1, sl);
+            g1 = __shfl_sync(kFull, g1, sl);
+            act = o < total;
+        }
         uint64_t live = 0;
         uint32_t x = 0;
-        if (o < total) {
+        if (act) {
             x = A.col[idx];
             const uint64_t t1 = plain ? tm1 : coin_tm1(A, idx, v);
             live = (mask & (mask - 1)) == 0 ? (fmix_le(A.he[idx] + g1, t1) ? mask : 0) : coin_lanes(A, idx, mask, t1, t);
@@ -979,7 +994,16 @@ SKIM_DEV void coin_expand(const TravArgs &A, Acc &acc, ulonglong2 *st, bool have
         S.put(A, live, x, t);
         if (S.n >= 32) S.visit(A, acc);
     }
-    while (S.n) S.visit(A, acc);  // before the items count as done
+    // what is left, fewer than 32, before the items count as done: in a search of few
+    // visits by a copy in place, which a chain waits for less (the cycle above: 6.95 and
+    // 5.92 s; in the search of many, R-MAT 13, p = 0.1, IC model: 92 and 98 ms with it)
+    if (FEW && S.n) {
+        __syncwarp();
+        const ulonglong2 e = lane < S.n ? st[lane] : make_ulonglong2(0, 0);
+        emit_rev(A, acc, lane < S.n, static_cast<uint32_t>(e.x), static_cast<uint32_t>(e.x >> 32), e.y);
+    } else if (S.n) {
+        S.visit(A, acc);
+    }
 }
 
 // ---- items of residual searches ----------------------------------------------------
@@ -1516,7 +1540,7 @@ __global__ void __launch_bounds__(kTravThreads, BLOCKS)
                 else if constexpr (FWD)
                     fwd_expand<MAT>(A, acc, ring, have, it, ginst);
                 else
-                    coin_expand(A, acc, s_coin[threadIdx.x >> 5], have, it);
+                    coin_expand<BLOCKS == kCoinBlocksFew>(A, acc, s_coin[threadIdx.x >> 5], have, it);
                 if constexpr (kLocal) {
                     // after the items' own pushes (their reservations are made)
                     __syncwarp();

@@ -67,3 +67,32 @@ def test_batches_of_few_and_many_visits(p, mode, l):
             want = oracle.skim_stops(pb, 15, rank_mode=mode)
             for a, b in zip(sk.greedy_stops(15), want):
                 assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("items", [None, "600"])
+@pytest.mark.parametrize("mode,l,bl", [(2, 1, 0), (2, 1, 64), (0, 64, 0)])
+@pytest.mark.parametrize("degree,p", [(1, 1.0), (1, 0.99), (2, 0.6), (8, 0.2), (31, 0.05), (32, 0.05)])
+def test_rows_of_one_length(degree, p, mode, l, bl, items, monkeypatch):
+    """Every node has as many in-edges: from a chain of single edges, where each lane
+    takes its own edge, to rows that the warp sweeps; a queue that is full at once
+    (items of many lanes come back) and one that is not."""
+    import paper_1408_6282_gb300 as pkg
+    if items:
+        monkeypatch.setenv("SKIM_QUEUE_ITEMS", items)
+    n, k = 700, 33
+    v = np.repeat(np.arange(n, dtype=np.uint32), degree)
+    u = ((v + np.tile(21 * np.arange(degree, dtype=np.uint32) + 1, n)) % n).astype(np.uint32)
+    key = np.unique(u.astype(np.uint64) << np.uint64(32) | v.astype(np.uint64))
+    src, dst = (key >> np.uint64(32)).astype(np.uint32), key.astype(np.uint32)
+    src, dst = src[src != dst], dst[src != dst]
+    ks = synth.Keys.from_seed(23)
+    pb = oracle.Problem(n, src, dst, l, k, 0, p, ks.coin, ks.rank, ks.prob)
+    ox, oln, _ = oracle.build_ic_sketches(pb) if mode == 2 else oracle.build_sketches(pb, rank_mode=mode)
+    with pkg.Skim(n, src, dst, l, k, 0, p, ks.coin, ks.rank, ks.prob, batch_lanes=bl, rank_mode=mode) as sk:
+        sk.set_live_rows(False)
+        sk.build_sketches()
+        x, ln = sk.sketches()
+        assert np.array_equal(ln, oln) and np.array_equal(x, ox)
+        if mode != 2:
+            for a, b in zip(sk.greedy_stops(10), oracle.skim_stops(pb, 10, rank_mode=mode)):
+                assert np.array_equal(a, b)
