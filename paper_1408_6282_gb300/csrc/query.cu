@@ -159,11 +159,11 @@ constexpr int small_threads(uint32_t queries) {
 }
 // Small queries go in one launch with the clusters of a few larger ones, in a block of
 // 1024 threads each and one per SM, while they are few: with clusters of 4 up to
-// kFewSmall, with clusters of 16, of which kClusterParts are resident at once, up to
-// kFewClusters of them in all.  Else they take a launch of their own (as above, beside one larger query
-// 152, 304, 608, 2000 small ones: 81, 108, 174, 438 us together, 96, 111, 116, 208 us
-// apart; 152 beside 6: 97 and 89 us).
-constexpr uint32_t kFewSmall = 2 * kSmsUsual, kFewClusters = 14;
+// kFewSmall, with clusters of 16, of which kClusterParts are resident at once, where all
+// take one round more at most.  Else they take a launch of their own (as above, beside one
+// larger query 152, 304, 608, 2000 small ones: 81, 108, 174, 438 us together, 96, 111, 116, 208 us
+// apart; beside 7 150, 250 132, 158 and 127, 139 us, beside 10 60, 150 113, 135 and 139, 148).
+constexpr uint32_t kFewSmall = 2 * kSmsUsual;
 constexpr uint32_t kPartEntries = 8000, kPartSlots = 12287;  // 192 KB
 constexpr int kPartThreads = 1024;
 constexpr uint32_t kStage = 64;  // pairs a warp collects
@@ -763,7 +763,9 @@ cudaError_t launch_query_multi(const uint64_t *X, const uint32_t *xlen, uint32_t
         f.ways = few ? std::max(1u, std::min(kClusterParts / f.n_large, wanted)) : 1;
         const uint32_t small = q - f.n_large - tables;
         const uint32_t with_small = f.n_large * f.ways + (q + cl - 1) / cl;
-        const bool together = small == 0 || (small <= kFewSmall && (!few || with_small <= kFewClusters));
+        const auto rounds = [](uint32_t n) { return (n + kClusterParts - 1) / kClusterParts; };
+        const bool together =
+            small == 0 || (small <= kFewSmall && (!few || rounds(with_small) <= rounds(f.n_large * f.ways) + 1));
         const uint32_t clusters = small && together ? with_small : f.n_large * f.ways;
         const cudaError_t ce =
             few ? cluster_launch<kCluster>(qs.clusters, k_q_few<kCluster>, clusters, kClusterSlots, s, X, xlen, n, k,

@@ -29,3 +29,20 @@ def test_large_queries(k, seeds):
         assert sk.query(s) == a
         ref = oracle.union_estimate(x, ln, l, s)
         assert abs(a - ref) <= 1e-12 * ref
+
+
+@pytest.mark.parametrize("large", [1, 7, 13, 16])
+@pytest.mark.parametrize("small", [4, 14, 100, 150, 300])
+def test_small_queries_beside_large_ones(large, small):
+    """In one launch with the clusters of 16 and in one of their own: the same bits as alone."""
+    import paper_1408_6282_gb300 as pkg
+    g = synth.erdos_renyi(5003, 20000, 62)
+    ks = synth.Keys.from_seed(62)
+    l, k, p = 40, 64, 0.3
+    rng = np.random.default_rng(100 * large + small)
+    sets = [rng.choice(g.n, s, replace=False).astype(np.uint32)
+            for s in [600] + list(rng.integers(44, 1000, large - 1)) + list(rng.integers(0, 43, small))]
+    sets = [sets[i] for i in rng.permutation(len(sets))]
+    with pkg.Skim(g.n, g.src, g.dst, l, k, 0, p, ks.coin, ks.rank, ks.prob) as sk:
+        sk.build_sketches()
+        assert np.array_equal(sk.query_batch(sets), [sk.query(s) for s in sets])

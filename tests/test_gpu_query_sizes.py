@@ -78,7 +78,7 @@ def test_without_clusters(monkeypatch, k):
 
 
 @pytest.mark.parametrize("large,small,launches", [(0, 152, 1), (0, 153, 1), (0, 456, 1), (0, 457, 1), (1, 207, 1),
-                                                  (1, 208, 2), (8, 88, 1), (8, 89, 2), (20, 304, 1), (20, 305, 2),
+                                                  (1, 208, 2), (8, 200, 1), (8, 201, 2), (20, 304, 1), (20, 305, 2),
                                                   (70, 300, 2), (1, 5000, 2)])
 def test_calls_with_many_small_queries(large, small, launches):
     """Blocks of 1024, 512 and 256 threads for small queries; beside larger ones in their
